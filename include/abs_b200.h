@@ -235,9 +235,10 @@ ABS_API float abs_alpha_from_amax(abs_fmt_t fmt, float amax);
  * unit (Sec. 5.2): the decoded codes of a pair of groups are multiplied and summed exactly, the sum is scaled by
  * Delta_a * Delta_b, and the FP32 factor 1, 6/7 or 36/49 is applied on the scale path when none, one or both of
  * the groups are stored as integers; alpha_a * alpha_b multiplies the result.  FP groups are NVFP4 groups (Sec. 3)
- * and go to the block-scaled FP4 MMA (tcgen05.mma kind::mxf4nvf4) unchanged; an integer code k in -7..7 is the sum
- * of two E2M1 values (5 = 4 + 1, 7 = 6 + 1), so each operand is first split into three NVFP4 planes in the
- * workspace and the three kinds of group pairs accumulate in three FP32 accumulators that meet in the epilogue.
+ * and go to the block-scaled FP4 MMA (tcgen05.mma kind::mxf4nvf4) unchanged; the 6/7 k that an integer code k stands
+ * for is h + l / 7 with two E2M1 values (1 - 1/7, 4 + 2/7, ...), so each operand is first split into two NVFP4 planes in
+ * the workspace and the products h h, h l + l h and l l accumulate in three FP32 accumulators that meet, with the factors
+ * 1, 1/7 and 1/49, in the epilogue.
  *   fmt                ABS_FMT_IF4 or ABS_FMT_NVFP4 (both operands)
  *   a_codes, a_scales  A as abs_quantize wrote it: [m, k] quantized along k, scales row-major [m, k/16]; a_alpha its alpha
  *   b_codes, b_scales  B likewise: [n, k]

@@ -4,23 +4,26 @@
 // groups stored as integers -- are applied in FP32 on the scale path, here in the epilogue.
 //
 // How integer groups reach an FP4 tensor core.  An FP4 group is an NVFP4 group (Sec. 3) and goes to
-// tcgen05.mma kind::mxf4nvf4 as it is.  An integer code k in -7..7 is not an E2M1 value, but it is the sum of
-// two: k = h + l with h in {0, 1, 2, 3, 4, 6} and l in {0, 1} (5 = 4 + 1, 7 = 6 + 1), signs equal.  So every
-// operand is split once into three NVFP4 "planes" that share the group scales:
-//     F: the codes of the FP groups (integer groups zero)     H, L: the two parts of the integer groups
-// and the product is  F_a F_b  +  6/7 (F_a (H_b + L_b) + (H_a + L_a) F_b)  +  36/49 (H_a + L_a)(H_b + L_b),
-// nine block-scaled MMAs per K-step into three FP32 accumulators that live in tensor memory side by side
-// (3 x 128 columns) and meet only in the epilogue.  Every product and partial sum is exact in the tensor core's
-// FP32 accumulation up to its rounding of the running sum, which is what the float64 reference is compared to.
+// tcgen05.mma kind::mxf4nvf4 as it is.  An integer code k in -8..7 stands for (6/7) k, which is no E2M1 value, but it is
+// h + l / 7 with two of them: for |k| = 1, 2, 3, 4, 6 take h = k, l = -k (k - k/7 = 6k/7); for 5, 7 and 8 take
+// (4, 2), (6, 0) and (6, 6).  So every operand is split once into two NVFP4 "planes" that share the group scales:
+//     H: the codes of the FP groups, h of the integer groups     L: zero in the FP groups, l of the integer groups
+// and the product is  H_a H_b  +  1/7 (H_a L_b + L_a H_b)  +  1/49 L_a L_b,  four block-scaled MMAs per K-step (an earlier
+// split of k itself into two summands, beside a plane of the FP groups, took nine) into three FP32 accumulators that live
+// in tensor memory side by side (3 x 128 columns) and meet only in the epilogue.  Every product and partial sum is exact
+// in the tensor core's FP32 accumulation up to its rounding of the running sum, which is what the float64 reference is
+// compared to; |l / 7| is at most a sixth of |h|, so what the two small accumulators round hardly reaches the result.
 //
-// Kernel: persistent, one block of ten warps per SM over the 128 x 128 tiles of C.  One thread feeds the pipeline with
-// TMA (cp.async.bulk.tensor.2d, 128-byte swizzle, each load for this CTA alone) and runs ahead into the next tile, one
-// thread issues the MMAs, four warps write the scales of every K-step into tensor memory (tcgen05.st), four warps read
-// the accumulators back (tcgen05.ld) and write C.  Every mbarrier wait is bounded in time: when a wait runs out the
-// block raises an error word, stops issuing, frees its tensor memory and returns.
+// Kernel: persistent, one block per SM over the 128 x 128 tiles of C.  One thread feeds the pipeline with TMA
+// (cp.async.bulk.tensor.2d, 128-byte swizzle, each load for this CTA alone) and runs ahead into the next tile, one
+// thread issues the MMAs, four warps write the scales of every K-step into tensor memory (tcgen05.st), four (NVFP4) or
+// eight (IF4) warps read the accumulators back (tcgen05.ld) and write C.  Every mbarrier wait is bounded in time: when a
+// wait runs out the block raises an error word, stops issuing, frees its tensor memory and returns.
 //
-// What bounds it: the rate at which the one MMA stream of a CTA completes -- about 87 cycles per 128 x 128 x 64
-// block-scaled MMA against the 64 the tensor pipe counts as active; the loads hide completely under it.
+// What bounds it: the feed of the operands from the L2, about 40 bytes per cycle and SM with one tile per block (both
+// formats spend some 1650 cycles on a stage of 64 KiB, of which the tensor pipe is active in 1024 for IF4 and in 512 for
+// NVFP4).  4096^3, operands and split included: IF4 195 -> 118 us (nine MMAs per K-block to four), 8192 x 14336 x 4096
+// 1440 -> 785 us; NVFP4 46 and 340 us.
 #include "../../include/abs_b200.h"
 #include "abs_device.cuh"
 
@@ -36,41 +39,53 @@ constexpr int kStageK = 256;                       // elements of K of one TMA b
 constexpr int kMmaK = 64;                          // K of one tcgen05.mma kind::mxf4nvf4
 constexpr int kPlaneBytes = kTileM * kStageK / 2;  // 16 KiB: one box (128 rows x 128 bytes) of one plane of one operand
 // A pipeline stage (one K-step) holds KBOXES boxes of each of the PLANES planes of A and of B (the scales do not pass
-// through shared memory).  IF4 (three planes, one box: K = 256, 96 KiB) has room for two stages.  Plain NVFP4 issues one
-// MMA per K-block, so the hand-overs of a step weigh more: its steps are two boxes long where K allows (K = 512, 64 KiB,
-// three stages), else one box (32 KiB, six stages).
+// through shared memory).  IF4 (two planes, one box: K = 256, 64 KiB) has three stages.  Plain NVFP4 issues one MMA per
+// K-block, so the hand-overs of a step weigh more: its steps are two boxes long where K allows (K = 512, 64 KiB, three
+// stages), else one box (32 KiB, six stages).
 template <int PLANES, int KBOXES> constexpr int kStageBytes = 2 * PLANES * KBOXES * kPlaneBytes;
-template <int PLANES, int KBOXES> constexpr int kStages = PLANES == 3 ? 2 : (KBOXES == 2 ? 3 : 6);
-// Epilogue staging: each of the four epilogue warps turns its 32 rows x 32 columns of a chunk through shared memory
-// (rows 36 floats apart: 16-byte aligned and free of bank conflicts for 128-bit accesses both ways).
+template <int PLANES, int KBOXES> constexpr int kStages = PLANES * KBOXES == 2 ? 3 : 6;
+// Epilogue warps: IF4, whose accumulators fill the tensor memory, takes eight, two per quarter of the accumulator lanes,
+// that have everything in registers before they store (the MMAs of the next tile wait only for that); NVFP4 has two sets
+// of accumulators and streams each through four warps.  Staging: a warp turns 16 rows x 128 bytes (IF4) or 32 rows x 128
+// bytes (NVFP4) of output at a time through shared memory, rows 144 bytes apart: 16-byte aligned and free of bank
+// conflicts for 128-bit accesses both ways.
+template <int PLANES> constexpr int kEpiWarps = PLANES == 2 ? 8 : 4;
+template <int PLANES> constexpr int kGemmThreads = 32 * (2 + kEpiWarps<PLANES> + 4);
 constexpr int kStagePitch = 36, kStagingBytes = 4 * 32 * kStagePitch * 4;
 template <int PLANES, int KBOXES> constexpr int kGemmSmemBytes =
     kStages<PLANES, KBOXES> * kStageBytes<PLANES, KBOXES> + 1024 /* alignment slack */ + 512 /* barriers */ + kStagingBytes;
+// The accumulators of a tile are summed in the tensor core over at most kChunkK of K; the epilogue adds the chunks in
+// registers.  The rounding error of one long chain grows with the square root of its steps: 8192 x 4096 x 14336, IF4,
+// 2-norm against float64: 1.3e-7 in one chain, 7.8e-8 in four (1.2e-7 with the nine-MMA split).  A hand-over costs what it
+// costs at the end of a tile, once per 4096 of K.
+constexpr int kChunkK = 4096;
 constexpr uint64_t kWaitLimitNs = 1000000000ull;   // one second: how long an mbarrier wait polls before the block gives up
 
 // ----------------------------------------------------------------------------- operand split
 
 // Splits eight integer codes (two's complement nibbles of one word) into the planes H and L, all nibbles at once:
-// sign s, magnitude m = |k|; H = s | e2m1(h), L = s | e2m1(l) with m = h + l, h in {0, 1, 2, 3, 4, 6} and l = 1 for
-// m = 5 or 7, l = 2 for m = 8 (the most negative code, which no quantizer writes but dequantize reads as -8), else
-// 0.  E2M1 codes of the integers 0, 1, 2, 3, 4, 6 are 0, 2, 4, 5, 6, 7.  No step carries from one nibble into the next.
+// sign s, magnitude m = |k|; h = m without bit 0 where m = 5 or 7 and 6 where m = 8 (the most negative code, which no
+// quantizer writes but dequantize reads as -8); l = -h, except 2 for m = 5, 0 for m = 7 and 6 for m = 8.  E2M1 codes of
+// the integers 0, 1, 2, 3, 4, 6 are 0, 2, 4, 5, 6, 7.  No step carries from one nibble into the next.
 __device__ __forceinline__ void split_int_word(uint32_t w, uint32_t& h, uint32_t& l) {
     constexpr uint32_t kOnes = 0x11111111u;
     const uint32_t s = w & 0x88888888u, neg = s >> 3;
     const uint32_t m = (w ^ (neg * 15u)) + neg;                      // |k| per nibble, 0 .. 8
-    const uint32_t l1 = (m >> 2) & m & kOnes;                         // m = 5 or 7
-    const uint32_t l2 = (m >> 3) & kOnes;                             // m = 8
-    const uint32_t mh = m - (l1 | (l2 << 1));                         // 0, 1, 2, 3, 4, 6
+    const uint32_t odd = (m >> 2) & m & kOnes;                        // m = 5 or 7
+    const uint32_t is8 = (m >> 3) & kOnes;                            // m = 8
+    const uint32_t mh = m - (odd | (is8 << 1));                       // h: 0, 1, 2, 3, 4, 6
     const uint32_t c0 = mh & kOnes, c1 = (mh >> 1) & kOnes, c2 = (mh >> 2) & kOnes;
-    h = s | ((c2 | c1) << 2) | ((c2 | (c0 & ~c1)) << 1) | (c1 & (c0 | c2));
-    l = (((l1 | l2) << 3) & s) | (l1 << 1) | (l2 << 2);
+    const uint32_t mag = ((c2 | c1) << 2) | ((c2 | (c0 & ~c1)) << 1) | (c1 & (c0 | c2));
+    const uint32_t is5 = odd & ~(m >> 1), is7 = odd & (m >> 1);
+    h = s | mag;
+    l = (s ^ (0x88888888u & ~((is5 | is8) << 3))) | (mag & ~((is5 << 1) | (is7 * 7u)));
 }
 
 // One operand of the product as the split kernel sees it.
 struct SplitOperand {
     const uint4* codes;            // [rows, k / 2] bytes as abs_quantize wrote them
     const uint8_t* scales;         // [rows, k / 16] row-major
-    uint4 *plane_f, *plane_h, *plane_l;
+    uint4 *plane_h, *plane_l;
     uint8_t* sf_tiled;             // magnitudes of the scales in the 128x4-tile layout
     int64_t rows;
     int64_t pairs;                 // rows * k / 32: pairs of groups (16 bytes of codes)
@@ -79,10 +94,10 @@ struct SplitOperand {
 };
 
 // Prepares both operands in one launch.  Code items (IF4 only; an NVFP4 operand is read by the product kernel where
-// it lies): 32 codes = two groups -> 16 bytes of each of the planes F, H, L.  Scale items: thread i of a warp reads 16
+// it lies): 32 codes = two groups -> 16 bytes of each of the planes H and L.  Scale items: thread i of a warp reads 16
 // scale bytes of each of the rows i, i + 32, i + 64, i + 96 of a 128-row block and writes, for each of four
 // consecutive 128x4 tiles, the 16 bytes that tile keeps for those four rows.  Also clears the error word.
-__global__ void __launch_bounds__(256) if4_split_kernel(const SplitOperand a, const SplitOperand b, bool has_int,
+__global__ void __launch_bounds__(256, 8) if4_split_kernel(const SplitOperand a, const SplitOperand b, bool has_int,
                                                         int* __restrict__ error) {
     pdl_launch_dependents();
     pdl_wait();
@@ -94,10 +109,9 @@ __global__ void __launch_bounds__(256) if4_split_kernel(const SplitOperand a, co
         const int64_t p = i < a.pairs ? i : i - a.pairs;
         const uint4 c = __ldg(o.codes + p);
         const uint32_t sb = __ldg(reinterpret_cast<const uint16_t*>(o.scales) + p);
-        uint4 f = c, h = make_uint4(0u, 0u, 0u, 0u), l = h;
-        if (sb & 0x80u) { f.x = 0u; f.y = 0u; split_int_word(c.x, h.x, l.x); split_int_word(c.y, h.y, l.y); }
-        if (sb & 0x8000u) { f.z = 0u; f.w = 0u; split_int_word(c.z, h.z, l.z); split_int_word(c.w, h.w, l.w); }
-        o.plane_f[p] = f;
+        uint4 h = c, l = make_uint4(0u, 0u, 0u, 0u);
+        if (sb & 0x80u) { split_int_word(c.x, h.x, l.x); split_int_word(c.y, h.y, l.y); }
+        if (sb & 0x8000u) { split_int_word(c.z, h.z, l.z); split_int_word(c.w, h.w, l.w); }
         o.plane_h[p] = h;
         o.plane_l[p] = l;
     }
@@ -206,6 +220,13 @@ __device__ __forceinline__ void tmem_load32(uint32_t addr, uint32_t (&r)[32]) {
                    "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                  : "r"(addr) : "memory");
 }
+// The same with 16 columns.
+__device__ __forceinline__ void tmem_load16(uint32_t addr, uint32_t (&r)[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(addr) : "memory");
+}
 // Two FP32 values rounded to nearest even bf16, the first in the low half.
 __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
     uint32_t r;
@@ -240,7 +261,7 @@ constexpr uint32_t kInstrDesc = (1u << 7) | (1u << 10) | ((uint32_t)(kTileN >> 3
 constexpr uint32_t kTmemCols = 512;
 
 struct GemmMaps {
-    CUtensorMap a[3], b[3];        // planes F, H, L of A [M, K/2 bytes] and B [N, K/2 bytes], boxes of 128 bytes x 128 rows
+    CUtensorMap a[2], b[2];        // planes H, L of A [M, K/2 bytes] and B [N, K/2 bytes], boxes of 128 bytes x 128 rows
 };
 
 // Tile t of the (tiles_m x tiles_n) grid of 128 x 128 tiles, walked in bands of eight tile rows, column by column
@@ -253,23 +274,25 @@ __device__ __forceinline__ void tile_of(int32_t t, int32_t tiles_m, int32_t tile
     tm = first + (in_band - tn * rows);
 }
 
-// PLANES = 3: IF4 operands (nine MMAs per K-step); PLANES = 1: plain NVFP4 (one).  error: device word set to a
+// PLANES = 2: IF4 operands (four MMAs per K-block); PLANES = 1: plain NVFP4 (one).  error: device word set to a
 // non-zero code when a wait ran out.
 //
-// Persistent: one block per SM walks the tiles blockIdx.x, blockIdx.x + gridDim.x, ...  Ten warps: warp 0 (one
-// thread) feeds the pipeline and runs ahead into the next tile while the current one is finished; warp 1 (one thread)
-// issues MMAs; warps 2-5 are the epilogue (warp w reads the 32 accumulator lanes of tensor-memory quarter w % 4);
-// warps 6-9 bring the scales: each loads the 128x4 scale tiles of a K-step from global memory into registers and
-// writes them to its quarter of tensor memory (tcgen05.st; every quarter holds the same four columns per MMA: rows
-// r, r+32, r+64, r+96 of the tile, which is the byte order of the 128x4 tile), two slots used alternately and handed
-// over through sf_full / sf_empty barriers -- a tcgen05.cp from shared memory by the MMA thread would stand in the
-// MMA queue for some 34 cycles per copy, 270 per K-step.  The accumulators pass between MMA and epilogue through
-// acc_full / acc_empty barriers; NVFP4, with one accumulator of 128 columns, alternates between two of them so that a
-// tile's epilogue overlaps the next tile's MMAs, IF4 (3 x 128 columns) has room for one set and overlaps the epilogue
-// only with the next tile's loads.
+// Persistent: one block per SM walks the tiles blockIdx.x, blockIdx.x + gridDim.x, ...  Warp 0 (one thread) feeds the
+// pipeline and runs ahead into the next tile while the current one is finished; warp 1 (one thread) issues MMAs; the next
+// kEpiWarps warps are the epilogue (warp w reads the 32 accumulator lanes of tensor-memory quarter w % 4); the last four
+// warps bring the scales: each loads the 128x4 scale tiles of a K-step from global memory into registers and writes them
+// to its quarter of tensor memory (tcgen05.st; every quarter holds the same four columns per MMA: rows r, r+32, r+64, r+96
+// of the tile, which is the byte order of the 128x4 tile), into slots handed over through sf_full / sf_empty barriers -- a
+// tcgen05.cp from shared memory by the MMA thread would stand in the MMA queue for some 34 cycles per copy.  (Scale tiles
+// brought to shared memory by bulk copies with the operands measured the same.)  The accumulators pass between MMA and
+// epilogue through acc_full / acc_empty barriers; NVFP4, with one accumulator of 128 columns, alternates between two of
+// them so that a tile's epilogue overlaps the next tile's MMAs, IF4 (3 x 128 columns) has room for one set and overlaps
+// only its stores and the next tile's loads.
+// A block stays below the registers and the shared memory that would keep a block of the next call's split kernel from
+// becoming resident beside it: without that overlap every call took 5 us longer.
 // OUT_BF16: C is written as bf16 (round to nearest even of the same FP32 value), else as FP32.
 template <int PLANES, bool OUT_BF16, int KBOXES = 1>
-__global__ void __launch_bounds__(320, 1)
+__global__ void __launch_bounds__(kGemmThreads<PLANES>, 1)
 if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict__ sfa, const uint8_t* __restrict__ sfb,
                 const float* __restrict__ alpha_a, const float* __restrict__ alpha_b, void* __restrict__ c_out, int32_t tiles_m,
                 int32_t tiles_n, int32_t k_iters, int32_t m_rows, int* __restrict__ error, int32_t stall_step,
@@ -277,14 +300,15 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
     constexpr int planes = PLANES, kStages = absq::kStages<PLANES, KBOXES>, kStageBytes = absq::kStageBytes<PLANES, KBOXES>;
     constexpr int kStepBlocks = KBOXES * (kStageK / kMmaK);          // MMA K-blocks (and scale tiles per operand) of one step
     constexpr int kAccBufs = PLANES == 1 ? 2 : 1;
+    constexpr int kEpiWarps = absq::kEpiWarps<PLANES>;
+    constexpr int kChunkSteps = PLANES == 2 ? kChunkK / kStageK : 1 << 30;    // NVFP4: the whole of K in one chain
     extern __shared__ uint8_t gemm_smem_raw[];
     const uint32_t raw = smem_u32(gemm_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;                    // 128-byte swizzle wants 1024-byte aligned tiles
-    // Scale slots in tensor memory: 32 columns each (16 of A scales, 16 of B scales).  IF4 has room for two behind its
-    // three accumulators; NVFP4, whose K-steps are only four MMAs long, takes eight behind its two accumulators so
-    // that the scale warps can run several steps ahead of the MMAs.
+    // Scale slots in tensor memory: 32 columns each (16 of A scales, 16 of B scales).  IF4 has room for four behind its
+    // three accumulators, NVFP4 for eight behind its two.
     constexpr uint32_t kSlotCols = 8u * kStepBlocks;                  // 4 columns per K-block and operand
-    constexpr uint32_t kSfSlots = PLANES == 1 ? 256u / kSlotCols : 2u, kSfBase = PLANES == 1 ? 2 * kTileN : 3 * kTileN;
+    constexpr uint32_t kSfSlots = PLANES == 1 ? 256u / kSlotCols : 4u, kSfBase = PLANES == 1 ? 2 * kTileN : 3 * kTileN;
     // barriers: full[], empty[] (stages), acc_full[2], acc_empty[2], sf_full[], sf_empty[] (slots); then the tmem address word
     const uint32_t bars = base + kStages * kStageBytes;
     uint32_t* tmem_word = reinterpret_cast<uint32_t*>(gemm_smem_raw + (bars - raw) + 320);
@@ -296,7 +320,7 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
-        for (int i = 0; i < kAccBufs; ++i) { mbar_init(acc_full0 + 8 * i, 1); mbar_init(acc_empty0 + 8 * i, 4); }
+        for (int i = 0; i < kAccBufs; ++i) { mbar_init(acc_full0 + 8 * i, 1); mbar_init(acc_empty0 + 8 * i, kEpiWarps); }
         for (int i = 0; i < (int)kSfSlots; ++i) { mbar_init(sf_full0 + 8 * i, 4); mbar_init(sf_empty0 + 8 * i, 1); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -310,7 +334,7 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
     if (warp == 0) {
         if (lane == 0) {
             // ---- producer: TMA loads of the operand planes
-            const uint32_t bytes = (uint32_t)planes * 2u * KBOXES * kPlaneBytes;
+            constexpr uint32_t bytes = kStageBytes;
             uint32_t it = 0;
             bool ok = true;
             for (int32_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
@@ -334,13 +358,14 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
     } else if (warp == 1) {
         if (lane == 0) {
             // ---- MMAs
-            uint32_t it = 0, j = 0;
+            uint32_t it = 0, j = 0;                     // K-steps and chunks so far
             bool ok = true;
-            for (int32_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++j) {
+            for (int32_t t = blockIdx.x, k0 = 0; t < num_tiles && ok; ++j) {
                 const uint32_t buf = j % kAccBufs, acc = tmem + buf * kTileN;
                 if (!mbar_wait(acc_empty0 + 8 * buf, ((j / kAccBufs) & 1u) ^ 1u)) { atomicExch(error, 4); ok = false; break; }
                 tc_fence_after();
-                for (int32_t kt = 0; kt < k_iters; ++kt, ++it) {
+                const int32_t k_end = min(k_iters - k0, kChunkSteps);
+                for (int32_t kt = 0; kt < k_end; ++kt, ++it) {
                     const uint32_t s = it % kStages;
                     const uint32_t slot = it % kSfSlots;
                     if (!mbar_wait(full0 + 8 * s, (it / kStages) & 1u)) { atomicExch(error, 2); ok = false; break; }
@@ -348,7 +373,6 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
                     tc_fence_after();
                     const uint32_t st = base + s * kStageBytes;
                     const uint32_t tsfa = tmem + kSfBase + slot * kSlotCols, tsfb = tsfa + kSlotCols / 2;
-                    // the MMAs of a step, one accumulator after the other (K order inside an accumulator is free)
                     // K-block kb of a step lies in box kb / 4 of its plane, 32 bytes per K-block inside the box's 128-byte rows
                     auto desc_a = [&](int p, int kb) {
                         return operand_desc(st + (p * KBOXES + (kb >> 2)) * kPlaneBytes + (kb & 3) * (kMmaK / 2));
@@ -356,34 +380,30 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
                     auto desc_b = [&](int p, int kb) {
                         return operand_desc(st + ((PLANES + p) * KBOXES + (kb >> 2)) * kPlaneBytes + (kb & 3) * (kMmaK / 2));
                     };
+                    if constexpr (PLANES == 1) {
 #pragma unroll
-                    for (int kb = 0; kb < kStepBlocks; ++kb)
-                        tc_mma_nvf4(acc, desc_a(0, kb), desc_b(0, kb), kInstrDesc, !(kt == 0 && kb == 0), tsfa + 4 * kb, tsfb + 4 * kb);   // F F
-                    if constexpr (PLANES == 3) {
-#pragma unroll
-                        for (int kb = 0; kb < kStepBlocks; ++kb) {
-                            const uint32_t fa = tsfa + 4 * kb, fb = tsfb + 4 * kb;
-                            tc_mma_nvf4<kFill>(acc + kTileN, desc_a(0, kb), desc_b(1, kb), kInstrDesc, !(kt == 0 && kb == 0), fa, fb);   // F H
-                            tc_mma_nvf4<kLastUse>(acc + kTileN, desc_a(0, kb), desc_b(2, kb), kInstrDesc, true, fa, fb);                 // F L
-                            tc_mma_nvf4(acc + kTileN, desc_a(1, kb), desc_b(0, kb), kInstrDesc, true, fa, fb);                           // H F
-                            tc_mma_nvf4(acc + kTileN, desc_a(2, kb), desc_b(0, kb), kInstrDesc, true, fa, fb);                           // L F
-                        }
+                        for (int kb = 0; kb < kStepBlocks; ++kb)
+                            tc_mma_nvf4(acc, desc_a(0, kb), desc_b(0, kb), kInstrDesc, !(kt == 0 && kb == 0), tsfa + 4 * kb, tsfb + 4 * kb);
+                    } else {
 #pragma unroll
                         for (int kb = 0; kb < kStepBlocks; ++kb) {
                             const uint32_t fa = tsfa + 4 * kb, fb = tsfb + 4 * kb;
-                            tc_mma_nvf4<kFill>(acc + 2 * kTileN, desc_a(1, kb), desc_b(1, kb), kInstrDesc, !(kt == 0 && kb == 0), fa, fb);  // H H
-                            tc_mma_nvf4<kLastUse>(acc + 2 * kTileN, desc_a(1, kb), desc_b(2, kb), kInstrDesc, true, fa, fb);              // H L
-                            tc_mma_nvf4<kFill>(acc + 2 * kTileN, desc_a(2, kb), desc_b(1, kb), kInstrDesc, true, fa, fb);                 // L H
-                            tc_mma_nvf4<kLastUse>(acc + 2 * kTileN, desc_a(2, kb), desc_b(2, kb), kInstrDesc, true, fa, fb);              // L L
+                            const bool go = !(kt == 0 && kb == 0);
+                            tc_mma_nvf4<kFill>(acc, desc_a(0, kb), desc_b(0, kb), kInstrDesc, go, fa, fb);                        // H H
+                            tc_mma_nvf4<kLastUse>(acc + kTileN, desc_a(0, kb), desc_b(1, kb), kInstrDesc, go, fa, fb);            // H L
+                            tc_mma_nvf4<kFill>(acc + kTileN, desc_a(1, kb), desc_b(0, kb), kInstrDesc, true, fa, fb);             // L H
+                            tc_mma_nvf4<kLastUse>(acc + 2 * kTileN, desc_a(1, kb), desc_b(1, kb), kInstrDesc, go, fa, fb);        // L L
                         }
                     }
                     tc_commit(empty0 + 8 * s);          // the stage's shared memory is free once these MMAs have run
                     tc_commit(sf_empty0 + 8 * slot);    // and so is the slot of scales
                 }
-                if (ok) tc_commit(acc_full0 + 8 * buf); // and the tile's accumulators are complete
+                if (ok) tc_commit(acc_full0 + 8 * buf); // and the chunk's accumulators are complete
+                k0 += k_end;
+                if (k0 == k_iters) { k0 = 0; t += gridDim.x; }
             }
         }
-    } else if (warp >= 6) {
+    } else if (warp >= 2 + kEpiWarps) {
         // ---- scales: this warp's copy of every K-step's scale tiles, global memory -> registers -> tensor memory
         // The loads of step it + 1 are in flight while step it waits for its slot and is written.
         const int32_t ktiles = k_iters * kStepBlocks;
@@ -436,89 +456,159 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
             }
         }
     } else {
-        // ---- epilogue: warp w owns the accumulator lanes (rows of the tile) 32 (w % 4) .. 32 (w % 4) + 31
+        // ---- epilogue
         const int quarter = warp & 3;
-        float* staging = reinterpret_cast<float*>(gemm_smem_raw + (bars - raw) + 512) + (warp - 2) * 32 * kStagePitch;
         const float scale = __fmul_rn(__ldg(alpha_a), __ldg(alpha_b));
-        const float c1 = __uint_as_float(0x3F5B6DB7u);                 // fp32(6/7)
-        const float c2 = __fdiv_rn(36.0f, 49.0f);
         uint32_t j = 0;
         uint32_t out_max = 0u;                  // bf16 output with next_alpha: largest |C| bit pattern this thread has written
         bool all_tiles = true;
-        for (int32_t t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
-            int32_t tile_m, tile_n;
-            tile_of(t, tiles_m, tiles_n, tile_m, tile_n);
-            const uint32_t buf = j % kAccBufs;
-            bool have = mbar_wait(acc_full0 + 8 * buf, (j / kAccBufs) & 1u);
-            if (!have && lane == 0) atomicExch(error, 3);
-            have = __all_sync(0xFFFFFFFFu, have);
-            if (!have) { all_tiles = false; break; }
-            tc_fence_after();
-            const bool own_row_valid = tile_m * kTileM + quarter * 32 + lane < m_rows;   // the row whose values this thread holds
-            // this thread's part of every store.  FP32: row (lane / 8) of each group of four rows, 16 bytes at column
-            // 4 (lane % 8); bf16: row (lane / 4) of each group of eight rows, 16 bytes at column 8 (lane % 4)
-            const int32_t row0 = tile_m * kTileM + quarter * 32 + (OUT_BF16 ? (lane >> 2) : (lane >> 3));
-            float* out = reinterpret_cast<float*>(c_out) + (size_t)row0 * (size_t)n_cols + (size_t)tile_n * kTileN + 4 * (lane & 7);
-            __nv_bfloat16* out16 = reinterpret_cast<__nv_bfloat16*>(c_out) + (size_t)row0 * (size_t)n_cols + (size_t)tile_n * kTileN +
-                                   8 * (lane & 3);
-            const uint32_t lane_base = tmem + buf * kTileN + ((uint32_t)(quarter * 32) << 16);
-            for (int chunk = 0; chunk < kTileN / 32; ++chunk) {
-                uint32_t r0[32], r1[32], r2[32];
-                tmem_load32(lane_base + chunk * 32, r0);
-                if (planes == 3) {
-                    tmem_load32(lane_base + kTileN + chunk * 32, r1);
-                    tmem_load32(lane_base + 2 * kTileN + chunk * 32, r2);
-                }
-                tmem_load_wait();
-                if (chunk == kTileN / 32 - 1) {         // everything is in registers: the MMAs of the next tile may start
+        if constexpr (PLANES == 2) {
+            // Two warps per quarter of tensor memory; a warp owns the accumulator lanes (rows of the tile) 32 (w % 4) ..
+            // 32 (w % 4) + 31 of one half (64) of the columns.  It takes its share into registers, hands the accumulators
+            // back, and only then stores.
+            constexpr int kCols = kTileN / 2;
+            const int col0 = ((warp - 2) >> 2) * kCols;
+            uint32_t* staging = reinterpret_cast<uint32_t*>(gemm_smem_raw + (bars - raw) + 512) + (warp - 2) * 16 * kStagePitch;
+            const float c1 = __uint_as_float(0x3E124925u), c2 = __uint_as_float(0x3CA72F05u);      // fp32(1/7), fp32(1/49)
+            for (int32_t t = blockIdx.x; t < num_tiles && all_tiles; t += gridDim.x) {
+                int32_t tile_m, tile_n;
+                tile_of(t, tiles_m, tiles_n, tile_m, tile_n);
+                const bool own_row_valid = tile_m * kTileM + quarter * 32 + lane < m_rows;   // the row whose values this thread holds
+                // this thread's part of every store: row (lane / 8) of each group of four rows, 16 bytes at byte 16 (lane % 8)
+                const int32_t row0 = tile_m * kTileM + quarter * 32 + (lane >> 3);
+                const size_t first = (size_t)row0 * (size_t)n_cols + (size_t)tile_n * kTileN + col0;
+                float v[kCols];
+                for (int32_t k0 = 0; k0 < k_iters; k0 += kChunkSteps, ++j) {
+                    const uint32_t buf = j % kAccBufs;
+                    bool have = mbar_wait(acc_full0 + 8 * buf, (j / kAccBufs) & 1u);
+                    if (!have && lane == 0) atomicExch(error, 3);
+                    have = __all_sync(0xFFFFFFFFu, have);
+                    if (!have) { all_tiles = false; break; }
+                    tc_fence_after();
+                    const uint32_t lane_base = tmem + buf * kTileN + col0 + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll
+                    for (int chunk = 0; chunk < kCols / 16; ++chunk) {
+                        uint32_t r0[16], r1[16], r2[16];
+                        tmem_load16(lane_base + chunk * 16, r0);
+                        tmem_load16(lane_base + kTileN + chunk * 16, r1);
+                        tmem_load16(lane_base + 2 * kTileN + chunk * 16, r2);
+                        tmem_load_wait();
+#pragma unroll
+                        for (int jj = 0; jj < 16; ++jj) {
+                            const float acc = __fadd_rn(__uint_as_float(r0[jj]), __fmaf_rn(c2, __uint_as_float(r2[jj]), __fmul_rn(c1, __uint_as_float(r1[jj]))));
+                            v[chunk * 16 + jj] = k0 == 0 ? acc : __fadd_rn(v[chunk * 16 + jj], acc);
+                        }
+                    }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(acc_empty0 + 8 * buf);
+                    if (lane == 0) mbar_arrive(acc_empty0 + 8 * buf);    // the MMAs of the next chunk or tile may start
                 }
-                float v[32];
+                if (!all_tiles) break;
+                // A thread holds 64 columns of ONE row; stored as they are, every store instruction of the warp would touch
+                // 32 different rows.  Through shared memory each instruction writes four rows of 128 contiguous bytes.
+                constexpr int kPart = OUT_BF16 ? 64 : 32;                 // columns of 128 bytes
 #pragma unroll
-                for (int jj = 0; jj < 32; ++jj) {
-                    float acc = __uint_as_float(r0[jj]);
-                    if (planes == 3) acc = __fmaf_rn(c2, __uint_as_float(r2[jj]), __fmaf_rn(c1, __uint_as_float(r1[jj]), acc));
-                    v[jj] = __fmul_rn(acc, scale);
-                }
-                // A thread holds 32 columns of ONE row; stored as they are, every store instruction of the warp would
-                // touch 32 different rows.  Through shared memory each instruction writes four rows of 128 contiguous bytes.
-                if constexpr (!OUT_BF16) {
+                for (int part = 0; part < kCols / kPart; ++part) {
+                    uint32_t pk[32];
 #pragma unroll
-                    for (int jj = 0; jj < 32; jj += 4)
-                        *reinterpret_cast<float4*>(staging + lane * kStagePitch + jj) = make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
-                    __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float4 x = *reinterpret_cast<const float4*>(staging + (4 * i + (lane >> 3)) * kStagePitch + 4 * (lane & 7));
-                        if (row0 + 4 * i < m_rows)                      // the last row block may be partial
-                            *reinterpret_cast<float4*>(out + (size_t)(4 * i) * n_cols + chunk * 32) = x;
+                    for (int e = 0; e < 32; ++e) {
+                        if constexpr (OUT_BF16) {
+                            pk[e] = bf16x2_bits(__fmul_rn(v[2 * e], scale), __fmul_rn(v[2 * e + 1], scale));
+                            if (next_alpha != nullptr && own_row_valid) out_max = max(out_max, max(pk[e] & 0x7FFFu, (pk[e] >> 16) & 0x7FFFu));
+                        } else {
+                            pk[e] = __float_as_uint(__fmul_rn(v[part * kPart + e], scale));
+                        }
                     }
-                } else {
-                    // 32 bf16 = 64 bytes per row, rows 20 words apart; a store instruction writes eight rows of 64 bytes
-                    uint32_t* stg = reinterpret_cast<uint32_t*>(staging);
+#pragma unroll 1
+                    for (int h = 0; h < 2; ++h) {                          // rows 16 h .. 16 h + 15 of the warp's 32
+                        if ((lane >> 4) == h) {
 #pragma unroll
-                    for (int jj = 0; jj < 32; jj += 8) {
-                        uint4 pk;
-                        pk.x = bf16x2_bits(v[jj], v[jj + 1]); pk.y = bf16x2_bits(v[jj + 2], v[jj + 3]);
-                        pk.z = bf16x2_bits(v[jj + 4], v[jj + 5]); pk.w = bf16x2_bits(v[jj + 6], v[jj + 7]);
-                        *reinterpret_cast<uint4*>(stg + lane * 20 + jj / 2) = pk;
-                        if (next_alpha != nullptr && own_row_valid) {
-                            const uint32_t w4[4] = {pk.x, pk.y, pk.z, pk.w};
+                            for (int q = 0; q < 8; ++q) *reinterpret_cast<uint4*>(staging + (lane & 15) * kStagePitch + 4 * q) = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+                        }
+                        __syncwarp();
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) out_max = max(out_max, max(w4[q] & 0x7FFFu, (w4[q] >> 16) & 0x7FFFu));
+                        for (int i = 0; i < 4; ++i) {
+                            const uint4 x = *reinterpret_cast<const uint4*>(staging + (4 * i + (lane >> 3)) * kStagePitch + 4 * (lane & 7));
+                            if (row0 + 16 * h + 4 * i < m_rows) {          // the last row block may be partial
+                                const size_t at = first + (size_t)(16 * h + 4 * i) * n_cols + part * kPart;
+                                if constexpr (OUT_BF16) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(c_out) + at + 8 * (lane & 7)) = x;
+                                else *reinterpret_cast<uint4*>(reinterpret_cast<float*>(c_out) + at + 4 * (lane & 7)) = x;
+                            }
+                        }
+                        __syncwarp();
+                    }
+                }
+            }
+        } else {
+            // A warp owns the accumulator lanes (rows of the tile) 32 (w % 4) .. 32 (w % 4) + 31.
+            float* staging = reinterpret_cast<float*>(gemm_smem_raw + (bars - raw) + 512) + (warp - 2) * 32 * kStagePitch;
+            for (int32_t t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
+                int32_t tile_m, tile_n;
+                tile_of(t, tiles_m, tiles_n, tile_m, tile_n);
+                const uint32_t buf = j % kAccBufs;
+                bool have = mbar_wait(acc_full0 + 8 * buf, (j / kAccBufs) & 1u);
+                if (!have && lane == 0) atomicExch(error, 3);
+                have = __all_sync(0xFFFFFFFFu, have);
+                if (!have) { all_tiles = false; break; }
+                tc_fence_after();
+                const bool own_row_valid = tile_m * kTileM + quarter * 32 + lane < m_rows;   // the row whose values this thread holds
+                // this thread's part of every store.  FP32: row (lane / 8) of each group of four rows, 16 bytes at column
+                // 4 (lane % 8); bf16: row (lane / 4) of each group of eight rows, 16 bytes at column 8 (lane % 4)
+                const int32_t row0 = tile_m * kTileM + quarter * 32 + (OUT_BF16 ? (lane >> 2) : (lane >> 3));
+                float* out = reinterpret_cast<float*>(c_out) + (size_t)row0 * (size_t)n_cols + (size_t)tile_n * kTileN + 4 * (lane & 7);
+                __nv_bfloat16* out16 = reinterpret_cast<__nv_bfloat16*>(c_out) + (size_t)row0 * (size_t)n_cols + (size_t)tile_n * kTileN +
+                                       8 * (lane & 3);
+                const uint32_t lane_base = tmem + buf * kTileN + ((uint32_t)(quarter * 32) << 16);
+                for (int chunk = 0; chunk < kTileN / 32; ++chunk) {
+                    uint32_t r0[32];
+                    tmem_load32(lane_base + chunk * 32, r0);
+                    tmem_load_wait();
+                    if (chunk == kTileN / 32 - 1) {         // everything is in registers: the MMAs of the next tile may start
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(acc_empty0 + 8 * buf);
+                    }
+                    float v[32];
+#pragma unroll
+                    for (int jj = 0; jj < 32; ++jj) v[jj] = __fmul_rn(__uint_as_float(r0[jj]), scale);
+                    // A thread holds 32 columns of ONE row; stored as they are, every store instruction of the warp would
+                    // touch 32 different rows.  Through shared memory each instruction writes four rows of 128 contiguous bytes.
+                    if constexpr (!OUT_BF16) {
+#pragma unroll
+                        for (int jj = 0; jj < 32; jj += 4)
+                            *reinterpret_cast<float4*>(staging + lane * kStagePitch + jj) = make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
+                        __syncwarp();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const float4 x = *reinterpret_cast<const float4*>(staging + (4 * i + (lane >> 3)) * kStagePitch + 4 * (lane & 7));
+                            if (row0 + 4 * i < m_rows)                      // the last row block may be partial
+                                *reinterpret_cast<float4*>(out + (size_t)(4 * i) * n_cols + chunk * 32) = x;
+                        }
+                    } else {
+                        // 32 bf16 = 64 bytes per row, rows 20 words apart; a store instruction writes eight rows of 64 bytes
+                        uint32_t* stg = reinterpret_cast<uint32_t*>(staging);
+#pragma unroll
+                        for (int jj = 0; jj < 32; jj += 8) {
+                            uint4 pk;
+                            pk.x = bf16x2_bits(v[jj], v[jj + 1]); pk.y = bf16x2_bits(v[jj + 2], v[jj + 3]);
+                            pk.z = bf16x2_bits(v[jj + 4], v[jj + 5]); pk.w = bf16x2_bits(v[jj + 6], v[jj + 7]);
+                            *reinterpret_cast<uint4*>(stg + lane * 20 + jj / 2) = pk;
+                            if (next_alpha != nullptr && own_row_valid) {
+                                const uint32_t w4[4] = {pk.x, pk.y, pk.z, pk.w};
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) out_max = max(out_max, max(w4[q] & 0x7FFFu, (w4[q] >> 16) & 0x7FFFu));
+                            }
+                        }
+                        __syncwarp();
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const uint4 x = *reinterpret_cast<const uint4*>(stg + (8 * i + (lane >> 2)) * 20 + 4 * (lane & 3));
+                            if (row0 + 8 * i < m_rows)
+                                *reinterpret_cast<uint4*>(out16 + (size_t)(8 * i) * n_cols + chunk * 32) = x;
                         }
                     }
                     __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const uint4 x = *reinterpret_cast<const uint4*>(stg + (8 * i + (lane >> 2)) * 20 + 4 * (lane & 3));
-                        if (row0 + 8 * i < m_rows)
-                            *reinterpret_cast<uint4*>(out16 + (size_t)(8 * i) * n_cols + chunk * 32) = x;
-                    }
                 }
-                __syncwarp();
             }
         }
         // The global maximum of |C| as written (bf16), for the next quantizer's tensor scale (Eq. 1): every epilogue
@@ -529,7 +619,7 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
                 atomicMax(reinterpret_cast<unsigned int*>(error) + 1, wmax);
                 __threadfence();
                 const int ticket = atomicAdd(error + 2, 1);
-                if (ticket == (int)gridDim.x * 4 - 1) {
+                if (ticket == (int)gridDim.x * kEpiWarps - 1) {
                     const float A = __uint_as_float(atomicMax(reinterpret_cast<unsigned int*>(error) + 1, 0u) << 16);
                     *next_alpha = (A == 0.0f) ? 1.0f : __fdiv_rn(A, next_denom);
                 }
@@ -609,8 +699,8 @@ GemmLayout gemm_layout(int64_t m, int64_t n, int64_t k) {
     L.sf_a = round1k((size_t)((m + kTileM - 1) / kTileM * kTileM) * k / 16);
     L.sf_b = round1k((size_t)n * k / 16);
     L.off_a = 1024;
-    L.off_b = L.off_a + 3 * L.plane_a;
-    L.off_sfa = L.off_b + 3 * L.plane_b;
+    L.off_b = L.off_a + 2 * L.plane_a;
+    L.off_sfa = L.off_b + 2 * L.plane_b;
     L.off_sfb = L.off_sfa + L.sf_a;
     L.total = L.off_sfb + L.sf_b;
     return L;
@@ -647,7 +737,7 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
     const bool has_int = fmt == ABS_FMT_IF4;
 
     GemmMaps maps;
-    for (int p = 0; p < 3; ++p) {
+    for (int p = 0; p < 2; ++p) {
         // NVFP4 needs no split: its single plane is the caller's codes
         void* pa = has_int ? (void*)(ws + L.off_a + p * L.plane_a) : const_cast<void*>(a_codes);
         void* pb = has_int ? (void*)(ws + L.off_b + p * L.plane_b) : const_cast<void*>(b_codes);
@@ -661,9 +751,8 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
         const size_t off = op ? L.off_b : L.off_a, plane = op ? L.plane_b : L.plane_a;
         so[op].codes = (const uint4*)(op ? b_codes : a_codes);
         so[op].scales = (const uint8_t*)(op ? b_scales : a_scales);
-        so[op].plane_f = (uint4*)(ws + off);
-        so[op].plane_h = (uint4*)(ws + off + plane);
-        so[op].plane_l = (uint4*)(ws + off + 2 * plane);
+        so[op].plane_h = (uint4*)(ws + off);
+        so[op].plane_l = (uint4*)(ws + off + plane);
         so[op].sf_tiled = ws + (op ? L.off_sfb : L.off_sfa);
         so[op].rows = rows;
         so[op].pairs = rows * (k / 32);
@@ -692,7 +781,7 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
     if (attr_err[dev] == cudaSuccess)                                                                                   \
         attr_err[dev] = cudaFuncSetAttribute(if4_gemm_kernel<P, O, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                                              kGemmSmemBytes<P, B>)
-        ABS_GEMM_ATTR(3, false, 1); ABS_GEMM_ATTR(3, true, 1);
+        ABS_GEMM_ATTR(2, false, 1); ABS_GEMM_ATTR(2, true, 1);
         ABS_GEMM_ATTR(1, false, 1); ABS_GEMM_ATTR(1, true, 1);
         ABS_GEMM_ATTR(1, false, 2); ABS_GEMM_ATTR(1, true, 2);
 #undef ABS_GEMM_ATTR
@@ -703,12 +792,12 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
     const dim3 pgrid((unsigned)(num_tiles < sm_count[dev] ? num_tiles : sm_count[dev]));
     cudaError_t e;
 #define ABS_LAUNCH_GEMM(P, O, B)                                                                                        \
-    e = launch_pdl(if4_gemm_kernel<P, O, B>, pgrid, 320, kGemmSmemBytes<P, B>, s, maps, (const uint8_t*)(ws + L.off_sfa), \
+    e = launch_pdl(if4_gemm_kernel<P, O, B>, pgrid, kGemmThreads<P>, kGemmSmemBytes<P, B>, s, maps, (const uint8_t*)(ws + L.off_sfa), \
                    (const uint8_t*)(ws + L.off_sfb), a_alpha, b_alpha, c_f32, tiles_m, tiles_n,                           \
                    (int32_t)(k / (kStageK * B)), (int32_t)m, (int*)ws, stall_step, next_alpha, next_denom)
     const bool long_steps = !has_int && k % (2 * kStageK) == 0;      // NVFP4: K-steps of 512 where K allows
-    if (has_int && out_bf16) ABS_LAUNCH_GEMM(3, true, 1);
-    else if (has_int) ABS_LAUNCH_GEMM(3, false, 1);
+    if (has_int && out_bf16) ABS_LAUNCH_GEMM(2, true, 1);
+    else if (has_int) ABS_LAUNCH_GEMM(2, false, 1);
     else if (long_steps && out_bf16) ABS_LAUNCH_GEMM(1, true, 2);
     else if (long_steps) ABS_LAUNCH_GEMM(1, false, 2);
     else if (out_bf16) ABS_LAUNCH_GEMM(1, true, 1);

@@ -1157,3 +1157,21 @@ def test_matmul_leaves_the_tensor_scale_of_its_output(B, oracle, fmt):
     c, alpha = B.abs_matmul(fmt, B.abs_quantize(fmt, z), B.abs_quantize(fmt, to_dev(I.generate("cfg3a", 128, 256, seed=9))),
                             128, 128, 256, bf16=True, next_fmt=1, check=True)
     assert float(alpha.item()) == 1.0 and bool((c == 0).all())
+
+
+@pytest.mark.parametrize("fmt", [1, 0])
+@pytest.mark.parametrize("m,n,k", [(130, 128, 4096), (127, 256, 4352), (1, 128, 8192), (129, 128, 12544)])
+def test_tensor_core_matmul_around_the_accumulation_chunks(B, oracle, fmt, m, n, k):
+    """abs_matmul accumulates IF4 products in the tensor core over at most 4096 of K and adds the chunks in registers:
+    whole chunks, a last chunk of one pipeline step, several chunks, partial row blocks, one row.  Both outputs against the
+    float64 MAC reference: k / 64 roundings of a running sum of at most sum |a b| (2^-24 each), and a final bf16 rounding."""
+    a, b = I.generate("cfg2", m, k, seed=21), I.generate("cfg3b", n, k, seed=22)
+    oa, ob = oracle.quantize(fmt, a, threads=THREADS), oracle.quantize(fmt, b, threads=THREADS)
+    ref = oracle.mac_matmul_reference(fmt, oa, ob, m, n, k)
+    qa, qb = B.abs_quantize(fmt, to_dev(a)), B.abs_quantize(fmt, to_dev(b))
+    c = B.abs_matmul(fmt, qa, qb, m, n, k, check=True)
+    da = np.abs(B.abs_dequantize(fmt, *qa, m, k).double().cpu().numpy())
+    db = np.abs(B.abs_dequantize(fmt, *qb, n, k).double().cpu().numpy())
+    bound = (k / 64 + 8) * 2.0 ** -24 * 1.5 * (da @ db.T)
+    assert (np.abs(c.double().cpu().numpy() - ref) <= bound).all()
+    assert torch.equal(B.abs_matmul(fmt, qa, qb, m, n, k, check=True, bf16=True), c.bfloat16())
