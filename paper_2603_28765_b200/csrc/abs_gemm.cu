@@ -25,7 +25,8 @@
 // NVFP4).  4096^3, operands and split included: IF4 195 -> 118 us (nine MMAs per K-block to four), 8192 x 14336 x 4096
 // 1440 -> 785 us; NVFP4 46 and 340 us.
 #include "../../include/abs_b200.h"
-#include "abs_device.cuh"
+#include "abs_tc.cuh"
+#include "abs_skinny.cuh"
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -34,10 +35,6 @@
 
 namespace absq {
 
-constexpr int kTileM = 128, kTileN = 128;
-constexpr int kStageK = 256;                       // elements of K of one TMA box: 128 bytes of packed codes per row
-constexpr int kMmaK = 64;                          // K of one tcgen05.mma kind::mxf4nvf4
-constexpr int kPlaneBytes = kTileM * kStageK / 2;  // 16 KiB: one box (128 rows x 128 bytes) of one plane of one operand
 // A pipeline stage (one K-step) holds KBOXES boxes of each of the PLANES planes of A and of B (the scales do not pass
 // through shared memory).  IF4 (two planes, one box: K = 256, 64 KiB) has three stages.  Plain NVFP4 issues one MMA per
 // K-block, so the hand-overs of a step weigh more: its steps are two boxes long where K allows (K = 512, 64 KiB, three
@@ -54,32 +51,8 @@ template <int PLANES> constexpr int kGemmThreads = 32 * (2 + kEpiWarps<PLANES> +
 constexpr int kStagePitch = 36, kStagingBytes = 4 * 32 * kStagePitch * 4;
 template <int PLANES, int KBOXES> constexpr int kGemmSmemBytes =
     kStages<PLANES, KBOXES> * kStageBytes<PLANES, KBOXES> + 1024 /* alignment slack */ + 512 /* barriers */ + kStagingBytes;
-// The accumulators of a tile are summed in the tensor core over at most kChunkK of K; the epilogue adds the chunks in
-// registers.  The rounding error of one long chain grows with the square root of its steps: 8192 x 4096 x 14336, IF4,
-// 2-norm against float64: 1.3e-7 in one chain, 7.8e-8 in four (1.2e-7 with the nine-MMA split).  A hand-over costs what it
-// costs at the end of a tile, once per 4096 of K.
-constexpr int kChunkK = 4096;
-constexpr uint64_t kWaitLimitNs = 1000000000ull;   // one second: how long an mbarrier wait polls before the block gives up
 
 // ----------------------------------------------------------------------------- operand split
-
-// Splits eight integer codes (two's complement nibbles of one word) into the planes H and L, all nibbles at once:
-// sign s, magnitude m = |k|; h = m without bit 0 where m = 5 or 7 and 6 where m = 8 (the most negative code, which no
-// quantizer writes but dequantize reads as -8); l = -h, except 2 for m = 5, 0 for m = 7 and 6 for m = 8.  E2M1 codes of
-// the integers 0, 1, 2, 3, 4, 6 are 0, 2, 4, 5, 6, 7.  No step carries from one nibble into the next.
-__device__ __forceinline__ void split_int_word(uint32_t w, uint32_t& h, uint32_t& l) {
-    constexpr uint32_t kOnes = 0x11111111u;
-    const uint32_t s = w & 0x88888888u, neg = s >> 3;
-    const uint32_t m = (w ^ (neg * 15u)) + neg;                      // |k| per nibble, 0 .. 8
-    const uint32_t odd = (m >> 2) & m & kOnes;                        // m = 5 or 7
-    const uint32_t is8 = (m >> 3) & kOnes;                            // m = 8
-    const uint32_t mh = m - (odd | (is8 << 1));                       // h: 0, 1, 2, 3, 4, 6
-    const uint32_t c0 = mh & kOnes, c1 = (mh >> 1) & kOnes, c2 = (mh >> 2) & kOnes;
-    const uint32_t mag = ((c2 | c1) << 2) | ((c2 | (c0 & ~c1)) << 1) | (c1 & (c0 | c2));
-    const uint32_t is5 = odd & ~(m >> 1), is7 = odd & (m >> 1);
-    h = s | mag;
-    l = (s ^ (0x88888888u & ~((is5 | is8) << 3))) | (mag & ~((is5 << 1) | (is7 * 7u)));
-}
 
 // One operand of the product as the split kernel sees it.
 struct SplitOperand {
@@ -138,121 +111,6 @@ __global__ void __launch_bounds__(256, 8) if4_split_kernel(const SplitOperand a,
         out[96] = make_uint4(r[0].w & kMag, r[1].w & kMag, r[2].w & kMag, r[3].w & kMag);
     }
 }
-
-// ----------------------------------------------------------------------------- PTX building blocks
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-    uint32_t done;
-    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    return done != 0;
-}
-__device__ __forceinline__ uint64_t global_timer_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-// Wait for the phase with the given parity, bounded in time (a try_wait may itself sleep for a while, so counting
-// polls would not bound it); false when the limit ran out.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = global_timer_ns();
-    do {
-        if (mbar_try_wait(bar, parity)) return true;
-    } while (global_timer_ns() - t0 < kWaitLimitNs);
-    return false;
-}
-// One 2-D tile (inner coordinate x in bytes, outer coordinate y in rows) from a tensor map into shared memory.
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int32_t x, int32_t y, uint32_t bar) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                 :: "r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void tmem_alloc(uint32_t smem_result, uint32_t columns) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_result), "r"(columns) : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() { asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_free(uint32_t addr, uint32_t columns) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(addr), "r"(columns) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// Arrives on the mbarrier once every tcgen05 operation this thread issued before has completed.
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
-}
-// D[tmem] (+)= A[smem] * B[smem]^T, 128 x 128 x 64, E2M1 operands, one UE4M3 scale per 16 elements read from tensor memory.
-// What happens to the A operand in the tensor core's collector buffer: read from shared memory and dropped, read and
-// kept (kFill), taken from the buffer and kept (kUse), taken from the buffer and dropped (kLastUse).  An MMA that
-// takes A from the buffer reads only B from shared memory.
-enum Collector { kDiscard, kFill, kUse, kLastUse };
-template <Collector C = kDiscard>
-__device__ __forceinline__ void tc_mma_nvf4(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate,
-                                            uint32_t sfa_tmem, uint32_t sfb_tmem) {
-#define ABS_MMA_NVF4(USAGE)                                                                                              \
-    asm volatile("{ .reg .pred p; setp.ne.b32 p, %4, 0;\n"                                                               \
-                 "  tcgen05.mma.cta_group::1.kind::mxf4nvf4.block_scale.block16" USAGE " [%0], %1, %2, %3, [%5], [%6], p; }" \
-                 :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(sfa_tmem), "r"(sfb_tmem) \
-                 : "memory")
-    if constexpr (C == kFill) ABS_MMA_NVF4(".collector::a::fill");
-    else if constexpr (C == kUse) ABS_MMA_NVF4(".collector::a::use");
-    else if constexpr (C == kLastUse) ABS_MMA_NVF4(".collector::a::lastuse");
-    else ABS_MMA_NVF4("");
-#undef ABS_MMA_NVF4
-}
-// 32 lanes x 32 columns of 32 bits: thread t of the warp gets columns c .. c+31 of lane (warp % 4) * 32 + t.
-__device__ __forceinline__ void tmem_load32(uint32_t addr, uint32_t (&r)[32]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(addr) : "memory");
-}
-// The same with 16 columns.
-__device__ __forceinline__ void tmem_load16(uint32_t addr, uint32_t (&r)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(addr) : "memory");
-}
-// Two FP32 values rounded to nearest even bf16, the first in the low half.
-__device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-__device__ __forceinline__ void tmem_load_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// 32 lanes x 16 columns of 32 bits: thread t of the warp writes columns c .. c+15 of lane (warp % 4) * 32 + t.
-__device__ __forceinline__ void tmem_store16(uint32_t addr, const uint4& a, const uint4& b, const uint4& c, const uint4& d) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-                 :: "r"(addr), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w), "r"(c.x), "r"(c.y),
-                    "r"(c.z), "r"(c.w), "r"(d.x), "r"(d.y), "r"(d.z), "r"(d.w)
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_store_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-// Shared-memory matrix descriptors (64 bits): start address, leading / stride byte offsets (all in 16-byte units),
-// descriptor version 1 (Blackwell) in bits 46-47, swizzle mode in bits 61-63.
-//   operand tiles: K-major rows of 128 bytes, 128-byte swizzle (mode 2), 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t operand_desc(uint32_t smem_addr) {
-    return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
-           ((uint64_t)2 << 61);
-}
-// Instruction descriptor of kind::mxf4nvf4: A and B E2M1 (format 1, bits 7-9 and 10-12), both K-major, N / 8 in bits
-// 17-22, scale format UE4M3 (bit 23 = 0), M / 16 in bits 24-28, dense, K = 64 (bit 31 = 0), scale ids 0.
-constexpr uint32_t kInstrDesc = (1u << 7) | (1u << 10) | ((uint32_t)(kTileN >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
 
 // ----------------------------------------------------------------------------- the product kernel
 
@@ -670,6 +528,17 @@ bool plane_map(CUtensorMap* map, void* base, uint64_t rows, uint64_t row_bytes) 
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Tensor map of row-major scales: bytes [rows, row_bytes], box 16 bytes x 128 rows, no swizzle.
+bool scale_map(CUtensorMap* map, void* base, uint64_t rows, uint64_t row_bytes) {
+    EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc) return false;
+    const cuuint64_t dims[2] = {row_bytes, rows};
+    const cuuint64_t strides[1] = {row_bytes};
+    const cuuint32_t box[2] = {16, 128}, elem[2] = {1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 size_t round1k(size_t n) { return (n + 1023) & ~(size_t)1023; }
 
 // Launch with programmatic stream serialization: the kernel may become resident while its predecessor in the stream
@@ -688,6 +557,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int block, size_t sm
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+constexpr int kMaxSms = 160;               // workspaces are sized for up to this many SMs
 struct GemmLayout {
     size_t plane_a, plane_b, sf_a, sf_b;       // sizes
     size_t off_a, off_b, off_sfa, off_sfb, total;
@@ -706,6 +576,25 @@ GemmLayout gemm_layout(int64_t m, int64_t n, int64_t k) {
     return L;
 }
 
+// Plan and workspace of the product with few rows of A (see abs_skinny.cuh): tickets, partial sums.
+struct SkinnyPlan {
+    int32_t units, grid;
+    size_t off_partials, total;
+};
+// The rule: IF4 with up to 32 rows of A, except where the whole of B is fewer than 64 steps, which the blocks of abs_gemm.cu's
+// kernel take in one go while here most of the time would be the sum of shared tiles (1024 x 1024: 9.0 -> 8.2 us with one
+// token, but 8.9 -> 9.5 us with 16; 4096 x 1024, 32 tokens: 10.7 -> 10.1).  With 33 to 64 rows (64 columns for the MMA's N side,
+// two stages) it lost at every size below 8192 x 8192.  NVFP4 has no planes to save and measured slower at all sizes.
+bool skinny_plan(abs_fmt_t fmt, int64_t m, int64_t n, int64_t k, int sm_count, SkinnyPlan& P) {
+    const int64_t units = n / kTileM * (k / kStageK);
+    if (fmt != ABS_FMT_IF4 || m > kSkinnyMaxRows || (m > 8 && units < 64) || units > 0x7FFFFFFF) return false;
+    P.units = (int32_t)units;
+    P.grid = P.units < sm_count ? P.units : sm_count;
+    P.off_partials = 1024 + round1k((size_t)(n / kTileM) * sizeof(int));
+    P.total = P.off_partials + (size_t)P.grid * 2 * kSkinnyTok * kTileM * sizeof(float);
+    return true;
+}
+
 bool gemm_shape_ok(abs_fmt_t fmt, int64_t m, int64_t n, int64_t k) {
     return (fmt == ABS_FMT_IF4 || fmt == ABS_FMT_NVFP4) && m > 0 && n > 0 && k > 0 && n % kTileN == 0 &&
            k % kStageK == 0 && m < ((int64_t)1 << 30) && n < ((int64_t)1 << 30) && k < ((int64_t)1 << 30);
@@ -717,7 +606,33 @@ extern "C" {
 
 size_t abs_matmul_workspace_bytes(abs_fmt_t fmt, int64_t m, int64_t n, int64_t k) {
     if (!gemm_shape_ok(fmt, m, n, k)) return 0;
-    return gemm_layout(m, n, k).total;
+    size_t total = gemm_layout(m, n, k).total;
+    SkinnyPlan P;
+    // for the largest grid: the size must not depend on the device that happens to be current
+    if (skinny_plan(fmt, m, n, k, kMaxSms, P) && P.total > total) total = P.total;
+    return total;
+}
+
+// The product with few rows of A.  Arguments are already validated.
+static abs_status_t skinny_matmul(const SkinnyPlan& P, const void* a_codes, const void* a_scales, const float* a_alpha,
+                                  const void* b_codes, const void* b_scales, const float* b_alpha, int64_t m, int64_t n, int64_t k,
+                                  void* out, uint8_t* ws, cudaStream_t s, bool out_bf16, float* next_alpha, float next_denom) {
+    SkinnyArgs p;
+    if (!plane_map(&p.w_codes, const_cast<void*>(b_codes), (uint64_t)n, (uint64_t)k / 2) ||
+        !scale_map(&p.w_scales, const_cast<void*>(b_scales), (uint64_t)n, (uint64_t)k / 16))
+        return ABS_ERR_CUDA;
+    p.x_codes = (const uint8_t*)a_codes; p.x_scales = (const uint8_t*)a_scales;
+    p.alpha_a = a_alpha; p.alpha_b = b_alpha;
+    p.out = out;
+    p.partials = (float*)(ws + P.off_partials);
+    p.tickets = (int*)(ws + 1024); p.error = (int*)ws;
+    p.m = (int32_t)m; p.n = (int32_t)n; p.k = (int32_t)k; p.units = P.units;
+    p.next_alpha = next_alpha; p.next_denom = next_denom;
+    if (launch_pdl(skinny_clear_kernel, dim3(1), 256, 0, s, (int*)ws, p.tickets, (int32_t)(n / kTileM)) != cudaSuccess) return ABS_ERR_CUDA;
+    const cudaError_t e = launch_pdl(out_bf16 ? skinny_kernel<true> : skinny_kernel<false>, dim3((unsigned)P.grid), kSkinnyThreads,
+                                     kSkinnySmemBytes, s, p);
+    if (e != cudaSuccess) return ABS_ERR_CUDA;
+    return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
 }
 
 static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* a_scales, const float* a_alpha, const void* b_codes,
@@ -730,11 +645,39 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
     if (!a_codes || !a_scales || !a_alpha || !b_codes || !b_scales || !b_alpha || !c_f32 || !workspace) return ABS_ERR_NULL;
     const uintptr_t all = (uintptr_t)a_codes | (uintptr_t)a_scales | (uintptr_t)b_codes | (uintptr_t)b_scales | (uintptr_t)c_f32;
     if ((all & 15u) || ((uintptr_t)workspace & 1023u)) return ABS_ERR_ALIGN;
+    if (workspace_bytes < abs_matmul_workspace_bytes(fmt, m, n, k)) return ABS_ERR_SIZE;
     const GemmLayout L = gemm_layout(m, n, k);
-    if (workspace_bytes < L.total) return ABS_ERR_SIZE;
     cudaStream_t s = (cudaStream_t)stream;
     uint8_t* ws = (uint8_t*)workspace;
     const bool has_int = fmt == ABS_FMT_IF4;
+    // the opt-in to more than 48 KiB of dynamic shared memory is per device
+    static std::once_flag attr_once[64];
+    static cudaError_t attr_err[64];
+    static int sm_count[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return ABS_ERR_CUDA;
+    std::call_once(attr_once[dev], [dev]() {
+        if (cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sm_count[dev] < 1)
+            sm_count[dev] = 1;
+        attr_err[dev] = cudaSuccess;
+#define ABS_GEMM_ATTR(P, O, B)                                                                                         \
+    if (attr_err[dev] == cudaSuccess)                                                                                   \
+        attr_err[dev] = cudaFuncSetAttribute(if4_gemm_kernel<P, O, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
+                                             kGemmSmemBytes<P, B>)
+        ABS_GEMM_ATTR(2, false, 1); ABS_GEMM_ATTR(2, true, 1);
+        ABS_GEMM_ATTR(1, false, 1); ABS_GEMM_ATTR(1, true, 1);
+        ABS_GEMM_ATTR(1, false, 2); ABS_GEMM_ATTR(1, true, 2);
+#undef ABS_GEMM_ATTR
+        if (attr_err[dev] == cudaSuccess)
+            attr_err[dev] = cudaFuncSetAttribute(skinny_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkinnySmemBytes);
+        if (attr_err[dev] == cudaSuccess)
+            attr_err[dev] = cudaFuncSetAttribute(skinny_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkinnySmemBytes);
+    });
+    if (attr_err[dev] != cudaSuccess) return ABS_ERR_CUDA;
+    SkinnyPlan P;
+    if (stall_step < 0 && skinny_plan(fmt, m, n, k, sm_count[dev] < kMaxSms ? sm_count[dev] : kMaxSms, P))
+        return skinny_matmul(P, a_codes, a_scales, a_alpha, b_codes, b_scales, b_alpha, m, n, k, c_f32, ws, s, out_bf16, next_alpha,
+                             next_denom);
 
     GemmMaps maps;
     for (int p = 0; p < 2; ++p) {
@@ -767,26 +710,6 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
         if (launch_pdl(if4_split_kernel, dim3((unsigned)blocks), 256, 0, s, so[0], so[1], has_int, (int*)ws) != cudaSuccess)
             return ABS_ERR_CUDA;
     }
-    // the opt-in to more than 48 KiB of dynamic shared memory is per device
-    static std::once_flag attr_once[64];
-    static cudaError_t attr_err[64];
-    static int sm_count[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return ABS_ERR_CUDA;
-    std::call_once(attr_once[dev], [dev]() {
-        if (cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sm_count[dev] < 1)
-            sm_count[dev] = 1;
-        attr_err[dev] = cudaSuccess;
-#define ABS_GEMM_ATTR(P, O, B)                                                                                         \
-    if (attr_err[dev] == cudaSuccess)                                                                                   \
-        attr_err[dev] = cudaFuncSetAttribute(if4_gemm_kernel<P, O, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
-                                             kGemmSmemBytes<P, B>)
-        ABS_GEMM_ATTR(2, false, 1); ABS_GEMM_ATTR(2, true, 1);
-        ABS_GEMM_ATTR(1, false, 1); ABS_GEMM_ATTR(1, true, 1);
-        ABS_GEMM_ATTR(1, false, 2); ABS_GEMM_ATTR(1, true, 2);
-#undef ABS_GEMM_ATTR
-    });
-    if (attr_err[dev] != cudaSuccess) return ABS_ERR_CUDA;
     const int32_t tiles_m = (int32_t)((m + kTileM - 1) / kTileM), tiles_n = (int32_t)(n / kTileN);
     const int64_t num_tiles = (int64_t)tiles_m * tiles_n;
     const dim3 pgrid((unsigned)(num_tiles < sm_count[dev] ? num_tiles : sm_count[dev]));

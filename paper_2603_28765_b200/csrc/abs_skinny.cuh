@@ -1,0 +1,412 @@
+// IF4 products with few rows of A (a decoder step's tokens, up to 32): C = A B^T with the arithmetic of abs_gemm.cu, in one
+// pass over the weights B where they lie.
+//
+// With so few rows the time is that of reading B once; abs_gemm.cu would first write B's planes and tiled scales to the
+// workspace, pad A to 128 rows, and run one block per 128 columns of C whatever their number.  Here
+//   - the weights are the M side of the MMA (128 rows) and the tokens the N side;
+//   - the work, (n / 128) tiles x (k / 256) steps, is cut into one run of equal length per SM, tile by tile, so that every SM
+//     reads the same number of bytes whatever the sizes; tiles that are shared between runs are summed by the last of their
+//     blocks, in the order of K, from partial sums in the workspace;
+//   - one lane brings codes and scales of B by TMA, three steps ahead; sixteen warps split the codes, and those of the
+//     tokens, into planes in the MMA's layout in shared memory; four warps write the scales into tensor memory and are the
+//     epilogue of every tile; one lane issues MMAs.
+//
+// The planes.  Every code of B passes through the integer pipe once per call, which is what bounds the kernel, so B's split
+// is the cheapest one and not the shortest: the codes of the FP groups (F), and for the integer groups
+// k = 8 y + 2 x with y in {0, 1/2, -1, -1/2} from the two high bits and x in {0, 1/2, 1, 3/2} the two low bits as they are --
+// eight word operations for eight codes against some twenty of split_int_word.  The tokens take the planes H and L of
+// abs_gemm.cu, one below the other as the N side of one MMA (an MMA of 128 x N x 64 takes 75 to 100 cycles for any N up to
+// 128), so there are three MMAs of 128 x 64 x 64 per K-block.
+//
+// Measured, product alone, weights not in the L2 (before: planes through the workspace): n = 14336, k = 4096: 1 token 52.5
+// -> 21.5 us, 24 tokens 53 -> 24 us; 4096 x 4096, 1 token 32.7 -> 14.3 us; 14336 x 14336, 32 tokens 133 -> 56 us.  A step
+// of 256 of K takes 1450 cycles on an SM, of which the integer pipe is busy for about 1000; the first data after some 3 us
+// and the sum of shared tiles, 2 us, are the rest.
+#pragma once
+#include "abs_tc.cuh"
+
+namespace absq {
+
+constexpr int kSkinnyMaxRows = 32, kSkinnyTok = 32;                       // rows of A; columns of the MMA they are padded to
+constexpr int kSkinnyDecWarps = 16;
+constexpr int kSkinnyThreads = 32 * (1 + 4 + kSkinnyDecWarps + 1);
+constexpr uint32_t kSkinnySfSlots = 4, kSkinnySlotCols = 32;              // 16 columns of weight scales, 16 of token scales
+// Steps of B as it lies, and steps of planes, in shared memory: decoding a step, the hand-over and its MMAs take about as
+// long as two steps, so there are three stages of planes.
+constexpr int kSkinnyRaw = 3, kSkinnyStages = 3;
+constexpr int kSkinnyRawBytes = kPlaneBytes + kTileM * 16;                // codes, then 16 scale bytes per row
+constexpr int kSkinnyStageBytes = 3 * kPlaneBytes + 2 * kSkinnyTok * 128; // F, Y, X of B; H, L of A
+constexpr int kSkinnySmemBytes = kSkinnyStages * kSkinnyStageBytes + kSkinnyRaw * kSkinnyRawBytes + 1024 + 512;
+
+struct SkinnyArgs {
+    CUtensorMap w_codes, w_scales;         // weights B [n, k] as abs_quantize wrote them: boxes of 128 rows x 128 and x 16 bytes
+    const uint8_t *x_codes, *x_scales;     // tokens A [m, k]
+    const float *alpha_a, *alpha_b;
+    void* out;                             // [m, n] bf16 or FP32
+    float* partials;                       // [blocks][2][32][128]
+    int *tickets, *error;                  // tickets: one per tile
+    int32_t m, n, k, units;
+    float* next_alpha;
+    float next_denom;
+};
+
+// Clears what skinny_kernel counts in: the three words at the start of the workspace (error word, output maximum, ticket of
+// the maximum) and the tickets of the tiles.
+__global__ void __launch_bounds__(256) skinny_clear_kernel(int* __restrict__ error, int* __restrict__ tickets, int32_t n_tickets) {
+    pdl_launch_dependents();
+    pdl_wait();
+    if (threadIdx.x < 3) error[threadIdx.x] = 0;
+    for (int32_t i = threadIdx.x; i < n_tickets; i += blockDim.x) tickets[i] = 0;
+}
+
+__device__ __forceinline__ uint4 mask_scales(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    constexpr uint32_t kMag = 0x7F7F7F7Fu;
+    return make_uint4(a & kMag, b & kMag, c & kMag, d & kMag);
+}
+
+template <bool OUT_BF16>
+__global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_constant__ SkinnyArgs p) {
+    constexpr int NT = kSkinnyTok, kRaw = kSkinnyRaw, kStages = kSkinnyStages, kStageBytes = kSkinnyStageBytes;
+    constexpr uint32_t kSfBase = 6 * NT;                                   // accumulators F H, F L, Y H, Y L, X H, X L
+    constexpr uint32_t kTmem = 512;                                        // of which 320 columns are used
+    constexpr int kChunkSteps = kChunkK / kStageK;
+    extern __shared__ uint8_t gemm_smem_raw[];
+    const uint32_t raw = smem_u32(gemm_smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    const uint32_t raw0 = base + kStages * kStageBytes, bars = raw0 + kRaw * kSkinnyRawBytes;
+    uint32_t* tmem_word = reinterpret_cast<uint32_t*>(gemm_smem_raw + (bars - raw) + 320);
+    const uint32_t full0 = bars, empty0 = bars + 64, acc_full = bars + 128, acc_empty = bars + 136;
+    const uint32_t sf_full0 = bars + 192, sf_empty0 = bars + 256, raw_full0 = bars + 384, raw_empty0 = bars + 424;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int32_t ksteps = p.k / kStageK;
+    const int32_t u0 = (int32_t)((int64_t)p.units * blockIdx.x / gridDim.x), u1 = (int32_t)((int64_t)p.units * (blockIdx.x + 1) / gridDim.x);
+    const size_t code_pitch = (size_t)p.k / 2, scale_pitch = (size_t)p.k / 16;
+
+    __shared__ int failed, last[2];
+    pdl_launch_dependents();
+    if (threadIdx.x == 0) {
+        failed = 0;
+        for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, kSkinnyDecWarps / 2); mbar_init(empty0 + 8 * s, 1); }
+        mbar_init(acc_full, 1);
+        mbar_init(acc_empty, 4);
+        for (int i = 0; i < (int)kSkinnySfSlots; ++i) { mbar_init(sf_full0 + 8 * i, 4); mbar_init(sf_empty0 + 8 * i, 1); }
+        for (int s = 0; s < kRaw; ++s) { mbar_init(raw_full0 + 8 * s, 1); mbar_init(raw_empty0 + 8 * s, kSkinnyDecWarps / 2 + 4); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) { tmem_alloc(smem_u32(tmem_word), kTmem); tmem_relinquish(); }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_word;
+    pdl_wait();
+
+    // A run is walked in spans: consecutive steps of one tile, no longer than a chunk of K (see kChunkK).
+    auto span = [&](int32_t u, int32_t k0) { return min(min(ksteps - k0, u1 - u), kChunkSteps - k0 % kChunkSteps); };
+
+    const float scale = __fmul_rn(*p.alpha_a, *p.alpha_b);
+    uint32_t out_max = 0u;                                                 // largest |C| bit pattern this thread has written as bf16
+    auto write_out = [&](int32_t token, size_t col, float sum) {
+        const float c = __fmul_rn(sum, scale);
+        const size_t at = (size_t)token * p.n + col;
+        if constexpr (OUT_BF16) {
+            const __nv_bfloat16 b = __float2bfloat16_rn(c);
+            reinterpret_cast<__nv_bfloat16*>(p.out)[at] = b;
+            out_max = max(out_max, (uint32_t)__bfloat16_as_ushort(b) & 0x7FFFu);
+        } else {
+            reinterpret_cast<float*>(p.out)[at] = c;
+        }
+    };
+
+    if (warp == 0) {
+        // ---- MMAs: weights are A (128 rows), tokens B (NT rows of H, then NT of L).  The whole warp walks the loop and one elected lane
+        // issues: descriptors and addresses are then known to be uniform and are not converted before every instruction
+        // (2400 cycles for the sixteen MMAs of a step when lane 0 alone ran the loop, beside eight busy warps).
+        constexpr uint32_t kDesc = (1u << 7) | (1u << 10) | ((uint32_t)(2 * NT >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
+        const uint64_t desc0 = operand_desc(base);
+        uint32_t it = 0, j = 0;
+        bool ok = true;
+        for (int32_t u = u0, k0 = u0 % ksteps; u < u1 && ok; ++j) {
+            const int32_t len = span(u, k0);
+            ok = mbar_wait_warp(acc_empty, (j & 1u) ^ 1u);
+            if (!ok) { if (lane == 0) atomicExch(p.error, 4); break; }
+            tc_fence_after();
+            for (int32_t kt = 0; kt < len; ++kt, ++it) {
+                const uint32_t s = it % kStages, slot = it % kSkinnySfSlots;
+                ok = mbar_wait_warp(full0 + 8 * s, (it / kStages) & 1u);
+                if (!ok) { if (lane == 0) atomicExch(p.error, 2); break; }
+                ok = mbar_wait_warp(sf_full0 + 8 * slot, (it / kSkinnySfSlots) & 1u);
+                if (!ok) { if (lane == 0) atomicExch(p.error, 5); break; }
+                tc_fence_after();
+                const uint64_t st = desc0 + (uint64_t)((s * kStageBytes) >> 4);
+                const uint32_t tsfa = tmem + kSfBase + slot * kSkinnySlotCols, tsfb = tsfa + kSkinnySlotCols / 2;
+                auto desc_a = [&](int pl, int kb) { return st + ((pl * kPlaneBytes + kb * (kMmaK / 2)) >> 4); };
+                auto desc_b = [&](int kb) { return st + ((3 * kPlaneBytes + kb * (kMmaK / 2)) >> 4); };
+                if (elect_one()) {
+#pragma unroll
+                    for (int kb = 0; kb < kStageK / kMmaK; ++kb) {
+                        const bool go = !(kt == 0 && kb == 0);
+#pragma unroll
+                        for (int pl = 0; pl < 3; ++pl)
+                            tc_mma_nvf4(tmem + 2 * pl * NT, desc_a(pl, kb), desc_b(kb), kDesc, go, tsfa + 4 * kb, tsfb + 4 * kb);
+                    }
+                    tc_commit(empty0 + 8 * s);
+                    tc_commit(sf_empty0 + 8 * slot);
+                    if (kt == len - 1) tc_commit(acc_full);
+                }
+                __syncwarp();
+            }
+            u += len;
+            k0 += len;
+            if (k0 == ksteps) k0 = 0;
+        }
+    } else if (warp <= 4) {
+        // ---- scales and epilogue: this warp's quarter of tensor memory (lanes 32 (w % 4) ..)
+        const int quarter = warp & 3;
+        const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16);
+        constexpr int kTokRows = NT / 32;
+        // 16 scale bytes of a step for this lane's tokens, one step ahead
+        uint4 xr[kTokRows];
+        int32_t kf = u0 % ksteps;                                          // the step loaded next
+        auto load_tokens = [&]() __attribute__((always_inline)) {
+            const uint8_t* xp = p.x_scales + (size_t)lane * scale_pitch + (size_t)kf * 16;
+#pragma unroll
+            for (int q = 0; q < kTokRows; ++q)
+                xr[q] = q * 32 + lane < p.m ? *reinterpret_cast<const uint4*>(xp + (size_t)(q * 32) * scale_pitch) : make_uint4(0u, 0u, 0u, 0u);
+            if (++kf == ksteps) kf = 0;
+        };
+        load_tokens();
+        // fp32(1/7), fp32(6/7), fp32(6/49)
+        const float c17 = __uint_as_float(0x3E124925u), c67 = __uint_as_float(0x3F5B6DB7u), c649 = __uint_as_float(0x3DFAC688u);
+        uint32_t it = 0, j = 0;
+        bool ok = true;
+        bool from_start = u0 % ksteps == 0, first_span = true;
+        // one step: its scales go to the next slot
+        auto step = [&]() __attribute__((always_inline)) {
+            const uint32_t slot = it % kSkinnySfSlots, rs = it % kRaw;
+            ok = mbar_wait_warp(raw_full0 + 8 * rs, (it / kRaw) & 1u) &&
+                 mbar_wait_warp(sf_empty0 + 8 * slot, ((it / kSkinnySfSlots) & 1u) ^ 1u);
+            if (!ok) { if (lane == 0) atomicExch(p.error, 6); return; }
+            const uint4* wp = reinterpret_cast<const uint4*>(gemm_smem_raw + (raw0 - raw) + rs * kSkinnyRawBytes + kPlaneBytes) + lane;
+            const uint4 w[4] = {wp[0], wp[32], wp[64], wp[96]};
+            tc_fence_after();
+            const uint32_t at = lanes + kSfBase + slot * kSkinnySlotCols;
+            tmem_store16(at, mask_scales(w[0].x, w[1].x, w[2].x, w[3].x), mask_scales(w[0].y, w[1].y, w[2].y, w[3].y),
+                         mask_scales(w[0].z, w[1].z, w[2].z, w[3].z), mask_scales(w[0].w, w[1].w, w[2].w, w[3].w));
+            uint32_t x4[4][4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint4 v = q < 2 * kTokRows ? xr[q % kTokRows] : make_uint4(0u, 0u, 0u, 0u);     // H rows, then L rows
+                x4[0][q] = v.x; x4[1][q] = v.y; x4[2][q] = v.z; x4[3][q] = v.w;
+            }
+            tmem_store16(at + 16, mask_scales(x4[0][0], x4[0][1], x4[0][2], x4[0][3]), mask_scales(x4[1][0], x4[1][1], x4[1][2], x4[1][3]),
+                         mask_scales(x4[2][0], x4[2][1], x4[2][2], x4[2][3]), mask_scales(x4[3][0], x4[3][1], x4[3][2], x4[3][3]));
+            load_tokens();
+            tmem_store_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) { mbar_arrive(sf_full0 + 8 * slot); mbar_arrive(raw_empty0 + 8 * rs); }
+            ++it;
+        };
+        for (int32_t u = u0; u < u1 && ok; ++j) {
+            const int32_t tile = u / ksteps, k0 = u - tile * ksteps, len = span(u, k0);
+            const uint32_t end = it + len;
+            while (ok && it < end) step();
+            if (!ok) break;
+            // the span's accumulators
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(acc_full, j & 1u));
+            if (!ok) { if (lane == 0) atomicExch(p.error, 3); break; }
+            tc_fence_after();
+            u += len;
+            const bool tile_end = k0 + len == ksteps, whole = tile_end && from_start;      // whole: this block has all of K
+            float* mine = p.partials + ((size_t)blockIdx.x * 2 + (from_start ? 1 : 0)) * (NT * kTileM) + quarter * 32 + lane;
+            const size_t col = (size_t)tile * kTileM + quarter * 32 + lane;
+            for (int32_t t0 = 0; t0 < p.m; t0 += 8) {
+                uint32_t r[6][8];
+#pragma unroll
+                for (int a = 0; a < 6; ++a) tmem_load8(lanes + a * NT + t0, r[a]);
+                tmem_load_wait();
+                float v[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    auto acc = [&](int a) { return __uint_as_float(r[a][e]); };
+                    const float kh = __fmaf_rn(8.0f, acc(2), __fmul_rn(2.0f, acc(4))), kl = __fmaf_rn(8.0f, acc(3), __fmul_rn(2.0f, acc(5)));
+                    v[e] = __fadd_rn(__fmaf_rn(c67, kh, acc(0)), __fmaf_rn(c649, kl, __fmul_rn(c17, acc(1))));
+                }
+                // columns of tokens beyond m are stored with the rest (the workspace has NT of them) and never read
+                if (!first_span) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[e] = __fadd_rn(mine[e * kTileM], v[e]);
+                }
+                if (whole) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (t0 + e < p.m) write_out(t0 + e, col, v[e]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) mine[e * kTileM] = v[e];
+                }
+                mine += 8 * kTileM;
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty);
+            first_span = tile_end;
+            if (tile_end) from_start = true;
+        }
+        __threadfence();                                                   // the shares, for the block that sums them
+        if (!ok) failed = 1;
+    } else if (warp < 5 + kSkinnyDecWarps) {
+        // ---- codes: thread i handles the 16 bytes (two groups) at place i % 8 of weight rows i / 8, i / 8 + 32, ... of a
+        // step, and of the tokens likewise.  Place c of row r holds bytes 16 (c ^ (r % 8)): the MMA's 128-byte swizzle, in
+        // which TMA has written the codes of B.
+        // Two groups of warps take the steps in turn, so that one computes while the other waits for its next step.
+        constexpr int kThreadsD = 16 * kSkinnyDecWarps, kW = 1024 / kThreadsD, kX = (NT * 8 + kThreadsD - 1) / kThreadsD;
+        const uint32_t group = warp >= 5 + kSkinnyDecWarps / 2;
+        const int i = (threadIdx.x - 160) % kThreadsD, r = i >> 3, c = (i & 7) ^ (r & 7);
+        struct Piece { uint4 codes; uint32_t two; };
+        // tokens of the group's next step
+        Piece x[kX];
+        int32_t kf = (u0 + (int32_t)group) % ksteps;
+        auto fetch = [&]() __attribute__((always_inline)) {
+#pragma unroll
+            for (int q = 0; q < kX; ++q) {
+                const size_t token = q * (kThreadsD / 8) + r;
+                if ((int32_t)token < p.m) {
+                    x[q].codes = *reinterpret_cast<const uint4*>(p.x_codes + token * code_pitch + (size_t)kf * 128 + c * 16);
+                    x[q].two = *reinterpret_cast<const uint16_t*>(p.x_scales + token * scale_pitch + (size_t)kf * 16 + c * 2);
+                }
+            }
+            kf = (kf + 2) % ksteps;
+        };
+        auto store = [&](uint32_t at, const uint4& v) {
+            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" :: "r"(at), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+        };
+        auto put_weights = [&](const Piece& f, uint32_t at) {
+            const uint32_t m0 = 0u - ((f.two >> 7) & 1u), m1 = 0u - (f.two >> 15);      // all ones for an integer group
+            auto low = [](uint32_t w, uint32_t mask) { return w & mask & 0x33333333u; };
+            // bits b3 b2 of k: code of 0, 1/2, -1, -1/2 = b3 << 3 | (b3 & ~b2) << 1 | b2
+            auto high = [](uint32_t w, uint32_t mask) {
+                const uint32_t w2 = w >> 2;
+                return ((w & 0x88888888u) | (w2 & 0x11111111u) | (w2 & ~(w >> 1) & 0x22222222u)) & mask;
+            };
+            store(at, make_uint4(f.codes.x & ~m0, f.codes.y & ~m0, f.codes.z & ~m1, f.codes.w & ~m1));
+            store(at + kPlaneBytes, make_uint4(high(f.codes.x, m0), high(f.codes.y, m0), high(f.codes.z, m1), high(f.codes.w, m1)));
+            store(at + 2 * kPlaneBytes, make_uint4(low(f.codes.x, m0), low(f.codes.y, m0), low(f.codes.z, m1), low(f.codes.w, m1)));
+        };
+        auto put_tokens = [&](const Piece& f, uint32_t at) {
+            uint4 h = f.codes, l = make_uint4(0u, 0u, 0u, 0u);
+            if (f.two & 0x80u) { split_int_word(f.codes.x, h.x, l.x); split_int_word(f.codes.y, h.y, l.y); }
+            if (f.two & 0x8000u) { split_int_word(f.codes.z, h.z, l.z); split_int_word(f.codes.w, h.w, l.w); }
+            store(at, h);
+            store(at + NT * 128, l);
+        };
+        fetch();
+        const uint32_t steps = (uint32_t)(u1 - u0);
+        for (uint32_t it = group; it < steps; it += 2) {
+            const uint32_t s = it % kStages, rs = it % kRaw;
+            const bool ok = mbar_wait_warp(raw_full0 + 8 * rs, (it / kRaw) & 1u) &&
+                            mbar_wait_warp(empty0 + 8 * s, ((it / kStages) & 1u) ^ 1u);
+            if (!ok) { if (lane == 0) atomicExch(p.error, 1); break; }
+            const uint8_t* codes = gemm_smem_raw + (raw0 - raw) + rs * kSkinnyRawBytes;
+            const uint32_t st = base + s * kStageBytes + 16 * i;
+#pragma unroll
+            for (int q = 0; q < kW; ++q) {
+                Piece f;
+                f.codes = *reinterpret_cast<const uint4*>(codes + 16 * (q * kThreadsD + i));
+                f.two = *reinterpret_cast<const uint16_t*>(codes + kPlaneBytes + 16 * (q * (kThreadsD / 8) + r) + 2 * c);
+                put_weights(f, st + 16 * q * kThreadsD);
+            }
+#pragma unroll
+            for (int q = 0; q < kX; ++q)
+                if (q * (kThreadsD / 8) + r < p.m) put_tokens(x[q], st + 3 * kPlaneBytes + 16 * q * kThreadsD);
+            fetch();
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");    // the MMA reads through the async proxy
+            __syncwarp();
+            if (lane == 0) { mbar_arrive(full0 + 8 * s); mbar_arrive(raw_empty0 + 8 * rs); }
+        }
+    } else {
+        // ---- B by TMA
+        int32_t tile = u0 / ksteps, k0 = u0 - tile * ksteps;
+        const uint32_t steps = (uint32_t)(u1 - u0);
+        for (uint32_t it = 0; it < steps; ++it) {
+            const uint32_t rs = it % kRaw;
+            const bool ok = mbar_wait_warp(raw_empty0 + 8 * rs, ((it / kRaw) & 1u) ^ 1u);
+            if (!ok) { if (lane == 0) atomicExch(p.error, 7); break; }
+            if (elect_one()) {
+                const uint32_t at = raw0 + rs * kSkinnyRawBytes, bar = raw_full0 + 8 * rs;
+                mbar_expect_tx(bar, kSkinnyRawBytes);
+                tma_load_2d(at, &p.w_codes, k0 * 128, tile * kTileM, bar);
+                tma_load_2d(at + kPlaneBytes, &p.w_scales, k0 * 16, tile * kTileM, bar);
+            }
+            __syncwarp();
+            if (++k0 == ksteps) { k0 = 0; ++tile; }
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_free(tmem, kTmem);
+    if (failed) return;
+
+    // ---- the tiles at the two ends of the run may be shared with other blocks: the last of a tile's blocks sums the
+    // shares in the order of K (in FP64: the shares carry all 24 bits, and this is no place to lose any)
+    const int32_t t_first = u0 / ksteps, t_last = (u1 - 1) / ksteps;
+    const bool share_first = u0 % ksteps != 0 || u1 - u0 < ksteps, share_last = t_last != t_first && u1 % ksteps != 0;
+    if (threadIdx.x == 0) {
+        __threadfence();
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            last[e] = 0;
+            if (e == 0 ? share_first : share_last) {
+                const int32_t tile = e == 0 ? t_first : t_last;
+                const int64_t bf = (((int64_t)tile * ksteps + 1) * gridDim.x - 1) / p.units;
+                const int64_t bl = (((int64_t)tile * ksteps + ksteps) * gridDim.x - 1) / p.units;
+                last[e] = atomicAdd(p.tickets + tile, 1) == (int)(bl - bf);
+            }
+        }
+        __threadfence();
+    }
+    __syncthreads();
+    int32_t done = t_last - t_first + 1 - (share_first ? 1 : 0) - (share_last ? 1 : 0);
+#pragma unroll 1
+    for (int e = 0; e < 2; ++e) {
+        if (!last[e]) continue;
+        ++done;
+        const int32_t tile = e == 0 ? t_first : t_last;
+        const int32_t bf = (int32_t)((((int64_t)tile * ksteps + 1) * gridDim.x - 1) / p.units);
+        const int32_t bl = (int32_t)((((int64_t)tile * ksteps + ksteps) * gridDim.x - 1) / p.units);
+        constexpr int kEach = 8;                                           // outputs per thread and trip
+        for (int32_t i0 = threadIdx.x; i0 < p.m * kTileM; i0 += kEach * kSkinnyThreads) {
+            double v[kEach];
+#pragma unroll
+            for (int q = 0; q < kEach; ++q) v[q] = 0.0;
+            for (int32_t b = bf; b <= bl; ++b) {
+                const float* share = p.partials + ((size_t)b * 2 + (b == bf ? 1 : 0)) * (NT * kTileM);
+#pragma unroll
+                for (int q = 0; q < kEach; ++q)
+                    if (i0 + q * kSkinnyThreads < p.m * kTileM) v[q] += (double)__ldcg(share + i0 + q * kSkinnyThreads);
+            }
+#pragma unroll
+            for (int q = 0; q < kEach; ++q) {
+                const int32_t i = i0 + q * kSkinnyThreads;
+                if (i < p.m * kTileM) write_out(i / kTileM, (size_t)tile * kTileM + i % kTileM, (float)v[q]);
+            }
+        }
+    }
+    // the global maximum of |C| as written, for the next quantizer's tensor scale (as in abs_gemm.cu); the ticket counts tiles
+    if (OUT_BF16 && p.next_alpha != nullptr) {
+        out_max = __reduce_max_sync(0xFFFFFFFFu, out_max);
+        if (lane == 0 && out_max) {
+            atomicMax(reinterpret_cast<unsigned int*>(p.error) + 1, out_max);
+            __threadfence();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && done > 0 && atomicAdd(p.error + 2, done) + done == p.n / kTileM) {
+            __threadfence();
+            const float A = __uint_as_float(atomicMax(reinterpret_cast<unsigned int*>(p.error) + 1, 0u) << 16);
+            *p.next_alpha = (A == 0.0f) ? 1.0f : __fdiv_rn(A, p.next_denom);
+        }
+    }
+}
+
+}  // namespace absq

@@ -1175,3 +1175,43 @@ def test_tensor_core_matmul_around_the_accumulation_chunks(B, oracle, fmt, m, n,
     bound = (k / 64 + 8) * 2.0 ** -24 * 1.5 * (da @ db.T)
     assert (np.abs(c.double().cpu().numpy() - ref) <= bound).all()
     assert torch.equal(B.abs_matmul(fmt, qa, qb, m, n, k, check=True, bf16=True), c.bfloat16())
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 128, 256), (8, 256, 1024), (9, 1024, 2048), (31, 128, 16384), (32, 384, 5632), (7, 2560, 256),
+                                   (32, 1024, 1024), (33, 256, 4096)])
+def test_matmul_with_few_rows(B, oracle, m, n, k):
+    """abs_matmul, IF4, around the dispatch of the few-row kernel (32 rows; 64 steps of 128 columns x 256 of K unless at most 8
+    rows): one unit, fewer units than SMs, tiles shared by many blocks, one step per tile, every row count at an edge.  The
+    bound is that of the accumulation-chunk test, plus the sums over shares of a tile."""
+    a, b = I.generate("cfg2", m, k, seed=31), I.generate("cfg3b", n, k, seed=32)
+    oa, ob = oracle.quantize(1, a, threads=THREADS), oracle.quantize(1, b, threads=THREADS)
+    ref = oracle.mac_matmul_reference(1, oa, ob, m, n, k)
+    qa, qb = B.abs_quantize(1, to_dev(a)), B.abs_quantize(1, to_dev(b))
+    guard = torch.full((m + 2, n), 7.0, dtype=torch.float32, device="cuda")
+    c = B.abs_matmul(1, qa, qb, m, n, k, out=guard, check=True)[:m]
+    assert (guard[m:] == 7.0).all()
+    da = np.abs(B.abs_dequantize(1, *qa, m, k).double().cpu().numpy())
+    db = np.abs(B.abs_dequantize(1, *qb, n, k).double().cpu().numpy())
+    assert (np.abs(c.double().cpu().numpy() - ref) <= (k / 64 + 8) * 2.0 ** -24 * 1.5 * (da @ db.T)).all()
+    c16, alpha = B.abs_matmul(1, qa, qb, m, n, k, bf16=True, next_fmt=1, check=True)
+    assert torch.equal(c16, c.bfloat16())
+    assert torch.equal(alpha, B.abs_quantize(1, c16)[2])
+
+
+def test_matmul_with_few_rows_agrees_with_the_tiled_kernel(B):
+    """The few-row kernel where blocks own whole tiles of several accumulation chunks (160 tiles, K = 8192), with random code
+    bytes (every nibble, -8 included), against the same rows of a product with more rows, which the tiled kernel computes."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    m, n, k = 32, 20480, 8192
+
+    def operand(rows):
+        codes = torch.randint(0, 256, (rows * k // 2,), generator=g, device="cuda", dtype=torch.uint8)
+        scales = torch.randint(0x20, 0x58, (rows * k // 16,), generator=g, device="cuda", dtype=torch.uint8)
+        scales |= torch.randint(0, 2, scales.shape, generator=g, device="cuda", dtype=torch.uint8) << 7
+        return codes, scales, torch.tensor([0.37], device="cuda")
+
+    qa, qb = operand(48), operand(n)
+    few = B.abs_matmul(1, (qa[0][: m * k // 2], qa[1][: m * k // 16], qa[2]), qb, m, n, k, check=True)
+    many = B.abs_matmul(1, qa, qb, 48, n, k, check=True)[:m]
+    mag = torch.mm(B.abs_dequantize(1, *qa, 48, k)[:m].abs().float(), B.abs_dequantize(1, *qb, n, k).abs().float().t())
+    assert ((few - many).abs() <= 2 * (k / 64 + 8) * 2.0 ** -24 * 1.5 * mag).all()
