@@ -1,7 +1,8 @@
 """Thin ctypes binding of ``libabs_b200.so`` (the C ABI declared in ``include/abs_b200.h``).
 
 Argument marshalling only: every step of quantize / dequantize runs in the library's CUDA
-kernels.  PyTorch supplies device memory and streams.  There is no CPU fallback -- if the
+kernels.  PyTorch supplies device memory and streams.  The calls that programs make in their
+loops go through the host module ``_abs_call`` (csrc/abs_call.cpp).  There is no CPU fallback -- if the
 library cannot be loaded, or a call fails, an exception is raised.
 """
 from __future__ import annotations
@@ -125,6 +126,26 @@ def lib():
     return _lib
 
 
+_native = None
+
+
+def _call():
+    """The host module ``_abs_call`` (csrc/abs_call.cpp), bound to the library's functions. Raises if unavailable."""
+    global _native
+    if _native is None:
+        import torch  # noqa: F401  (its libraries have to be loaded first)
+        L = lib()
+        with _lock:
+            if _native is None:
+                _build.build_call()
+                from . import _abs_call
+                _abs_call.init(*(C.cast(f, C.c_void_p).value for f in (
+                    L.abs_quantize_ex, L.abs_quantize_transposed, L.abs_quantize_dequantize, L.abs_dequantize_ex, L.abs_matmul,
+                    L.abs_matmul_bf16, L.abs_matmul_bf16_scaled, L.abs_matmul_workspace_bytes, L.abs_scales_bytes_swizzled)))
+                _native = _abs_call
+    return _native
+
+
 def status_string(status: int) -> str:
     return lib().abs_status_string(status).decode()
 
@@ -169,24 +190,7 @@ def abs_quantize(fmt: int, x, codes=None, scales=None, tensor_scale=None, opts: 
 
     Output buffers are allocated with torch when not given.  Returns (codes u8, scales u8,
     tensor_scale f32[1]); with ABS_F_ALPHA_GIVEN ``tensor_scale`` is the input alpha."""
-    import torch
-    assert x.is_cuda and x.dtype == torch.bfloat16 and x.dim() == 2 and x.is_contiguous()
-    rows, cols = x.shape
-    L = lib()
-    if codes is None:
-        codes = torch.empty(max(L.abs_codes_bytes(fmt, rows, cols), 1) if cols % 16 == 0 else 1, dtype=torch.uint8,
-                            device=x.device)
-    if scales is None:
-        if opts is not None and (opts.flags & ABS_F_SCALES_SWIZZLED):
-            scales = torch.zeros(max(L.abs_scales_bytes_swizzled(fmt, rows, cols), 1), dtype=torch.uint8, device=x.device)
-        else:
-            scales = torch.empty(max(rows * cols // FMT_GROUP[fmt], 1), dtype=torch.uint8, device=x.device)
-    if tensor_scale is None:
-        tensor_scale = torch.zeros(1, dtype=torch.float32, device=x.device)
-    with torch.cuda.device(x.device):
-        rc = L.abs_quantize_ex(fmt, x.data_ptr(), rows, cols, codes.data_ptr(), scales.data_ptr(),
-                               tensor_scale.data_ptr(), C.byref(opts) if opts is not None else None,
-                               _stream_ptr(stream))
+    rc, codes, scales, tensor_scale = (_native or _call()).quantize(fmt, x, codes, scales, tensor_scale, opts, stream)
     _check(rc, "abs_quantize")
     return codes, scales, tensor_scale
 
@@ -195,19 +199,7 @@ def abs_quantize_transposed(fmt: int, x, codes_t=None, scales_t=None, tensor_sca
                             stream=None):
     """Quantize the transpose of the CUDA bf16 matrix ``x`` [rows, cols] (groups of 16 down the columns)
     without materialising it.  Returns (codes_t u8 [cols*rows*b/8], scales_t u8 [cols*rows/16], alpha)."""
-    import torch
-    assert x.is_cuda and x.dtype == torch.bfloat16 and x.dim() == 2 and x.is_contiguous()
-    rows, cols = x.shape
-    if codes_t is None:
-        codes_t = torch.empty(max(rows * cols * FMT_BITS[fmt] // 8, 1), dtype=torch.uint8, device=x.device)
-    if scales_t is None:
-        scales_t = torch.empty(max(rows * cols // 16, 1), dtype=torch.uint8, device=x.device)
-    if tensor_scale is None:
-        tensor_scale = torch.zeros(1, dtype=torch.float32, device=x.device)
-    with torch.cuda.device(x.device):
-        rc = lib().abs_quantize_transposed(fmt, x.data_ptr(), rows, cols, codes_t.data_ptr(), scales_t.data_ptr(),
-                                           tensor_scale.data_ptr(), C.byref(opts) if opts is not None else None,
-                                           _stream_ptr(stream))
+    rc, codes_t, scales_t, tensor_scale = (_native or _call()).quantize_transposed(fmt, x, codes_t, scales_t, tensor_scale, opts, stream)
     _check(rc, "abs_quantize_transposed")
     return codes_t, scales_t, tensor_scale
 
@@ -216,18 +208,7 @@ def abs_quantize_dequantize(fmt: int, x, out=None, codes=None, scales=None, tens
                             opts: AbsOpts | None = None, stream=None):
     """Quantize the CUDA bf16 matrix ``x`` and dequantize it in the same pass (the emulation of Sec. 4.1).
     ``codes`` and ``scales`` are optional outputs (both or neither).  Returns (out bf16 [rows, cols], alpha)."""
-    import torch
-    assert x.is_cuda and x.dtype == torch.bfloat16 and x.dim() == 2 and x.is_contiguous()
-    rows, cols = x.shape
-    if out is None:
-        out = torch.empty((rows, cols), dtype=torch.bfloat16, device=x.device)
-    if tensor_scale is None:
-        tensor_scale = torch.zeros(1, dtype=torch.float32, device=x.device)
-    with torch.cuda.device(x.device):
-        rc = lib().abs_quantize_dequantize(fmt, x.data_ptr(), rows, cols, out.data_ptr(),
-                                           codes.data_ptr() if codes is not None else None,
-                                           scales.data_ptr() if scales is not None else None, tensor_scale.data_ptr(),
-                                           C.byref(opts) if opts is not None else None, _stream_ptr(stream))
+    rc, out, tensor_scale = (_native or _call()).quantize_dequantize(fmt, x, out, codes, scales, tensor_scale, opts, stream)
     _check(rc, "abs_quantize_dequantize")
     return out, tensor_scale
 
@@ -248,13 +229,7 @@ def abs_quantize_noalloc(fmt: int, x, codes, scales, tensor_scale, stream=None):
 def abs_dequantize(fmt: int, codes, scales, tensor_scale, rows: int, cols: int, out=None,
                    opts: AbsOpts | None = None, stream=None):
     """Dequantize to a CUDA bf16 matrix (float32 with ABS_F_OUT_FP32)."""
-    import torch
-    fp32 = bool(opts is not None and (opts.flags & ABS_F_OUT_FP32))
-    if out is None:
-        out = torch.empty((rows, cols), dtype=torch.float32 if fp32 else torch.bfloat16, device=codes.device)
-    with torch.cuda.device(codes.device):
-        rc = lib().abs_dequantize_ex(fmt, codes.data_ptr(), scales.data_ptr(), tensor_scale.data_ptr(), rows, cols,
-                                     out.data_ptr(), C.byref(opts) if opts is not None else None, _stream_ptr(stream))
+    rc, out = (_native or _call()).dequantize(fmt, codes, scales, tensor_scale, rows, cols, out, opts, stream)
     _check(rc, "abs_dequantize")
     return out
 
@@ -267,36 +242,17 @@ def abs_matmul(fmt: int, qa, qb, m: int, n: int, k: int, out=None, workspace=Non
     leaves the tensor scale that ``abs_quantize(next_fmt, C)`` would compute in ``next_alpha`` (a CUDA float32[1],
     allocated when not given) and the call returns (C, next_alpha).  ``check`` synchronises and raises if a wait inside
     the kernel ran out."""
-    import torch
-    L = lib()
-    need = L.abs_matmul_workspace_bytes(fmt, m, n, k)
-    if need == 0:
+    rc, *tensors = (_native or _call()).matmul(fmt, qa, qb, m, n, k, out, workspace, stream, bf16, next_fmt, next_alpha)
+    if rc == -1:
         raise AbsError(2, "abs_matmul: n a multiple of 128 and k a multiple of 256; IF4 or NVFP4")
-    if workspace is None:
-        workspace = torch.empty(need + 1024, dtype=torch.uint8, device=qa[0].device)
-    off = (-workspace.data_ptr()) % 1024
-    if out is None:
-        out = torch.empty((m, n), dtype=torch.bfloat16 if bf16 else torch.float32, device=qa[0].device)
-    assert out.dtype == (torch.bfloat16 if bf16 else torch.float32)
-    with torch.cuda.device(qa[0].device):
-        sp = _stream_ptr(stream)
-        if next_fmt is not None:
-            assert bf16
-            if next_alpha is None:
-                next_alpha = torch.zeros(1, dtype=torch.float32, device=qa[0].device)
-            rc = L.abs_matmul_bf16_scaled(fmt, qa[0].data_ptr(), qa[1].data_ptr(), qa[2].data_ptr(), qb[0].data_ptr(),
-                                          qb[1].data_ptr(), qb[2].data_ptr(), m, n, k, out.data_ptr(), next_fmt,
-                                          next_alpha.data_ptr(), workspace.data_ptr() + off, workspace.numel() - off, sp)
-            _check(rc, "abs_matmul_bf16_scaled")
-            if check:
-                _check(L.abs_matmul_check(workspace.data_ptr() + off, sp), "abs_matmul (a wait inside the kernel ran out)")
-            return out, next_alpha
-        rc = (L.abs_matmul_bf16 if bf16 else L.abs_matmul)(fmt, qa[0].data_ptr(), qa[1].data_ptr(), qa[2].data_ptr(), qb[0].data_ptr(), qb[1].data_ptr(),
-                          qb[2].data_ptr(), m, n, k, out.data_ptr(), workspace.data_ptr() + off, workspace.numel() - off, sp)
-        _check(rc, "abs_matmul")
-        if check:
-            _check(L.abs_matmul_check(workspace.data_ptr() + off, sp), "abs_matmul (a wait inside the kernel ran out)")
-    return out
+    _check(rc, "abs_matmul" if next_fmt is None else "abs_matmul_bf16_scaled")
+    if check:
+        import torch
+        workspace = tensors[1]
+        with torch.cuda.device(workspace.device):
+            rc = lib().abs_matmul_check(workspace.data_ptr() + (-workspace.data_ptr()) % 1024, _stream_ptr(stream))
+        _check(rc, "abs_matmul (a wait inside the kernel ran out)")
+    return tensors[0] if next_fmt is None else (tensors[0], tensors[2])
 
 
 def abs_amax(x, opts: AbsOpts | None = None, out=None, stream=None):

@@ -1,4 +1,4 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Builds the CUDA library in-tree with nvcc for sm_100a, and the host module that calls it with torch tensors."""
 from __future__ import annotations
 
 import os
@@ -21,15 +21,44 @@ NVCC_FLAGS = [
 ]
 
 
-def needs_build() -> bool:
-    if not os.path.exists(LIB_PATH):
+CALL_PATH = os.path.join(_HERE, "_abs_call.so")
+CALL_SOURCES = [os.path.join(CSRC, "abs_call.cpp"), os.path.join(os.path.dirname(_HERE), "include", "abs_b200.h")]
+
+
+def _older(target: str, sources) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB_PATH)
-    return any(os.path.getmtime(p) > t for p in SOURCES + HEADERS)
+    t = os.path.getmtime(target)
+    return any(os.path.getmtime(p) > t for p in sources)
+
+
+def needs_build() -> bool:
+    return _older(LIB_PATH, SOURCES + HEADERS)
+
+
+def build_call(force: bool = False) -> str:
+    """Compile the host module ``_abs_call`` (torch's C++ interface, no kernels) if it is missing or older than its sources."""
+    if not force and not _older(CALL_PATH, CALL_SOURCES):
+        return CALL_PATH
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    tmp = CALL_PATH + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd += [x for p in inc for x in ("-isystem", p)] + ["-o", tmp, CALL_SOURCES[0], "-L" + os.path.join(root, "lib")]
+    cmd += ["-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10", "-Wl,-rpath," + os.path.join(root, "lib")]
+    subprocess.run(cmd, check=True)
+    os.replace(tmp, CALL_PATH)
+    return CALL_PATH
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile libabs_b200.so if it is missing or older than its sources. Returns its path."""
+    """Compile libabs_b200.so and the host module if they are missing or older than their sources. Returns the library's path."""
+    build_call(force)
     if not force and not needs_build():
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -1215,3 +1215,55 @@ def test_matmul_with_few_rows_agrees_with_the_tiled_kernel(B):
     many = B.abs_matmul(1, qa, qb, 48, n, k, check=True)[:m]
     mag = torch.mm(B.abs_dequantize(1, *qa, 48, k)[:m].abs().float(), B.abs_dequantize(1, *qb, n, k).abs().float().t())
     assert ((few - many).abs() <= 2 * (k / 64 + 8) * 2.0 ** -24 * 1.5 * mag).all()
+
+
+def test_calls_with_given_and_with_own_buffers(B):
+    """The host module behind the calls: given buffers are used and returned, own ones have the sizes of the library, nothing is
+    written for an empty matrix (tensor scale 0), a given alpha is an input, another stream and other threads work, and
+    what the calls refuse they refuse with an exception."""
+    import threading
+    x = to_dev(I.generate("cfg1", 48, 256, seed=3))
+    codes, scales, alpha = B.abs_quantize(1, x)
+    assert codes.numel() == 48 * 128 and scales.numel() == 48 * 16 and alpha.shape == (1,)
+    given = torch.zeros_like(codes), torch.zeros_like(scales), torch.zeros_like(alpha)
+    got = B.abs_quantize(1, x, *given)
+    assert all(a.data_ptr() == b.data_ptr() for a, b in zip(got, given)) and torch.equal(got[0], codes) and torch.equal(got[2], alpha)
+    empty = torch.empty((0, 64), dtype=torch.bfloat16, device="cuda")
+    assert B.abs_quantize(1, empty)[2].item() == 0.0 and B.abs_quantize_dequantize(1, empty)[0].shape == (0, 64)
+    again = B.abs_quantize(1, x, tensor_scale=alpha, opts=B.make_opts(B.ABS_F_ALPHA_GIVEN))
+    assert torch.equal(again[0], codes) and torch.equal(again[1], scales)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    other = B.abs_quantize(1, x, stream=side)
+    side.synchronize()
+    assert torch.equal(other[0], codes)
+    results = [None] * 4
+
+    def work(i):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            results[i] = [B.abs_quantize(1, x)[0] for _ in range(50)][-1]
+            torch.cuda.current_stream().synchronize()
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    torch.cuda.synchronize()
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert all(torch.equal(r, codes) for r in results)
+    for bad in (x.float(), x.t(), x.cpu(), x[0]):
+        with pytest.raises(AssertionError):
+            B.abs_quantize(1, bad)
+    with pytest.raises(TypeError):
+        B.abs_quantize(1, x, opts=b"no options")
+    with pytest.raises(TypeError):
+        B.abs_quantize(1, [1.0])
+    with pytest.raises(KeyError):
+        B.abs_quantize(99, x)
+    with pytest.raises(B.AbsError):
+        B.abs_quantize(1, x[:, :40].contiguous())
+    with pytest.raises(B.AbsError):
+        B.abs_matmul(1, (codes, scales, alpha), (codes, scales, alpha), 48, 48, 256)
+    with pytest.raises(AssertionError):
+        B.abs_matmul(1, (codes, scales, alpha), B.abs_quantize(1, to_dev(I.generate("cfg1", 128, 256, seed=4))), 48, 128, 256,
+                     out=torch.empty((48, 128), dtype=torch.bfloat16, device="cuda"))
