@@ -26,19 +26,26 @@ constexpr int kMaxDevices = 64;
 
 // Launch with programmatic stream serialization: the kernel may be scheduled while the previous
 // kernel of the stream drains; every kernel here calls pdl_wait() before its first global access.
+// cooperative: the blocks wait for one another (one_pass_alpha), so all of them have to be resident.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
+cudaError_t launch_any(bool cooperative, void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cooperative ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
+    return launch_any(false, kernel, grid, block, s, args...);
 }
 
 // ------------------------------------------------------------------------------------------ host state
@@ -49,6 +56,7 @@ struct DeviceState {
     std::once_flag once;
     cudaError_t init_err = cudaSuccess;
     uint32_t* ring = nullptr;          // ABS_MAX_INFLIGHT slots of 16 bytes: tagged maximum (u64), ticket (u32), pad
+    unsigned long long* cells = nullptr;   // per slot kMaxCells tagged maxima, for the calls that are one kernel (5 MiB)
     std::mutex slot_mu;                // guards `next` and the clearing of the ring when the generation wraps
     uint64_t next = 0;                 // calls that took a slot so far; generation = low 32 bits
     uint32_t* overrun_host = nullptr;  // pinned, mapped word a kernel sets when its slot was reused under it
@@ -72,6 +80,8 @@ abs_status_t device_state(DeviceState** out) {
     std::call_once(st.once, [&]() {
         st.init_err = cudaMalloc(&st.ring, ABS_MAX_INFLIGHT * 4 * sizeof(uint32_t));
         if (st.init_err == cudaSuccess) st.init_err = cudaMemset(st.ring, 0, ABS_MAX_INFLIGHT * 4 * sizeof(uint32_t));
+        if (st.init_err == cudaSuccess) st.init_err = cudaMalloc(&st.cells, (size_t)ABS_MAX_INFLIGHT * kMaxCells * sizeof(unsigned long long));
+        if (st.init_err == cudaSuccess) st.init_err = cudaMemset(st.cells, 0, (size_t)ABS_MAX_INFLIGHT * kMaxCells * sizeof(unsigned long long));
         if (st.init_err == cudaSuccess) st.init_err = cudaHostAlloc(&st.overrun_host, sizeof(uint32_t), cudaHostAllocMapped);
         if (st.init_err == cudaSuccess) {
             *st.overrun_host = 0u;
@@ -145,6 +155,7 @@ abs_status_t next_slot(DeviceState& st, unsigned long long** slot, uint32_t* gen
     if (g == 0) {
         if (cudaDeviceSynchronize() != cudaSuccess) return ABS_ERR_CUDA;
         if (cudaMemset(st.ring, 0, ABS_MAX_INFLIGHT * 4 * sizeof(uint32_t)) != cudaSuccess) return ABS_ERR_CUDA;
+        if (cudaMemset(st.cells, 0, (size_t)ABS_MAX_INFLIGHT * kMaxCells * sizeof(unsigned long long)) != cudaSuccess) return ABS_ERR_CUDA;
         g = (uint32_t)++st.next;
     }
     *gen = g;
@@ -180,6 +191,22 @@ constexpr int kDeqIters = 2;   // groups per thread of the 4-bit dequantize kern
 constexpr int kFastIters = 7;   // groups per thread the IF4 round-to-nearest kernel is launched for
 constexpr int kOptIters = 12;   // same for the Hadamard / stochastic-rounding kernel
 
+// Whether a call finds its maximum inside the quantize kernel (one_pass_alpha): the format and options have a packed kernel,
+// and every group has a thread of one resident wave of it.  (1 to 2.4 million elements, by the blocks per SM that the
+// kernel is compiled for.)
+bool one_pass(int fmt, const abs_opts_t& o, int sm_count, int64_t ngroups, bool emulate) {
+    const bool rht = o.flags & ABS_F_HADAMARD16, sr = o.flags & ABS_F_STOCHASTIC;
+    int per_sm = 0;
+    switch (fmt) {
+        case ABS_FMT_NVFP4: case ABS_FMT_IF4: per_sm = (rht || sr || emulate) ? opt_blocks_per_sm(sr, rht) : kFastMinBlocks; break;
+        case ABS_FMT_NVFP4_BS8: case ABS_FMT_IF4_BS8: per_sm = (rht || sr) ? 0 : 4; break;
+        default: per_sm = (rht || sr) ? 0 : 3; break;       // IF3, IF6
+    }
+    int64_t blocks = (int64_t)sm_count * per_sm;
+    if (blocks > kMaxCells) blocks = kMaxCells;
+    return !(o.flags & ABS_F_INDEX64) && (ngroups + kThreads - 1) / kThreads <= blocks;
+}
+
 template <int FMT>
 // emul_out != nullptr asks for the emulation pass (abs_quantize_dequantize) of the formats handled by the
 // kernels of abs_fastx.cuh: bf16 output, codes stored only when emul_store.  *handled tells the caller whether
@@ -210,23 +237,27 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
             // L2 prefetch ahead of the loads unless the amax pass of this call has just streamed an input that
             // fits the L2 (about 100 MB of the 126 MB stay resident behind a streaming read)
             const bool pf = !alpha.slot || ngroups * 32 > (int64_t)96 << 20;
-#define ABS_LAUNCH_F3(IDX, A32, SLOT, MUL)                                                                           \
-    e = swz ? launch_pdl(quantize4_fast_kernel<kInt, IDX, A32, SLOT, MUL, true>, pgrid, kThreads, s,                  \
-                         (const uint4*)in, (uint2*)codes, (uint8_t*)scales, alpha, (IDX)ngroups, gpr, ktiles, pf)     \
-            : launch_pdl(quantize4_fast_kernel<kInt, IDX, A32, SLOT, MUL, false>, pgrid, kThreads, s,                 \
-                         (const uint4*)in, (uint2*)codes, (uint8_t*)scales, alpha, (IDX)ngroups, gpr, ktiles, pf)
+#define ABS_LAUNCH_F3(IDX, A32, SRC, MUL)                                                                            \
+    e = launch_any(SRC == kOnePass, swz ? quantize4_fast_kernel<kInt, IDX, A32, SRC, MUL, true>                       \
+                                        : quantize4_fast_kernel<kInt, IDX, A32, SRC, MUL, false>, pgrid, kThreads, s, \
+                   (const uint4*)in, (uint2*)codes, (uint8_t*)scales, alpha, (IDX)ngroups, gpr, ktiles, pf)
+#define ABS_LAUNCH_F2(IDX, A32, SRC)                                                                                 \
+    do {                                                                                                             \
+        if (mul != 1.0f) ABS_LAUNCH_F3(IDX, A32, SRC, true);                                                         \
+        else ABS_LAUNCH_F3(IDX, A32, SRC, false);                                                                    \
+    } while (0)
 #define ABS_LAUNCH_F(IDX, A32)                                                                                       \
     do {                                                                                                             \
-        if (alpha.slot && mul != 1.0f) ABS_LAUNCH_F3(IDX, A32, true, true);                                          \
-        else if (alpha.slot) ABS_LAUNCH_F3(IDX, A32, true, false);                                                   \
-        else if (mul != 1.0f) ABS_LAUNCH_F3(IDX, A32, false, true);                                                  \
-        else ABS_LAUNCH_F3(IDX, A32, false, false);                                                                  \
+        if (alpha.cells) ABS_LAUNCH_F2(int32_t, A32, kOnePass);      /* few groups: always 32-bit indices */          \
+        else if (alpha.slot) ABS_LAUNCH_F2(IDX, A32, kFromSlot);                                                     \
+        else ABS_LAUNCH_F2(IDX, A32, kGiven);                                                                        \
     } while (0)
             if (i32 && a32) ABS_LAUNCH_F(int32_t, true);
             else if (i32) ABS_LAUNCH_F(int32_t, false);
             else if (a32) ABS_LAUNCH_F(int64_t, true);
             else ABS_LAUNCH_F(int64_t, false);
 #undef ABS_LAUNCH_F
+#undef ABS_LAUNCH_F2
 #undef ABS_LAUNCH_F3
             if (e != cudaSuccess) return ABS_ERR_CUDA;
             if (g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
@@ -241,12 +272,11 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             cudaError_t e;
 #define ABS_LAUNCH_O(R, S)                                                                                        \
-    e = alpha.slot ? launch_pdl(quantize4_opt_kernel<kInt, R, S, true, false>, ogrid, kThreads, s, (const uint4*)in, \
-                                (uint2*)codes, (uint8_t*)scales, alpha, (int32_t)ngroups, mul,                    \
-                                (uint32_t)o.had_sign_mask, pk, ctr, a32, (uint4*)nullptr, false, true)             \
-                   : launch_pdl(quantize4_opt_kernel<kInt, R, S, false, false>, ogrid, kThreads, s, (const uint4*)in, \
-                                (uint2*)codes, (uint8_t*)scales, alpha, (int32_t)ngroups, mul,                    \
-                                (uint32_t)o.had_sign_mask, pk, ctr, a32, (uint4*)nullptr, false, true)
+    e = launch_any(alpha.cells != nullptr, alpha.cells ? quantize4_opt_kernel<kInt, R, S, kOnePass, false>         \
+                                           : alpha.slot ? quantize4_opt_kernel<kInt, R, S, kFromSlot, false>       \
+                                                        : quantize4_opt_kernel<kInt, R, S, kGiven, false>,         \
+                   ogrid, kThreads, s, (const uint4*)in, (uint2*)codes, (uint8_t*)scales, alpha, (int32_t)ngroups, mul, \
+                   (uint32_t)o.had_sign_mask, pk, ctr, a32, (uint4*)nullptr, false, true)
             if (rht && sr) ABS_LAUNCH_O(true, true);
             else if (rht) ABS_LAUNCH_O(true, false);
             else ABS_LAUNCH_O(false, true);
@@ -263,13 +293,10 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
         if (!rht && !sr && !(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)bgrid * kThreads) {
             if (handled) *handled = true;
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
-            const cudaError_t e =
-                alpha.slot ? (emul_out ? launch_pdl(quantize4_bs8_kernel<kInt, true, true>, bgrid, kThreads, s, (const uint4*)in, (uint2*)codes,
-                                        (uint16_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store) : launch_pdl(quantize4_bs8_kernel<kInt, true, false>, bgrid, kThreads, s, (const uint4*)in, (uint2*)codes,
-                                        (uint16_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)nullptr, false, true))
-                           : (emul_out ? launch_pdl(quantize4_bs8_kernel<kInt, false, true>, bgrid, kThreads, s, (const uint4*)in, (uint2*)codes,
-                                        (uint16_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store) : launch_pdl(quantize4_bs8_kernel<kInt, false, false>, bgrid, kThreads, s, (const uint4*)in, (uint2*)codes,
-                                        (uint16_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)nullptr, false, true));
+            const auto kernel = emul_out ? (alpha.cells ? quantize4_bs8_kernel<kInt, kOnePass, true> : alpha.slot ? quantize4_bs8_kernel<kInt, kFromSlot, true> : quantize4_bs8_kernel<kInt, kGiven, true>)
+                                         : (alpha.cells ? quantize4_bs8_kernel<kInt, kOnePass, false> : alpha.slot ? quantize4_bs8_kernel<kInt, kFromSlot, false> : quantize4_bs8_kernel<kInt, kGiven, false>);
+            const cudaError_t e = launch_any(alpha.cells != nullptr, kernel, bgrid, kThreads, s, (const uint4*)in, (uint2*)codes, (uint16_t*)scales, alpha,
+                                             (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
             if (e != cudaSuccess) return ABS_ERR_CUDA;
             if (g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
             return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
@@ -281,13 +308,10 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
         if (!rht && !sr && !(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)sgrid * kThreads) {
             if (handled) *handled = true;
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
-            const cudaError_t e =
-                alpha.slot ? (emul_out ? launch_pdl(quantize6_fast_kernel<FMT, true, true>, sgrid, kThreads, s, (const uint4*)in, (uint32_t*)codes,
-                                        (uint8_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store) : launch_pdl(quantize6_fast_kernel<FMT, true, false>, sgrid, kThreads, s, (const uint4*)in, (uint32_t*)codes,
-                                        (uint8_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)nullptr, false, true))
-                           : (emul_out ? launch_pdl(quantize6_fast_kernel<FMT, false, true>, sgrid, kThreads, s, (const uint4*)in, (uint32_t*)codes,
-                                        (uint8_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store) : launch_pdl(quantize6_fast_kernel<FMT, false, false>, sgrid, kThreads, s, (const uint4*)in, (uint32_t*)codes,
-                                        (uint8_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)nullptr, false, true));
+            const auto kernel = emul_out ? (alpha.cells ? quantize6_fast_kernel<FMT, kOnePass, true> : alpha.slot ? quantize6_fast_kernel<FMT, kFromSlot, true> : quantize6_fast_kernel<FMT, kGiven, true>)
+                                         : (alpha.cells ? quantize6_fast_kernel<FMT, kOnePass, false> : alpha.slot ? quantize6_fast_kernel<FMT, kFromSlot, false> : quantize6_fast_kernel<FMT, kGiven, false>);
+            const cudaError_t e = launch_any(alpha.cells != nullptr, kernel, sgrid, kThreads, s, (const uint4*)in, (uint32_t*)codes, (uint8_t*)scales, alpha,
+                                             (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
             if (e != cudaSuccess) return ABS_ERR_CUDA;
             if (g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
             return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
@@ -300,13 +324,10 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
         if (!rht && !sr && !(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)tgrid * kThreads) {
             if (handled) *handled = true;
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
-            const cudaError_t e =
-                alpha.slot ? (emul_out ? launch_pdl(quantize3_fast_kernel<kG, true, true>, tgrid, kThreads, s, (const uint4*)in, (uint16_t*)codes,
-                                        (uint8_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store) : launch_pdl(quantize3_fast_kernel<kG, true, false>, tgrid, kThreads, s, (const uint4*)in, (uint16_t*)codes,
-                                        (uint8_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)nullptr, false, true))
-                           : (emul_out ? launch_pdl(quantize3_fast_kernel<kG, false, true>, tgrid, kThreads, s, (const uint4*)in, (uint16_t*)codes,
-                                        (uint8_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store) : launch_pdl(quantize3_fast_kernel<kG, false, false>, tgrid, kThreads, s, (const uint4*)in, (uint16_t*)codes,
-                                        (uint8_t*)scales, alpha, (int32_t)ngroups, mul, a32, (uint4*)nullptr, false, true));
+            const auto kernel = emul_out ? (alpha.cells ? quantize3_fast_kernel<kG, kOnePass, true> : alpha.slot ? quantize3_fast_kernel<kG, kFromSlot, true> : quantize3_fast_kernel<kG, kGiven, true>)
+                                         : (alpha.cells ? quantize3_fast_kernel<kG, kOnePass, false> : alpha.slot ? quantize3_fast_kernel<kG, kFromSlot, false> : quantize3_fast_kernel<kG, kGiven, false>);
+            const cudaError_t e = launch_any(alpha.cells != nullptr, kernel, tgrid, kThreads, s, (const uint4*)in, (uint16_t*)codes, (uint8_t*)scales, alpha,
+                                             (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
             if (e != cudaSuccess) return ABS_ERR_CUDA;
             if (g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
             return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
@@ -592,18 +613,21 @@ abs_status_t abs_quantize_ex(abs_fmt_t fmt, const void* in_bf16, int64_t rows, i
     if (device_state(&st) != ABS_OK) return ABS_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t ngroups = rows * cols / 16;
-    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr};
+    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr};
     if (!(o.flags & ABS_F_ALPHA_GIVEN)) {
         unsigned long long* slot = nullptr;
         uint32_t gen = 0;
         if ((rc = next_slot(*st, &slot, &gen)) != ABS_OK) return rc;
-        const float denom = fmt_mfp((int)fmt) * 448.0f;
-        rc = launch_amax(st->sm_count, in_bf16, ngroups, o, false, slot, gen, tensor_scale_f32, denom, s);
-        if (rc != ABS_OK) return rc;
-        src.slot = slot;
         src.gen = gen;
-        src.denom = denom;
+        src.denom = fmt_mfp((int)fmt) * 448.0f;
         src.overrun = st->overrun_dev;
+        if (one_pass(fmt, o, st->sm_count, ngroups, false)) {
+            src.cells = st->cells + (size_t)(gen % ABS_MAX_INFLIGHT) * kMaxCells;
+        } else {
+            rc = launch_amax(st->sm_count, in_bf16, ngroups, o, false, slot, gen, tensor_scale_f32, src.denom, s);
+            if (rc != ABS_OK) return rc;
+            src.slot = slot;
+        }
     }
     switch (fmt) {
         case ABS_FMT_NVFP4: return launch_quantize_fmt<0>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
@@ -651,18 +675,21 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
     const bool rht = o.flags & ABS_F_HADAMARD16, sr = o.flags & ABS_F_STOCHASTIC;
     const int grid = grid_waves(st->sm_count, ngroups, opt_blocks_per_sm(sr, rht), (rht || sr) ? kOptIters : kFastIters);
     if (ngroups >= (int64_t)0x7FFFFFFF - (int64_t)grid * kThreads) return ABS_ERR_SIZE;    // 32-bit group indices only
-    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr};
+    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr};
     if (!(o.flags & ABS_F_ALPHA_GIVEN)) {
         unsigned long long* slot = nullptr;
         uint32_t gen = 0;
         if ((rc = next_slot(*st, &slot, &gen)) != ABS_OK) return rc;
-        const float denom = fmt_mfp((int)fmt) * 448.0f;
-        rc = launch_amax(st->sm_count, in_bf16, ngroups, o, false, slot, gen, tensor_scale_f32, denom, s);
-        if (rc != ABS_OK) return rc;
-        src.slot = slot;
         src.gen = gen;
-        src.denom = denom;
+        src.denom = fmt_mfp((int)fmt) * 448.0f;
         src.overrun = st->overrun_dev;
+        if (one_pass(fmt, o, st->sm_count, ngroups, true)) {
+            src.cells = st->cells + (size_t)(gen % ABS_MAX_INFLIGHT) * kMaxCells;
+        } else {
+            rc = launch_amax(st->sm_count, in_bf16, ngroups, o, false, slot, gen, tensor_scale_f32, src.denom, s);
+            if (rc != ABS_OK) return rc;
+            src.slot = slot;
+        }
     }
     const bool store = codes_u8 != nullptr;
     if (!four_bit) {
@@ -682,15 +709,12 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
     const PhiloxKeys pk = philox_keys(o.sr_seed);
     const bool a32 = (reinterpret_cast<uintptr_t>(in_bf16) & 31u) == 0, o32 = (reinterpret_cast<uintptr_t>(out_bf16) & 31u) == 0;
     cudaError_t e = cudaSuccess;
-#define ABS_LAUNCH_E3(I, R, S, SLOT)                                                                                \
-    e = launch_pdl(quantize4_opt_kernel<I, R, S, SLOT, true>, grid, kThreads, s, (const uint4*)in_bf16, (uint2*)codes_u8, \
-                   (uint8_t*)scales_e4m3, src, (int32_t)ngroups, mul, (uint32_t)o.had_sign_mask, pk, ctr, a32,       \
-                   (uint4*)out_bf16, o32, store)
 #define ABS_LAUNCH_E2(I, R, S)                                                                                      \
-    do {                                                                                                            \
-        if (src.slot) ABS_LAUNCH_E3(I, R, S, true);                                                                 \
-        else ABS_LAUNCH_E3(I, R, S, false);                                                                         \
-    } while (0)
+    e = launch_any(src.cells != nullptr, src.cells ? quantize4_opt_kernel<I, R, S, kOnePass, true>                   \
+                                         : src.slot ? quantize4_opt_kernel<I, R, S, kFromSlot, true>                 \
+                                                    : quantize4_opt_kernel<I, R, S, kGiven, true>, grid, kThreads, s, \
+                   (const uint4*)in_bf16, (uint2*)codes_u8, (uint8_t*)scales_e4m3, src, (int32_t)ngroups, mul,        \
+                   (uint32_t)o.had_sign_mask, pk, ctr, a32, (uint4*)out_bf16, o32, store)
 #define ABS_LAUNCH_E(I)                                                                                             \
     do {                                                                                                            \
         if (rht && sr) ABS_LAUNCH_E2(I, true, true);                                                                \
@@ -702,7 +726,6 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
     else ABS_LAUNCH_E(false);
 #undef ABS_LAUNCH_E
 #undef ABS_LAUNCH_E2
-#undef ABS_LAUNCH_E3
     return (e == cudaSuccess && cudaGetLastError() == cudaSuccess) ? ABS_OK : ABS_ERR_CUDA;
 }
 
@@ -792,7 +815,7 @@ static abs_status_t quantize_transposed_impl(abs_fmt_t fmt, const void* in_bf16,
     const float mul = (o.flags & ABS_F_SR_SCALE_17_16) ? 1.0625f : 1.0f;
     const uint64_t ctr = o.sr_index_offset / 8;
     const PhiloxKeys pk = philox_keys(o.sr_seed);
-    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr};
+    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr};
     if (!(o.flags & ABS_F_ALPHA_GIVEN)) {
         unsigned long long* slot = nullptr;
         uint32_t gen = 0;
@@ -867,7 +890,7 @@ abs_status_t abs_quantize_noalloc(abs_fmt_t fmt, const void* in_bf16, int64_t ro
                                                         fmt_mfp((int)fmt) * 448.0f);
     if (cudaGetLastError() != cudaSuccess) return ABS_ERR_CUDA;
     const abs_opts_t o = {0, 0, 0, 0, 0};
-    const AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr};   // alpha was written by the chunked pass
+    const AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr};   // alpha was written by the chunked pass
     switch (fmt) {
         case ABS_FMT_NVFP4: return launch_quantize_fmt<0>(na.sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
         case ABS_FMT_IF4: return launch_quantize_fmt<1>(na.sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);

@@ -142,10 +142,11 @@ constexpr int kFastMinBlocks = 4;   // resident blocks of 256 threads per SM the
 // grid as a few waves of resident blocks) and fetches the next group's 32 bytes before it works on the
 // current one, so loads stay in flight under the math.
 // IdxT is int32_t whenever the group count allows it (shorter address arithmetic).
-template <bool HAS_INT, typename IdxT, bool ALIGNED32, bool FROM_SLOT, bool SCALE_MUL, bool SWZ>
+template <bool HAS_INT, typename IdxT, bool ALIGNED32, int SRC, bool SCALE_MUL, bool SWZ>
 __global__ void __launch_bounds__(256, HAS_INT ? kFastMinBlocks : 5)
 quantize4_fast_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, uint8_t* __restrict__ scales,
                       const AlphaSrc alpha_src, IdxT ngroups, uint32_t gpr, uint32_t ktiles, bool l2_prefetch) {
+    constexpr bool FROM_SLOT = SRC == kFromSlot;
     pdl_launch_dependents();
     const IdxT stride = (IdxT)(gridDim.x * blockDim.x);
     IdxT g = (IdxT)(blockIdx.x * blockDim.x + threadIdx.x);
@@ -160,7 +161,7 @@ quantize4_fast_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, u
     // instance is bound by arithmetic and measured 1 % slower that way, so it walks forwards.
     auto at = [&](IdxT gg) -> IdxT { return (FROM_SLOT && !HAS_INT) ? (IdxT)(ngroups - 1 - gg) : gg; };
     if (active) load32B<ALIGNED32>(in + 2 * (size_t)at(g), w);
-    const float alpha = resolve_alpha_per_thread<FROM_SLOT>(alpha_src);      // T2
+    const float alpha = alpha_of<SRC>(alpha_src, w, active);                 // T2
     // G5 once per block for every scale byte 0x00..0x7E: d = Delta * alpha, 1 / d, d * 6/7 (8192x4096: 16.68 -> 16.56 us)
     __shared__ float4 scale_lut[128];
     if (threadIdx.x < 127) {

@@ -138,7 +138,7 @@ __device__ __forceinline__ void encode_half4(const float* x, uint32_t sb, float 
 // EMUL (all kernels of this file): the emulation pass of Sec. 4.1, as in quantize4_opt_kernel: the group is decoded
 // from the registers that hold its codes and scale and written to `out` as bf16; codes and scale bytes are
 // stored only when `store_codes` is set.
-template <bool HAS_INT, bool FROM_SLOT, bool EMUL = false>
+template <bool HAS_INT, int SRC, bool EMUL = false>
 __global__ void __launch_bounds__(256, HAS_INT ? 4 : 5)
 quantize4_bs8_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, uint16_t* __restrict__ scales,
                      const AlphaSrc alpha_src, int32_t nblocks16, float scale_mul, bool aligned32,
@@ -154,7 +154,7 @@ quantize4_bs8_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
         if (aligned32) load32B<true>(in + 2 * (size_t)g, w);
         else load32B<false>(in + 2 * (size_t)g, w);
     }
-    const float alpha = resolve_alpha_per_thread<FROM_SLOT>(alpha_src);      // T2
+    const float alpha = alpha_of<SRC>(alpha_src, w, active);                 // T2
     __shared__ float2 scale_table[128];
     fill_scale_table(scale_table, alpha);                                    // G5 for every scale byte, once per block
     if (!active) return;
@@ -322,7 +322,7 @@ __device__ __forceinline__ void encode_body6(const float (&x)[16], uint32_t sb, 
     sbyte = sb | (flag ? 0x80u : 0u);                                           // S3
 }
 
-template <int FMT, bool FROM_SLOT, bool EMUL = false>
+template <int FMT, int SRC, bool EMUL = false>
 __global__ void __launch_bounds__(256, 3)
 quantize6_fast_kernel(const uint4* __restrict__ in, uint32_t* __restrict__ codes, uint8_t* __restrict__ scales,
                       const AlphaSrc alpha_src, int32_t ngroups, float scale_mul, bool aligned32,
@@ -339,7 +339,7 @@ quantize6_fast_kernel(const uint4* __restrict__ in, uint32_t* __restrict__ codes
         if (aligned32) load32B<true>(in + 2 * (size_t)g, w);
         else load32B<false>(in + 2 * (size_t)g, w);
     }
-    const float alpha = resolve_alpha_per_thread<FROM_SLOT>(alpha_src);      // T2
+    const float alpha = alpha_of<SRC>(alpha_src, w, active);                 // T2
     if (!active) return;
     const float inv_a6 = __frcp_rn(__fmul_rn(alpha, F::M_FP));               // T3
     const float c_pre = __fdiv_rn(F::M_INT, F::M_FP), c_post = __fdiv_rn(F::M_FP, F::M_INT);
@@ -511,7 +511,7 @@ __device__ __forceinline__ void encode_body3(const float (&x)[16], const uint32_
 constexpr int kIf3MinBlocks = 3;   // resident blocks of 256 threads per SM the IF3 kernel is compiled for
 
 // G = 16: one scale per thread's 16 values.  G = 8 (IF3-BS8): each half has its own scale and selection.
-template <int G, bool FROM_SLOT, bool EMUL = false>
+template <int G, int SRC, bool EMUL = false>
 __global__ void __launch_bounds__(256, kIf3MinBlocks)
 quantize3_fast_kernel(const uint4* __restrict__ in, uint16_t* __restrict__ codes, uint8_t* __restrict__ scales,
                       const AlphaSrc alpha_src, int32_t ngroups, float scale_mul, bool aligned32,
@@ -527,7 +527,7 @@ quantize3_fast_kernel(const uint4* __restrict__ in, uint16_t* __restrict__ codes
         if (aligned32) load32B<true>(in + 2 * (size_t)g, w);
         else load32B<false>(in + 2 * (size_t)g, w);
     }
-    const float alpha = resolve_alpha_per_thread<FROM_SLOT>(alpha_src);      // T2
+    const float alpha = alpha_of<SRC>(alpha_src, w, active);                 // T2
     if (!active) return;
     const float inv_a6 = __frcp_rn(__fmul_rn(alpha, 4.0f));                  // T3
     // one block of 16 values held in `w`, index `g`

@@ -172,7 +172,7 @@ constexpr int opt_blocks_per_sm(bool sr, bool rht = true) { return sr ? 2 : (rht
 // quantizing): the group is decoded from the registers that hold its codes and scale, with the arithmetic of
 // the dequantize kernel, and written to `out` as bf16; codes and scale bytes are stored only when
 // `store_codes` is set.
-template <bool HAS_INT, bool RHT, bool SR, bool FROM_SLOT, bool EMUL>
+template <bool HAS_INT, bool RHT, bool SR, int SRC, bool EMUL>
 __global__ void __launch_bounds__(256, opt_blocks_per_sm(SR, RHT))
 quantize4_opt_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, uint8_t* __restrict__ scales,
                      const AlphaSrc alpha_src, int32_t ngroups, float scale_mul, uint32_t sign_mask,
@@ -189,15 +189,27 @@ quantize4_opt_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
         if (aligned32) load32B<true>(in + 2 * (size_t)g, w);
         else load32B<false>(in + 2 * (size_t)g, w);
     }
-    const float alpha = resolve_alpha_per_thread<FROM_SLOT>(alpha_src);      // T2
-    __shared__ float2 scale_table[128];
-    fill_scale_table(scale_table, alpha);                                    // G5 for every scale byte, once per block
-    if (!active) return;
-    const float inv_a6 = __frcp_rn(__fmul_rn(alpha, 6.0f));                  // T3
     uint32_t smask[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
         smask[i] = (((sign_mask >> (2 * i)) & 1u) << 15) | (((sign_mask >> (2 * i + 1)) & 1u) << 31);
+    float alpha;                                                             // T2
+    if constexpr (SRC == kOnePass && RHT) {
+        float m = 0.0f;
+        if (active) {
+            float x[16];
+            hadamard16_packed(w, smask, x);
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) m = max3abs(m, x[i], x[i + 1]);
+        }
+        alpha = one_pass_alpha(alpha_src, __float_as_uint(m));
+    } else {
+        alpha = alpha_of<SRC>(alpha_src, w, active);
+    }
+    __shared__ float2 scale_table[128];
+    fill_scale_table(scale_table, alpha);                                    // G5 for every scale byte, once per block
+    if (!active) return;
+    const float inv_a6 = __frcp_rn(__fmul_rn(alpha, 6.0f));                  // T3
     while (true) {
         const int32_t gn = g + stride;
         const bool more = gn < ngroups;

@@ -1267,3 +1267,28 @@ def test_calls_with_given_and_with_own_buffers(B):
     with pytest.raises(AssertionError):
         B.abs_matmul(1, (codes, scales, alpha), B.abs_quantize(1, to_dev(I.generate("cfg1", 128, 256, seed=4))), 48, 128, 256,
                      out=torch.empty((48, 128), dtype=torch.bfloat16, device="cuda"))
+
+
+@pytest.mark.parametrize("fmt,flags", [(f, 0) for f in ALL_FMTS] + [(0, 1), (1, 1), (1, 2), (1, 7), (1, 64)])
+def test_one_kernel_quantize_agrees_with_the_two_kernel_route(B, fmt, flags):
+    """Tensors whose groups fit one resident wave are quantized by one kernel that finds the maximum itself; others, and all calls
+    with a given alpha, are not.  Bytes and alpha must agree with abs_amax followed by a call with that alpha: one group, one
+    block less one group, several blocks, a block of one group, the whole wave and one group more, 16-byte aligned input."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g = torch.Generator(device="cuda").manual_seed(fmt * 100 + flags)
+    for groups, shift in ((1, 0), (255, 0), (2049, 8), (37889, 0), (2 * sms * 256, 8), (3 * sms * 256, 0), (4 * sms * 256, 8),
+                          (4 * sms * 256 + 1, 0), (5 * sms * 256 + 3, 8)):
+        flat = torch.randn(groups * 16 + shift, generator=g, device="cuda").bfloat16()
+        flat[shift + groups * 16 - 1] = 9.0
+        x = flat[shift:].view(groups, 16)
+        opts = B.make_opts(flags, 0x5A3C, 17)
+        codes, scales, alpha = B.abs_quantize(fmt, x, opts=opts)
+        amax = B.abs_amax(x, opts=B.make_opts(flags & B.ABS_F_HADAMARD16, 0x5A3C))
+        want = torch.tensor([B.abs_alpha_from_amax(fmt, amax.item())], device="cuda")
+        assert torch.equal(alpha, want), (groups, shift)
+        ref = B.abs_quantize(fmt, x, tensor_scale=want, opts=B.make_opts(flags | B.ABS_F_ALPHA_GIVEN, 0x5A3C, 17))
+        assert torch.equal(codes, ref[0]) and torch.equal(scales, ref[1]), (groups, shift)
+        if not flags & B.ABS_F_SCALES_SWIZZLED:
+            out, alpha2 = B.abs_quantize_dequantize(fmt, x, opts=opts)
+            assert torch.equal(alpha2, want)
+            assert torch.equal(out.view(torch.int16), B.abs_dequantize(fmt, codes, scales, alpha, groups, 16).view(torch.int16)), (groups, shift)
