@@ -34,6 +34,7 @@ constexpr uint32_t kSkinnySfSlots = 4, kSkinnySlotCols = 32;              // 16 
 // Steps of B as it lies, and steps of planes, in shared memory: decoding a step, the hand-over and its MMAs take about as
 // long as two steps, so there are three stages of planes.
 constexpr int kSkinnyRaw = 3, kSkinnyStages = 3;
+static_assert(kSkinnyRaw == kSkinnyStages, "the decoders' waits rely on it");
 constexpr int kSkinnyRawBytes = kPlaneBytes + kTileM * 16;                // codes, then 16 scale bytes per row
 constexpr int kSkinnyStageBytes = 3 * kPlaneBytes + 2 * kSkinnyTok * 128; // F, Y, X of B; H, L of A
 constexpr int kSkinnySmemBytes = kSkinnyStages * kSkinnyStageBytes + kSkinnyRaw * kSkinnyRawBytes + 1024 + 512;
@@ -304,8 +305,12 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
         const uint32_t steps = (uint32_t)(u1 - u0);
         for (uint32_t it = group; it < steps; it += 2) {
             const uint32_t s = it % kStages, rs = it % kRaw;
-            const bool ok = mbar_wait_warp(raw_full0 + 8 * rs, (it / kRaw) & 1u) &&
-                            mbar_wait_warp(empty0 + 8 * s, ((it / kStages) & 1u) ^ 1u);
+            // The order matters.  This group sees only every second phase of raw_full[rs], always with the same parity, and a
+            // parity wait also passes two phases early: while the load of step it - 3 (the other group's) has not landed.  The
+            // wait on empty, for the MMAs of step it - 3, rules that out; it is itself covered by the one of step it - 2, since
+            // MMAs complete in order.  A wait that skips phases of its barrier needs one before it that does not.
+            const bool ok = mbar_wait_warp(empty0 + 8 * s, ((it / kStages) & 1u) ^ 1u) &&
+                            mbar_wait_warp(raw_full0 + 8 * rs, (it / kRaw) & 1u);
             if (!ok) { if (lane == 0) atomicExch(p.error, 1); break; }
             const uint8_t* codes = gemm_smem_raw + (raw0 - raw) + rs * kSkinnyRawBytes;
             const uint32_t st = base + s * kStageBytes + 16 * i;

@@ -1,0 +1,191 @@
+"""The hand-over of the few-row product kernel (csrc/abs_skinny.cuh), modelled on the CPU: warps, barriers with phases and
+parities, loads that land whenever they like, MMAs that complete in order.
+
+The model's constants and the order in which each role waits are read from the source; what each role does between its waits
+is stated here.  A parity wait passes when the phase before the current one has the parity asked for, so a role that
+does not visit every phase of a barrier can pass two phases early; the model shows such a pass as a read of another step's data.
+"""
+import heapq
+import os
+import random
+import re
+
+import pytest
+
+SOURCE = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2603_28765_b200", "csrc", "abs_skinny.cuh")
+ROLES = {"mma": "// ---- MMAs", "scales": "// ---- scales and epilogue", "codes": "// ---- codes", "loads": "// ---- B by TMA", "end": "// ---- the tiles at"}
+
+
+def protocol():
+    """Constants of the kernel and, per role, the barriers it waits on in the order of the text."""
+    text = open(SOURCE).read()
+    const = {name: int(re.search(rf"\b{name} = (\d+)", text).group(1)) for name in ("kSkinnyDecWarps", "kSkinnySfSlots", "kSkinnyRaw", "kSkinnyStages")}
+    at = [text.index(mark) for mark in ROLES.values()]
+    waits = {role: re.findall(r"mbar_wait(?:_warp)?\((\w+?)0?\b(?: \+|,)", text[a:b]) for role, a, b in zip(ROLES, at, at[1:])}
+    return const, waits
+
+
+class Barrier:
+    def __init__(self, count):
+        self.count, self.pending, self.phases, self.waiting = count, count, 0, []
+
+    def passes(self, parity):
+        return self.phases % 2 != parity
+
+
+class Model:
+    """One block over `steps` K-steps in spans of `span` steps.  delay(role, step) draws how long a piece of work takes."""
+
+    def __init__(self, steps, span, delay, decoder_waits=None):
+        self.const, self.waits = protocol()
+        assert sorted(self.waits["mma"]) == ["acc_empty", "full", "sf_full"] and self.waits["loads"] == ["raw_empty"]
+        assert sorted(self.waits["scales"]) == ["acc_full", "raw_full", "sf_empty"] and sorted(self.waits["codes"]) == ["empty", "raw_full"]
+        self.decoder_waits = decoder_waits or self.waits["codes"]
+        self.steps, self.span, self.delay = steps, span, delay
+        dec, self.raw_n, self.stage_n, self.slot_n = (self.const[k] for k in ("kSkinnyDecWarps", "kSkinnyRaw", "kSkinnyStages", "kSkinnySfSlots"))
+        self.dec = dec
+        bar = lambda n, count: [Barrier(count) for _ in range(n)]                              # noqa: E731
+        self.bars = {"raw_full": bar(self.raw_n, 1), "raw_empty": bar(self.raw_n, dec // 2 + 4), "full": bar(self.stage_n, dec // 2),
+                     "empty": bar(self.stage_n, 1), "sf_full": bar(self.slot_n, 4), "sf_empty": bar(self.slot_n, 1),
+                     "acc_full": bar(1, 1), "acc_empty": bar(1, 4)}
+        self.raw = [None] * self.raw_n                                  # step whose bytes the raw stage holds
+        self.planes = [[None] * (dec // 2) for _ in range(self.stage_n)]
+        self.slots = [[None] * 4 for _ in range(self.slot_n)]
+        self.acc, self.wrong, self.now, self.queue, self.serial = None, [], 0, [], 0
+        self.mma_free = 0
+
+    # barrier, index and parity of a wait of step `it` (accumulator barriers: of span `it`)
+    def wait(self, name, it):
+        n = len(self.bars[name])
+        return self.bars[name][it % n], (it // n) % 2 if name.endswith("full") else (it // n) % 2 ^ 1
+
+    def expect(self, what, got, it):
+        if got != it:
+            self.wrong.append((what, it, got))
+
+    def at(self, time, action):
+        self.serial += 1
+        heapq.heappush(self.queue, (time, self.serial, action))
+
+    def arrive(self, bar):
+        bar.pending -= 1
+        if bar.pending == 0:
+            bar.pending, bar.phases = bar.count, bar.phases + 1
+            waiting, bar.waiting = bar.waiting, []
+            for process, parity in waiting:
+                if bar.passes(parity):
+                    self.at(self.now, lambda p=process: self.resume(p))
+                else:
+                    bar.waiting.append((process, parity))
+
+    def resume(self, process):
+        for kind, *what in process:                                     # generator: runs on until it has to wait
+            if kind == "delay":
+                self.at(self.now + what[0], lambda: self.resume(process))
+                return
+            bar, parity = what
+            if not bar.passes(parity):
+                bar.waiting.append((process, parity))
+                return
+        self.running -= 1
+
+    def loads(self):
+        for it in range(self.steps):
+            bar, parity = self.wait("raw_empty", it)
+            yield "wait", bar, parity
+
+            def land(it=it):
+                self.raw[it % self.raw_n] = it
+                self.arrive(self.bars["raw_full"][it % self.raw_n])
+            self.at(self.now + self.delay("load", it), land)
+
+    def decoder(self, warp):
+        group, lane = divmod(warp, self.dec // 2)
+        for it in range(group, self.steps, 2):
+            for name in self.decoder_waits:
+                yield ("wait", *self.wait(name, it))
+            self.expect("decode", self.raw[it % self.raw_n], it)
+            yield "delay", self.delay("decode", it)
+            self.expect("decode", self.raw[it % self.raw_n], it)
+            self.planes[it % self.stage_n][lane] = it
+            self.arrive(self.bars["full"][it % self.stage_n])
+            self.arrive(self.bars["raw_empty"][it % self.raw_n])
+
+    def scales(self, quarter):
+        it = j = 0
+        while it < self.steps:
+            end = min(it + self.span, self.steps)
+            while it < end:
+                for name in self.waits["scales"][:2]:
+                    yield ("wait", *self.wait(name, it))
+                self.expect("scales", self.raw[it % self.raw_n], it)
+                yield "delay", self.delay("scales", it)
+                self.expect("scales", self.raw[it % self.raw_n], it)
+                self.slots[it % self.slot_n][quarter] = it
+                self.arrive(self.bars["sf_full"][it % self.slot_n])
+                self.arrive(self.bars["raw_empty"][it % self.raw_n])
+                it += 1
+            yield ("wait", *self.wait("acc_full", j))
+            self.expect("accumulators", self.acc, j)
+            yield "delay", self.delay("epilogue", j)
+            self.expect("accumulators", self.acc, j)
+            self.arrive(self.bars["acc_empty"][0])
+            j += 1
+
+    def mma(self):
+        it = j = 0
+        while it < self.steps:
+            yield ("wait", *self.wait("acc_empty", j))
+            end = min(it + self.span, self.steps)
+            while it < end:
+                for name in self.waits["mma"][1:]:
+                    yield ("wait", *self.wait(name, it))
+
+                def complete(it=it, j=j, last=it == end - 1):
+                    self.expect("planes", set(self.planes[it % self.stage_n]), {it})
+                    self.expect("slot", set(self.slots[it % self.slot_n]), {it})
+                    self.acc = j
+                    self.arrive(self.bars["empty"][it % self.stage_n])
+                    self.arrive(self.bars["sf_empty"][it % self.slot_n])
+                    if last:
+                        self.arrive(self.bars["acc_full"][0])
+                self.mma_free = max(self.mma_free, self.now) + self.delay("mma", it)
+                self.at(self.mma_free, complete)
+                it += 1
+            j += 1
+
+    def run(self):
+        processes = [self.loads(), self.mma()] + [self.decoder(w) for w in range(self.dec)] + [self.scales(q) for q in range(4)]
+        self.running = len(processes)
+        for p in processes:
+            self.at(0, lambda p=p: self.resume(p))
+        while self.queue:
+            self.now, _, action = heapq.heappop(self.queue)
+            action()
+        assert self.running == 0, "a role waits for ever"
+        return self.wrong
+
+
+def ordinary(role, it):
+    return {"load": 1500, "decode": 1000, "scales": 150, "mma": 900, "epilogue": 1200}[role]
+
+
+@pytest.mark.parametrize("late", [1200, 2500, 20000, 1000000])
+@pytest.mark.parametrize("step", range(0, 24))
+def test_one_late_load_is_waited_for(step, late):
+    """One load that lands late, beside its ordinary successors: nobody reads its stage before it is there."""
+    assert Model(24, 16, lambda role, it: late if (role, it) == ("load", step) else ordinary(role, it)).run() == []
+
+
+@pytest.mark.parametrize("steps,span", [(1, 1), (2, 16), (3, 2), (7, 3), (16, 16), (40, 7)])
+def test_any_order_of_loads_and_any_pace_of_the_warps(steps, span):
+    for seed in range(60):
+        rng = random.Random(seed * 1000 + steps)
+        assert Model(steps, span, lambda role, it: int(10 ** rng.uniform(0, 5))).run() == [], seed
+
+
+def test_the_model_sees_a_wait_that_passes_two_phases_early():
+    """With the load's barrier asked before the stage's, whose wait is what rules the earlier phase out, the model reports stale reads."""
+    late = lambda role, it: 20000 if (role, it) == ("load", 9) else ordinary(role, it)         # noqa: E731
+    assert Model(24, 16, late, decoder_waits=["raw_full", "empty"]).run() != []
+    assert Model(24, 16, late, decoder_waits=["empty", "raw_full"]).run() == []
