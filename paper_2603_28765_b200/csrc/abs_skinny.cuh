@@ -401,15 +401,15 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
     // the global maximum of |C| as written, for the next quantizer's tensor scale (as in abs_gemm.cu); the ticket counts tiles
     if (OUT_BF16 && p.next_alpha != nullptr) {
         out_max = __reduce_max_sync(0xFFFFFFFFu, out_max);
-        if (lane == 0 && out_max) {
-            atomicMax(reinterpret_cast<unsigned int*>(p.error) + 1, out_max);
-            __threadfence();
-        }
+        if (lane == 0 && out_max) atomicMax(reinterpret_cast<unsigned int*>(p.error) + 1, out_max);
         __syncthreads();
-        if (threadIdx.x == 0 && done > 0 && atomicAdd(p.error + 2, done) + done == p.n / kTileM) {
-            __threadfence();
-            const float A = __uint_as_float(atomicMax(reinterpret_cast<unsigned int*>(p.error) + 1, 0u) << 16);
-            *p.next_alpha = (A == 0.0f) ? 1.0f : __fdiv_rn(A, p.next_denom);
+        if (threadIdx.x == 0 && done > 0) {
+            __threadfence();                 // by the thread that takes the ticket, after the barrier: the block's maxima come before it
+            if (atomicAdd(p.error + 2, done) + done == p.n / kTileM) {
+                __threadfence();
+                const float A = __uint_as_float(atomicMax(reinterpret_cast<unsigned int*>(p.error) + 1, 0u) << 16);
+                *p.next_alpha = (A == 0.0f) ? 1.0f : __fdiv_rn(A, p.next_denom);
+            }
         }
     }
 }
