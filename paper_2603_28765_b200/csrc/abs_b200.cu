@@ -47,6 +47,9 @@ template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
     return launch_any(false, kernel, grid, block, s, args...);
 }
+// Internal status: a cooperative grid was refused because its blocks do not all fit what the stream may use (a green context, an
+// MPS share: fewer SMs than the device has).  Nothing was enqueued; the call takes the two kernels.
+constexpr abs_status_t kNotResident = (abs_status_t)-1;
 
 // ------------------------------------------------------------------------------------------ host state
 
@@ -72,6 +75,17 @@ DeviceState g_dev[kMaxDevices];
 
 // Optional CUDA events recorded around the group-quantize kernel (abs_profile_events).
 cudaEvent_t g_ev_quant_begin = nullptr, g_ev_quant_end = nullptr;
+
+// Status of the launch of a quantize kernel on s; also ends the interval of abs_profile_events.
+abs_status_t quantize_launched(cudaError_t e, cudaStream_t s, bool profile = true) {
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();                  // the refusal is answered here: it is not left for the caller's own error checks
+        return kNotResident;
+    }
+    if (e != cudaSuccess) return ABS_ERR_CUDA;
+    if (profile && g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
+    return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
+}
 
 abs_status_t device_state(DeviceState** out) {
     int dev = 0;
@@ -259,9 +273,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
 #undef ABS_LAUNCH_F
 #undef ABS_LAUNCH_F2
 #undef ABS_LAUNCH_F3
-            if (e != cudaSuccess) return ABS_ERR_CUDA;
-            if (g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
-            return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
+            return quantize_launched(e, s);
         }
     }
     if constexpr (FMT == ABS_FMT_NVFP4 || FMT == ABS_FMT_IF4) {
@@ -281,9 +293,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
             else if (rht) ABS_LAUNCH_O(true, false);
             else ABS_LAUNCH_O(false, true);
 #undef ABS_LAUNCH_O
-            if (e != cudaSuccess) return ABS_ERR_CUDA;
-            if (g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
-            return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
+            return quantize_launched(e, s);
         }
     }
     if constexpr (FMT == ABS_FMT_NVFP4_BS8 || FMT == ABS_FMT_IF4_BS8) {
@@ -297,9 +307,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
                                          : (alpha.cells ? quantize4_bs8_kernel<kInt, kOnePass, false> : alpha.slot ? quantize4_bs8_kernel<kInt, kFromSlot, false> : quantize4_bs8_kernel<kInt, kGiven, false>);
             const cudaError_t e = launch_any(alpha.cells != nullptr, kernel, bgrid, kThreads, s, (const uint4*)in, (uint2*)codes, (uint16_t*)scales, alpha,
                                              (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
-            if (e != cudaSuccess) return ABS_ERR_CUDA;
-            if (g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
-            return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
+            return quantize_launched(e, s);
         }
     }
     if constexpr (FMT == ABS_FMT_IF6_E2M3 || FMT == ABS_FMT_IF6_E3M2) {
@@ -312,9 +320,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
                                          : (alpha.cells ? quantize6_fast_kernel<FMT, kOnePass, false> : alpha.slot ? quantize6_fast_kernel<FMT, kFromSlot, false> : quantize6_fast_kernel<FMT, kGiven, false>);
             const cudaError_t e = launch_any(alpha.cells != nullptr, kernel, sgrid, kThreads, s, (const uint4*)in, (uint32_t*)codes, (uint8_t*)scales, alpha,
                                              (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
-            if (e != cudaSuccess) return ABS_ERR_CUDA;
-            if (g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
-            return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
+            return quantize_launched(e, s);
         }
     }
     if constexpr (FMT == ABS_FMT_IF3 || FMT == ABS_FMT_IF3_BS8) {
@@ -328,9 +334,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
                                          : (alpha.cells ? quantize3_fast_kernel<kG, kOnePass, false> : alpha.slot ? quantize3_fast_kernel<kG, kFromSlot, false> : quantize3_fast_kernel<kG, kGiven, false>);
             const cudaError_t e = launch_any(alpha.cells != nullptr, kernel, tgrid, kThreads, s, (const uint4*)in, (uint16_t*)codes, (uint8_t*)scales, alpha,
                                              (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
-            if (e != cudaSuccess) return ABS_ERR_CUDA;
-            if (g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
-            return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
+            return quantize_launched(e, s);
         }
     }
     if (emul_out) return ABS_ERR_FLAGS;          // no emulation kernel for this format / option combination
@@ -614,6 +618,19 @@ abs_status_t abs_quantize_ex(abs_fmt_t fmt, const void* in_bf16, int64_t rows, i
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t ngroups = rows * cols / 16;
     AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr};
+    // the quantize kernel, with src as it then is
+    auto quantize = [&]() {
+        switch (fmt) {
+            case ABS_FMT_NVFP4: return launch_quantize_fmt<0>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
+            case ABS_FMT_IF4: return launch_quantize_fmt<1>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
+            case ABS_FMT_IF3: return launch_quantize_fmt<2>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
+            case ABS_FMT_IF6_E2M3: return launch_quantize_fmt<3>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
+            case ABS_FMT_IF6_E3M2: return launch_quantize_fmt<4>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
+            case ABS_FMT_NVFP4_BS8: return launch_quantize_fmt<5>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
+            case ABS_FMT_IF4_BS8: return launch_quantize_fmt<6>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
+            default: return launch_quantize_fmt<7>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
+        }
+    };
     if (!(o.flags & ABS_F_ALPHA_GIVEN)) {
         unsigned long long* slot = nullptr;
         uint32_t gen = 0;
@@ -623,22 +640,14 @@ abs_status_t abs_quantize_ex(abs_fmt_t fmt, const void* in_bf16, int64_t rows, i
         src.overrun = st->overrun_dev;
         if (one_pass(fmt, o, st->sm_count, ngroups, false)) {
             src.cells = st->cells + (size_t)(gen % ABS_MAX_INFLIGHT) * kMaxCells;
-        } else {
-            rc = launch_amax(st->sm_count, in_bf16, ngroups, o, false, slot, gen, tensor_scale_f32, src.denom, s);
-            if (rc != ABS_OK) return rc;
-            src.slot = slot;
+            if ((rc = quantize()) != kNotResident) return rc;
+            src.cells = nullptr;
         }
+        rc = launch_amax(st->sm_count, in_bf16, ngroups, o, false, slot, gen, tensor_scale_f32, src.denom, s);
+        if (rc != ABS_OK) return rc;
+        src.slot = slot;
     }
-    switch (fmt) {
-        case ABS_FMT_NVFP4: return launch_quantize_fmt<0>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
-        case ABS_FMT_IF4: return launch_quantize_fmt<1>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
-        case ABS_FMT_IF3: return launch_quantize_fmt<2>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
-        case ABS_FMT_IF6_E2M3: return launch_quantize_fmt<3>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
-        case ABS_FMT_IF6_E3M2: return launch_quantize_fmt<4>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
-        case ABS_FMT_NVFP4_BS8: return launch_quantize_fmt<5>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
-        case ABS_FMT_IF4_BS8: return launch_quantize_fmt<6>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
-        default: return launch_quantize_fmt<7>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
-    }
+    return quantize();
 }
 
 abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t rows, int64_t cols, void* out_bf16,
@@ -676,6 +685,46 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
     const int grid = grid_waves(st->sm_count, ngroups, opt_blocks_per_sm(sr, rht), (rht || sr) ? kOptIters : kFastIters);
     if (ngroups >= (int64_t)0x7FFFFFFF - (int64_t)grid * kThreads) return ABS_ERR_SIZE;    // 32-bit group indices only
     AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr};
+    const bool store = codes_u8 != nullptr;
+    const float mul = (o.flags & ABS_F_SR_SCALE_17_16) ? 1.0625f : 1.0f;
+    const uint64_t ctr = o.sr_index_offset / 8;
+    const PhiloxKeys pk = philox_keys(o.sr_seed);
+    const bool a32 = (reinterpret_cast<uintptr_t>(in_bf16) & 31u) == 0, o32 = (reinterpret_cast<uintptr_t>(out_bf16) & 31u) == 0;
+    // the quantize kernel, with src as it then is
+    auto quantize = [&]() -> abs_status_t {
+        if (!four_bit) {
+            bool handled = false;
+            abs_status_t r;
+            switch (fmt) {
+                case ABS_FMT_IF3: r = launch_quantize_fmt<2>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
+                case ABS_FMT_IF6_E2M3: r = launch_quantize_fmt<3>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
+                case ABS_FMT_IF6_E3M2: r = launch_quantize_fmt<4>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
+                case ABS_FMT_NVFP4_BS8: r = launch_quantize_fmt<5>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
+                case ABS_FMT_IF4_BS8: r = launch_quantize_fmt<6>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
+                default: r = launch_quantize_fmt<7>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
+            }
+            return (!handled && r == ABS_ERR_FLAGS) ? ABS_ERR_SIZE : r;
+        }
+        cudaError_t e = cudaSuccess;
+#define ABS_LAUNCH_E2(I, R, S)                                                                                      \
+        e = launch_any(src.cells != nullptr, src.cells ? quantize4_opt_kernel<I, R, S, kOnePass, true>                   \
+                                             : src.slot ? quantize4_opt_kernel<I, R, S, kFromSlot, true>                 \
+                                                        : quantize4_opt_kernel<I, R, S, kGiven, true>, grid, kThreads, s, \
+                       (const uint4*)in_bf16, (uint2*)codes_u8, (uint8_t*)scales_e4m3, src, (int32_t)ngroups, mul,        \
+                       (uint32_t)o.had_sign_mask, pk, ctr, a32, (uint4*)out_bf16, o32, store)
+#define ABS_LAUNCH_E(I)                                                                                             \
+        do {                                                                                                            \
+            if (rht && sr) ABS_LAUNCH_E2(I, true, true);                                                                \
+            else if (rht) ABS_LAUNCH_E2(I, true, false);                                                                \
+            else if (sr) ABS_LAUNCH_E2(I, false, true);                                                                 \
+            else ABS_LAUNCH_E2(I, false, false);                                                                        \
+        } while (0)
+        if (fmt == ABS_FMT_IF4) ABS_LAUNCH_E(true);
+        else ABS_LAUNCH_E(false);
+#undef ABS_LAUNCH_E
+#undef ABS_LAUNCH_E2
+        return quantize_launched(e, s, false);
+    };
     if (!(o.flags & ABS_F_ALPHA_GIVEN)) {
         unsigned long long* slot = nullptr;
         uint32_t gen = 0;
@@ -685,48 +734,14 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
         src.overrun = st->overrun_dev;
         if (one_pass(fmt, o, st->sm_count, ngroups, true)) {
             src.cells = st->cells + (size_t)(gen % ABS_MAX_INFLIGHT) * kMaxCells;
-        } else {
-            rc = launch_amax(st->sm_count, in_bf16, ngroups, o, false, slot, gen, tensor_scale_f32, src.denom, s);
-            if (rc != ABS_OK) return rc;
-            src.slot = slot;
+            if ((rc = quantize()) != kNotResident) return rc;
+            src.cells = nullptr;
         }
+        rc = launch_amax(st->sm_count, in_bf16, ngroups, o, false, slot, gen, tensor_scale_f32, src.denom, s);
+        if (rc != ABS_OK) return rc;
+        src.slot = slot;
     }
-    const bool store = codes_u8 != nullptr;
-    if (!four_bit) {
-        bool handled = false;
-        switch (fmt) {
-            case ABS_FMT_IF3: rc = launch_quantize_fmt<2>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
-            case ABS_FMT_IF6_E2M3: rc = launch_quantize_fmt<3>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
-            case ABS_FMT_IF6_E3M2: rc = launch_quantize_fmt<4>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
-            case ABS_FMT_NVFP4_BS8: rc = launch_quantize_fmt<5>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
-            case ABS_FMT_IF4_BS8: rc = launch_quantize_fmt<6>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
-            default: rc = launch_quantize_fmt<7>(st->sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols, out_bf16, store, &handled); break;
-        }
-        return (!handled && rc == ABS_ERR_FLAGS) ? ABS_ERR_SIZE : rc;
-    }
-    const float mul = (o.flags & ABS_F_SR_SCALE_17_16) ? 1.0625f : 1.0f;
-    const uint64_t ctr = o.sr_index_offset / 8;
-    const PhiloxKeys pk = philox_keys(o.sr_seed);
-    const bool a32 = (reinterpret_cast<uintptr_t>(in_bf16) & 31u) == 0, o32 = (reinterpret_cast<uintptr_t>(out_bf16) & 31u) == 0;
-    cudaError_t e = cudaSuccess;
-#define ABS_LAUNCH_E2(I, R, S)                                                                                      \
-    e = launch_any(src.cells != nullptr, src.cells ? quantize4_opt_kernel<I, R, S, kOnePass, true>                   \
-                                         : src.slot ? quantize4_opt_kernel<I, R, S, kFromSlot, true>                 \
-                                                    : quantize4_opt_kernel<I, R, S, kGiven, true>, grid, kThreads, s, \
-                   (const uint4*)in_bf16, (uint2*)codes_u8, (uint8_t*)scales_e4m3, src, (int32_t)ngroups, mul,        \
-                   (uint32_t)o.had_sign_mask, pk, ctr, a32, (uint4*)out_bf16, o32, store)
-#define ABS_LAUNCH_E(I)                                                                                             \
-    do {                                                                                                            \
-        if (rht && sr) ABS_LAUNCH_E2(I, true, true);                                                                \
-        else if (rht) ABS_LAUNCH_E2(I, true, false);                                                                \
-        else if (sr) ABS_LAUNCH_E2(I, false, true);                                                                 \
-        else ABS_LAUNCH_E2(I, false, false);                                                                        \
-    } while (0)
-    if (fmt == ABS_FMT_IF4) ABS_LAUNCH_E(true);
-    else ABS_LAUNCH_E(false);
-#undef ABS_LAUNCH_E
-#undef ABS_LAUNCH_E2
-    return (e == cudaSuccess && cudaGetLastError() == cudaSuccess) ? ABS_OK : ABS_ERR_CUDA;
+    return quantize();
 }
 
 abs_status_t abs_quantize(abs_fmt_t fmt, const void* in_bf16, int64_t rows, int64_t cols, void* codes_u8,

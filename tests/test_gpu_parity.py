@@ -284,19 +284,25 @@ def test_amax_entry_point(B, oracle):
             assert a.view(np.uint32) == np.float32(oracle.alpha_from_amax(fmt, want)).view(np.uint32)
 
 
-def test_back_to_back_calls_reuse_scratch(B, oracle):
-    """The amax scratch slot re-arms itself: many calls in a row, on two streams, stay exact."""
+@pytest.mark.parametrize("flags", [0, 32], ids=["one_kernel", "two_kernels"])
+def test_back_to_back_calls_reuse_scratch(B, oracle, flags):
+    """The scratch of a call re-arms itself: many calls in a row, on two streams, stay exact.  Small calls find their maximum in the
+    cells of the one-kernel route; with ABS_F_INDEX64 (32) the same calls take the slots of the two-kernel route."""
+    assert flags in (0, B.ABS_F_INDEX64)
     xs = [I.generate("cfg1", 64, 256, seed=s) for s in range(4)]
     want = [oracle.quantize(1, x) for x in xs]
     devs = [to_dev(x) for x in xs]
     s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    opts = B.make_opts(flags) if flags else None
     torch.cuda.synchronize()
     outs = []
-    for rep in range(600):      # wraps the scratch ring more than once across both streams
+    for rep in range(2200):     # wraps the scratch ring of 1024 twice; waits now and then, so that fewer than 1024 are in flight
         k = rep % 4
-        outs.append((k, B.abs_quantize(1, devs[k], stream=(s1 if rep % 2 else s2))))
+        outs.append((k, B.abs_quantize(1, devs[k], opts=opts, stream=(s1 if rep % 2 else s2))))
+        if rep % 500 == 499:
+            torch.cuda.synchronize()
     torch.cuda.synchronize()
-    for k, (c, s, a) in outs[-16:]:
+    for k, (c, s, a) in outs[-16:] + outs[::97]:
         assert np.float32(a.item()) == want[k][2]
         assert np.array_equal(c.cpu().numpy().reshape(64, -1), want[k][0])
         assert np.array_equal(s.cpu().numpy().reshape(64, -1), want[k][1])
@@ -940,12 +946,13 @@ def test_tensor_core_matmul_on_arbitrary_bytes(B, oracle, fmt):
         assert err < 2e-5, (fmt, a_flags, b_flags, err)
 
 
-def test_scratch_ring_overrun_is_reported(B, oracle):
-    """More than ABS_MAX_INFLIGHT amax-carrying calls enqueued between the two kernels of one call: that call loses
-    its maximum.  Provoked without any fault: stream A first runs a bounded delay kernel, then one abs_quantize;
-    while A is delayed, stream B runs 1100 abs_quantize calls, which wraps the ring of 1024 slots past A's slot.
-    A's group-quantize kernel then finds another call's tag in its slot and raises the flag: the next call that
-    takes a slot returns ABS_ERR_SIZE (7) exactly once, and the library works normally afterwards."""
+@pytest.mark.parametrize("flags", [0, 32], ids=["one_kernel", "two_kernels"])
+def test_scratch_ring_overrun_is_reported(B, oracle, flags):
+    """More than ABS_MAX_INFLIGHT scratch-taking calls enqueued before an earlier one has run: that call loses its maximum.
+    Provoked without any fault: stream A first runs a bounded delay kernel, then one abs_quantize; while A is delayed,
+    stream B runs 1100 abs_quantize calls, which wraps the ring of 1024 past A's place in it.  A's kernel then finds another
+    call's tag -- in the cells of the one-kernel route, or with ABS_F_INDEX64 (32) in the slot of the two-kernel route -- and raises
+    the flag: the next call that takes scratch returns ABS_ERR_SIZE (7) exactly once, and the library works normally afterwards."""
     import ctypes
     L = B.lib()
     xb = I.generate("cfg1", 64, 256)
@@ -956,9 +963,9 @@ def test_scratch_ring_overrun_is_reported(B, oracle):
     torch.cuda.synchronize()
     with torch.cuda.stream(a):
         torch.cuda._sleep(400_000_000)                  # about 0.2 s at 2 GHz: a bounded busy-wait, nothing else
-        B.abs_quantize(1, x, codes_a, scales_a, ts_a, stream=a)
+        B.abs_quantize(1, x, codes_a, scales_a, ts_a, opts=B.make_opts(flags), stream=a)
     for _ in range(1100):
-        B.abs_quantize(1, x, outs_b[0], outs_b[1], outs_b[2], stream=b)
+        B.abs_quantize(1, x, outs_b[0], outs_b[1], outs_b[2], opts=B.make_opts(flags), stream=b)
     torch.cuda.synchronize()
     sp = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     args = (1, x.data_ptr(), 64, 256, outs_b[0].data_ptr(), outs_b[1].data_ptr(), outs_b[2].data_ptr(), sp)
@@ -1292,3 +1299,72 @@ def test_one_kernel_quantize_agrees_with_the_two_kernel_route(B, fmt, flags):
             out, alpha2 = B.abs_quantize_dequantize(fmt, x, opts=opts)
             assert torch.equal(alpha2, want)
             assert torch.equal(out.view(torch.int16), B.abs_dequantize(fmt, codes, scales, alpha, groups, 16).view(torch.int16)), (groups, shift)
+
+
+def test_small_quantize_with_fewer_sms_than_the_device(B):
+    """In a green context of a few SMs the cooperative grid of the one-kernel route does not fit from some size on: the call then
+    takes the two kernels.  Every packed kernel family, at a size that fits, the first that cannot, and a whole wave of the device;
+    bytes and alpha equal those outside the context, and no error is left behind."""
+    if not torch.cuda.green_contexts.SUPPORTED:
+        pytest.skip("torch without green contexts")
+    sms, few = torch.cuda.get_device_properties(0).multi_processor_count, 16
+    g = torch.Generator(device="cuda").manual_seed(11)
+    cases = []
+    for fmt, flags, per_sm in [(1, 0, 4), (0, 0, 4), (6, 0, 4), (2, 0, 3), (3, 0, 3), (1, 1, 3), (1, 7, 2), (0, 2, 2)]:
+        for blocks in (1, few * 5 + 1, sms * per_sm):
+            x = torch.randn((blocks * 256, 16), generator=g, device="cuda").bfloat16()
+            opts = B.make_opts(flags, 0x5A3C, 3)
+            emulated = B.abs_quantize_dequantize(fmt, x, opts=opts)
+            cases.append((fmt, x, opts, (*B.abs_quantize(fmt, x, opts=opts), *emulated)))
+    torch.cuda.synchronize()
+    green = torch.cuda.GreenContext.create(few, 0)
+    green.set_context()
+    try:
+        got = [(*B.abs_quantize(fmt, x, opts=opts), *B.abs_quantize_dequantize(fmt, x, opts=opts)) for fmt, x, opts, _ in cases]
+        torch.cuda.synchronize()
+    finally:
+        green.pop_context()
+    for (fmt, x, opts, want), have in zip(cases, got):
+        assert all(torch.equal(a.view(torch.int16) if a.dtype == torch.bfloat16 else a, b.view(torch.int16) if b.dtype == torch.bfloat16 else b)
+                   for a, b in zip(want, have)), (fmt, opts.flags, x.shape)
+
+
+def test_full_wave_one_kernel_quantize_on_several_streams(B):
+    """Grids that fill the device (2, 3 and 4 blocks per SM) and wait for all of their blocks, on four streams from four threads,
+    among larger two-kernel calls and products: every call's bytes as when it ran alone."""
+    import threading
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g = torch.Generator(device="cuda").manual_seed(12)
+    kinds = []
+    for fmt, flags, groups in [(1, 0, 4 * sms * 256), (2, 0, 3 * sms * 256), (1, 7, 2 * sms * 256), (1, 0, 4 * sms * 256 + 1), (6, 0, 4 * sms * 256)]:
+        x = torch.randn((groups, 16), generator=g, device="cuda").bfloat16()
+        kinds.append((fmt, x, B.make_opts(flags, 0x5A3C, 3)))
+    qa = B.abs_quantize(1, torch.randn((512, 1024), generator=g, device="cuda").bfloat16())
+    want = [B.abs_quantize(fmt, x, opts=opts) for fmt, x, opts in kinds]
+    product = B.abs_matmul(1, qa, qa, 512, 512, 1024, check=True)
+    torch.cuda.synchronize()
+    wrong, failures = [], []
+
+    def work(i):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                for rep in range(40):
+                    j = (rep + i) % len(kinds)
+                    fmt, x, opts = kinds[j]
+                    got = B.abs_quantize(fmt, x, opts=opts)
+                    wrong.append(torch.stack([(a != b).any() for a, b in zip(got, want[j])]).any())
+                    if rep % 3 == 0:
+                        wrong.append((B.abs_matmul(1, qa, qa, 512, 512, 1024) != product).any())
+                stream.synchronize()
+        except BaseException as e:                                       # noqa: BLE001
+            failures.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failures
+    assert not any(bool(w) for w in wrong)
+    B.abs_quantize(1, kinds[0][1])                                       # no wait ran out: nothing is reported here
