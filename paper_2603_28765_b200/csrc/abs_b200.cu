@@ -93,9 +93,11 @@ abs_status_t device_state(DeviceState** out) {
     DeviceState& st = g_dev[dev];
     std::call_once(st.once, [&]() {
         st.init_err = cudaMalloc(&st.ring, ABS_MAX_INFLIGHT * 4 * sizeof(uint32_t));
-        if (st.init_err == cudaSuccess) st.init_err = cudaMemset(st.ring, 0, ABS_MAX_INFLIGHT * 4 * sizeof(uint32_t));
+        if (st.init_err == cudaSuccess) st.init_err = cudaMemsetAsync(st.ring, 0, ABS_MAX_INFLIGHT * 4 * sizeof(uint32_t), cudaStreamLegacy);
         if (st.init_err == cudaSuccess) st.init_err = cudaMalloc(&st.cells, (size_t)ABS_MAX_INFLIGHT * kMaxCells * sizeof(unsigned long long));
-        if (st.init_err == cudaSuccess) st.init_err = cudaMemset(st.cells, 0, (size_t)ABS_MAX_INFLIGHT * kMaxCells * sizeof(unsigned long long));
+        if (st.init_err == cudaSuccess) st.init_err = cudaMemsetAsync(st.cells, 0, (size_t)ABS_MAX_INFLIGHT * kMaxCells * sizeof(unsigned long long), cudaStreamLegacy);
+        // the memsets are on the legacy stream, which streams created as non-blocking do not wait for
+        if (st.init_err == cudaSuccess) st.init_err = cudaStreamSynchronize(cudaStreamLegacy);
         if (st.init_err == cudaSuccess) st.init_err = cudaHostAlloc(&st.overrun_host, sizeof(uint32_t), cudaHostAllocMapped);
         if (st.init_err == cudaSuccess) {
             *st.overrun_host = 0u;
@@ -168,8 +170,9 @@ abs_status_t next_slot(DeviceState& st, unsigned long long** slot, uint32_t* gen
     uint32_t g = (uint32_t)++st.next;
     if (g == 0) {
         if (cudaDeviceSynchronize() != cudaSuccess) return ABS_ERR_CUDA;
-        if (cudaMemset(st.ring, 0, ABS_MAX_INFLIGHT * 4 * sizeof(uint32_t)) != cudaSuccess) return ABS_ERR_CUDA;
-        if (cudaMemset(st.cells, 0, (size_t)ABS_MAX_INFLIGHT * kMaxCells * sizeof(unsigned long long)) != cudaSuccess) return ABS_ERR_CUDA;
+        if (cudaMemsetAsync(st.ring, 0, ABS_MAX_INFLIGHT * 4 * sizeof(uint32_t), cudaStreamLegacy) != cudaSuccess) return ABS_ERR_CUDA;
+        if (cudaMemsetAsync(st.cells, 0, (size_t)ABS_MAX_INFLIGHT * kMaxCells * sizeof(unsigned long long), cudaStreamLegacy) != cudaSuccess) return ABS_ERR_CUDA;
+        if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return ABS_ERR_CUDA;     // as in device_state
         g = (uint32_t)++st.next;
     }
     *gen = g;

@@ -6,6 +6,7 @@ outputs (alpha, dequantized bf16 / fp32) are compared by bit pattern too, becaus
 fix the same FP32 operation order.
 """
 import os
+import sys
 
 import numpy as np
 import pytest
@@ -1368,3 +1369,23 @@ def test_full_wave_one_kernel_quantize_on_several_streams(B):
     assert not failures
     assert not any(bool(w) for w in wrong)
     B.abs_quantize(1, kinds[0][1])                                       # no wait ran out: nothing is reported here
+
+
+def test_scratch_is_clear_before_the_first_call_runs(B):
+    """The first call of a process, on a stream that does not wait for the legacy default stream, while that one is busy (a bounded
+    delay kernel): the clearing of the scratch, which is queued there, has to be over when the call's kernel is enqueued."""
+    import subprocess
+    code = """
+import torch
+from paper_2603_28765_b200 import binding as B
+x = (torch.arange(64 * 256, device="cuda").view(64, 256) % 251 - 125).bfloat16()
+side = torch.cuda.Stream()
+torch.cuda.synchronize()
+torch.cuda._sleep(1_000_000_000)
+first = B.abs_quantize(1, x, stream=side)
+assert torch.cuda.default_stream().query()
+torch.cuda.synchronize()
+for a, b in zip(first, B.abs_quantize(1, x)):
+    assert torch.equal(a, b)
+"""
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=300, cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
