@@ -260,7 +260,9 @@ def abs_amax(x, opts: AbsOpts | None = None, out=None, stream=None):
     import torch
     rows, cols = x.shape
     if out is None:
-        out = torch.zeros(1, dtype=torch.float32, device=x.device)
+        out = torch.empty(1, dtype=torch.float32, device=x.device)      # always written, on `stream`
+        if stream is not None:
+            out.record_stream(torch.cuda.ExternalStream(stream.cuda_stream, device=x.device))
     with torch.cuda.device(x.device):
         rc = lib().abs_amax(x.data_ptr(), rows, cols, C.byref(opts) if opts is not None else None, out.data_ptr(),
                             _stream_ptr(stream))

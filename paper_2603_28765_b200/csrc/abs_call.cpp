@@ -3,6 +3,7 @@
 // include/abs_b200.h, whose addresses binding.py passes in.  A quantize call is two kernels of a few microseconds on small
 // tensors, and marshalling it from Python took 31 us, with a fill kernel for the one float of the tensor scale.
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
@@ -62,20 +63,47 @@ struct Opts {
         ptr = &value;
     }
 };
-// With the guard of the tensor's device in force.
-void* stream_of(PyObject* o, c10::Device device) {
-    if (o == Py_None) return (void*)c10::cuda::getCurrentCUDAStream(device.index()).stream();
-    PyObject* s = PyObject_GetAttrString(o, "cuda_stream");
-    if (!s) throw Raised();
-    void* p = PyLong_AsVoidPtr(s);
-    Py_DECREF(s);
-    if (!p && PyErr_Occurred()) throw Raised();
-    return p;
-}
-at::Tensor bytes(int64_t n, c10::Device device, bool zero = false) {
-    const auto o = at::TensorOptions().dtype(at::kByte).device(device);
-    return zero ? at::zeros({n}, o) : at::empty({n}, o);
-}
+// The stream a call's kernels run on, with the guard of the tensor's device in force.  What a call allocates comes from the
+// current stream's pool.  Where the caller names another stream, the allocator is told that it is used there (a workspace that is
+// released when the call returns, or an output that is dropped, must not be handed out again while the kernels are pending), and
+// fills run there too, before the kernels.
+class Work {
+    c10::Device device;
+    bool other = false;                  // not the current stream
+
+    c10::cuda::CUDAStream torch_stream() const { return c10::cuda::getStreamFromExternal((cudaStream_t)stream, device.index()); }
+
+  public:
+    void* stream;
+    Work(PyObject* o, c10::Device d) : device(d) {
+        void* const current = (void*)c10::cuda::getCurrentCUDAStream(device.index()).stream();
+        stream = current;
+        if (o == Py_None) return;
+        PyObject* s = PyObject_GetAttrString(o, "cuda_stream");
+        if (!s) throw Raised();
+        stream = PyLong_AsVoidPtr(s);
+        Py_DECREF(s);
+        if (!stream && PyErr_Occurred()) throw Raised();
+        other = stream != current;
+    }
+    at::Tensor empty(at::IntArrayRef sizes, at::ScalarType type) const {
+        at::Tensor t = at::empty(sizes, at::TensorOptions().dtype(type).device(device));
+        if (other && t.numel() > 0) c10::cuda::CUDACachingAllocator::recordStream(t.storage().data_ptr(), torch_stream());
+        return t;
+    }
+    at::Tensor zeros(at::IntArrayRef sizes, at::ScalarType type) const {
+        at::Tensor t = empty(sizes, type);
+        if (!other) return t.zero_();
+        const c10::cuda::CUDAStreamGuard on(torch_stream());
+        return t.zero_();
+    }
+    at::Tensor bytes(int64_t n) const { return empty({n}, at::kByte); }
+    // One float: the kernels always write the tensor scale of a tensor that has elements, unless it is an input.
+    at::Tensor tensor_scale(PyObject* o, bool written) const {
+        if (o != Py_None) return tensor(o, "tensor_scale");
+        return written ? empty({1}, at::kFloat) : zeros({1}, at::kFloat);
+    }
+};
 at::Tensor given_or(PyObject* o, const char* what, const std::function<at::Tensor()>& make) { return o == Py_None ? make() : tensor(o, what); }
 int bits_of(int64_t fmt) {
     switch (fmt) {
@@ -93,12 +121,6 @@ int known_bits(int64_t fmt) {
         throw Raised();
     }
     return b;
-}
-// One float: the kernels always write the tensor scale of a tensor that has elements, unless it is an input.
-at::Tensor tensor_scale_for(PyObject* o, bool written, c10::Device device) {
-    if (o != Py_None) return tensor(o, "tensor_scale");
-    const auto opt = at::TensorOptions().dtype(at::kFloat).device(device);
-    return written ? at::empty({1}, opt) : at::zeros({1}, opt);
 }
 at::Tensor input_matrix(PyObject* o) {
     at::Tensor x = tensor(o, "x");
@@ -163,16 +185,17 @@ PyObject* quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int64_t rows = x.size(0), cols = x.size(1);
     const c10::Device dev = x.device();
     const c10::cuda::CUDAGuard guard(dev);
-    const at::Tensor codes = given_or(a[2], "codes", [&] { return bytes(std::max<int64_t>(cols % 16 == 0 ? rows * cols / 16 * (2 * bits_of(fmt)) : 0, 1), dev); });
+    const Work work(a[6], dev);
+    const at::Tensor codes = given_or(a[2], "codes", [&] { return work.bytes(std::max<int64_t>(cols % 16 == 0 ? rows * cols / 16 * (2 * bits_of(fmt)) : 0, 1)); });
     const at::Tensor scales = given_or(a[3], "scales", [&] {
         if (opts.value.flags & ABS_F_SCALES_SWIZZLED)
-            return bytes(std::max<int64_t>((int64_t)entry.scales_bytes_swizzled((abs_fmt_t)fmt, rows, cols), 1), dev, true);
+            return work.zeros({std::max<int64_t>((int64_t)entry.scales_bytes_swizzled((abs_fmt_t)fmt, rows, cols), 1)}, at::kByte);
         known_bits(fmt);
-        return bytes(std::max<int64_t>(rows * cols / group_of(fmt), 1), dev);
+        return work.bytes(std::max<int64_t>(rows * cols / group_of(fmt), 1));
     });
     const bool written = rows * cols > 0 && cols % 16 == 0 && bits_of(fmt) && !(opts.value.flags & ABS_F_ALPHA_GIVEN);
-    const at::Tensor ts = tensor_scale_for(a[4], written, dev);
-    void *px = x.data_ptr(), *pc = codes.data_ptr(), *ps = scales.data_ptr(), *s = stream_of(a[6], dev);
+    const at::Tensor ts = work.tensor_scale(a[4], written);
+    void *px = x.data_ptr(), *pc = codes.data_ptr(), *ps = scales.data_ptr(), *s = work.stream;
     float* pt = (float*)ts.data_ptr();
     return result(unlocked([&] { return entry.quantize((abs_fmt_t)fmt, px, rows, cols, pc, ps, pt, opts.ptr, s); }), {codes, scales, ts});
     ABS_CALL_END
@@ -187,11 +210,12 @@ PyObject* quantize_transposed(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int64_t rows = x.size(0), cols = x.size(1);
     const c10::Device dev = x.device();
     const c10::cuda::CUDAGuard guard(dev);
-    const at::Tensor codes = given_or(a[2], "codes_t", [&] { return bytes(std::max<int64_t>(rows * cols * known_bits(fmt) / 8, 1), dev); });
-    const at::Tensor scales = given_or(a[3], "scales_t", [&] { return bytes(std::max<int64_t>(rows * cols / 16, 1), dev); });
+    const Work work(a[6], dev);
+    const at::Tensor codes = given_or(a[2], "codes_t", [&] { return work.bytes(std::max<int64_t>(rows * cols * known_bits(fmt) / 8, 1)); });
+    const at::Tensor scales = given_or(a[3], "scales_t", [&] { return work.bytes(std::max<int64_t>(rows * cols / 16, 1)); });
     const bool written = rows * cols > 0 && rows % 16 == 0 && cols % 16 == 0 && !(opts.value.flags & ABS_F_ALPHA_GIVEN);
-    const at::Tensor ts = tensor_scale_for(a[4], written, dev);
-    void *px = x.data_ptr(), *pc = codes.data_ptr(), *ps = scales.data_ptr(), *s = stream_of(a[6], dev);
+    const at::Tensor ts = work.tensor_scale(a[4], written);
+    void *px = x.data_ptr(), *pc = codes.data_ptr(), *ps = scales.data_ptr(), *s = work.stream;
     float* pt = (float*)ts.data_ptr();
     return result(unlocked([&] { return entry.quantize_transposed((abs_fmt_t)fmt, px, rows, cols, pc, ps, pt, opts.ptr, s); }),
                   {codes, scales, ts});
@@ -207,12 +231,13 @@ PyObject* quantize_dequantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int64_t rows = x.size(0), cols = x.size(1);
     const c10::Device dev = x.device();
     const c10::cuda::CUDAGuard guard(dev);
-    const at::Tensor out = given_or(a[2], "out", [&] { return at::empty({rows, cols}, at::TensorOptions().dtype(at::kBFloat16).device(dev)); });
+    const Work work(a[7], dev);
+    const at::Tensor out = given_or(a[2], "out", [&] { return work.empty({rows, cols}, at::kBFloat16); });
     void* pc = a[3] == Py_None ? nullptr : tensor(a[3], "codes").data_ptr();
     void* ps = a[4] == Py_None ? nullptr : tensor(a[4], "scales").data_ptr();
     const bool written = rows * cols > 0 && cols % 16 == 0 && bits_of(fmt) && !(opts.value.flags & ABS_F_ALPHA_GIVEN);
-    const at::Tensor ts = tensor_scale_for(a[5], written, dev);
-    void *px = x.data_ptr(), *po = out.data_ptr(), *s = stream_of(a[7], dev);
+    const at::Tensor ts = work.tensor_scale(a[5], written);
+    void *px = x.data_ptr(), *po = out.data_ptr(), *s = work.stream;
     float* pt = (float*)ts.data_ptr();
     return result(unlocked([&] { return entry.quantize_dequantize((abs_fmt_t)fmt, px, rows, cols, po, pc, ps, pt, opts.ptr, s); }), {out, ts});
     ABS_CALL_END
@@ -226,10 +251,9 @@ PyObject* dequantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const Opts opts(a[7]);
     const c10::Device dev = codes.device();
     const c10::cuda::OptionalCUDAGuard guard(dev);      // a tensor that is not on a GPU raises
-    const at::Tensor out = given_or(a[6], "out", [&] {
-        return at::empty({rows, cols}, at::TensorOptions().dtype(opts.value.flags & ABS_F_OUT_FP32 ? at::kFloat : at::kBFloat16).device(dev));
-    });
-    void *pc = codes.data_ptr(), *ps = scales.data_ptr(), *po = out.data_ptr(), *s = stream_of(a[8], dev);
+    const Work work(a[8], dev);
+    const at::Tensor out = given_or(a[6], "out", [&] { return work.empty({rows, cols}, opts.value.flags & ABS_F_OUT_FP32 ? at::kFloat : at::kBFloat16); });
+    void *pc = codes.data_ptr(), *ps = scales.data_ptr(), *po = out.data_ptr(), *s = work.stream;
     const float* pt = (const float*)ts.data_ptr();
     return result(unlocked([&] { return entry.dequantize((abs_fmt_t)fmt, pc, ps, pt, rows, cols, po, opts.ptr, s); }), {out});
     ABS_CALL_END
@@ -263,18 +287,19 @@ PyObject* matmul(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (bf16 < 0) throw Raised();
     const c10::Device dev = q[0].device();
     const c10::cuda::OptionalCUDAGuard guard(dev);
-    const at::Tensor ws = given_or(a[7], "workspace", [&] { return bytes(need + 1024, dev); });
-    const at::Tensor out = given_or(a[6], "out", [&] { return at::empty({M, N}, at::TensorOptions().dtype(bf16 ? at::kBFloat16 : at::kFloat).device(dev)); });
+    const Work work(a[8], dev);
+    const at::Tensor ws = given_or(a[7], "workspace", [&] { return work.bytes(need + 1024); });
+    const at::Tensor out = given_or(a[6], "out", [&] { return work.empty({M, N}, bf16 ? at::kBFloat16 : at::kFloat); });
     require(out.scalar_type() == (bf16 ? at::kBFloat16 : at::kFloat), "out: float32, or bfloat16 with bf16");
     const int64_t off = (int64_t)((0 - (uintptr_t)ws.data_ptr()) & 1023u);
-    void *pw = (uint8_t*)ws.data_ptr() + off, *po = out.data_ptr(), *s = stream_of(a[8], dev);
+    void *pw = (uint8_t*)ws.data_ptr() + off, *po = out.data_ptr(), *s = work.stream;
     const size_t ws_bytes = (size_t)std::max<int64_t>(ws.numel() - off, 0);
     void* p[6];
     for (int i = 0; i < 6; ++i) p[i] = q[i].data_ptr();
     if (a[10] != Py_None) {
         require(bf16, "next_fmt: bf16 output only");
         const int64_t next_fmt = integer(a[10]);
-        const at::Tensor next = tensor_scale_for(a[11], true, dev);
+        const at::Tensor next = work.tensor_scale(a[11], true);
         float* pn = (float*)next.data_ptr();
         return result(unlocked([&] {
                           return entry.matmul_bf16_scaled((abs_fmt_t)fmt, p[0], p[1], (const float*)p[2], p[3], p[4], (const float*)p[5], M, N, K,

@@ -1389,3 +1389,38 @@ for a, b in zip(first, B.abs_quantize(1, x)):
     assert torch.equal(a, b)
 """
     subprocess.run([sys.executable, "-c", code], check=True, timeout=300, cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+
+
+def test_what_a_call_allocates_is_ordered_with_its_stream(B):
+    """Calls on a stream other than the current one, with their own buffers: fills run on that stream, before the kernels, and what
+    the call releases is not handed out again while its kernels are pending.  (a) The current stream is behind a bounded delay:
+    the zero fill of tiled scales must not come after the kernel that writes them.  (b) The call's stream is behind one: buffers of
+    the workspace's size, allocated and filled on the current stream meanwhile, must not be the workspace of the pending product."""
+    side = torch.cuda.Stream()
+    x = to_dev(I.generate("cfg1", 100, 512, seed=5))
+    opts = B.make_opts(B.ABS_F_SCALES_SWIZZLED)
+    want, amax = B.abs_quantize(1, x, opts=opts), B.abs_amax(x)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(400_000_000)
+    got, got_amax = B.abs_quantize(1, x, opts=opts, stream=side), B.abs_amax(x, stream=side)
+    empty = B.abs_quantize(1, x[:0], stream=side)
+    assert not torch.cuda.current_stream().query()
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(want, got)) and torch.equal(amax, got_amax) and empty[2].item() == 0.0
+
+    for m in (8, 256):                                                   # few-row and tiled product
+        n, k = 1024, 2048
+        qa, qb = B.abs_quantize(1, to_dev(I.generate("cfg2", m, k))), B.abs_quantize(1, to_dev(I.generate("cfg3a", n, k, seed=9)))
+        want = B.abs_matmul(1, qa, qb, m, n, k, check=True)
+        need = B.lib().abs_matmul_workspace_bytes(1, m, n, k) + 1024
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(400_000_000)
+        got = B.abs_matmul(1, qa, qb, m, n, k, stream=side)
+        fills = [torch.full((need,), 0x77, dtype=torch.uint8, device="cuda") for _ in range(8)]
+        dropped = B.abs_quantize(1, x, stream=side)[0].data_ptr()        # its outputs are released at once, the kernel is pending
+        assert all(torch.empty(100 * 256, dtype=torch.uint8, device="cuda").data_ptr() != dropped for _ in range(4))
+        torch.cuda.current_stream().synchronize()
+        assert not side.query()
+        torch.cuda.synchronize()
+        assert torch.equal(got, want) and all(bool((f == 0x77).all()) for f in fills)
