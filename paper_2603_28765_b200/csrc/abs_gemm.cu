@@ -591,7 +591,7 @@ bool skinny_plan(abs_fmt_t fmt, int64_t m, int64_t n, int64_t k, int sm_count, S
     P.units = (int32_t)units;
     P.grid = P.units < sm_count ? P.units : sm_count;
     P.off_partials = 1024 + round1k((size_t)(n / kTileM) * sizeof(int));
-    P.total = P.off_partials + (size_t)P.grid * 2 * kSkinnyTok * kTileM * sizeof(float);
+    P.total = P.off_partials + (size_t)P.grid * 2 * kSkinnyTok * kTileM * sizeof(double);
     return true;
 }
 
@@ -624,7 +624,7 @@ static abs_status_t skinny_matmul(const SkinnyPlan& P, const void* a_codes, cons
     p.x_codes = (const uint8_t*)a_codes; p.x_scales = (const uint8_t*)a_scales;
     p.alpha_a = a_alpha; p.alpha_b = b_alpha;
     p.out = out;
-    p.partials = (float*)(ws + P.off_partials);
+    p.partials = (double*)(ws + P.off_partials);
     p.tickets = (int*)(ws + 1024); p.error = (int*)ws;
     p.m = (int32_t)m; p.n = (int32_t)n; p.k = (int32_t)k; p.units = P.units;
     p.next_alpha = next_alpha; p.next_denom = next_denom;

@@ -13,10 +13,16 @@
 //
 // The planes.  Every code of B passes through the integer pipe once per call, which is what bounds the kernel, so B's split
 // is the cheapest one and not the shortest: the codes of the FP groups (F), and for the integer groups
-// k = 8 y + 2 x with y in {0, 1/2, -1, -1/2} from the two high bits and x in {0, 1/2, 1, 3/2} the two low bits as they are --
-// eight word operations for eight codes against some twenty of split_int_word.  The tokens take the planes H and L of
-// abs_gemm.cu, one below the other as the N side of one MMA (an MMA of 128 x N x 64 takes 75 to 100 cycles for any N up to
-// 128), so there are three MMAs of 128 x 64 x 64 per K-block.
+// k / 2 = y + x with y in {0, 2, -4, -2} from the two high bits and x in {0, 1/2, 1, 3/2} the two low bits as they are --
+// eight word operations for eight codes against some twenty of split_int_word.  y and x have one factor and one accumulator:
+// x is never negative, and with tokens of one sign a sum of its own would grow and cancel against that of y.  The
+// tokens take the planes H and L of abs_gemm.cu, one below the other as the N side of one MMA (an MMA of 128 x N x 64 takes 75
+// to 100 cycles for any N up to 128), so there are three MMAs of 128 x 64 x 64 per K-block.
+//
+// Roundings.  The accumulators hardly round (products of E2M1 codes and narrow ranges of scales); what is lost is lost where they
+// meet.  The products with L, some tenth of the result, are added up in FP32; everything else -- the products with H, spans of a
+// tile, shares of blocks, the scale -- is FP64 up to the one rounding of the result.  2-norm error against 64 bits, 24 x 14336 x 4096 and
+// 8 x 4096 x 14336: 2.6e-8 and 2.6e-8; with FP32 sums and k = 8 y + 2 x in accumulators of their own 5.3e-8 and 5.6e-8 (same time).
 //
 // Measured, product alone, weights not in the L2 (before: planes through the workspace): n = 14336, k = 4096: 1 token 52.5
 // -> 21.5 us, 24 tokens 53 -> 24 us; 4096 x 4096, 1 token 32.7 -> 14.3 us; 14336 x 14336, 32 tokens 133 -> 56 us.  A step
@@ -44,7 +50,7 @@ struct SkinnyArgs {
     const uint8_t *x_codes, *x_scales;     // tokens A [m, k]
     const float *alpha_a, *alpha_b;
     void* out;                             // [m, n] bf16 or FP32
-    float* partials;                       // [blocks][2][32][128]
+    double* partials;                      // [blocks][2][32][128]
     int *tickets, *error;                  // tickets: one per tile
     int32_t m, n, k, units;
     float* next_alpha;
@@ -68,8 +74,9 @@ __device__ __forceinline__ uint4 mask_scales(uint32_t a, uint32_t b, uint32_t c,
 template <bool OUT_BF16>
 __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_constant__ SkinnyArgs p) {
     constexpr int NT = kSkinnyTok, kRaw = kSkinnyRaw, kStages = kSkinnyStages, kStageBytes = kSkinnyStageBytes;
-    constexpr uint32_t kSfBase = 6 * NT;                                   // accumulators F H, F L, Y H, Y L, X H, X L
-    constexpr uint32_t kTmem = 512;                                        // of which 320 columns are used
+    constexpr uint32_t kSfBase = 4 * NT;                                   // accumulators F H, F L, (Y + X) H, (Y + X) L
+    constexpr uint32_t kTmem = kSfBase + kSkinnySfSlots * kSkinnySlotCols;
+    static_assert(kTmem == 256, "a power of two");
     constexpr int kChunkSteps = kChunkK / kStageK;
     extern __shared__ uint8_t gemm_smem_raw[];
     const uint32_t raw = smem_u32(gemm_smem_raw);
@@ -106,8 +113,8 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
 
     const float scale = __fmul_rn(*p.alpha_a, *p.alpha_b);
     uint32_t out_max = 0u;                                                 // largest |C| bit pattern this thread has written as bf16
-    auto write_out = [&](int32_t token, size_t col, float sum) {
-        const float c = __fmul_rn(sum, scale);
+    auto write_out = [&](int32_t token, size_t col, double sum) {
+        const float c = __double2float_rn(__dmul_rn(sum, (double)scale));
         const size_t at = (size_t)token * p.n + col;
         if constexpr (OUT_BF16) {
             const __nv_bfloat16 b = __float2bfloat16_rn(c);
@@ -146,9 +153,10 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
 #pragma unroll
                     for (int kb = 0; kb < kStageK / kMmaK; ++kb) {
                         const bool go = !(kt == 0 && kb == 0);
-#pragma unroll
-                        for (int pl = 0; pl < 3; ++pl)
-                            tc_mma_nvf4(tmem + 2 * pl * NT, desc_a(pl, kb), desc_b(kb), kDesc, go, tsfa + 4 * kb, tsfb + 4 * kb);
+                        const uint32_t fa = tsfa + 4 * kb, fb = tsfb + 4 * kb;
+                        tc_mma_nvf4(tmem, desc_a(0, kb), desc_b(kb), kDesc, go, fa, fb);
+                        tc_mma_nvf4(tmem + 2 * NT, desc_a(1, kb), desc_b(kb), kDesc, go, fa, fb);
+                        tc_mma_nvf4(tmem + 2 * NT, desc_a(2, kb), desc_b(kb), kDesc, true, fa, fb);
                     }
                     tc_commit(empty0 + 8 * s);
                     tc_commit(sf_empty0 + 8 * slot);
@@ -176,8 +184,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
             if (++kf == ksteps) kf = 0;
         };
         load_tokens();
-        // fp32(1/7), fp32(6/7), fp32(6/49)
-        const float c17 = __uint_as_float(0x3E124925u), c67 = __uint_as_float(0x3F5B6DB7u), c649 = __uint_as_float(0x3DFAC688u);
+        const float c17 = __uint_as_float(0x3E124925u), c1249 = __uint_as_float(0x3E7AC688u);      // fp32(1/7), fp32(12/49)
         uint32_t it = 0, j = 0;
         bool ok = true;
         bool from_start = u0 % ksteps == 0, first_span = true;
@@ -219,24 +226,24 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
             tc_fence_after();
             u += len;
             const bool tile_end = k0 + len == ksteps, whole = tile_end && from_start;      // whole: this block has all of K
-            float* mine = p.partials + ((size_t)blockIdx.x * 2 + (from_start ? 1 : 0)) * (NT * kTileM) + quarter * 32 + lane;
+            double* mine = p.partials + ((size_t)blockIdx.x * 2 + (from_start ? 1 : 0)) * (NT * kTileM) + quarter * 32 + lane;
             const size_t col = (size_t)tile * kTileM + quarter * 32 + lane;
             for (int32_t t0 = 0; t0 < p.m; t0 += 8) {
-                uint32_t r[6][8];
+                uint32_t r[4][8];
 #pragma unroll
-                for (int a = 0; a < 6; ++a) tmem_load8(lanes + a * NT + t0, r[a]);
+                for (int a = 0; a < 4; ++a) tmem_load8(lanes + a * NT + t0, r[a]);
                 tmem_load_wait();
-                float v[8];
+                double v[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     auto acc = [&](int a) { return __uint_as_float(r[a][e]); };
-                    const float kh = __fmaf_rn(8.0f, acc(2), __fmul_rn(2.0f, acc(4))), kl = __fmaf_rn(8.0f, acc(3), __fmul_rn(2.0f, acc(5)));
-                    v[e] = __fadd_rn(__fmaf_rn(c67, kh, acc(0)), __fmaf_rn(c649, kl, __fmul_rn(c17, acc(1))));
+                    const float low = __fmaf_rn(c1249, acc(3), __fmul_rn(c17, acc(1)));
+                    v[e] = __fma_rn(12.0 / 7.0, (double)acc(2), __dadd_rn((double)acc(0), (double)low));
                 }
                 // columns of tokens beyond m are stored with the rest (the workspace has NT of them) and never read
                 if (!first_span) {
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = __fadd_rn(mine[e * kTileM], v[e]);
+                    for (int e = 0; e < 8; ++e) v[e] = __dadd_rn(mine[e * kTileM], v[e]);
                 }
                 if (whole) {
 #pragma unroll
@@ -285,10 +292,10 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
         auto put_weights = [&](const Piece& f, uint32_t at) {
             const uint32_t m0 = 0u - ((f.two >> 7) & 1u), m1 = 0u - (f.two >> 15);      // all ones for an integer group
             auto low = [](uint32_t w, uint32_t mask) { return w & mask & 0x33333333u; };
-            // bits b3 b2 of k: code of 0, 1/2, -1, -1/2 = b3 << 3 | (b3 & ~b2) << 1 | b2
+            // bits b3 b2 of k: code of 0, 2, -4, -2 = b3 << 3 | (b3 | b2) << 2 | (b3 & ~b2) << 1
             auto high = [](uint32_t w, uint32_t mask) {
-                const uint32_t w2 = w >> 2;
-                return ((w & 0x88888888u) | (w2 & 0x11111111u) | (w2 & ~(w >> 1) & 0x22222222u)) & mask;
+                const uint32_t w1 = w >> 1;
+                return ((w & 0x88888888u) | ((w | w1) & 0x44444444u) | ((w >> 2) & ~w1 & 0x22222222u)) & mask;
             };
             store(at, make_uint4(f.codes.x & ~m0, f.codes.y & ~m0, f.codes.z & ~m1, f.codes.w & ~m1));
             store(at + kPlaneBytes, make_uint4(high(f.codes.x, m0), high(f.codes.y, m0), high(f.codes.z, m1), high(f.codes.w, m1)));
@@ -354,7 +361,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
     if (failed) return;
 
     // ---- the tiles at the two ends of the run may be shared with other blocks: the last of a tile's blocks sums the
-    // shares in the order of K (in FP64: the shares carry all 24 bits, and this is no place to lose any)
+    // shares in the order of K
     const int32_t t_first = u0 / ksteps, t_last = (u1 - 1) / ksteps;
     const bool share_first = u0 % ksteps != 0 || u1 - u0 < ksteps, share_last = t_last != t_first && u1 % ksteps != 0;
     if (threadIdx.x == 0) {
@@ -386,15 +393,15 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
 #pragma unroll
             for (int q = 0; q < kEach; ++q) v[q] = 0.0;
             for (int32_t b = bf; b <= bl; ++b) {
-                const float* share = p.partials + ((size_t)b * 2 + (b == bf ? 1 : 0)) * (NT * kTileM);
+                const double* share = p.partials + ((size_t)b * 2 + (b == bf ? 1 : 0)) * (NT * kTileM);
 #pragma unroll
                 for (int q = 0; q < kEach; ++q)
-                    if (i0 + q * kSkinnyThreads < p.m * kTileM) v[q] += (double)__ldcg(share + i0 + q * kSkinnyThreads);
+                    if (i0 + q * kSkinnyThreads < p.m * kTileM) v[q] += __ldcg(share + i0 + q * kSkinnyThreads);
             }
 #pragma unroll
             for (int q = 0; q < kEach; ++q) {
                 const int32_t i = i0 + q * kSkinnyThreads;
-                if (i < p.m * kTileM) write_out(i / kTileM, (size_t)tile * kTileM + i % kTileM, (float)v[q]);
+                if (i < p.m * kTileM) write_out(i / kTileM, (size_t)tile * kTileM + i % kTileM, v[q]);
             }
         }
     }

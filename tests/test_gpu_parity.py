@@ -1424,3 +1424,31 @@ def test_what_a_call_allocates_is_ordered_with_its_stream(B):
         assert not side.query()
         torch.cuda.synchronize()
         assert torch.equal(got, want) and all(bool((f == 0x77).all()) for f in fills)
+
+
+def decoded_float64(q, rows, k):
+    """Codes times group scales of an IF4 operand (6/7 of the integer codes), without the tensor scale, in 64 bits."""
+    fp = torch.tensor([0, 0.5, 1, 1.5, 2, 3, 4, 6], dtype=torch.float64, device="cuda")
+    integer = torch.tensor([*range(8), *range(-8, 0)], dtype=torch.float64, device="cuda") * 6 / 7
+    e4m3 = torch.arange(128, dtype=torch.uint8, device="cuda").view(torch.float8_e4m3fn).double()
+    codes = q[0][: rows * k // 2].view(rows, k // 2)
+    codes = torch.stack([codes & 15, codes >> 4], -1).view(rows, k).long()
+    scales = q[1][: rows * k // 16].view(rows, k // 16)
+    values = torch.where((scales >> 7).bool().repeat_interleave(16, 1), integer[codes], torch.cat([fp, -fp])[codes])
+    return values * e4m3[(scales & 127).long()].repeat_interleave(16, 1)
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 4096, 4096), (24, 2560, 4096), (8, 1024, 14336), (32, 20480, 8192)])
+@pytest.mark.parametrize("tokens", ["both_signs", "one_sign"])
+def test_few_row_product_rounds_once(B, m, n, k, tokens):
+    """The few-row kernel keeps its sums in FP64 outside the tensor core: shared tiles, whole tiles, tiles of several spans.  Rounding
+    once to FP32 is an error of 2^-23 / sqrt(12) times 0.68 (log-uniform mantissas) = 2.3e-8 in the 2-norm; a second rounding of
+    the same size inside the tensor core would make it 3.3e-8, which is the limit."""
+    g = torch.Generator(device="cuda").manual_seed(m)
+    x = torch.randn((m, k), generator=g, device="cuda")
+    one, half = torch.tensor([1.0], device="cuda"), torch.tensor([0.5], device="cuda")     # tensor scales whose product is exact
+    qa = (*B.abs_quantize(1, (x.abs() if tokens == "one_sign" else x).bfloat16())[:2], one)
+    qb = (*B.abs_quantize(1, (torch.randn((n, k), generator=g, device="cuda") * 0.02).bfloat16())[:2], half)
+    c = B.abs_matmul(1, qa, qb, m, n, k, check=True).double()
+    want = 0.5 * decoded_float64(qa, m, k) @ decoded_float64(qb, n, k).t()
+    assert (c - want).norm() <= 3.3e-8 * want.norm()
