@@ -246,8 +246,8 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
 #pragma unroll
                         for (int kb = 0; kb < kStepBlocks; ++kb) {
                             const uint32_t fa = tsfa + 4 * kb, fb = tsfb + 4 * kb;
-                            const bool go = !(kt == 0 && kb == 0);
-                            tc_mma_nvf4<kFill>(acc, desc_a(0, kb), desc_b(0, kb), kInstrDesc, go, fa, fb);                        // H H
+                            const bool go0 = !(kt == 0 && kb == 0), go = go0 || k0 != 0;      // H H: anew in every chunk
+                            tc_mma_nvf4<kFill>(acc, desc_a(0, kb), desc_b(0, kb), kInstrDesc, go0, fa, fb);                       // H H
                             tc_mma_nvf4<kLastUse>(acc + kTileN, desc_a(0, kb), desc_b(1, kb), kInstrDesc, go, fa, fb);            // H L
                             tc_mma_nvf4<kFill>(acc + kTileN, desc_a(1, kb), desc_b(0, kb), kInstrDesc, true, fa, fb);             // L H
                             tc_mma_nvf4<kLastUse>(acc + 2 * kTileN, desc_a(1, kb), desc_b(1, kb), kInstrDesc, go, fa, fb);        // L L
@@ -344,17 +344,26 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
                     if (!have) { all_tiles = false; break; }
                     tc_fence_after();
                     const uint32_t lane_base = tmem + buf * kTileN + col0 + ((uint32_t)(quarter * 32) << 16);
+                    // H H of a chunk is added to that of the chunks before it; the other two accumulators run on to the last (see kChunkK)
 #pragma unroll
                     for (int chunk = 0; chunk < kCols / 16; ++chunk) {
-                        uint32_t r0[16], r1[16], r2[16];
+                        uint32_t r0[16];
                         tmem_load16(lane_base + chunk * 16, r0);
-                        tmem_load16(lane_base + kTileN + chunk * 16, r1);
-                        tmem_load16(lane_base + 2 * kTileN + chunk * 16, r2);
                         tmem_load_wait();
 #pragma unroll
-                        for (int jj = 0; jj < 16; ++jj) {
-                            const float acc = __fadd_rn(__uint_as_float(r0[jj]), __fmaf_rn(c2, __uint_as_float(r2[jj]), __fmul_rn(c1, __uint_as_float(r1[jj]))));
-                            v[chunk * 16 + jj] = k0 == 0 ? acc : __fadd_rn(v[chunk * 16 + jj], acc);
+                        for (int jj = 0; jj < 16; ++jj)
+                            v[chunk * 16 + jj] = k0 == 0 ? __uint_as_float(r0[jj]) : __fadd_rn(v[chunk * 16 + jj], __uint_as_float(r0[jj]));
+                    }
+                    if (k_iters - k0 <= kChunkSteps) {
+#pragma unroll
+                        for (int chunk = 0; chunk < kCols / 16; ++chunk) {
+                            uint32_t r1[16], r2[16];
+                            tmem_load16(lane_base + kTileN + chunk * 16, r1);
+                            tmem_load16(lane_base + 2 * kTileN + chunk * 16, r2);
+                            tmem_load_wait();
+#pragma unroll
+                            for (int jj = 0; jj < 16; ++jj)
+                                v[chunk * 16 + jj] = __fadd_rn(v[chunk * 16 + jj], __fmaf_rn(c2, __uint_as_float(r2[jj]), __fmul_rn(c1, __uint_as_float(r1[jj]))));
                         }
                     }
                     tc_fence_before();

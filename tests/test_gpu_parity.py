@@ -1452,3 +1452,18 @@ def test_few_row_product_rounds_once(B, m, n, k, tokens):
     c = B.abs_matmul(1, qa, qb, m, n, k, check=True).double()
     want = 0.5 * decoded_float64(qa, m, k) @ decoded_float64(qb, n, k).t()
     assert (c - want).norm() <= 3.3e-8 * want.norm()
+
+
+@pytest.mark.parametrize("k", [4096, 8192, 12544, 14336])
+def test_tiled_product_rounds_little_over_chunks_of_k(B, k):
+    """The tiled IF4 kernel over one chunk of the accumulators, two, three and a step, three and a half: the chunks' sums lie on a
+    coarse grid and add up almost without rounding.  One rounding to FP32 is 2.3e-8 in the 2-norm (see above; tensor scales with an
+    exact product); two are 3.3e-8, three 4.0e-8, which is the limit; rounded in every chunk it was 5e-8 and more."""
+    g = torch.Generator(device="cuda").manual_seed(k)
+    m, n = 96, 512
+    one, half = torch.tensor([1.0], device="cuda"), torch.tensor([0.5], device="cuda")
+    qa = (*B.abs_quantize(1, torch.randn((m, k), generator=g, device="cuda").bfloat16())[:2], one)
+    qb = (*B.abs_quantize(1, (torch.randn((n, k), generator=g, device="cuda") * 0.02).bfloat16())[:2], half)
+    c = B.abs_matmul(1, qa, qb, m, n, k, check=True).double()
+    want = 0.5 * decoded_float64(qa, m, k) @ decoded_float64(qb, n, k).t()
+    assert (c - want).norm() <= 4.0e-8 * want.norm()
