@@ -8,6 +8,8 @@ library cannot be loaded, or a call fails, an exception is raised.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 import threading
 
@@ -137,8 +139,9 @@ def _call():
         L = lib()
         with _lock:
             if _native is None:
-                _build.build_call()
-                from . import _abs_call
+                loader = importlib.machinery.ExtensionFileLoader(f"{__package__}._abs_call", _build.build_call())
+                _abs_call = importlib.util.module_from_spec(importlib.util.spec_from_file_location(loader.name, loader.path, loader=loader))
+                loader.exec_module(_abs_call)
                 _abs_call.init(*(C.cast(f, C.c_void_p).value for f in (
                     L.abs_quantize_ex, L.abs_quantize_transposed, L.abs_quantize_dequantize, L.abs_dequantize_ex, L.abs_matmul,
                     L.abs_matmul_bf16, L.abs_matmul_bf16_scaled, L.abs_matmul_workspace_bytes, L.abs_scales_bytes_swizzled)))

@@ -4,6 +4,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
@@ -21,7 +22,6 @@ NVCC_FLAGS = [
 ]
 
 
-CALL_PATH = os.path.join(_HERE, "_abs_call.so")
 CALL_SOURCES = [os.path.join(CSRC, "abs_call.cpp"), os.path.join(os.path.dirname(_HERE), "include", "abs_b200.h")]
 
 
@@ -36,29 +36,33 @@ def needs_build() -> bool:
     return _older(LIB_PATH, SOURCES + HEADERS)
 
 
+def call_path() -> str:
+    """The host module of this interpreter and this torch: it is bound to the binary interface of both, so both are in its name."""
+    import torch
+    return os.path.join(_HERE, f"_abs_call-torch{torch.__version__}" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
 def build_call(force: bool = False) -> str:
     """Compile the host module ``_abs_call`` (torch's C++ interface, no kernels) if it is missing or older than its sources."""
-    if not force and not _older(CALL_PATH, CALL_SOURCES):
-        return CALL_PATH
-    import sysconfig
-
+    path = call_path()
+    if not force and not _older(path, CALL_SOURCES):
+        return path
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
     inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
            sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
-    tmp = CALL_PATH + f".tmp{os.getpid()}"
+    tmp = path + f".tmp{os.getpid()}"
     cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
     cmd += [x for p in inc for x in ("-isystem", p)] + ["-o", tmp, CALL_SOURCES[0], "-L" + os.path.join(root, "lib")]
     cmd += ["-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10", "-Wl,-rpath," + os.path.join(root, "lib")]
     subprocess.run(cmd, check=True)
-    os.replace(tmp, CALL_PATH)
-    return CALL_PATH
+    os.replace(tmp, path)
+    return path
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile libabs_b200.so and the host module if they are missing or older than their sources. Returns the library's path."""
-    build_call(force)
+    """Compile libabs_b200.so if it is missing or older than its sources (nvcc only: no torch needed). Returns its path."""
     if not force and not needs_build():
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -71,3 +75,4 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))
+    print(build_call(force="--force" in sys.argv))

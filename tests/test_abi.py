@@ -101,3 +101,22 @@ def test_product_does_not_import_oracle():
         if f.endswith((".py", ".c", ".h")):
             text = open(os.path.join(ROOT, "oracle", f)).read()
             assert "paper_2603_28765_b200" not in text and "abs_b200" not in text, f
+
+
+def test_host_module_is_built_for_this_torch_and_the_library_without_it(B, monkeypatch):
+    """The host module is bound to one torch and one interpreter: a tree in which either has changed must not load the old binary.
+    The C library itself is built by nvcc alone, without torch's headers."""
+    import sysconfig
+
+    import torch
+    from paper_2603_28765_b200 import build
+    B._call()
+    path = build.call_path()
+    assert os.path.exists(path) and path.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and torch.__version__ in path
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert build.call_path() != path
+    commands = []
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, **kw: commands.append(cmd))
+    monkeypatch.setattr(build.os, "replace", lambda a, b: None)
+    build.build(force=True)
+    assert len(commands) == 1 and "nvcc" in commands[0][0]
