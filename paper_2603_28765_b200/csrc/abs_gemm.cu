@@ -625,7 +625,7 @@ size_t abs_matmul_workspace_bytes(abs_fmt_t fmt, int64_t m, int64_t n, int64_t k
 // The product with few rows of A.  Arguments are already validated.
 static abs_status_t skinny_matmul(const SkinnyPlan& P, const void* a_codes, const void* a_scales, const float* a_alpha,
                                   const void* b_codes, const void* b_scales, const float* b_alpha, int64_t m, int64_t n, int64_t k,
-                                  void* out, uint8_t* ws, cudaStream_t s, bool out_bf16, float* next_alpha, float next_denom) {
+                                  void* out, uint8_t* ws, cudaStream_t s, int32_t stall_step, bool out_bf16, float* next_alpha, float next_denom) {
     SkinnyArgs p;
     if (!plane_map(&p.w_codes, const_cast<void*>(b_codes), (uint64_t)n, (uint64_t)k / 2) ||
         !scale_map(&p.w_scales, const_cast<void*>(b_scales), (uint64_t)n, (uint64_t)k / 16))
@@ -635,7 +635,7 @@ static abs_status_t skinny_matmul(const SkinnyPlan& P, const void* a_codes, cons
     p.out = out;
     p.partials = (double*)(ws + P.off_partials);
     p.tickets = (int*)(ws + 1024); p.error = (int*)ws;
-    p.m = (int32_t)m; p.n = (int32_t)n; p.k = (int32_t)k; p.units = P.units;
+    p.m = (int32_t)m; p.n = (int32_t)n; p.k = (int32_t)k; p.units = P.units; p.stall_step = stall_step;
     p.next_alpha = next_alpha; p.next_denom = next_denom;
     if (launch_pdl(skinny_clear_kernel, dim3(1), 256, 0, s, (int*)ws, p.tickets, (int32_t)(n / kTileM)) != cudaSuccess) return ABS_ERR_CUDA;
     const cudaError_t e = launch_pdl(out_bf16 ? skinny_kernel<true> : skinny_kernel<false>, dim3((unsigned)P.grid), kSkinnyThreads,
@@ -684,9 +684,9 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
     });
     if (attr_err[dev] != cudaSuccess) return ABS_ERR_CUDA;
     SkinnyPlan P;
-    if (stall_step < 0 && skinny_plan(fmt, m, n, k, sm_count[dev] < kMaxSms ? sm_count[dev] : kMaxSms, P))
-        return skinny_matmul(P, a_codes, a_scales, a_alpha, b_codes, b_scales, b_alpha, m, n, k, c_f32, ws, s, out_bf16, next_alpha,
-                             next_denom);
+    if (skinny_plan(fmt, m, n, k, sm_count[dev] < kMaxSms ? sm_count[dev] : kMaxSms, P))
+        return skinny_matmul(P, a_codes, a_scales, a_alpha, b_codes, b_scales, b_alpha, m, n, k, c_f32, ws, s, stall_step, out_bf16,
+                             next_alpha, next_denom);
 
     GemmMaps maps;
     for (int p = 0; p < 2; ++p) {

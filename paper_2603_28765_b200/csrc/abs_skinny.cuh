@@ -53,6 +53,7 @@ struct SkinnyArgs {
     double* partials;                      // [blocks][2][32][128]
     int *tickets, *error;                  // tickets: one per tile
     int32_t m, n, k, units;
+    int32_t stall_step;                    // self-test: the bytes of this step of a block are announced and never loaded (-1: none)
     float* next_alpha;
     float next_denom;
 };
@@ -347,8 +348,10 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
             if (elect_one()) {
                 const uint32_t at = raw0 + rs * kSkinnyRawBytes, bar = raw_full0 + 8 * rs;
                 mbar_expect_tx(bar, kSkinnyRawBytes);
-                tma_load_2d(at, &p.w_codes, k0 * 128, tile * kTileM, bar);
-                tma_load_2d(at + kPlaneBytes, &p.w_scales, k0 * 16, tile * kTileM, bar);
+                if ((int32_t)it != p.stall_step) {
+                    tma_load_2d(at, &p.w_codes, k0 * 128, tile * kTileM, bar);
+                    tma_load_2d(at + kPlaneBytes, &p.w_scales, k0 * 16, tile * kTileM, bar);
+                }
             }
             __syncwarp();
             if (++k0 == ksteps) { k0 = 0; ++tile; }

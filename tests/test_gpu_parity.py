@@ -1467,3 +1467,46 @@ def test_tiled_product_rounds_little_over_chunks_of_k(B, k):
     c = B.abs_matmul(1, qa, qb, m, n, k, check=True).double()
     want = 0.5 * decoded_float64(qa, m, k) @ decoded_float64(qb, n, k).t()
     assert (c - want).norm() <= 4.0e-8 * want.norm()
+
+
+@pytest.mark.parametrize("stall_step", [0, 1, 2])
+def test_few_row_waits_run_out_and_are_reported(B, stall_step):
+    """The bounded waits of the few-row kernel: the loads of one step of every block that has it are announced and never issued
+    (blocks of three or four steps; steps of either group of decoder warps).  The waits run out after their limit, the error word is
+    set and reported, and the next call in the same workspace is bit-identical to one before."""
+    import time
+    m, n, k = 8, 4096, 4096
+    qa, qb = B.abs_quantize(1, to_dev(I.generate("cfg2", m, k))), B.abs_quantize(1, to_dev(I.generate("cfg3a", n, k, seed=9)))
+    good = B.abs_matmul(1, qa, qb, m, n, k, check=True)
+    L = B.lib()
+    need = L.abs_matmul_workspace_bytes(1, m, n, k)
+    ws = torch.empty(need + 1024, dtype=torch.uint8, device="cuda")
+    off = (-ws.data_ptr()) % 1024
+    out = torch.empty((m, n), dtype=torch.float32, device="cuda")
+    args = (1, *(t.data_ptr() for t in (*qa, *qb)), m, n, k, out.data_ptr(), ws.data_ptr() + off, need, None)
+    torch.cuda.synchronize()
+    t0 = time.time()
+    assert L.abs_selftest_matmul_stall(*args, stall_step) == 0
+    assert L.abs_matmul_check(ws.data_ptr() + off, None) == 6
+    assert time.time() - t0 < 20.0
+    assert torch.equal(B.abs_matmul(1, qa, qb, m, n, k, workspace=ws, check=True), good)
+
+
+def test_few_row_product_with_nan_scales_and_zero_operands(B, oracle):
+    """E4M3 NaN scale bytes (0x7F, 0xFF) in the few-row kernel poison exactly the rows of their tokens and the columns of their
+    weights, in whole and in shared tiles, and leave every other entry as it was; an all-zero operand gives an all-zero product."""
+    m, n, k = 20, 1280, 4096
+    qa, qb = B.abs_quantize(1, to_dev(I.generate("cfg2", m, k))), B.abs_quantize(1, to_dev(I.generate("cfg3a", n, k, seed=9)))
+    good = B.abs_matmul(1, qa, qb, m, n, k, check=True)
+    sa, sb = qa[1].clone().view(m, k // 16), qb[1].clone().view(n, k // 16)
+    sa[5, 3] = 0x7F
+    sa[19, 255] = 0xFF
+    sb[77, 31] = 0x7F
+    sb[1279, 0] = 0xFF
+    c = B.abs_matmul(1, (qa[0], sa.flatten(), qa[2]), (qb[0], sb.flatten(), qb[2]), m, n, k, check=True)
+    bad = torch.zeros((m, n), dtype=torch.bool, device="cuda")
+    bad[[5, 19], :] = True
+    bad[:, [77, 1279]] = True
+    assert bool(torch.isnan(c[bad]).all()) and torch.equal(c[~bad], good[~bad])
+    zero = B.abs_quantize(1, to_dev(np.zeros((m, k), dtype=np.uint16)))
+    assert bool((B.abs_matmul(1, zero, qb, m, n, k, check=True) == 0).all())
