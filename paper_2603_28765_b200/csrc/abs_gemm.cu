@@ -615,11 +615,12 @@ extern "C" {
 
 size_t abs_matmul_workspace_bytes(abs_fmt_t fmt, int64_t m, int64_t n, int64_t k) {
     if (!gemm_shape_ok(fmt, m, n, k)) return 0;
-    size_t total = gemm_layout(m, n, k).total;
+    // For the largest grid: the size must not depend on the device that happens to be current (which kernel runs does not).  A
+    // workspace for many rows also serves fewer: programs take one for their largest m.
     SkinnyPlan P;
-    // for the largest grid: the size must not depend on the device that happens to be current
-    if (skinny_plan(fmt, m, n, k, kMaxSms, P) && P.total > total) total = P.total;
-    return total;
+    if (skinny_plan(fmt, m, n, k, kMaxSms, P)) return P.total;
+    const size_t total = gemm_layout(m, n, k).total;
+    return skinny_plan(fmt, 1, n, k, kMaxSms, P) && P.total > total ? P.total : total;
 }
 
 // The product with few rows of A.  Arguments are already validated.

@@ -120,3 +120,21 @@ def test_host_module_is_built_for_this_torch_and_the_library_without_it(B, monke
     monkeypatch.setattr(build.os, "replace", lambda a, b: None)
     build.build(force=True)
     assert len(commands) == 1 and "nvcc" in commands[0][0]
+
+
+def test_workspace_of_a_product_with_few_rows(B):
+    """With up to 32 rows of A (IF4) the weights are not copied: header, a ticket per 128 columns and the partial sums of at most 160
+    blocks, whatever the size of B."""
+    for m, n, k in ((1, 128, 256), (24, 14336, 4096), (32, 14336, 14336), (8, 1024, 1024)):
+        blocks = min(160, n // 128 * (k // 256))
+        assert 0 < B.lib().abs_matmul_workspace_bytes(1, m, n, k) <= 2048 + 1024 * (n // 128 * 4 // 1024 + 1) + blocks * 2 * 32 * 128 * 8
+    assert B.lib().abs_matmul_workspace_bytes(1, 33, 14336, 4096) > 14336 * 4096
+
+
+def test_workspace_for_many_rows_serves_fewer(B):
+    """A program that takes one workspace for its largest number of rows must not be refused with fewer, whichever kernel these take."""
+    rows = (1, 8, 9, 31, 32, 33, 128, 129, 1000)
+    for fmt in (0, 1):
+        for n, k in ((128, 256), (1024, 1024), (1280, 2048), (2048, 2048), (4096, 4096), (14336, 4096), (128, 16384), (16384, 256)):
+            sizes = [B.lib().abs_matmul_workspace_bytes(fmt, m, n, k) for m in rows]
+            assert all(sizes) and sizes == sorted(sizes), (fmt, n, k, sizes)
