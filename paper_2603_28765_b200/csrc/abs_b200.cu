@@ -59,7 +59,7 @@ struct DeviceState {
     std::once_flag once;
     cudaError_t init_err = cudaSuccess;
     uint32_t* ring = nullptr;          // ABS_MAX_INFLIGHT slots of 16 bytes: tagged maximum (u64), ticket (u32), pad
-    unsigned long long* cells = nullptr;   // per slot kMaxCells tagged maxima, for the calls that are one kernel (5 MiB)
+    unsigned long long* cells = nullptr;   // per slot kMaxCells tagged maxima, for the calls that are one kernel (1.25 MiB)
     std::mutex slot_mu;                // guards `next` and the clearing of the ring when the generation wraps
     uint64_t next = 0;                 // calls that took a slot so far; generation = low 32 bits
     uint32_t* overrun_host = nullptr;  // pinned, mapped word a kernel sets when its slot was reused under it
@@ -208,20 +208,24 @@ constexpr int kDeqIters = 2;   // groups per thread of the 4-bit dequantize kern
 constexpr int kFastIters = 7;   // groups per thread the IF4 round-to-nearest kernel is launched for
 constexpr int kOptIters = 12;   // same for the Hadamard / stochastic-rounding kernel
 
-// Whether a call finds its maximum inside the quantize kernel (one_pass_alpha): the format and options have a packed kernel,
-// and every group has a thread of one resident wave of it.  (1 to 2.4 million elements, by the blocks per SM that the
-// kernel is compiled for.)
+// Whether a call finds its maximum inside the quantize kernel (one_pass_alpha), on a grid of at most one block per SM: the format
+// and options have a packed kernel, and a thread has no more than two to four groups, by what the kernel
+// computes per group: 1.2 to 2.4 million elements.  At the upper end, IF4, 2.4 million, both routes take about the same on the
+// device (10.2 us against 10.2 to 11.3), and one of two launches is saved on the host.
 bool one_pass(int fmt, const abs_opts_t& o, int sm_count, int64_t ngroups, bool emulate) {
     const bool rht = o.flags & ABS_F_HADAMARD16, sr = o.flags & ABS_F_STOCHASTIC;
-    int per_sm = 0;
+    int per_thread = 0;
     switch (fmt) {
-        case ABS_FMT_NVFP4: case ABS_FMT_IF4: per_sm = (rht || sr || emulate) ? opt_blocks_per_sm(sr, rht) : kFastMinBlocks; break;
-        case ABS_FMT_NVFP4_BS8: case ABS_FMT_IF4_BS8: per_sm = (rht || sr) ? 0 : 4; break;
-        default: per_sm = (rht || sr) ? 0 : 3; break;       // IF3, IF6
+        case ABS_FMT_NVFP4: case ABS_FMT_IF4: per_thread = (rht || sr || emulate) ? opt_blocks_per_sm(sr, rht) : kFastMinBlocks; break;
+        case ABS_FMT_NVFP4_BS8: case ABS_FMT_IF4_BS8: per_thread = (rht || sr) ? 0 : 4; break;
+        default: per_thread = (rht || sr) ? 0 : 3; break;       // IF3, IF6
     }
-    int64_t blocks = (int64_t)sm_count * per_sm;
-    if (blocks > kMaxCells) blocks = kMaxCells;
-    return !(o.flags & ABS_F_INDEX64) && (ngroups + kThreads - 1) / kThreads <= blocks;
+    return !(o.flags & ABS_F_INDEX64) && ngroups <= (int64_t)grid_for(sm_count < kMaxCells ? sm_count : kMaxCells, ngroups, 1) * kThreads * per_thread;
+}
+// Grid of a quantize kernel: see one_pass and grid_waves.
+int quantize_grid(const AlphaSrc& alpha, int sm_count, int64_t ngroups, int resident_per_sm, int target_iters) {
+    if (alpha.cells) return grid_for(sm_count < kMaxCells ? sm_count : kMaxCells, ngroups, 1);
+    return grid_waves(sm_count, ngroups, resident_per_sm, target_iters);
 }
 
 template <int FMT>
@@ -243,7 +247,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
     if constexpr (FMT == ABS_FMT_NVFP4 || FMT == ABS_FMT_IF4) {
         if (emul_out) return ABS_ERR_FLAGS;      // the 4-bit emulation pass is launched by abs_quantize_dequantize
         if (!rht && !sr) {   // the 4-bit round-to-nearest fast path
-            const int pgrid = FMT == ABS_FMT_IF4 ? grid_waves(sm_count, ngroups, kFastMinBlocks, kFastIters) : grid_waves(sm_count, ngroups, 5, kNvIters);
+            const int pgrid = FMT == ABS_FMT_IF4 ? quantize_grid(alpha, sm_count, ngroups, kFastMinBlocks, kFastIters) : quantize_grid(alpha, sm_count, ngroups, 5, kNvIters);
             constexpr bool kInt = FMT == ABS_FMT_IF4;
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             // the kernel looks three grid strides past the current group (next group, and its L2 prefetch)
@@ -281,7 +285,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
     }
     if constexpr (FMT == ABS_FMT_NVFP4 || FMT == ABS_FMT_IF4) {
         // Hadamard / stochastic-rounding options of the 4-bit formats: the packed persistent kernel
-        const int ogrid = grid_waves(sm_count, ngroups, opt_blocks_per_sm(sr, rht), kOptIters);
+        const int ogrid = quantize_grid(alpha, sm_count, ngroups, opt_blocks_per_sm(sr, rht), kOptIters);
         if (!(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)ogrid * kThreads) {
             constexpr bool kInt = FMT == ABS_FMT_IF4;
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
@@ -302,7 +306,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
     if constexpr (FMT == ABS_FMT_NVFP4_BS8 || FMT == ABS_FMT_IF4_BS8) {
         // block-size-8 variants of the 4-bit formats, round-to-nearest: two groups of 8 per thread
         constexpr bool kInt = FMT == ABS_FMT_IF4_BS8;
-        const int bgrid = grid_waves(sm_count, ngroups, kInt ? 4 : 5, kInt ? kIf6Iters : 5);
+        const int bgrid = quantize_grid(alpha, sm_count, ngroups, kInt ? 4 : 5, kInt ? kIf6Iters : 5);
         if (!rht && !sr && !(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)bgrid * kThreads) {
             if (handled) *handled = true;
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
@@ -315,7 +319,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
     }
     if constexpr (FMT == ABS_FMT_IF6_E2M3 || FMT == ABS_FMT_IF6_E3M2) {
         // 6-bit formats, round-to-nearest
-        const int sgrid = grid_waves(sm_count, ngroups, 3, kIf6Iters);
+        const int sgrid = quantize_grid(alpha, sm_count, ngroups, 3, kIf6Iters);
         if (!rht && !sr && !(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)sgrid * kThreads) {
             if (handled) *handled = true;
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
@@ -329,7 +333,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
     if constexpr (FMT == ABS_FMT_IF3 || FMT == ABS_FMT_IF3_BS8) {
         // IF3 and its block-size-8 variant, round-to-nearest
         constexpr int kG = FMT == ABS_FMT_IF3 ? 16 : 8;
-        const int tgrid = grid_waves(sm_count, ngroups, kIf3MinBlocks, kIf6Iters);
+        const int tgrid = quantize_grid(alpha, sm_count, ngroups, kIf3MinBlocks, kIf6Iters);
         if (!rht && !sr && !(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)tgrid * kThreads) {
             if (handled) *handled = true;
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
@@ -709,10 +713,11 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
             return (!handled && r == ABS_ERR_FLAGS) ? ABS_ERR_SIZE : r;
         }
         cudaError_t e = cudaSuccess;
+        const int egrid = quantize_grid(src, st->sm_count, ngroups, opt_blocks_per_sm(sr, rht), (rht || sr) ? kOptIters : kFastIters);
 #define ABS_LAUNCH_E2(I, R, S)                                                                                      \
         e = launch_any(src.cells != nullptr, src.cells ? quantize4_opt_kernel<I, R, S, kOnePass, true>                   \
                                              : src.slot ? quantize4_opt_kernel<I, R, S, kFromSlot, true>                 \
-                                                        : quantize4_opt_kernel<I, R, S, kGiven, true>, grid, kThreads, s, \
+                                                        : quantize4_opt_kernel<I, R, S, kGiven, true>, egrid, kThreads, s, \
                        (const uint4*)in_bf16, (uint2*)codes_u8, (uint8_t*)scales_e4m3, src, (int32_t)ngroups, mul,        \
                        (uint32_t)o.had_sign_mask, pk, ctr, a32, (uint4*)out_bf16, o32, store)
 #define ABS_LAUNCH_E(I)                                                                                             \

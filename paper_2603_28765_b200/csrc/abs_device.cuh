@@ -351,7 +351,7 @@ struct AlphaSrc {
 };
 // How a kernel learns alpha.
 enum AlphaKind { kGiven = 0, kFromSlot = 1, kOnePass = 2 };
-constexpr int kMaxCells = 640;            // blocks of a one-pass grid: four per SM on up to 160 SMs
+constexpr int kMaxCells = 160;            // blocks of a one-pass grid: one per SM on up to 160 SMs
 // After the amax pass of the same call the slot holds this call's generation.  Any other generation means
 // that a later call reused the slot while this one was still in flight (more than ABS_MAX_INFLIGHT calls
 // between the two): the maximum is lost.  The kernel then reports it through the host-mapped word, which
@@ -393,12 +393,14 @@ __device__ __forceinline__ float resolve_alpha_per_thread(const AlphaSrc& a) {
     return alpha;
 }
 
-// Eq. 1 inside the quantize kernel itself, for tensors whose groups all fit one resident wave of threads: every block
+// Eq. 1 inside the quantize kernel itself, for small tensors (a few groups per thread of a grid of one block per SM): every block
 // publishes the maximum of its groups (local: the bit pattern of this thread's largest |x|) in its cell, tagged like the
 // slots of the two-kernel calls, and waits for the cells of the whole grid, which is launched cooperatively.  The second
 // read of the input and one of two launches go (host time of a small abs_quantize 12.5 -> 8.8 us; on the device 3.1 us
 // against 1.9 + 2.4 us and the gap between them, 1 x 4096).  No atomics are shared between blocks; a cell that carries a
 // later call's tag means the same as in slot_amax.  The wait is bounded (one second) and reports like an overrun.
+// One block per SM, because the whole grid has to find room at once: beside a library GEMM of one block per SM on another
+// stream, grids of two and four blocks per SM waited for its end (251 and 273 us, two-kernel calls 17 and 24), one of one did not.
 __device__ __forceinline__ float one_pass_alpha(const AlphaSrc& a, uint32_t local) {
     __shared__ uint32_t warp_max[32];
     __shared__ float alpha_shared;
@@ -451,10 +453,25 @@ __device__ __forceinline__ uint32_t group_max_bits(const uint32_t (&w)[8]) {
     for (int i = 1; i < 8; ++i) m = __vmaxu2(m, w[i] & 0x7FFF7FFFu);
     return max(m & 0xFFFFu, m >> 16) << 16;
 }
-// alpha of a kernel of kind SRC; w holds the thread's first (one-pass: only) group where it has one.
-template <int SRC>
-__device__ __forceinline__ float alpha_of(const AlphaSrc& a, const uint32_t (&w)[8], bool active) {
-    if constexpr (SRC == kOnePass) return one_pass_alpha(a, active ? group_max_bits(w) : 0u);
+// Largest bits(group) over a thread's groups g, g + stride, ...; w holds the first, if there is one.
+template <typename IdxT, typename Bits>
+__device__ __forceinline__ uint32_t thread_max_bits(const uint32_t (&w)[8], const uint4* in, IdxT g, IdxT stride, IdxT ngroups, bool aligned32,
+                                                    Bits bits) {
+    uint32_t m = g < ngroups ? bits(w) : 0u;
+    for (IdxT gn = g + stride; gn < ngroups; gn += stride) {
+        uint32_t r[8];
+        if (aligned32) load32B<true>(in + 2 * (size_t)gn, r);
+        else load32B<false>(in + 2 * (size_t)gn, r);
+        m = max(m, bits(r));
+    }
+    return m;
+}
+// alpha of a kernel of kind SRC; w holds the thread's first group where it has one.
+template <int SRC, typename IdxT>
+__device__ __forceinline__ float alpha_of(const AlphaSrc& a, const uint32_t (&w)[8], const uint4* in, IdxT g, IdxT stride, IdxT ngroups,
+                                          bool aligned32) {
+    if constexpr (SRC == kOnePass)
+        return one_pass_alpha(a, thread_max_bits(w, in, g, stride, ngroups, aligned32, [](const uint32_t (&r)[8]) { return group_max_bits(r); }));
     else return resolve_alpha_per_thread<SRC == kFromSlot>(a);
 }
 

@@ -161,7 +161,7 @@ quantize4_fast_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, u
     // instance is bound by arithmetic and measured 1 % slower that way, so it walks forwards.
     auto at = [&](IdxT gg) -> IdxT { return (FROM_SLOT && !HAS_INT) ? (IdxT)(ngroups - 1 - gg) : gg; };
     if (active) load32B<ALIGNED32>(in + 2 * (size_t)at(g), w);
-    const float alpha = alpha_of<SRC>(alpha_src, w, active);                 // T2
+    const float alpha = alpha_of<SRC>(alpha_src, w, in, g, stride, ngroups, ALIGNED32);          // T2
     // G5 once per block for every scale byte 0x00..0x7E: d = Delta * alpha, 1 / d, d * 6/7 (8192x4096: 16.68 -> 16.56 us)
     __shared__ float4 scale_lut[128];
     if (threadIdx.x < 127) {

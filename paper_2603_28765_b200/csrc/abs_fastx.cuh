@@ -154,7 +154,7 @@ quantize4_bs8_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
         if (aligned32) load32B<true>(in + 2 * (size_t)g, w);
         else load32B<false>(in + 2 * (size_t)g, w);
     }
-    const float alpha = alpha_of<SRC>(alpha_src, w, active);                 // T2
+    const float alpha = alpha_of<SRC>(alpha_src, w, in, g, stride, nblocks16, aligned32);        // T2
     __shared__ float2 scale_table[128];
     fill_scale_table(scale_table, alpha);                                    // G5 for every scale byte, once per block
     if (!active) return;
@@ -339,7 +339,7 @@ quantize6_fast_kernel(const uint4* __restrict__ in, uint32_t* __restrict__ codes
         if (aligned32) load32B<true>(in + 2 * (size_t)g, w);
         else load32B<false>(in + 2 * (size_t)g, w);
     }
-    const float alpha = alpha_of<SRC>(alpha_src, w, active);                 // T2
+    const float alpha = alpha_of<SRC>(alpha_src, w, in, g, stride, ngroups, aligned32);          // T2
     if (!active) return;
     const float inv_a6 = __frcp_rn(__fmul_rn(alpha, F::M_FP));               // T3
     const float c_pre = __fdiv_rn(F::M_INT, F::M_FP), c_post = __fdiv_rn(F::M_FP, F::M_INT);
@@ -527,7 +527,7 @@ quantize3_fast_kernel(const uint4* __restrict__ in, uint16_t* __restrict__ codes
         if (aligned32) load32B<true>(in + 2 * (size_t)g, w);
         else load32B<false>(in + 2 * (size_t)g, w);
     }
-    const float alpha = alpha_of<SRC>(alpha_src, w, active);                 // T2
+    const float alpha = alpha_of<SRC>(alpha_src, w, in, g, stride, ngroups, aligned32);          // T2
     if (!active) return;
     const float inv_a6 = __frcp_rn(__fmul_rn(alpha, 4.0f));                  // T3
     // one block of 16 values held in `w`, index `g`

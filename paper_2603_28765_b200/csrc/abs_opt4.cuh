@@ -195,16 +195,16 @@ quantize4_opt_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
         smask[i] = (((sign_mask >> (2 * i)) & 1u) << 15) | (((sign_mask >> (2 * i + 1)) & 1u) << 31);
     float alpha;                                                             // T2
     if constexpr (SRC == kOnePass && RHT) {
-        float m = 0.0f;
-        if (active) {
-            float x[16];
-            hadamard16_packed(w, smask, x);
+        auto bits = [&](const uint32_t (&r)[8]) {
+            float x[16], m = 0.0f;
+            hadamard16_packed(r, smask, x);
 #pragma unroll
             for (int i = 0; i < 16; i += 2) m = max3abs(m, x[i], x[i + 1]);
-        }
-        alpha = one_pass_alpha(alpha_src, __float_as_uint(m));
+            return __float_as_uint(m);
+        };
+        alpha = one_pass_alpha(alpha_src, thread_max_bits(w, in, g, stride, ngroups, aligned32, bits));
     } else {
-        alpha = alpha_of<SRC>(alpha_src, w, active);
+        alpha = alpha_of<SRC>(alpha_src, w, in, g, stride, ngroups, aligned32);
     }
     __shared__ float2 scale_table[128];
     fill_scale_table(scale_table, alpha);                                    // G5 for every scale byte, once per block

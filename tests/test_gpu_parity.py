@@ -1331,8 +1331,8 @@ def test_small_quantize_with_fewer_sms_than_the_device(B):
 
 
 def test_full_wave_one_kernel_quantize_on_several_streams(B):
-    """Grids that fill the device (2, 3 and 4 blocks per SM) and wait for all of their blocks, on four streams from four threads,
-    among larger two-kernel calls and products: every call's bytes as when it ran alone."""
+    """The largest calls of the one-kernel route (2, 3 and 4 groups per thread of a grid of one block per SM that waits for all of its
+    blocks), on four streams from four threads, among larger two-kernel calls and products: every call's bytes as when it ran alone."""
     import threading
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     g = torch.Generator(device="cuda").manual_seed(12)
@@ -1510,3 +1510,29 @@ def test_few_row_product_with_nan_scales_and_zero_operands(B, oracle):
     assert bool(torch.isnan(c[bad]).all()) and torch.equal(c[~bad], good[~bad])
     zero = B.abs_quantize(1, to_dev(np.zeros((m, k), dtype=np.uint16)))
     assert bool((B.abs_matmul(1, zero, qb, m, n, k, check=True) == 0).all())
+
+
+def test_small_quantize_beside_a_long_kernel(B):
+    """The largest one-kernel call on one stream while a library GEMM of most of a millisecond, one block per SM, runs on another: its
+    grid finds room beside the GEMM's blocks.  It takes some 17 us there; grids of two and four blocks per SM took 250 us and more."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    x = torch.randn((4 * sms * 256, 16), device="cuda").bfloat16()
+    want = B.abs_quantize(1, x)
+    a = torch.randn((8192, 8192), device="cuda").bfloat16()
+    out = torch.mm(a, a)
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    times = []
+    for _ in range(9):
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s1):
+            torch.mm(a, a, out=out)
+        begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        with torch.cuda.stream(s2):
+            torch.cuda._sleep(60000)                                     # the GEMM is under way
+            begin.record()
+            got = B.abs_quantize(1, x)
+            end.record()
+        torch.cuda.synchronize()
+        times.append(begin.elapsed_time(end))
+        assert all(torch.equal(p, q) for p, q in zip(want, got))
+    assert sorted(times)[4] < 0.1, times
