@@ -104,9 +104,9 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
 }
 // D[tmem] (+)= A[smem] * B[smem]^T, 128 x 128 x 64, E2M1 operands, one UE4M3 scale per 16 elements read from tensor memory.
 // What happens to the A operand in the tensor core's collector buffer: read from shared memory and dropped, read and
-// kept (kFill), taken from the buffer and kept (kUse), taken from the buffer and dropped (kLastUse).  An MMA that
-// takes A from the buffer reads only B from shared memory.
-enum Collector { kDiscard, kFill, kUse, kLastUse };
+// kept (kFill), taken from the buffer and dropped (kLastUse).  An MMA that takes A from the buffer reads only B from shared
+// memory.
+enum Collector { kDiscard, kFill, kLastUse };
 template <Collector C = kDiscard>
 __device__ __forceinline__ void tc_mma_nvf4(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate,
                                             uint32_t sfa_tmem, uint32_t sfb_tmem) {
@@ -116,7 +116,6 @@ __device__ __forceinline__ void tc_mma_nvf4(uint32_t d_tmem, uint64_t a_desc, ui
                  :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(sfa_tmem), "r"(sfb_tmem) \
                  : "memory")
     if constexpr (C == kFill) ABS_MMA_NVF4(".collector::a::fill");
-    else if constexpr (C == kUse) ABS_MMA_NVF4(".collector::a::use");
     else if constexpr (C == kLastUse) ABS_MMA_NVF4(".collector::a::lastuse");
     else ABS_MMA_NVF4("");
 #undef ABS_MMA_NVF4
