@@ -250,7 +250,10 @@ ABS_API float abs_alpha_from_amax(abs_fmt_t fmt, float amax);
  *   b_codes, b_scales  B likewise: [n, k]
  *   c_f32              out, [m, n] float, row-major
  *   workspace          device memory, 1024-byte aligned, at least abs_matmul_workspace_bytes(fmt, m, n, k) bytes
- * With up to 32 rows of A (IF4) the weights are read where they lie and split on the way to the tensor cores instead.
+ * With up to 32 rows of A (IF4) the weights are read where they lie and split on the way to the tensor cores instead, and the
+ * order of the sums over K follows the number of SMs: a row of C may then differ, by rounding only (2-norm error against
+ * 64 bits 2.6e-8, above 32 rows 4e-8), from the same row of a product with more rows, and from that of a GPU with other SMs.
+ * A workspace taken for m rows also serves fewer (n, k and fmt the same).
  * m is any positive number of rows; n must be a multiple of 128, k a multiple of 256 (ABS_ERR_SHAPE otherwise; abs_matmul_workspace_bytes
  * returns 0).  Asynchronous like the other calls.  Every wait inside the kernel is bounded; if one runs out (it
  * never should) the kernel stops and leaves a non-zero word at the start of the workspace, which

@@ -20,9 +20,9 @@
 // eight (IF4) warps read the accumulators back (tcgen05.ld) and write C.  Every mbarrier wait is bounded in time: when a
 // wait runs out the block raises an error word, stops issuing, frees its tensor memory and returns.
 //
-// What bounds it: the feed of the operands from the L2, about 40 bytes per cycle and SM with one tile per block (both
-// formats spend some 1650 cycles on a stage of 64 KiB, of which the tensor pipe is active in 1024 for IF4 and in 512 for
-// NVFP4).  4096^3, operands and split included: IF4 195 -> 118 us (nine MMAs per K-block to four), 8192 x 14336 x 4096
+// What bounds it, by the counts: shared memory at 128 bytes per cycle.  IF4: an MMA takes 97 cycles, 64 of them tensor work;
+// beside it stand up to 8 KiB of operand reads (less where A comes from the collector buffer) and 4 KiB of TMA writes, 64
+// + 32 cycles.  NVFP4: 160 KiB per step of two boxes.  The feed from the L2 is at a third of its peak.  4096^3, operands and split included: IF4 195 -> 118 us (nine MMAs per K-block to four), 8192 x 14336 x 4096
 // 1440 -> 785 us; NVFP4 46 and 340 us.
 #include "../../include/abs_b200.h"
 #include "abs_tc.cuh"
