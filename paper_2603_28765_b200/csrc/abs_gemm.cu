@@ -26,6 +26,7 @@
 // 1440 -> 785 us; NVFP4 46 and 340 us.
 #include "../../include/abs_b200.h"
 #include "abs_tc.cuh"
+#include "abs_rows.cuh"
 #include "abs_skinny.cuh"
 
 #include <cuda.h>
@@ -604,6 +605,29 @@ bool skinny_plan(abs_fmt_t fmt, int64_t m, int64_t n, int64_t k, int sm_count, S
     return true;
 }
 
+// The product with very few rows of A (see abs_rows.cuh).
+int rows_instance(int64_t m) { return m <= 1 ? 1 : m <= 2 ? 2 : m <= 4 ? 4 : 8; }
+// The rule: its time grows with rows times the size of B from next to nothing, while the tensor-core kernels for few rows start at 9 us (IF4)
+// and 8 us (NVFP4) and hardly depend on the rows; the lines cross where the rows (of the instance) times n k are 224 million.
+// us here / there, IF4: 1 row 14336 x 14336 (206 million) 48.8 / 48.2, 2 rows 14336 x 4096 (117) 15.0 / 19.1, 4 rows 14336 x 4096 (235) 18.0 /
+// 19.1, 8 rows 4096 x 4096 (134) 10.4 / 13.3, 8 rows 14336 x 4096 (470) 25.6 / 19.1; NVFP4: 45 / 50, 14.0 / 16.8, 17.9 / 16.8, 9.9 / 11.2, 25 / 16.8.
+bool rows_rule(int64_t m, int64_t n, int64_t k) {
+    return m <= kRowsMax && n * k <= 224000000 / rows_instance(m) && rows_smem_bytes(rows_instance(m), k) <= (size_t)kRowsMaxSmem;
+}
+typedef void (*RowsKernel)(RowsArgs);
+template <int M> RowsKernel rows_kernel_for(bool has_int, bool out_bf16) {
+    return has_int ? (out_bf16 ? rows_kernel<M, true, true> : rows_kernel<M, true, false>)
+                   : (out_bf16 ? rows_kernel<M, false, true> : rows_kernel<M, false, false>);
+}
+RowsKernel rows_kernel_of(int64_t m, bool has_int, bool out_bf16) {
+    switch (rows_instance(m)) {
+        case 1: return rows_kernel_for<1>(has_int, out_bf16);
+        case 2: return rows_kernel_for<2>(has_int, out_bf16);
+        case 4: return rows_kernel_for<4>(has_int, out_bf16);
+        default: return rows_kernel_for<8>(has_int, out_bf16);
+    }
+}
+
 bool gemm_shape_ok(abs_fmt_t fmt, int64_t m, int64_t n, int64_t k) {
     return (fmt == ABS_FMT_IF4 || fmt == ABS_FMT_NVFP4) && m > 0 && n > 0 && k > 0 && n % kTileN == 0 &&
            k % kStageK == 0 && m < ((int64_t)1 << 30) && n < ((int64_t)1 << 30) && k < ((int64_t)1 << 30);
@@ -645,6 +669,27 @@ static abs_status_t skinny_matmul(const SkinnyPlan& P, const void* a_codes, cons
     return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
 }
 
+// The product with very few rows of A.  Arguments are already validated.
+static abs_status_t rows_matmul(bool has_int, const void* a_codes, const void* a_scales, const float* a_alpha, const void* b_codes,
+                                const void* b_scales, const float* b_alpha, int64_t m, int64_t n, int64_t k, void* out, uint8_t* ws,
+                                cudaStream_t s, int sm_count, bool out_bf16, float* next_alpha, float next_denom) {
+    RowsArgs p;
+    p.w_codes = (const uint8_t*)b_codes; p.w_scales = (const uint8_t*)b_scales;
+    p.x_codes = (const uint8_t*)a_codes; p.x_scales = (const uint8_t*)a_scales;
+    p.alpha_a = a_alpha; p.alpha_b = b_alpha;
+    p.out = out; p.error = (int*)ws;
+    p.m = (int32_t)m; p.n = (int32_t)n; p.k = (int32_t)k;
+    p.next_alpha = next_alpha; p.next_denom = next_denom;
+    // the maximum and its ticket start at zero; without them the kernel clears the error word itself
+    if (next_alpha && launch_pdl(skinny_clear_kernel, dim3(1), 32, 0, s, (int*)ws, (int*)ws, 0) != cudaSuccess) return ABS_ERR_CUDA;
+    const size_t smem = rows_smem_bytes(rows_instance(m), k);
+    const int64_t turns = n / kRowsPerTurn;
+    const int64_t fit = kRowsMaxSmem / (int64_t)smem, blocks = (int64_t)sm_count * (fit < rows_blocks(rows_instance(m)) ? fit : rows_blocks(rows_instance(m)));
+    if (launch_pdl(rows_kernel_of(m, has_int, out_bf16), dim3((unsigned)(turns < blocks ? turns : blocks)), kRowsThreads, smem, s, p) != cudaSuccess)
+        return ABS_ERR_CUDA;
+    return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
+}
+
 static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* a_scales, const float* a_alpha, const void* b_codes,
                                 const void* b_scales, const float* b_alpha, int64_t m, int64_t n, int64_t k, void* c_f32,
                                 void* workspace, size_t workspace_bytes, void* stream, int32_t stall_step, bool out_bf16 = false,
@@ -682,8 +727,14 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
             attr_err[dev] = cudaFuncSetAttribute(skinny_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkinnySmemBytes);
         if (attr_err[dev] == cudaSuccess)
             attr_err[dev] = cudaFuncSetAttribute(skinny_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkinnySmemBytes);
+        for (int i = 0; i < 16; ++i)
+            if (attr_err[dev] == cudaSuccess)
+                attr_err[dev] = cudaFuncSetAttribute(rows_kernel_of(1 << (i >> 2), i & 1, i & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsMaxSmem);
     });
     if (attr_err[dev] != cudaSuccess) return ABS_ERR_CUDA;
+    if (stall_step < 0 && rows_rule(m, n, k))      // (the self-test of the waits is for kernels that have some)
+        return rows_matmul(has_int, a_codes, a_scales, a_alpha, b_codes, b_scales, b_alpha, m, n, k, c_f32, ws, s, sm_count[dev], out_bf16,
+                           next_alpha, next_denom);
     SkinnyPlan P;
     if (skinny_plan(fmt, m, n, k, sm_count[dev] < kMaxSms ? sm_count[dev] : kMaxSms, P))
         return skinny_matmul(P, a_codes, a_scales, a_alpha, b_codes, b_scales, b_alpha, m, n, k, c_f32, ws, s, stall_step, out_bf16,

@@ -1,0 +1,224 @@
+// IF4 and NVFP4 products with very few rows of A (a decoder step's tokens, up to 8): C = A B^T with the arithmetic of
+// abs_gemm.cu on the integer and FP64 pipes, in one pass over the weights B where they lie.
+//
+// With one token a product is 16 multiply-adds per 9 bytes of weights: what counts is how early the weights are asked for and how
+// little stands around that.  Here a warp owns two rows of B at a time and all of K (lane i: two groups of
+// each 1024 values, 16 bytes), so nothing is shared between blocks and no partial sum leaves a warp; the rows of its first
+// turn are requested into the L2 before the kernel waits for its predecessor, those of the next one at the start of each.
+// Product alone, weights not in the L2, IF4 (before: abs_skinny.cuh; NVFP4: abs_gemm.cu's kernel): 1 row 4096 x 4096 14.3 -> 5.4 us, 14336 x 4096
+// 21.5 -> 13.1; 8 rows 4096 x 4096 16.5 -> 10.4; NVFP4 1 row 4096 x 4096 11.2 -> 5.2.  What bounds it: issue slots are used to 51 %, the
+// integer pipe to 48 %, the rest is waiting for the weights of the first turn (two thirds of B at 14336 x 4096) and a last turn
+// that not all warps have.
+//
+// Arithmetic.  A code stands for an integer u, twice the E2M1 value in an FP group and k in an integer group (-12 .. 12), times
+// its scale times 1/2 or 6/7.  The tokens are laid out once per block as signed bytes in shared memory; the bytes u + 16 of
+// four weights come from two byte permutes (their sign mode gives zero for the half of the codes that the table does not hold,
+// so an "or" joins both), and dp4a sums the products of a pair of groups exactly.  Its first addend removes the 16 and adds 2^31, so that
+// the sum is the low word of a double above 2^52 and needs no conversion.  Everything after that is FP64 up to the one rounding of
+// the result (2-norm error against 64 bits 2.3e-8, that rounding alone).
+#pragma once
+#include "abs_tc.cuh"
+
+namespace absq {
+
+constexpr int kRowsMax = 8;                          // rows of A
+constexpr int kRowsWarps = 8, kRowsThreads = 32 * kRowsWarps, kRowsPerTurn = 2;
+constexpr int kRowsChunk = 1024;                     // of K: two groups per lane
+// Shared memory: scale byte -> its value times 1/2 or 6/7; then per chunk, half of a lane's pair of groups, token and lane: 16 bytes of
+// A, its scale as a double, the first addend of the dot product.
+constexpr int kRowsTable = 256 * 8, kRowsMaxSmem = 220 * 1024;
+constexpr size_t rows_smem_bytes(int tokens, int64_t k) { return kRowsTable + (size_t)((k + kRowsChunk - 1) / kRowsChunk) * 64 * tokens * 28; }
+
+// Blocks per SM: as many warps as the registers of the instance allow (62, 64, 80, 128 a thread).
+constexpr int rows_blocks(int tokens) { return tokens <= 2 ? 4 : tokens <= 4 ? 3 : 2; }
+
+struct RowsArgs {
+    const uint8_t *w_codes, *w_scales, *x_codes, *x_scales;
+    const float *alpha_a, *alpha_b;
+    void* out;                                       // [m, n] bf16 or FP32
+    int* error;                                      // error word (cleared here), output maximum, ticket of the maximum
+    int32_t m, n, k;
+    float* next_alpha;
+    float next_denom;
+};
+
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return r;
+}
+// c + the sum of four products, unsigned bytes of a times signed bytes of b
+__device__ __forceinline__ uint32_t dot4(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t d;
+    asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+// The sixteen codes of a group as bytes u + 16.  FP: 0, 1, 2, 3, 4, 6, 8, 12 and their negatives; integer: two's complement.
+template <bool HAS_INT>
+__device__ __forceinline__ void group_bytes(uint32_t w0, uint32_t w1, bool is_int, uint32_t (&u)[4]) {
+    uint32_t p0 = 0x13121110u, p1 = 0x1C181614u, n0 = 0x0D0E0F10u, n1 = 0x04080A0Cu;
+    if (HAS_INT && is_int) { p1 = 0x17161514u; n0 = 0x0B0A0908u; n1 = 0x0F0E0D0Cu; }     // codes 0 .. 7 and -8 .. -1
+    const uint32_t v0 = w0 ^ 0x88888888u, v1 = w1 ^ 0x88888888u;
+    u[0] = prmt(p0, p1, w0) | prmt(n0, n1, v0);
+    u[1] = prmt(p0, p1, w0 >> 16) | prmt(n0, n1, v0 >> 16);
+    u[2] = prmt(p0, p1, w1) | prmt(n0, n1, v1);
+    u[3] = prmt(p0, p1, w1 >> 16) | prmt(n0, n1, v1 >> 16);
+}
+
+// M: rows of A the instance is made for (p.m <= M).
+template <int M, bool HAS_INT, bool OUT_BF16>
+__global__ void __launch_bounds__(kRowsThreads, rows_blocks(M)) rows_kernel(const __grid_constant__ RowsArgs p) {
+    constexpr int R = kRowsPerTurn;
+    extern __shared__ __align__(16) uint8_t rows_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int32_t chunks = (p.k + kRowsChunk - 1) / kRowsChunk, turns = p.n / R, step = (int32_t)gridDim.x * kRowsWarps;
+    const uint32_t code_pitch = (uint32_t)p.k / 2, scale_pitch = (uint32_t)p.k / 16;
+    double* const table = reinterpret_cast<double*>(rows_smem);
+    uint4* const xs = reinterpret_cast<uint4*>(rows_smem + kRowsTable);
+    double* const xd = reinterpret_cast<double*>(xs + (size_t)chunks * 64 * M);
+    uint32_t* const xi = reinterpret_cast<uint32_t*>(xd + (size_t)chunks * 64 * M);
+
+    pdl_launch_dependents();
+    int32_t turn = warp * (int32_t)gridDim.x + (int32_t)blockIdx.x;
+    auto request = [&](int32_t t) {                  // the rows of a turn into the L2: consecutive bytes
+        if (t >= turns) return;
+        const uint8_t* c = p.w_codes + (size_t)t * R * code_pitch;
+        const uint8_t* s = p.w_scales + (size_t)t * R * scale_pitch;
+        for (uint32_t at = lane * 128u; at < R * code_pitch; at += 4096u) prefetch_l2(c + at);
+        for (uint32_t at = lane * 128u; at < R * scale_pitch; at += 4096u) prefetch_l2(s + at);
+    };
+    request(turn);
+    if (threadIdx.x < 256) {
+        const float v = (threadIdx.x & 0x7Fu) == 0x7Fu ? __uint_as_float(0x7FC00000u) : e4m3_value(threadIdx.x & 0x7Fu);
+        table[threadIdx.x] = HAS_INT && (threadIdx.x & 0x80u) ? __dmul_rn((double)v, 6.0 / 7.0) : __dmul_rn((double)v, 0.5);
+    }
+    pdl_wait();
+
+    // this lane's 32 codes and two scales of a chunk of the rows of a turn
+    struct Piece { uint4 codes; uint32_t two; };
+    Piece w[R], wn[R];
+    auto load = [&](Piece (&q)[R], int32_t t, int32_t chunk) {
+        const uint32_t at = (uint32_t)chunk * 64u + 2u * lane;                       // first of the two groups
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            q[r].codes = make_uint4(0u, 0u, 0u, 0u);
+            q[r].two = 0u;
+            if (at < scale_pitch) {
+                const size_t row = (size_t)t * R + r;
+                q[r].codes = __ldg(reinterpret_cast<const uint4*>(p.w_codes + row * code_pitch + at * 8u));
+                q[r].two = __ldg(reinterpret_cast<const uint16_t*>(p.w_scales + row * scale_pitch + at));
+            }
+        }
+    };
+    if (turn < turns) load(w, turn, 0);
+    __syncthreads();                                                                 // the table
+
+    // the tokens: one group per thread and trip
+    for (int32_t i = threadIdx.x; i < chunks * 64 * M; i += kRowsThreads) {
+        const int32_t l = i & 31, t = (i >> 5) % M, half = (i >> 5) / M;             // place i = ((chunk * 2 + half) * M + token) * 32 + lane
+        const uint32_t g = (uint32_t)(half >> 1) * 64u + 2u * l + (half & 1);
+        uint32_t u[4] = {0x10101010u, 0x10101010u, 0x10101010u, 0x10101010u}, sb = 0u;
+        if (t < p.m && g < scale_pitch) {
+            const uint2 c = __ldg(reinterpret_cast<const uint2*>(p.x_codes + (size_t)t * code_pitch + g * 8u));
+            sb = __ldg(p.x_scales + (size_t)t * scale_pitch + g);
+            group_bytes<HAS_INT>(c.x, c.y, sb & 0x80u, u);
+        }
+        uint32_t sum16 = 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            u[q] = ((u[q] | 0x80808080u) - 0x10101010u) ^ 0x80808080u;               // bytes u, two's complement
+            sum16 = dot4(0x10101010u, u[q], sum16);
+        }
+        xs[i] = make_uint4(u[0], u[1], u[2], u[3]);
+        xd[i] = table[sb];
+        xi[i] = 0x80000000u - sum16;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.error[0] = 0;
+    __syncthreads();
+
+    const float scale = __fmul_rn(*p.alpha_a, *p.alpha_b);
+    uint32_t out_max = 0u;
+    for (; turn < turns; turn += step) {
+        request(turn + step);
+        double acc[R * M];
+#pragma unroll
+        for (int v = 0; v < R * M; ++v) acc[v] = 0.0;
+        for (int32_t chunk = 0; chunk < chunks; ++chunk) {
+            // the next piece is on its way while this one is worked on, across turns too
+            if (chunk + 1 < chunks) load(wn, turn, chunk + 1);
+            else if (turn + step < turns) load(wn, turn + step, 0);
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t u[R][4];
+                double wb[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const uint32_t sb = half ? w[r].two >> 8 : w[r].two & 0xFFu;
+                    group_bytes<HAS_INT>(half ? w[r].codes.z : w[r].codes.x, half ? w[r].codes.w : w[r].codes.y, sb & 0x80u, u[r]);
+                    wb[r] = table[sb];
+                }
+                const int32_t at = (chunk * 2 + half) * M * 32 + lane;
+#pragma unroll
+                for (int t = 0; t < M; ++t) {
+                    const uint4 x = xs[at + t * 32];
+                    const double xa = xd[at + t * 32];
+                    const uint32_t first = xi[at + t * 32];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const uint32_t s = dot4(u[r][3], x.w, dot4(u[r][2], x.z, dot4(u[r][1], x.y, dot4(u[r][0], x.x, first))));
+                        const double d = __dsub_rn(__hiloint2double(0x43300000, (int)s), 4503601774854144.0 /* 2^52 + 2^31 */);
+                        acc[r * M + t] = __fma_rn(d, __dmul_rn(xa, wb[r]), acc[r * M + t]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) w[r] = wn[r];
+        }
+        // sum over the lanes: every exchange halves what a lane holds, while it holds more than one
+        int held = R * M;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            if (held > 1) {
+                held /= 2;
+                const bool up = lane & off;
+#pragma unroll
+                for (int v = 0; v < R * M / 2; ++v)
+                    if (v < held) {
+                        const double send = up ? acc[v] : acc[v + held], keep = up ? acc[v + held] : acc[v];
+                        acc[v] = __dadd_rn(keep, __shfl_xor_sync(0xFFFFFFFFu, send, off));
+                    }
+            } else {
+                acc[0] = __dadd_rn(acc[0], __shfl_xor_sync(0xFFFFFFFFu, acc[0], off));
+            }
+        }
+        constexpr int kEach = 32 / (R * M);                                          // lanes that hold the same sum
+        const int v = lane / kEach, t = v % M;
+        if (lane % kEach == 0 && t < p.m) {
+            const float c = __double2float_rn(__dmul_rn(acc[0], (double)scale));
+            const size_t at = (size_t)t * p.n + (size_t)turn * R + v / M;
+            if constexpr (OUT_BF16) {
+                const __nv_bfloat16 b = __float2bfloat16_rn(c);
+                reinterpret_cast<__nv_bfloat16*>(p.out)[at] = b;
+                out_max = max(out_max, (uint32_t)__bfloat16_as_ushort(b) & 0x7FFFu);
+            } else {
+                reinterpret_cast<float*>(p.out)[at] = c;
+            }
+        }
+    }
+    // the global maximum of |C| as written, for the next quantizer's tensor scale (as in abs_gemm.cu)
+    if (OUT_BF16 && p.next_alpha != nullptr) {
+        out_max = __reduce_max_sync(0xFFFFFFFFu, out_max);
+        if (lane == 0 && out_max) atomicMax(reinterpret_cast<unsigned int*>(p.error) + 1, out_max);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();                 // by the thread that takes the ticket, after the barrier: the block's maxima come before it
+            if (atomicAdd(p.error + 2, 1) == (int)gridDim.x - 1) {
+                __threadfence();
+                const float A = __uint_as_float(atomicMax(reinterpret_cast<unsigned int*>(p.error) + 1, 0u) << 16);
+                *p.next_alpha = (A == 0.0f) ? 1.0f : __fdiv_rn(A, p.next_denom);
+            }
+        }
+    }
+}
+
+}  // namespace absq

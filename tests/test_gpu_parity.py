@@ -1454,6 +1454,41 @@ def test_few_row_product_rounds_once(B, m, n, k, tokens):
     assert (c - want).norm() <= 3.3e-8 * want.norm()
 
 
+@pytest.mark.parametrize("fmt", [0, 1])
+@pytest.mark.parametrize("m,n,k", [(1, 128, 256), (1, 4096, 4096), (2, 1024, 1280), (3, 13568, 4096), (4, 1024, 13568), (5, 384, 2304),
+                                   (7, 2560, 256), (8, 128, 768), (8, 256, 14336), (8, 6784, 4096)])
+def test_product_with_very_few_rows(B, fmt, m, n, k):
+    """The kernel for up to eight rows: every instance with all and with fewer rows, K below, at and beside a multiple of its 1024 values,
+    one turn and several per warp, the ends of its range; random bytes (every code, -8 and subnormal scales included) against 64 bits
+    with the bound of one rounding (see test_few_row_product_rounds_once), the outputs' scale, rows beyond m untouched, and NaN scales, which
+    poison their rows and columns alone."""
+    g = torch.Generator(device="cuda").manual_seed(m * k + fmt)
+
+    def operand(rows):
+        codes = torch.randint(0, 256, (rows * k // 2,), generator=g, device="cuda", dtype=torch.uint8)
+        scales = torch.randint(0, 127, (rows * k // 16,), generator=g, device="cuda", dtype=torch.uint8)
+        if fmt:
+            scales |= torch.randint(0, 2, scales.shape, generator=g, device="cuda", dtype=torch.uint8) << 7
+        return codes, scales, torch.tensor([0.5], device="cuda")
+
+    qa, qb = operand(m), operand(n)
+    guard = torch.full((m + 2, n), 7.0, dtype=torch.float32, device="cuda")
+    c = B.abs_matmul(fmt, qa, qb, m, n, k, out=guard, check=True)[:m].clone()
+    assert (guard[m:] == 7.0).all()
+    want = 0.25 * decoded_float64(qa, m, k) @ decoded_float64(qb, n, k).t()
+    # 3.3e-8 for many results; a single one may be at its half ulp, 2^-24 of it, of up to 2^-24 sqrt(128) of the norm of 128 equal ones
+    assert (c.double() - want).norm() <= 3.3e-8 * want.norm() * (1.0 if m * n >= 1024 else 1.8)
+    c16, alpha = B.abs_matmul(fmt, qa, qb, m, n, k, bf16=True, next_fmt=fmt, check=True)
+    assert torch.equal(c16, c.bfloat16()) and torch.equal(alpha, B.abs_quantize(fmt, c16)[2])
+    sa, sb = qa[1].clone(), qb[1].clone()
+    sa[(m - 1) * k // 16] = 0x7F
+    sb[77 * k // 16 + 5] = 0xFF if fmt else 0x7F
+    bad = torch.zeros((m, n), dtype=torch.bool, device="cuda")
+    bad[m - 1, :], bad[:, 77] = True, True
+    got = B.abs_matmul(fmt, (qa[0], sa, qa[2]), (qb[0], sb, qb[2]), m, n, k, check=True)
+    assert bool(torch.isnan(got[bad]).all()) and torch.equal(got[~bad], c[~bad])
+
+
 @pytest.mark.parametrize("k", [4096, 8192, 12544, 14336])
 def test_tiled_product_rounds_little_over_chunks_of_k(B, k):
     """The tiled IF4 kernel over one chunk of the accumulators, two, three and a step, three and a half: the chunks' sums lie on a
