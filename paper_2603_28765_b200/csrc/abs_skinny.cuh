@@ -24,10 +24,12 @@
 // tile, shares of blocks, the scale -- is FP64 up to the one rounding of the result.  2-norm error against 64 bits, 24 x 14336 x 4096 and
 // 8 x 4096 x 14336: 2.6e-8 and 2.6e-8; with FP32 sums and k = 8 y + 2 x in accumulators of their own 5.3e-8 and 5.6e-8 (same time).
 //
-// Measured, product alone, weights not in the L2 (before: planes through the workspace): n = 14336, k = 4096: 1 token 52.5
-// -> 21.5 us, 24 tokens 53 -> 24 us; 4096 x 4096, 1 token 32.7 -> 14.3 us; 14336 x 14336, 32 tokens 133 -> 56 us.  A step
-// of 256 of K takes 1450 cycles on an SM, of which the integer pipe is busy for about 1000; the first data after some 3 us
-// and the sum of shared tiles, 2 us, are the rest.
+// Measured, product alone, weights not in the L2 (before: planes through the workspace; then with the ends of the kernel as they were at first):
+// n = 14336, k = 4096, 9 tokens 53 -> 22.6 -> 19.1 us; 4096 x 4096, 9 tokens 33 -> 16.5 -> 13.3 us; 14336 x 14336, 9 tokens 50.6 -> 48.2 us.  A step
+// of 256 of K takes 1340 cycles on an SM, of which the integer pipe is busy for about 1000.  The rest is fixed: launch and the wait for the kernel that
+// clears the counters 2 us, first data and first decoded step 2 us, the last accumulators 2 us, tickets and the sum of shared tiles
+// 4 us.  That last part was 9 us: one thread took the tickets of both ends in turn, after 64-bit divisions, behind two fences, and the
+// shares were loaded one after the other; the first data came 1 us later without the request into the L2.
 #pragma once
 #include "abs_tc.cuh"
 
@@ -36,6 +38,7 @@ namespace absq {
 constexpr int kSkinnyMaxRows = 32, kSkinnyTok = 32;                       // rows of A; columns of the MMA they are padded to
 constexpr int kSkinnyDecWarps = 16;
 constexpr int kSkinnyThreads = 32 * (1 + 4 + kSkinnyDecWarps + 1);
+constexpr int kSkinnyAhead = 8;                                           // steps of a run requested into the L2 in advance
 constexpr uint32_t kSkinnySfSlots = 4, kSkinnySlotCols = 32;              // 16 columns of weight scales, 16 of token scales
 // Steps of B as it lies, and steps of planes, in shared memory: decoding a step, the hand-over and its MMAs take about as
 // long as two steps, so there are three stages of planes.
@@ -91,7 +94,9 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
     const int32_t u0 = (int32_t)((int64_t)p.units * blockIdx.x / gridDim.x), u1 = (int32_t)((int64_t)p.units * (blockIdx.x + 1) / gridDim.x);
     const size_t code_pitch = (size_t)p.k / 2, scale_pitch = (size_t)p.k / 16;
 
-    __shared__ int failed, last[2];
+    // The tiles at the two ends of the run may be shared with other blocks: the first and the last block of each, and whether this
+    // block's share was the last to be stored.
+    __shared__ int failed, last[2], first_block[2], last_block[2];
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
         failed = 0;
@@ -103,6 +108,19 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) { tmem_alloc(smem_u32(tmem_word), kTmem); tmem_relinquish(); }
+    if (warp == 5 + kSkinnyDecWarps) {
+        // The first steps of B into the L2, before the wait (see prefetch_l2): the blocks are often resident while the tokens are still
+        // being quantized.
+        if (lane < kSkinnyAhead && u0 + lane < u1) {
+            const int32_t tile = (u0 + lane) / ksteps, k0 = u0 + lane - tile * ksteps;
+            tma_prefetch_2d(&p.w_codes, k0 * 128, tile * kTileM);
+            tma_prefetch_2d(&p.w_scales, k0 * 16, tile * kTileM);
+        }
+    } else if (warp == 5 && lane < 2) {
+        const int64_t tile = (lane == 0 ? u0 : u1 - 1) / ksteps;
+        first_block[lane] = (int)(((tile * ksteps + 1) * gridDim.x - 1) / p.units);
+        last_block[lane] = (int)(((tile * ksteps + ksteps) * gridDim.x - 1) / p.units);
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -262,7 +280,6 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
             first_span = tile_end;
             if (tile_end) from_start = true;
         }
-        __threadfence();                                                   // the shares, for the block that sums them
         if (!ok) failed = 1;
     } else if (warp < 5 + kSkinnyDecWarps) {
         // ---- codes: thread i handles the 16 bytes (two groups) at place i % 8 of weight rows i / 8, i / 8 + 32, ... of a
@@ -367,19 +384,13 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
     // shares in the order of K
     const int32_t t_first = u0 / ksteps, t_last = (u1 - 1) / ksteps;
     const bool share_first = u0 % ksteps != 0 || u1 - u0 < ksteps, share_last = t_last != t_first && u1 % ksteps != 0;
-    if (threadIdx.x == 0) {
-        __threadfence();
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            last[e] = 0;
-            if (e == 0 ? share_first : share_last) {
-                const int32_t tile = e == 0 ? t_first : t_last;
-                const int64_t bf = (((int64_t)tile * ksteps + 1) * gridDim.x - 1) / p.units;
-                const int64_t bl = (((int64_t)tile * ksteps + ksteps) * gridDim.x - 1) / p.units;
-                last[e] = atomicAdd(p.tickets + tile, 1) == (int)(bl - bf);
-            }
+    if (warp == 1 && lane < 2) {
+        last[lane] = 0;
+        if (lane == 0 ? share_first : share_last) {
+            __threadfence();                 // by the thread that takes the ticket, after the barrier: the block's shares come before it
+            last[lane] = atomicAdd(p.tickets + (lane == 0 ? t_first : t_last), 1) == last_block[lane] - first_block[lane];
+            __threadfence();
         }
-        __threadfence();
     }
     __syncthreads();
     int32_t done = t_last - t_first + 1 - (share_first ? 1 : 0) - (share_last ? 1 : 0);
@@ -388,18 +399,27 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_
         if (!last[e]) continue;
         ++done;
         const int32_t tile = e == 0 ? t_first : t_last;
-        const int32_t bf = (int32_t)((((int64_t)tile * ksteps + 1) * gridDim.x - 1) / p.units);
-        const int32_t bl = (int32_t)((((int64_t)tile * ksteps + ksteps) * gridDim.x - 1) / p.units);
-        constexpr int kEach = 8;                                           // outputs per thread and trip
+        const int32_t bf = first_block[e], bl = last_block[e];
+        constexpr int kEach = 4, kLoads = 4;                               // outputs per thread and trip; shares loaded at a time
         for (int32_t i0 = threadIdx.x; i0 < p.m * kTileM; i0 += kEach * kSkinnyThreads) {
             double v[kEach];
 #pragma unroll
             for (int q = 0; q < kEach; ++q) v[q] = 0.0;
-            for (int32_t b = bf; b <= bl; ++b) {
-                const double* share = p.partials + ((size_t)b * 2 + (b == bf ? 1 : 0)) * (NT * kTileM);
+            for (int32_t b0 = bf; b0 <= bl; b0 += kLoads) {
+                double s[kLoads][kEach];
 #pragma unroll
-                for (int q = 0; q < kEach; ++q)
-                    if (i0 + q * kSkinnyThreads < p.m * kTileM) v[q] += __ldcg(share + i0 + q * kSkinnyThreads);
+                for (int a = 0; a < kLoads; ++a) {
+                    const double* share = p.partials + ((size_t)(b0 + a) * 2 + (b0 + a == bf ? 1 : 0)) * (NT * kTileM);
+#pragma unroll
+                    for (int q = 0; q < kEach; ++q) {
+                        const int32_t i = i0 + q * kSkinnyThreads;
+                        s[a][q] = b0 + a <= bl && i < p.m * kTileM ? __ldcg(share + i) : 0.0;
+                    }
+                }
+#pragma unroll
+                for (int a = 0; a < kLoads; ++a)
+#pragma unroll
+                    for (int q = 0; q < kEach; ++q) v[q] = __dadd_rn(v[q], s[a][q]);
             }
 #pragma unroll
             for (int q = 0; q < kEach; ++q) {
