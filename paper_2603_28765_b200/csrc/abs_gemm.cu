@@ -20,10 +20,13 @@
 // eight (IF4) warps read the accumulators back (tcgen05.ld) and write C.  Every mbarrier wait is bounded in time: when a
 // wait runs out the block raises an error word, stops issuing, frees its tensor memory and returns.
 //
-// What bounds it, by the counts: shared memory at 128 bytes per cycle.  IF4: an MMA takes 97 cycles, 64 of them tensor work;
-// beside it stand up to 8 KiB of operand reads (less where A comes from the collector buffer) and 4 KiB of TMA writes, 64
-// + 32 cycles.  NVFP4: 160 KiB per step of two boxes.  The feed from the L2 is at a third of its peak.  4096^3, operands and split included: IF4 195 -> 118 us (nine MMAs per K-block to four), 8192 x 14336 x 4096
-// 1440 -> 785 us; NVFP4 46 and 340 us.
+// What bounds it: power.  Back to back, the GPU is at its power cap and lowers the clock (IF4, 8192 x 14336 x 4096: 1450 MHz), so what counts is
+// energy and, below the cap, the cycles in which no MMA runs.  An MMA takes 64 cycles whatever else the SM's memories do (bulk
+// copies at 50, shared loads at 120, tensor-memory loads at 280 bytes per cycle beside it change nothing, and neither do commits),
+// the copy engine brings 110 bytes per cycle and SM, and the tensor core queues two MMAs: what used to take 93 cycles per MMA was the issuing thread,
+// busy for 470 cycles between the MMAs of two steps.  Operands and split included, back to back: IF4 2048 x 4096 x 4096 72.2 -> 64.2
+// us, 1000 x 14336 x 4096 133 -> 122 us, 8192 x 14336 x 4096 845 -> 787 us; NVFP4, whose scales (two groups of warps now) were late as well, 26.8 ->
+// 25.5, 45.6 -> 43.4 and 324 -> 313 us.  (Nine MMAs per K-block in IF4: 1440 us for the largest.)
 #include "../../include/abs_b200.h"
 #include "abs_tc.cuh"
 #include "abs_rows.cuh"
@@ -36,49 +39,49 @@
 
 namespace absq {
 
-// A pipeline stage (one K-step) holds KBOXES boxes of each of the PLANES planes of A and of B (the scales do not pass
-// through shared memory).  IF4 (two planes, one box: K = 256, 64 KiB) has three stages.  Plain NVFP4 issues one MMA per
-// K-block, so the hand-overs of a step weigh more: its steps are two boxes long where K allows (K = 512, 64 KiB, three
-// stages), else one box (32 KiB, six stages).
+// A pipeline stage (one K-step) holds KBOXES boxes of each of the PLANES planes of A and of B; 192 KiB of stages are on their way or in use.
+// IF4 (two planes, one box: K = 256, 64 KiB) has three stages.  Plain NVFP4 issues one MMA per K-block, so the hand-overs of a step weigh
+// more: its steps are two boxes long where K allows (K = 512, 64 KiB, three stages), else one box (32 KiB, six stages).
+// The scales.  IF4: boxes of 16 bytes x 128 rows as they lie, in a ring of their own.  The copy engine takes about a cycle per row of a box
+// whatever its width, so beside the boxes of codes of an NVFP4 step, which has a quarter of the MMAs, there is no room for that (28.3 us
+// instead of 25.5 for 2048 x 4096 x 4096), and boxes for eight steps cost two stages (26.2 us): there the scales are tiled first
+// (sf_tile_kernel) and come through registers.
 template <int PLANES, int KBOXES> constexpr int kStageBytes = 2 * PLANES * KBOXES * kPlaneBytes;
 template <int PLANES, int KBOXES> constexpr int kStages = PLANES * KBOXES == 2 ? 3 : 6;
+constexpr int kSfBufs = 3, kScaleBoxBytes = kTileM * (kStageK / 16);
+template <int PLANES> constexpr int kSfRingBytes = PLANES == 2 ? kSfBufs * 2 * kScaleBoxBytes : 0;
 // Epilogue warps: IF4, whose accumulators fill the tensor memory, takes eight, two per quarter of the accumulator lanes,
 // that have everything in registers before they store (the MMAs of the next tile wait only for that); NVFP4 has two sets
 // of accumulators and streams each through four warps.  Staging: a warp turns 16 rows x 128 bytes (IF4) or 32 rows x 128
 // bytes (NVFP4) of output at a time through shared memory, rows 144 bytes apart: 16-byte aligned and free of bank
 // conflicts for 128-bit accesses both ways.
 template <int PLANES> constexpr int kEpiWarps = PLANES == 2 ? 8 : 4;
-template <int PLANES> constexpr int kGemmThreads = 32 * (2 + kEpiWarps<PLANES> + 4);
+// Scale warps: four, one per quarter of tensor memory.  NVFP4, whose steps are short, has two groups of four that take the steps in
+// turn, so that the loads of one step are waited for while another's scales are written.
+template <int PLANES> constexpr int kScaleGroups = PLANES == 2 ? 1 : 2;
+template <int PLANES> constexpr int kGemmThreads = 32 * (2 + kEpiWarps<PLANES> + 4 * kScaleGroups<PLANES>);
 constexpr int kStagePitch = 36, kStagingBytes = 4 * 32 * kStagePitch * 4;
 template <int PLANES, int KBOXES> constexpr int kGemmSmemBytes =
-    kStages<PLANES, KBOXES> * kStageBytes<PLANES, KBOXES> + 1024 /* alignment slack */ + 512 /* barriers */ + kStagingBytes;
+    kStages<PLANES, KBOXES> * kStageBytes<PLANES, KBOXES> + kSfRingBytes<PLANES> + 1024 /* alignment slack */ + 512 /* barriers */ + kStagingBytes;
 
 // ----------------------------------------------------------------------------- operand split
 
-// One operand of the product as the split kernel sees it.
+// One operand of an IF4 product as the split kernel sees it.
 struct SplitOperand {
     const uint4* codes;            // [rows, k / 2] bytes as abs_quantize wrote them
     const uint8_t* scales;         // [rows, k / 16] row-major
     uint4 *plane_h, *plane_l;
-    uint8_t* sf_tiled;             // magnitudes of the scales in the 128x4-tile layout
-    int64_t rows;
     int64_t pairs;                 // rows * k / 32: pairs of groups (16 bytes of codes)
-    int64_t sf_items;              // ceil(rows / 128) * ktiles / 4 * 32: one item = 4 rows x 16 scales
-    uint32_t gpr, ktiles;          // groups per row (a multiple of 16), gpr / 4
 };
 
-// Prepares both operands in one launch.  Code items (IF4 only; an NVFP4 operand is read by the product kernel where
-// it lies): 32 codes = two groups -> 16 bytes of each of the planes H and L.  Scale items: thread i of a warp reads 16
-// scale bytes of each of the rows i, i + 32, i + 64, i + 96 of a 128-row block and writes, for each of four
-// consecutive 128x4 tiles, the 16 bytes that tile keeps for those four rows.  Also clears the error word.
-__global__ void __launch_bounds__(256, 8) if4_split_kernel(const SplitOperand a, const SplitOperand b, bool has_int,
-                                                        int* __restrict__ error) {
+// Writes the planes H and L of both operands of an IF4 product in one launch (an NVFP4 operand is read by the product kernel where it
+// lies): 32 codes = two groups -> 16 bytes of each plane.  Also clears the error word.
+__global__ void __launch_bounds__(256, 8) if4_split_kernel(const SplitOperand a, const SplitOperand b, int* __restrict__ error) {
     pdl_launch_dependents();
     pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (first == 0) { error[0] = 0; error[1] = 0; error[2] = 0; }     // error word, output maximum, ticket
-    const int64_t code_items = has_int ? a.pairs + b.pairs : 0;
-    for (int64_t i = first; i < code_items; i += stride) {
+    for (int64_t i = first; i < a.pairs + b.pairs; i += stride) {
         const SplitOperand& o = i < a.pairs ? a : b;
         const int64_t p = i < a.pairs ? i : i - a.pairs;
         const uint4 c = __ldg(o.codes + p);
@@ -89,27 +92,39 @@ __global__ void __launch_bounds__(256, 8) if4_split_kernel(const SplitOperand a,
         o.plane_h[p] = h;
         o.plane_l[p] = l;
     }
-    const int64_t sf_items = a.sf_items + b.sf_items;
-    for (int64_t i = first; i < sf_items; i += stride) {
-        const SplitOperand& o = i < a.sf_items ? a : b;
-        const int64_t j = i < a.sf_items ? i : i - a.sf_items;
+}
+
+// The scales of both operands of an NVFP4 product in the 128x4-tile layout (16 bytes: the four K-blocks' bytes of rows r, r + 32, r + 64,
+// r + 96 of a 128-row block): thread i of a warp reads 16 scale bytes of each of its four rows and writes 16 bytes of each of four
+// consecutive tiles.  Also clears the error word.
+struct TileOperand {
+    const uint8_t* scales;         // [rows, k / 16] row-major
+    uint8_t* tiled;
+    int64_t rows;
+    int64_t items;                 // ceil(rows / 128) * k / 256 * 32: one item = 4 rows x 16 scales
+};
+__global__ void __launch_bounds__(256, 8) sf_tile_kernel(const TileOperand a, const TileOperand b, uint32_t ksteps, int* __restrict__ error) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (first == 0) { error[0] = 0; error[1] = 0; error[2] = 0; }     // error word, output maximum, ticket
+    for (int64_t i = first; i < a.items + b.items; i += stride) {
+        const TileOperand& o = i < a.items ? a : b;
+        const int64_t j = i < a.items ? i : i - a.items;
         const uint32_t lane = (uint32_t)(j & 31);
-        const int64_t t4 = j >> 5;                                    // (row block, group of four tiles)
-        const uint32_t quads = o.ktiles >> 2;
-        const int64_t rb = t4 / quads;
-        const uint32_t kq = (uint32_t)(t4 - rb * quads);
+        const int64_t step = j >> 5, rb = step / ksteps;              // (row block, K-step), row block
+        const uint32_t kt = (uint32_t)(step - rb * ksteps);
         uint4 r[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int64_t row = rb * 128 + q * 32 + lane;       // rows beyond the operand (last row block) get zero scales
-            r[q] = row < o.rows ? __ldg(reinterpret_cast<const uint4*>(o.scales + row * o.gpr) + kq) : make_uint4(0u, 0u, 0u, 0u);
+            const int64_t row = rb * 128 + q * 32 + lane;             // rows beyond the operand (last row block) get zero scales
+            r[q] = row < o.rows ? __ldg(reinterpret_cast<const uint4*>(o.scales + row * (ksteps * 16)) + kt) : make_uint4(0u, 0u, 0u, 0u);
         }
-        uint4* out = reinterpret_cast<uint4*>(o.sf_tiled + ((size_t)rb * o.ktiles + (size_t)kq * 4u) * 512u) + lane;
-        constexpr uint32_t kMag = 0x7F7F7F7Fu;
-        out[0] = make_uint4(r[0].x & kMag, r[1].x & kMag, r[2].x & kMag, r[3].x & kMag);
-        out[32] = make_uint4(r[0].y & kMag, r[1].y & kMag, r[2].y & kMag, r[3].y & kMag);
-        out[64] = make_uint4(r[0].z & kMag, r[1].z & kMag, r[2].z & kMag, r[3].z & kMag);
-        out[96] = make_uint4(r[0].w & kMag, r[1].w & kMag, r[2].w & kMag, r[3].w & kMag);
+        uint4* out = reinterpret_cast<uint4*>(o.tiled + step * 2048) + lane;
+        out[0] = mask_scales(r[0].x, r[1].x, r[2].x, r[3].x);
+        out[32] = mask_scales(r[0].y, r[1].y, r[2].y, r[3].y);
+        out[64] = mask_scales(r[0].z, r[1].z, r[2].z, r[3].z);
+        out[96] = mask_scales(r[0].w, r[1].w, r[2].w, r[3].w);
     }
 }
 
@@ -121,6 +136,7 @@ constexpr uint32_t kTmemCols = 512;
 
 struct GemmMaps {
     CUtensorMap a[2], b[2];        // planes H, L of A [M, K/2 bytes] and B [N, K/2 bytes], boxes of 128 bytes x 128 rows
+    CUtensorMap sa, sb;            // IF4: their scales as abs_quantize wrote them [rows, K/16 bytes], boxes of 16 bytes x 128 rows
 };
 
 // Tile t of the (tiles_m x tiles_n) grid of 128 x 128 tiles, walked in bands of eight tile rows, column by column
@@ -138,12 +154,10 @@ __device__ __forceinline__ void tile_of(int32_t t, int32_t tiles_m, int32_t tile
 //
 // Persistent: one block per SM walks the tiles blockIdx.x, blockIdx.x + gridDim.x, ...  Warp 0 (one thread) feeds the
 // pipeline and runs ahead into the next tile while the current one is finished; warp 1 (one thread) issues MMAs; the next
-// kEpiWarps warps are the epilogue (warp w reads the 32 accumulator lanes of tensor-memory quarter w % 4); the last four
-// warps bring the scales: each loads the 128x4 scale tiles of a K-step from global memory into registers and writes them
-// to its quarter of tensor memory (tcgen05.st; every quarter holds the same four columns per MMA: rows r, r+32, r+64, r+96
-// of the tile, which is the byte order of the 128x4 tile), into slots handed over through sf_full / sf_empty barriers -- a
-// tcgen05.cp from shared memory by the MMA thread would stand in the MMA queue for some 34 cycles per copy.  (Scale tiles
-// brought to shared memory by bulk copies with the operands measured the same.)  The accumulators pass between MMA and
+// kEpiWarps warps are the epilogue (warp w reads the 32 accumulator lanes of tensor-memory quarter w % 4); the last four or eight
+// warps bring the scales of every K-step through registers to their quarter of tensor memory (tcgen05.st; every quarter holds the same four
+// columns per MMA: rows r, r+32, r+64, r+96 of the tile); a stage's full barrier counts them with the loads of its operands -- a
+// tcgen05.cp from shared memory by the MMA thread would stand in the MMA queue for some 34 cycles per copy.  The accumulators pass between MMA and
 // epilogue through acc_full / acc_empty barriers; NVFP4, with one accumulator of 128 columns, alternates between two of
 // them so that a tile's epilogue overlaps the next tile's MMAs, IF4 (3 x 128 columns) has room for one set and overlaps
 // only its stores and the next tile's loads.
@@ -156,7 +170,7 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
                 const float* __restrict__ alpha_a, const float* __restrict__ alpha_b, void* __restrict__ c_out, int32_t tiles_m,
                 int32_t tiles_n, int32_t k_iters, int32_t m_rows, int* __restrict__ error, int32_t stall_step,
                 float* __restrict__ next_alpha, float next_denom) {
-    constexpr int planes = PLANES, kStages = absq::kStages<PLANES, KBOXES>, kStageBytes = absq::kStageBytes<PLANES, KBOXES>;
+    constexpr int kStages = absq::kStages<PLANES, KBOXES>, kStageBytes = absq::kStageBytes<PLANES, KBOXES>;
     constexpr int kStepBlocks = KBOXES * (kStageK / kMmaK);          // MMA K-blocks (and scale tiles per operand) of one step
     constexpr int kAccBufs = PLANES == 1 ? 2 : 1;
     constexpr int kEpiWarps = absq::kEpiWarps<PLANES>;
@@ -164,48 +178,61 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
     extern __shared__ uint8_t gemm_smem_raw[];
     const uint32_t raw = smem_u32(gemm_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;                    // 128-byte swizzle wants 1024-byte aligned tiles
-    // Scale slots in tensor memory: 32 columns each (16 of A scales, 16 of B scales).  IF4 has room for four behind its
-    // three accumulators, NVFP4 for eight behind its two.
+    // Scales in tensor memory: a slot per stage behind the accumulators (IF4: three, NVFP4: two), A scales, then B scales.
     constexpr uint32_t kSlotCols = 8u * kStepBlocks;                  // 4 columns per K-block and operand
-    constexpr uint32_t kSfSlots = PLANES == 1 ? 256u / kSlotCols : 4u, kSfBase = PLANES == 1 ? 2 * kTileN : 3 * kTileN;
-    // barriers: full[], empty[] (stages), acc_full[2], acc_empty[2], sf_full[], sf_empty[] (slots); then the tmem address word
-    const uint32_t bars = base + kStages * kStageBytes;
+    constexpr uint32_t kSfBase = PLANES == 1 ? 2 * kTileN : 3 * kTileN;
+    static_assert(kSfBase + kStages * kSlotCols <= kTmemCols, "tensor memory");
+    // barriers: full[], empty[] (stages), acc_full[2], acc_empty[2], sf_full[], sf_empty[] (scale boxes); then the tmem address word
+    const uint32_t sf0 = base + kStages * kStageBytes, bars = sf0 + kSfRingBytes<PLANES>;
     uint32_t* tmem_word = reinterpret_cast<uint32_t*>(gemm_smem_raw + (bars - raw) + 320);
-    const uint32_t full0 = bars, empty0 = bars + 64, acc_full0 = bars + 128, acc_empty0 = bars + 144;
-    const uint32_t sf_full0 = bars + 192, sf_empty0 = bars + 256;
+    const uint32_t full0 = bars, empty0 = bars + 64, acc_full0 = bars + 128, acc_empty0 = bars + 144, sf_full0 = bars + 192, sf_empty0 = bars + 256;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int32_t num_tiles = tiles_m * tiles_n, n_cols = tiles_n * kTileN;
 
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(full0 + 8 * s, 1 + 4);              // loads of the operands, scale warps
+            mbar_init(empty0 + 8 * s, 1);
+        }
+        for (int i = 0; i < kSfBufs; ++i) { mbar_init(sf_full0 + 8 * i, 1); mbar_init(sf_empty0 + 8 * i, 4); }
         for (int i = 0; i < kAccBufs; ++i) { mbar_init(acc_full0 + 8 * i, 1); mbar_init(acc_empty0 + 8 * i, kEpiWarps); }
-        for (int i = 0; i < (int)kSfSlots; ++i) { mbar_init(sf_full0 + 8 * i, 4); mbar_init(sf_empty0 + 8 * i, 1); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) { tmem_alloc(smem_u32(tmem_word), kTmemCols); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_word;
+    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tmem_word, 0);
     pdl_wait();
 
     if (warp == 0) {
         if (lane == 0) {
             // ---- producer: TMA loads of the operand planes
-            constexpr uint32_t bytes = kStageBytes;
             uint32_t it = 0;
             bool ok = true;
             for (int32_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
                 int32_t tile_m, tile_n;
                 tile_of(t, tiles_m, tiles_n, tile_m, tile_n);
                 for (int32_t kt = 0; kt < k_iters; ++kt, ++it) {
+                    const bool stalled = (int32_t)it == stall_step;      // self-test only: the bytes announced never arrive
+                    if constexpr (PLANES == 2) {
+                        const uint32_t b = it % kSfBufs, at = sf0 + b * 2 * kScaleBoxBytes, bar = sf_full0 + 8 * b;
+                        if (!mbar_wait(sf_empty0 + 8 * b, ((it / kSfBufs) & 1u) ^ 1u)) { atomicExch(error, 7); ok = false; break; }
+                        mbar_expect_tx(bar, 2 * kScaleBoxBytes);
+                        if (!stalled) {
+                            tma_load_2d(at, &maps.sa, kt * (kStageK / 16), tile_m * kTileM, bar);
+                            tma_load_2d(at + kScaleBoxBytes, &maps.sb, kt * (kStageK / 16), tile_n * kTileN, bar);
+                        }
+                    }
                     const uint32_t s = it % kStages;
                     if (!mbar_wait(empty0 + 8 * s, ((it / kStages) & 1u) ^ 1u)) { atomicExch(error, 1); ok = false; break; }
                     const uint32_t st = base + s * kStageBytes, bar = full0 + 8 * s;
-                    mbar_expect_tx(bar, bytes);
-                    if ((int32_t)it == stall_step) continue;      // self-test only: the bytes announced never arrive
-                    for (int p = 0; p < planes; ++p)
+                    mbar_expect_tx(bar, kStageBytes);
+                    if (stalled) continue;
+#pragma unroll
+                    for (int p = 0; p < PLANES; ++p)
+#pragma unroll
                         for (int box = 0; box < KBOXES; ++box) {
                             const int32_t x = (kt * KBOXES + box) * (kStageK / 2);
                             tma_load_2d(st + (p * KBOXES + box) * kPlaneBytes, &maps.a[p], x, tile_m * kTileM, bar);
@@ -216,101 +243,121 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            // ---- MMAs
-            uint32_t it = 0, j = 0;                     // K-steps and chunks so far
-            bool ok = true;
+            // ---- MMAs.  The tensor core's queue holds about two MMAs of 64 cycles, so what this thread does between two of them must
+            // take less than that: descriptors by one addition, stages and parities kept and not computed, and the wait for the next step's
+            // operands in the middle of this step's MMAs.  (Warp-wide loop with votes, remainders, and the wait after the step's MMAs: 470 cycles
+            // a step without an MMA running.)
+            const uint64_t desc0 = operand_desc(base);
+            uint32_t s = 0, parity = 0, j = 0;          // stage and its parity; chunks so far
+            bool ok = mbar_wait(full0, 0);
             for (int32_t t = blockIdx.x, k0 = 0; t < num_tiles && ok; ++j) {
                 const uint32_t buf = j % kAccBufs, acc = tmem + buf * kTileN;
-                if (!mbar_wait(acc_empty0 + 8 * buf, ((j / kAccBufs) & 1u) ^ 1u)) { atomicExch(error, 4); ok = false; break; }
+                if (!mbar_wait(acc_empty0 + 8 * buf, ((j / kAccBufs) & 1u) ^ 1u)) { atomicExch(error, 4); break; }
                 tc_fence_after();
                 const int32_t k_end = min(k_iters - k0, kChunkSteps);
-                for (int32_t kt = 0; kt < k_end; ++kt, ++it) {
-                    const uint32_t s = it % kStages;
-                    const uint32_t slot = it % kSfSlots;
-                    if (!mbar_wait(full0 + 8 * s, (it / kStages) & 1u)) { atomicExch(error, 2); ok = false; break; }
-                    if (!mbar_wait(sf_full0 + 8 * slot, (it / kSfSlots) & 1u)) { atomicExch(error, 5); ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t st = base + s * kStageBytes;
-                    const uint32_t tsfa = tmem + kSfBase + slot * kSlotCols, tsfb = tsfa + kSlotCols / 2;
+                const bool last_chunk = k0 + k_end == k_iters && t + (int32_t)gridDim.x >= num_tiles;
+                for (int32_t kt = 0; kt < k_end && ok; ++kt) {
+                    const uint32_t s1 = s + 1 == kStages ? 0u : s + 1, parity1 = s1 ? parity : parity ^ 1u;
+                    const uint64_t st = desc0 + (uint64_t)s * (kStageBytes >> 4);
+                    const uint32_t tsfa = tmem + kSfBase + s * kSlotCols, tsfb = tsfa + kSlotCols / 2;
+                    const bool first = kt == 0, go = !first || k0 != 0;           // H H: anew in every chunk
                     // K-block kb of a step lies in box kb / 4 of its plane, 32 bytes per K-block inside the box's 128-byte rows
-                    auto desc_a = [&](int p, int kb) {
-                        return operand_desc(st + (p * KBOXES + (kb >> 2)) * kPlaneBytes + (kb & 3) * (kMmaK / 2));
-                    };
-                    auto desc_b = [&](int p, int kb) {
-                        return operand_desc(st + ((PLANES + p) * KBOXES + (kb >> 2)) * kPlaneBytes + (kb & 3) * (kMmaK / 2));
-                    };
-                    if constexpr (PLANES == 1) {
-#pragma unroll
-                        for (int kb = 0; kb < kStepBlocks; ++kb)
-                            tc_mma_nvf4(acc, desc_a(0, kb), desc_b(0, kb), kInstrDesc, !(kt == 0 && kb == 0), tsfa + 4 * kb, tsfb + 4 * kb);
-                    } else {
-#pragma unroll
-                        for (int kb = 0; kb < kStepBlocks; ++kb) {
-                            const uint32_t fa = tsfa + 4 * kb, fb = tsfb + 4 * kb;
-                            const bool go0 = !(kt == 0 && kb == 0), go = go0 || k0 != 0;      // H H: anew in every chunk
-                            tc_mma_nvf4<kFill>(acc, desc_a(0, kb), desc_b(0, kb), kInstrDesc, go0, fa, fb);                       // H H
-                            tc_mma_nvf4<kLastUse>(acc + kTileN, desc_a(0, kb), desc_b(1, kb), kInstrDesc, go, fa, fb);            // H L
-                            tc_mma_nvf4<kFill>(acc + kTileN, desc_a(1, kb), desc_b(0, kb), kInstrDesc, true, fa, fb);             // L H
-                            tc_mma_nvf4<kLastUse>(acc + 2 * kTileN, desc_a(1, kb), desc_b(1, kb), kInstrDesc, go, fa, fb);        // L L
+                    auto mmas = [&](int kb) __attribute__((always_inline)) {
+                        const uint64_t a = st + (((kb >> 2) * kPlaneBytes + (kb & 3) * (kMmaK / 2)) >> 4), b = a + ((PLANES * KBOXES * kPlaneBytes) >> 4);
+                        const uint32_t fa = tsfa + 4 * kb, fb = tsfb + 4 * kb;
+                        if constexpr (PLANES == 1) {
+                            tc_mma_nvf4(acc, a, b, kInstrDesc, kb > 0 || !first, fa, fb);
+                        } else {
+                            constexpr uint64_t L = kPlaneBytes >> 4;
+                            tc_mma_nvf4<kFill>(acc, a, b, kInstrDesc, kb > 0 || !first, fa, fb);                     // H H
+                            tc_mma_nvf4<kLastUse>(acc + kTileN, a, b + L, kInstrDesc, kb > 0 || go, fa, fb);         // H L
+                            tc_mma_nvf4<kFill>(acc + kTileN, a + L, b, kInstrDesc, true, fa, fb);                    // L H
+                            tc_mma_nvf4<kLastUse>(acc + 2 * kTileN, a + L, b + L, kInstrDesc, kb > 0 || go, fa, fb); // L L
                         }
-                    }
-                    tc_commit(empty0 + 8 * s);          // the stage's shared memory is free once these MMAs have run
-                    tc_commit(sf_empty0 + 8 * slot);    // and so is the slot of scales
+                    };
+                    constexpr int kBefore = PLANES == 2 ? kStepBlocks - 1 : kStepBlocks - 2;
+#pragma unroll
+                    for (int kb = 0; kb < kBefore; ++kb) mmas(kb);
+                    // The next step's stage was handed back kStages - 1 commits ago, so this waits for loads and scales alone.
+                    if (!(last_chunk && kt == k_end - 1)) ok = mbar_wait(full0 + 8 * s1, parity1);
+                    tc_fence_after();
+#pragma unroll
+                    for (int kb = kBefore; kb < kStepBlocks; ++kb) mmas(kb);
+                    tc_commit(empty0 + 8 * s);          // the stage's shared memory and scales are free once these MMAs have run
+                    s = s1;
+                    parity = parity1;
                 }
-                if (ok) tc_commit(acc_full0 + 8 * buf); // and the chunk's accumulators are complete
+                tc_commit(acc_full0 + 8 * buf);         // and the chunk's accumulators are complete
                 k0 += k_end;
                 if (k0 == k_iters) { k0 = 0; t += gridDim.x; }
             }
+            if (!ok) atomicExch(error, 2);
         }
     } else if (warp >= 2 + kEpiWarps) {
-        // ---- scales: this warp's copy of every K-step's scale tiles, global memory -> registers -> tensor memory
-        // The loads of step it + 1 are in flight while step it waits for its slot and is written.
-        const int32_t ktiles = k_iters * kStepBlocks;
+        // ---- scales: this warp's copy of every K-step's scales, through registers into tensor memory
+        constexpr uint32_t kGroups = kScaleGroups<PLANES>;
+        const uint32_t group = (uint32_t)(warp - 2 - kEpiWarps) >> 2;
         const uint32_t lane_base = tmem + kSfBase + ((uint32_t)((warp & 3) * 32) << 16);
-        int32_t t = blockIdx.x, kt = 0;                                   // the step whose tiles are loaded next
-        const uint4 *pa = nullptr, *pb = nullptr;
-        auto load_next = [&](uint4 (&a)[kStepBlocks], uint4 (&b)[kStepBlocks]) {   // false when there is no further step
-            if (t >= num_tiles) return false;
-            if (kt == 0) {
-                int32_t tile_m, tile_n;
-                tile_of(t, tiles_m, tiles_n, tile_m, tile_n);
-                pa = reinterpret_cast<const uint4*>(sfa + (size_t)tile_m * ktiles * 512) + lane;
-                pb = reinterpret_cast<const uint4*>(sfb + (size_t)tile_n * ktiles * 512) + lane;
-            }
+        if constexpr (PLANES == 2) {
+            const uint32_t steps = (uint32_t)((num_tiles - (int32_t)blockIdx.x + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x) * (uint32_t)k_iters;
+            for (uint32_t it = 0; it < steps; ++it) {
+                const uint32_t s = it % kStages, bx = it % kSfBufs;
+                const bool ok = mbar_wait_warp(sf_full0 + 8 * bx, (it / kSfBufs) & 1u) && mbar_wait_warp(empty0 + 8 * s, ((it / kStages) & 1u) ^ 1u);
+                if (!ok) { if (lane == 0) atomicExch(error, 6); break; }
+                // 16 scale bytes (four K-blocks) of each of the rows r, r + 32, r + 64, r + 96 of either operand, flag bits stripped
+                const uint4* at = reinterpret_cast<const uint4*>(gemm_smem_raw + (sf0 - raw) + bx * 2 * kScaleBoxBytes) + lane;
+                tc_fence_after();
 #pragma unroll
-            for (int kb = 0; kb < kStepBlocks; ++kb) {                     // tile kb of the step: 16 bytes per lane, tiles 512 bytes apart
-                a[kb] = __ldg(pa + (kt * kStepBlocks + kb) * 32);
-                b[kb] = __ldg(pb + (kt * kStepBlocks + kb) * 32);
+                for (int op = 0; op < 2; ++op) {
+                    const uint4 r0 = at[op * 128], r1 = at[op * 128 + 32], r2 = at[op * 128 + 64], r3 = at[op * 128 + 96];
+                    tmem_store16(lane_base + s * kSlotCols + op * (kSlotCols / 2), mask_scales(r0.x, r1.x, r2.x, r3.x), mask_scales(r0.y, r1.y, r2.y, r3.y),
+                                 mask_scales(r0.z, r1.z, r2.z, r3.z), mask_scales(r0.w, r1.w, r2.w, r3.w));
+                }
+                tmem_store_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) { mbar_arrive(full0 + 8 * s); mbar_arrive(sf_empty0 + 8 * bx); }
             }
-            if (++kt == k_iters) { kt = 0; t += gridDim.x; }
-            return true;
-        };
-        // One step of lookahead in registers where a step is one box long; with two-box steps the four scale slots
-        // already let these warps run three steps ahead of the MMAs.
-        constexpr bool kLookahead = KBOXES == 1;
-        uint4 a[kStepBlocks], b[kStepBlocks], an[kLookahead ? kStepBlocks : 1], bn[kLookahead ? kStepBlocks : 1];
-        bool more = load_next(a, b);
-        for (uint32_t it = 0; more; ++it) {
-            if constexpr (kLookahead) more = load_next(an, bn);
-            const uint32_t slot = it % kSfSlots;
-            bool have = mbar_wait(sf_empty0 + 8 * slot, ((it / kSfSlots) & 1u) ^ 1u);
-            if (!have && lane == 0) atomicExch(error, 6);
-            have = __all_sync(0xFFFFFFFFu, have);
-            if (!have) break;
-            tc_fence_after();
+        } else {
+            // The loads of the group's next step are in flight while this one waits for its slot and is written.
+            // With two groups and three stages a group sees only every second phase of a stage's barrier.  That is unambiguous: its step before, two
+            // steps earlier, waited for MMAs later than those of the phase before.
+            const int32_t ktiles = k_iters * kStepBlocks;
+            int32_t t = blockIdx.x, kt = (int32_t)group, t_at = -1;       // the step whose tiles are loaded next; the tile of pa and pb
+            const uint4 *pa = nullptr, *pb = nullptr;
+            auto load_next = [&](uint4 (&a)[kStepBlocks], uint4 (&b)[kStepBlocks]) {   // false when there is no further step
+                while (kt >= k_iters) { kt -= k_iters; t += gridDim.x; }
+                if (t >= num_tiles) return false;
+                if (t != t_at) {
+                    t_at = t;
+                    int32_t tile_m, tile_n;
+                    tile_of(t, tiles_m, tiles_n, tile_m, tile_n);
+                    pa = reinterpret_cast<const uint4*>(sfa + (size_t)tile_m * ktiles * 512) + lane;
+                    pb = reinterpret_cast<const uint4*>(sfb + (size_t)tile_n * ktiles * 512) + lane;
+                }
 #pragma unroll
-            for (int g = 0; g < KBOXES; ++g) {
-                tmem_store16(lane_base + slot * kSlotCols + 16u * g, a[4 * g], a[4 * g + 1], a[4 * g + 2], a[4 * g + 3]);
-                tmem_store16(lane_base + slot * kSlotCols + kSlotCols / 2 + 16u * g, b[4 * g], b[4 * g + 1], b[4 * g + 2], b[4 * g + 3]);
-            }
-            tmem_store_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(sf_full0 + 8 * slot);
-            if constexpr (kLookahead) {
+                for (int kb = 0; kb < kStepBlocks; ++kb) {                 // tile kb of the step: 16 bytes per lane, tiles 512 bytes apart
+                    a[kb] = __ldg(pa + (kt * kStepBlocks + kb) * 32);
+                    b[kb] = __ldg(pb + (kt * kStepBlocks + kb) * 32);
+                }
+                kt += kGroups;
+                return true;
+            };
+            uint4 a[kStepBlocks], b[kStepBlocks];
+            bool more = load_next(a, b);
+            for (uint32_t it = group; more; it += kGroups) {
+                const uint32_t s = it % kStages;
+                if (!mbar_wait_warp(empty0 + 8 * s, ((it / kStages) & 1u) ^ 1u)) { if (lane == 0) atomicExch(error, 6); break; }
+                tc_fence_after();
 #pragma unroll
-                for (int kb = 0; kb < kStepBlocks; ++kb) { a[kb] = an[kb]; b[kb] = bn[kb]; }
-            } else {
+                for (int g = 0; g < KBOXES; ++g) {
+                    tmem_store16(lane_base + s * kSlotCols + 16u * g, a[4 * g], a[4 * g + 1], a[4 * g + 2], a[4 * g + 3]);
+                    tmem_store16(lane_base + s * kSlotCols + kSlotCols / 2 + 16u * g, b[4 * g], b[4 * g + 1], b[4 * g + 2], b[4 * g + 3]);
+                }
+                tmem_store_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(full0 + 8 * s);
                 more = load_next(a, b);
             }
         }
@@ -569,7 +616,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int block, size_t sm
 }
 constexpr int kMaxSms = 160;               // workspaces are sized for up to this many SMs
 struct GemmLayout {
-    size_t plane_a, plane_b, sf_a, sf_b;       // sizes
+    size_t plane_a, plane_b, sf_a, sf_b;       // sizes (planes: IF4; tiled scales: NVFP4)
     size_t off_a, off_b, off_sfa, off_sfb, total;
 };
 GemmLayout gemm_layout(int64_t m, int64_t n, int64_t k) {
@@ -748,27 +795,33 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
         if (!plane_map(&maps.a[p], pa, (uint64_t)m, (uint64_t)k / 2) || !plane_map(&maps.b[p], pb, (uint64_t)n, (uint64_t)k / 2))
             return ABS_ERR_CUDA;
     }
-    const uint32_t gpr = (uint32_t)(k / 16), ktiles = gpr / 4u;
-    SplitOperand so[2];
-    for (int op = 0; op < 2; ++op) {
-        const int64_t rows = op ? n : m;
-        const size_t off = op ? L.off_b : L.off_a, plane = op ? L.plane_b : L.plane_a;
-        so[op].codes = (const uint4*)(op ? b_codes : a_codes);
-        so[op].scales = (const uint8_t*)(op ? b_scales : a_scales);
-        so[op].plane_h = (uint4*)(ws + off);
-        so[op].plane_l = (uint4*)(ws + off + plane);
-        so[op].sf_tiled = ws + (op ? L.off_sfb : L.off_sfa);
-        so[op].rows = rows;
-        so[op].pairs = rows * (k / 32);
-        so[op].sf_items = (rows + 127) / 128 * (int64_t)(ktiles / 4u) * 32;
-        so[op].gpr = gpr;
-        so[op].ktiles = ktiles;
-    }
-    {
-        const int64_t items = has_int ? so[0].pairs + so[1].pairs : so[0].sf_items + so[1].sf_items;
-        int64_t blocks = (items + 255) / 256;
+    if (has_int) {
+        if (!scale_map(&maps.sa, const_cast<void*>(a_scales), (uint64_t)m, (uint64_t)k / 16) ||
+            !scale_map(&maps.sb, const_cast<void*>(b_scales), (uint64_t)n, (uint64_t)k / 16))
+            return ABS_ERR_CUDA;
+        SplitOperand so[2];
+        for (int op = 0; op < 2; ++op) {
+            const size_t off = op ? L.off_b : L.off_a, plane = op ? L.plane_b : L.plane_a;
+            so[op].codes = (const uint4*)(op ? b_codes : a_codes);
+            so[op].scales = (const uint8_t*)(op ? b_scales : a_scales);
+            so[op].plane_h = (uint4*)(ws + off);
+            so[op].plane_l = (uint4*)(ws + off + plane);
+            so[op].pairs = (op ? n : m) * (k / 32);
+        }
+        int64_t blocks = (so[0].pairs + so[1].pairs + 255) / 256;
         if (blocks > 148 * 8) blocks = 148 * 8;
-        if (launch_pdl(if4_split_kernel, dim3((unsigned)blocks), 256, 0, s, so[0], so[1], has_int, (int*)ws) != cudaSuccess)
+        if (launch_pdl(if4_split_kernel, dim3((unsigned)blocks), 256, 0, s, so[0], so[1], (int*)ws) != cudaSuccess) return ABS_ERR_CUDA;
+    } else {
+        TileOperand to[2];
+        for (int op = 0; op < 2; ++op) {
+            to[op].scales = (const uint8_t*)(op ? b_scales : a_scales);
+            to[op].tiled = ws + (op ? L.off_sfb : L.off_sfa);
+            to[op].rows = op ? n : m;
+            to[op].items = (to[op].rows + 127) / 128 * (k / kStageK) * 32;
+        }
+        int64_t blocks = (to[0].items + to[1].items + 255) / 256;
+        if (blocks > 148 * 8) blocks = 148 * 8;
+        if (launch_pdl(sf_tile_kernel, dim3((unsigned)blocks), 256, 0, s, to[0], to[1], (uint32_t)(k / kStageK), (int*)ws) != cudaSuccess)
             return ABS_ERR_CUDA;
     }
     const int32_t tiles_m = (int32_t)((m + kTileM - 1) / kTileM), tiles_n = (int32_t)(n / kTileN);

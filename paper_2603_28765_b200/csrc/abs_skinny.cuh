@@ -70,11 +70,6 @@ __global__ void __launch_bounds__(256) skinny_clear_kernel(int* __restrict__ err
     for (int32_t i = threadIdx.x; i < n_tickets; i += blockDim.x) tickets[i] = 0;
 }
 
-__device__ __forceinline__ uint4 mask_scales(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    constexpr uint32_t kMag = 0x7F7F7F7Fu;
-    return make_uint4(a & kMag, b & kMag, c & kMag, d & kMag);
-}
-
 template <bool OUT_BF16>
 __global__ void __launch_bounds__(kSkinnyThreads, 1) skinny_kernel(const __grid_constant__ SkinnyArgs p) {
     constexpr int NT = kSkinnyTok, kRaw = kSkinnyRaw, kStages = kSkinnyStages, kStageBytes = kSkinnyStageBytes;

@@ -163,6 +163,12 @@ __device__ __forceinline__ void tmem_store16(uint32_t addr, const uint4& a, cons
 }
 __device__ __forceinline__ void tmem_store_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// Magnitudes of sixteen scale bytes: an integer group carries its flag in the sign bit.
+__device__ __forceinline__ uint4 mask_scales(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    constexpr uint32_t kMag = 0x7F7F7F7Fu;
+    return make_uint4(a & kMag, b & kMag, c & kMag, d & kMag);
+}
+
 // Shared-memory matrix descriptors (64 bits): start address, leading / stride byte offsets (all in 16-byte units),
 // descriptor version 1 (Blackwell) in bits 46-47, swizzle mode in bits 61-63.
 //   operand tiles: K-major rows of 128 bytes, 128-byte swizzle (mode 2), 8-row groups 1024 bytes apart
