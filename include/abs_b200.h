@@ -250,7 +250,8 @@ ABS_API float abs_alpha_from_amax(abs_fmt_t fmt, float amax);
  *   b_codes, b_scales  B likewise: [n, k]
  *   c_f32              out, [m, n] float, row-major
  *   workspace          device memory, 1024-byte aligned, at least abs_matmul_workspace_bytes(fmt, m, n, k) bytes
- * With up to 32 rows of A (IF4) the weights are read where they lie and split on the way to the tensor cores instead, and the
+ * With up to 8 rows of A, while rows times n k are small enough, the product runs on the integer and FP64 pipes instead (both formats); with up to 32 rows
+ * (IF4) the weights are read where they lie and split on the way to the tensor cores, and the
  * order of the sums over K follows the number of SMs: a row of C may then differ, by rounding only (2-norm error against
  * 64 bits 2.6e-8, above 32 rows 4e-8), from the same row of a product with more rows, and from that of a GPU with other SMs.
  * A workspace taken for m rows also serves fewer (n, k and fmt the same).
