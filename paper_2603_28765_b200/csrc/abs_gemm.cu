@@ -25,8 +25,8 @@
 // copies at 50, shared loads at 120, tensor-memory loads at 280 bytes per cycle beside it change nothing, and neither do commits),
 // the copy engine brings 110 bytes per cycle and SM, and the tensor core queues two MMAs: what used to take 93 cycles per MMA was the issuing thread,
 // busy for 470 cycles between the MMAs of two steps.  Operands and split included, back to back: IF4 2048 x 4096 x 4096 72.2 -> 64.2
-// us, 1000 x 14336 x 4096 133 -> 122 us, 8192 x 14336 x 4096 845 -> 787 us; NVFP4, whose scales (two groups of warps now) were late as well, 26.8 ->
-// 25.5, 45.6 -> 43.4 and 324 -> 313 us.  (Nine MMAs per K-block in IF4: 1440 us for the largest.)
+// us, 1000 x 14336 x 4096 133 -> 122 us, 8192 x 14336 x 4096 845 -> 787 us.  (Nine MMAs per K-block: 1440 us for the largest.)  NVFP4 26.8, 45.6 and
+// 324 us: its issuing thread is as it was (see there).
 #include "../../include/abs_b200.h"
 #include "abs_tc.cuh"
 #include "abs_rows.cuh"
@@ -42,10 +42,10 @@ namespace absq {
 // A pipeline stage (one K-step) holds KBOXES boxes of each of the PLANES planes of A and of B; 192 KiB of stages are on their way or in use.
 // IF4 (two planes, one box: K = 256, 64 KiB) has three stages.  Plain NVFP4 issues one MMA per K-block, so the hand-overs of a step weigh
 // more: its steps are two boxes long where K allows (K = 512, 64 KiB, three stages), else one box (32 KiB, six stages).
-// The scales.  IF4: boxes of 16 bytes x 128 rows as they lie, in a ring of their own.  The copy engine takes about a cycle per row of a box
-// whatever its width, so beside the boxes of codes of an NVFP4 step, which has a quarter of the MMAs, there is no room for that (28.3 us
-// instead of 25.5 for 2048 x 4096 x 4096), and boxes for eight steps cost two stages (26.2 us): there the scales are tiled first
-// (sf_tile_kernel) and come through registers.
+// The scales.  IF4: boxes of 16 bytes x 128 rows as they lie, in a ring of their own (with the codes in their stage: 821 us instead of 790 for
+// 8192 x 14336 x 4096).  The copy engine takes about a cycle per row of a box
+// whatever its width, so beside the boxes of codes of an NVFP4 step, which has a quarter of the MMAs, there is no room for that: there the
+// scales are tiled first (sf_tile_kernel) and come through registers.
 template <int PLANES, int KBOXES> constexpr int kStageBytes = 2 * PLANES * KBOXES * kPlaneBytes;
 template <int PLANES, int KBOXES> constexpr int kStages = PLANES * KBOXES == 2 ? 3 : 6;
 constexpr int kSfBufs = 3, kScaleBoxBytes = kTileM * (kStageK / 16);
@@ -56,10 +56,7 @@ template <int PLANES> constexpr int kSfRingBytes = PLANES == 2 ? kSfBufs * 2 * k
 // bytes (NVFP4) of output at a time through shared memory, rows 144 bytes apart: 16-byte aligned and free of bank
 // conflicts for 128-bit accesses both ways.
 template <int PLANES> constexpr int kEpiWarps = PLANES == 2 ? 8 : 4;
-// Scale warps: four, one per quarter of tensor memory.  NVFP4, whose steps are short, has two groups of four that take the steps in
-// turn, so that the loads of one step are waited for while another's scales are written.
-template <int PLANES> constexpr int kScaleGroups = PLANES == 2 ? 1 : 2;
-template <int PLANES> constexpr int kGemmThreads = 32 * (2 + kEpiWarps<PLANES> + 4 * kScaleGroups<PLANES>);
+template <int PLANES> constexpr int kGemmThreads = 32 * (2 + kEpiWarps<PLANES> + 4);
 constexpr int kStagePitch = 36, kStagingBytes = 4 * 32 * kStagePitch * 4;
 template <int PLANES, int KBOXES> constexpr int kGemmSmemBytes =
     kStages<PLANES, KBOXES> * kStageBytes<PLANES, KBOXES> + kSfRingBytes<PLANES> + 1024 /* alignment slack */ + 512 /* barriers */ + kStagingBytes;
@@ -154,9 +151,9 @@ __device__ __forceinline__ void tile_of(int32_t t, int32_t tiles_m, int32_t tile
 //
 // Persistent: one block per SM walks the tiles blockIdx.x, blockIdx.x + gridDim.x, ...  Warp 0 (one thread) feeds the
 // pipeline and runs ahead into the next tile while the current one is finished; warp 1 (one thread) issues MMAs; the next
-// kEpiWarps warps are the epilogue (warp w reads the 32 accumulator lanes of tensor-memory quarter w % 4); the last four or eight
+// kEpiWarps warps are the epilogue (warp w reads the 32 accumulator lanes of tensor-memory quarter w % 4); the last four
 // warps bring the scales of every K-step through registers to their quarter of tensor memory (tcgen05.st; every quarter holds the same four
-// columns per MMA: rows r, r+32, r+64, r+96 of the tile); a stage's full barrier counts them with the loads of its operands -- a
+// columns per MMA: rows r, r+32, r+64, r+96 of the tile); in IF4 a stage's full barrier counts them with the loads of its operands -- a
 // tcgen05.cp from shared memory by the MMA thread would stand in the MMA queue for some 34 cycles per copy.  The accumulators pass between MMA and
 // epilogue through acc_full / acc_empty barriers; NVFP4, with one accumulator of 128 columns, alternates between two of
 // them so that a tile's epilogue overlaps the next tile's MMAs, IF4 (3 x 128 columns) has room for one set and overlaps
@@ -178,11 +175,13 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
     extern __shared__ uint8_t gemm_smem_raw[];
     const uint32_t raw = smem_u32(gemm_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;                    // 128-byte swizzle wants 1024-byte aligned tiles
-    // Scales in tensor memory: a slot per stage behind the accumulators (IF4: three, NVFP4: two), A scales, then B scales.
+    // Scales in tensor memory: slots behind the accumulators (IF4: three, NVFP4: two), A scales, then B scales.
     constexpr uint32_t kSlotCols = 8u * kStepBlocks;                  // 4 columns per K-block and operand
     constexpr uint32_t kSfBase = PLANES == 1 ? 2 * kTileN : 3 * kTileN;
-    static_assert(kSfBase + kStages * kSlotCols <= kTmemCols, "tensor memory");
-    // barriers: full[], empty[] (stages), acc_full[2], acc_empty[2], sf_full[], sf_empty[] (scale boxes); then the tmem address word
+    // IF4: a slot per stage, NVFP4: as many as fit (four of a two-box step, eight of a one-box step)
+    constexpr uint32_t kSfSlots = PLANES == 1 ? (kTmemCols - kSfBase) / kSlotCols : (uint32_t)kStages;
+    static_assert(kSfBase + kSfSlots * kSlotCols <= kTmemCols && kSfSlots <= 8, "tensor memory, barriers");
+    // barriers: full[], empty[] (stages), acc_full[2], acc_empty[2], sf_full[], sf_empty[] (scale boxes, slots); then the tmem address word
     const uint32_t sf0 = base + kStages * kStageBytes, bars = sf0 + kSfRingBytes<PLANES>;
     uint32_t* tmem_word = reinterpret_cast<uint32_t*>(gemm_smem_raw + (bars - raw) + 320);
     const uint32_t full0 = bars, empty0 = bars + 64, acc_full0 = bars + 128, acc_empty0 = bars + 144, sf_full0 = bars + 192, sf_empty0 = bars + 256;
@@ -192,10 +191,14 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(full0 + 8 * s, 1 + 4);              // loads of the operands, scale warps
+            mbar_init(full0 + 8 * s, PLANES == 2 ? 1 + 4 : 1);     // loads of the operands; IF4: and scale warps
             mbar_init(empty0 + 8 * s, 1);
         }
-        for (int i = 0; i < kSfBufs; ++i) { mbar_init(sf_full0 + 8 * i, 1); mbar_init(sf_empty0 + 8 * i, 4); }
+        // IF4: boxes of scales, filled by loads and emptied by the scale warps; NVFP4: slots, filled by these and emptied by the MMAs
+        for (int i = 0; i < (PLANES == 2 ? kSfBufs : (int)kSfSlots); ++i) {
+            mbar_init(sf_full0 + 8 * i, PLANES == 2 ? 1 : 4);
+            mbar_init(sf_empty0 + 8 * i, PLANES == 2 ? 4 : 1);
+        }
         for (int i = 0; i < kAccBufs; ++i) { mbar_init(acc_full0 + 8 * i, 1); mbar_init(acc_empty0 + 8 * i, kEpiWarps); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -242,7 +245,7 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (PLANES == 2 && lane == 0) {
             // ---- MMAs.  The tensor core's queue holds about two MMAs of 64 cycles, so what this thread does between two of them must
             // take less than that: descriptors by one addition, stages and parities kept and not computed, and the wait for the next step's
             // operands in the middle of this step's MMAs.  (Warp-wide loop with votes, remainders, and the wait after the step's MMAs: 470 cycles
@@ -261,21 +264,17 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
                     const uint64_t st = desc0 + (uint64_t)s * (kStageBytes >> 4);
                     const uint32_t tsfa = tmem + kSfBase + s * kSlotCols, tsfb = tsfa + kSlotCols / 2;
                     const bool first = kt == 0, go = !first || k0 != 0;           // H H: anew in every chunk
-                    // K-block kb of a step lies in box kb / 4 of its plane, 32 bytes per K-block inside the box's 128-byte rows
+                    // 32 bytes per K-block inside a box's 128-byte rows
                     auto mmas = [&](int kb) __attribute__((always_inline)) {
-                        const uint64_t a = st + (((kb >> 2) * kPlaneBytes + (kb & 3) * (kMmaK / 2)) >> 4), b = a + ((PLANES * KBOXES * kPlaneBytes) >> 4);
+                        constexpr uint64_t L = kPlaneBytes >> 4;
+                        const uint64_t a = st + ((kb * (kMmaK / 2)) >> 4), b = a + 2 * L;
                         const uint32_t fa = tsfa + 4 * kb, fb = tsfb + 4 * kb;
-                        if constexpr (PLANES == 1) {
-                            tc_mma_nvf4(acc, a, b, kInstrDesc, kb > 0 || !first, fa, fb);
-                        } else {
-                            constexpr uint64_t L = kPlaneBytes >> 4;
-                            tc_mma_nvf4<kFill>(acc, a, b, kInstrDesc, kb > 0 || !first, fa, fb);                     // H H
-                            tc_mma_nvf4<kLastUse>(acc + kTileN, a, b + L, kInstrDesc, kb > 0 || go, fa, fb);         // H L
-                            tc_mma_nvf4<kFill>(acc + kTileN, a + L, b, kInstrDesc, true, fa, fb);                    // L H
-                            tc_mma_nvf4<kLastUse>(acc + 2 * kTileN, a + L, b + L, kInstrDesc, kb > 0 || go, fa, fb); // L L
-                        }
+                        tc_mma_nvf4<kFill>(acc, a, b, kInstrDesc, kb > 0 || !first, fa, fb);                     // H H
+                        tc_mma_nvf4<kLastUse>(acc + kTileN, a, b + L, kInstrDesc, kb > 0 || go, fa, fb);         // H L
+                        tc_mma_nvf4<kFill>(acc + kTileN, a + L, b, kInstrDesc, true, fa, fb);                    // L H
+                        tc_mma_nvf4<kLastUse>(acc + 2 * kTileN, a + L, b + L, kInstrDesc, kb > 0 || go, fa, fb); // L L
                     };
-                    constexpr int kBefore = PLANES == 2 ? kStepBlocks - 1 : kStepBlocks - 2;
+                    constexpr int kBefore = kStepBlocks - 1;
 #pragma unroll
                     for (int kb = 0; kb < kBefore; ++kb) mmas(kb);
                     // The next step's stage was handed back kStages - 1 commits ago, so this waits for loads and scales alone.
@@ -293,10 +292,41 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
             }
             if (!ok) atomicExch(error, 2);
         }
+        if (PLANES == 1 && lane == 0) {
+            // ---- MMAs, NVFP4.  With the loop above and a second group of scale warps, which it needs, products back to back take 4 % less (45.6 ->
+            // 43.5 us), but a pass with its quantizers more (1000 x 14336 x 4096 chained 55.9 -> 58.0 us, a layer's backward pass 133.4 -> 135.1):
+            // the next kernel's blocks find less room beside the larger block.
+            uint32_t it = 0, j = 0;                     // K-steps and chunks so far
+            bool ok = true;
+            for (int32_t t = blockIdx.x, k0 = 0; t < num_tiles && ok; ++j) {
+                const uint32_t buf = j % kAccBufs, acc = tmem + buf * kTileN;
+                if (!mbar_wait(acc_empty0 + 8 * buf, ((j / kAccBufs) & 1u) ^ 1u)) { atomicExch(error, 4); ok = false; break; }
+                tc_fence_after();
+                const int32_t k_end = min(k_iters - k0, kChunkSteps);
+                for (int32_t kt = 0; kt < k_end; ++kt, ++it) {
+                    const uint32_t s = it % kStages;
+                    const uint32_t slot = it % kSfSlots;
+                    if (!mbar_wait(full0 + 8 * s, (it / kStages) & 1u)) { atomicExch(error, 2); ok = false; break; }
+                    if (!mbar_wait(sf_full0 + 8 * slot, (it / kSfSlots) & 1u)) { atomicExch(error, 5); ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t st = base + s * kStageBytes;
+                    const uint32_t tsfa = tmem + kSfBase + slot * kSlotCols, tsfb = tsfa + kSlotCols / 2;
+                    // K-block kb of a step lies in box kb / 4 of its plane, 32 bytes per K-block inside the box's 128-byte rows
+                    auto desc_a = [&](int kb) { return operand_desc(st + (kb >> 2) * kPlaneBytes + (kb & 3) * (kMmaK / 2)); };
+                    auto desc_b = [&](int kb) { return operand_desc(st + (KBOXES + (kb >> 2)) * kPlaneBytes + (kb & 3) * (kMmaK / 2)); };
+#pragma unroll
+                    for (int kb = 0; kb < kStepBlocks; ++kb)
+                        tc_mma_nvf4(acc, desc_a(kb), desc_b(kb), kInstrDesc, !(kt == 0 && kb == 0), tsfa + 4 * kb, tsfb + 4 * kb);
+                    tc_commit(empty0 + 8 * s);          // the stage's shared memory is free once these MMAs have run
+                    tc_commit(sf_empty0 + 8 * slot);    // and so is the slot of scales
+                }
+                if (ok) tc_commit(acc_full0 + 8 * buf); // and the chunk's accumulators are complete
+                k0 += k_end;
+                if (k0 == k_iters) { k0 = 0; t += gridDim.x; }
+            }
+        }
     } else if (warp >= 2 + kEpiWarps) {
         // ---- scales: this warp's copy of every K-step's scales, through registers into tensor memory
-        constexpr uint32_t kGroups = kScaleGroups<PLANES>;
-        const uint32_t group = (uint32_t)(warp - 2 - kEpiWarps) >> 2;
         const uint32_t lane_base = tmem + kSfBase + ((uint32_t)((warp & 3) * 32) << 16);
         if constexpr (PLANES == 2) {
             const uint32_t steps = (uint32_t)((num_tiles - (int32_t)blockIdx.x + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x) * (uint32_t)k_iters;
@@ -319,46 +349,54 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict
                 if (lane == 0) { mbar_arrive(full0 + 8 * s); mbar_arrive(sf_empty0 + 8 * bx); }
             }
         } else {
-            // The loads of the group's next step are in flight while this one waits for its slot and is written.
-            // With two groups and three stages a group sees only every second phase of a stage's barrier.  That is unambiguous: its step before, two
-            // steps earlier, waited for MMAs later than those of the phase before.
+            // The loads of step it + 1 are in flight while step it waits for its slot and is written.
             const int32_t ktiles = k_iters * kStepBlocks;
-            int32_t t = blockIdx.x, kt = (int32_t)group, t_at = -1;       // the step whose tiles are loaded next; the tile of pa and pb
+            int32_t t = blockIdx.x, kt = 0;                                   // the step whose tiles are loaded next
             const uint4 *pa = nullptr, *pb = nullptr;
             auto load_next = [&](uint4 (&a)[kStepBlocks], uint4 (&b)[kStepBlocks]) {   // false when there is no further step
-                while (kt >= k_iters) { kt -= k_iters; t += gridDim.x; }
                 if (t >= num_tiles) return false;
-                if (t != t_at) {
-                    t_at = t;
+                if (kt == 0) {
                     int32_t tile_m, tile_n;
                     tile_of(t, tiles_m, tiles_n, tile_m, tile_n);
                     pa = reinterpret_cast<const uint4*>(sfa + (size_t)tile_m * ktiles * 512) + lane;
                     pb = reinterpret_cast<const uint4*>(sfb + (size_t)tile_n * ktiles * 512) + lane;
                 }
 #pragma unroll
-                for (int kb = 0; kb < kStepBlocks; ++kb) {                 // tile kb of the step: 16 bytes per lane, tiles 512 bytes apart
+                for (int kb = 0; kb < kStepBlocks; ++kb) {                     // tile kb of the step: 16 bytes per lane, tiles 512 bytes apart
                     a[kb] = __ldg(pa + (kt * kStepBlocks + kb) * 32);
                     b[kb] = __ldg(pb + (kt * kStepBlocks + kb) * 32);
                 }
-                kt += kGroups;
+                if (++kt == k_iters) { kt = 0; t += gridDim.x; }
                 return true;
             };
-            uint4 a[kStepBlocks], b[kStepBlocks];
+            // One step of lookahead in registers where a step is one box long; with two-box steps the four scale slots
+            // already let these warps run three steps ahead of the MMAs.
+            constexpr bool kLookahead = KBOXES == 1;
+            uint4 a[kStepBlocks], b[kStepBlocks], an[kLookahead ? kStepBlocks : 1], bn[kLookahead ? kStepBlocks : 1];
             bool more = load_next(a, b);
-            for (uint32_t it = group; more; it += kGroups) {
-                const uint32_t s = it % kStages;
-                if (!mbar_wait_warp(empty0 + 8 * s, ((it / kStages) & 1u) ^ 1u)) { if (lane == 0) atomicExch(error, 6); break; }
+            for (uint32_t it = 0; more; ++it) {
+                if constexpr (kLookahead) more = load_next(an, bn);
+                const uint32_t slot = it % kSfSlots;
+                bool have = mbar_wait(sf_empty0 + 8 * slot, ((it / kSfSlots) & 1u) ^ 1u);
+                if (!have && lane == 0) atomicExch(error, 6);
+                have = __all_sync(0xFFFFFFFFu, have);
+                if (!have) break;
                 tc_fence_after();
 #pragma unroll
                 for (int g = 0; g < KBOXES; ++g) {
-                    tmem_store16(lane_base + s * kSlotCols + 16u * g, a[4 * g], a[4 * g + 1], a[4 * g + 2], a[4 * g + 3]);
-                    tmem_store16(lane_base + s * kSlotCols + kSlotCols / 2 + 16u * g, b[4 * g], b[4 * g + 1], b[4 * g + 2], b[4 * g + 3]);
+                    tmem_store16(lane_base + slot * kSlotCols + 16u * g, a[4 * g], a[4 * g + 1], a[4 * g + 2], a[4 * g + 3]);
+                    tmem_store16(lane_base + slot * kSlotCols + kSlotCols / 2 + 16u * g, b[4 * g], b[4 * g + 1], b[4 * g + 2], b[4 * g + 3]);
                 }
                 tmem_store_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(full0 + 8 * s);
-                more = load_next(a, b);
+                if (lane == 0) mbar_arrive(sf_full0 + 8 * slot);
+                if constexpr (kLookahead) {
+#pragma unroll
+                    for (int kb = 0; kb < kStepBlocks; ++kb) { a[kb] = an[kb]; b[kb] = bn[kb]; }
+                } else {
+                    more = load_next(a, b);
+                }
             }
         }
     } else {
