@@ -99,8 +99,9 @@ struct TileOperand {
     uint8_t* tiled;
     int64_t rows;
     int64_t items;                 // ceil(rows / 128) * k / 256 * 32: one item = 4 rows x 16 scales
+    uint32_t pitch, ksteps;        // k / 16, k / 256
 };
-__global__ void __launch_bounds__(256, 8) sf_tile_kernel(const TileOperand a, const TileOperand b, uint32_t ksteps, int* __restrict__ error) {
+__global__ void __launch_bounds__(256, 8) sf_tile_kernel(const TileOperand a, const TileOperand b, int* __restrict__ error) {
     pdl_launch_dependents();
     pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -109,19 +110,22 @@ __global__ void __launch_bounds__(256, 8) sf_tile_kernel(const TileOperand a, co
         const TileOperand& o = i < a.items ? a : b;
         const int64_t j = i < a.items ? i : i - a.items;
         const uint32_t lane = (uint32_t)(j & 31);
-        const int64_t step = j >> 5, rb = step / ksteps;              // (row block, K-step), row block
+        const int64_t step = j >> 5;                                  // (row block, K-step)
+        const uint32_t ksteps = o.ksteps;
+        const int64_t rb = step / ksteps;
         const uint32_t kt = (uint32_t)(step - rb * ksteps);
         uint4 r[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int64_t row = rb * 128 + q * 32 + lane;             // rows beyond the operand (last row block) get zero scales
-            r[q] = row < o.rows ? __ldg(reinterpret_cast<const uint4*>(o.scales + row * (ksteps * 16)) + kt) : make_uint4(0u, 0u, 0u, 0u);
+            r[q] = row < o.rows ? __ldg(reinterpret_cast<const uint4*>(o.scales + row * o.pitch) + kt) : make_uint4(0u, 0u, 0u, 0u);
         }
-        uint4* out = reinterpret_cast<uint4*>(o.tiled + step * 2048) + lane;
-        out[0] = mask_scales(r[0].x, r[1].x, r[2].x, r[3].x);
-        out[32] = mask_scales(r[0].y, r[1].y, r[2].y, r[3].y);
-        out[64] = mask_scales(r[0].z, r[1].z, r[2].z, r[3].z);
-        out[96] = mask_scales(r[0].w, r[1].w, r[2].w, r[3].w);
+        uint4* out = reinterpret_cast<uint4*>(o.tiled + ((size_t)rb * ksteps + kt) * 2048u) + lane;
+        constexpr uint32_t kMag = 0x7F7F7F7Fu;
+        out[0] = make_uint4(r[0].x & kMag, r[1].x & kMag, r[2].x & kMag, r[3].x & kMag);
+        out[32] = make_uint4(r[0].y & kMag, r[1].y & kMag, r[2].y & kMag, r[3].y & kMag);
+        out[64] = make_uint4(r[0].z & kMag, r[1].z & kMag, r[2].z & kMag, r[3].z & kMag);
+        out[96] = make_uint4(r[0].w & kMag, r[1].w & kMag, r[2].w & kMag, r[3].w & kMag);
     }
 }
 
@@ -131,10 +135,10 @@ __global__ void __launch_bounds__(256, 8) sf_tile_kernel(const TileOperand a, co
 // then the scale slots: 16 columns of A scales and 16 of B scales each (four per MMA of K = 64).
 constexpr uint32_t kTmemCols = 512;
 
-struct GemmMaps {
-    CUtensorMap a[2], b[2];        // planes H, L of A [M, K/2 bytes] and B [N, K/2 bytes], boxes of 128 bytes x 128 rows
-    CUtensorMap sa, sb;            // IF4: their scales as abs_quantize wrote them [rows, K/16 bytes], boxes of 16 bytes x 128 rows
-};
+// Planes of A [M, K/2 bytes] and of B [N, K/2 bytes], boxes of 128 bytes x 128 rows: the codes (NVFP4), or H and L and, as abs_quantize wrote
+// them, the scales [rows, K/16 bytes], boxes of 16 bytes x 128 rows (IF4).
+template <int PLANES> struct GemmMaps { CUtensorMap a[1], b[1]; };
+template <> struct GemmMaps<2> { CUtensorMap a[2], b[2], sa, sb; };
 
 // Tile t of the (tiles_m x tiles_n) grid of 128 x 128 tiles, walked in bands of eight tile rows, column by column
 // inside a band, so that the blocks running at the same time share few rows of A and few of B (L2 reuse).
@@ -163,7 +167,7 @@ __device__ __forceinline__ void tile_of(int32_t t, int32_t tiles_m, int32_t tile
 // OUT_BF16: C is written as bf16 (round to nearest even of the same FP32 value), else as FP32.
 template <int PLANES, bool OUT_BF16, int KBOXES = 1>
 __global__ void __launch_bounds__(kGemmThreads<PLANES>, 1)
-if4_gemm_kernel(const __grid_constant__ GemmMaps maps, const uint8_t* __restrict__ sfa, const uint8_t* __restrict__ sfb,
+if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const uint8_t* __restrict__ sfa, const uint8_t* __restrict__ sfb,
                 const float* __restrict__ alpha_a, const float* __restrict__ alpha_b, void* __restrict__ c_out, int32_t tiles_m,
                 int32_t tiles_n, int32_t k_iters, int32_t m_rows, int* __restrict__ error, int32_t stall_step,
                 float* __restrict__ next_alpha, float next_denom) {
@@ -825,17 +829,15 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
         return skinny_matmul(P, a_codes, a_scales, a_alpha, b_codes, b_scales, b_alpha, m, n, k, c_f32, ws, s, stall_step, out_bf16,
                              next_alpha, next_denom);
 
-    GemmMaps maps;
-    for (int p = 0; p < 2; ++p) {
-        // NVFP4 needs no split: its single plane is the caller's codes
-        void* pa = has_int ? (void*)(ws + L.off_a + p * L.plane_a) : const_cast<void*>(a_codes);
-        void* pb = has_int ? (void*)(ws + L.off_b + p * L.plane_b) : const_cast<void*>(b_codes);
-        if (!plane_map(&maps.a[p], pa, (uint64_t)m, (uint64_t)k / 2) || !plane_map(&maps.b[p], pb, (uint64_t)n, (uint64_t)k / 2))
-            return ABS_ERR_CUDA;
-    }
+    GemmMaps<1> maps1;
+    GemmMaps<2> maps2;
     if (has_int) {
-        if (!scale_map(&maps.sa, const_cast<void*>(a_scales), (uint64_t)m, (uint64_t)k / 16) ||
-            !scale_map(&maps.sb, const_cast<void*>(b_scales), (uint64_t)n, (uint64_t)k / 16))
+        for (int p = 0; p < 2; ++p)
+            if (!plane_map(&maps2.a[p], ws + L.off_a + p * L.plane_a, (uint64_t)m, (uint64_t)k / 2) ||
+                !plane_map(&maps2.b[p], ws + L.off_b + p * L.plane_b, (uint64_t)n, (uint64_t)k / 2))
+                return ABS_ERR_CUDA;
+        if (!scale_map(&maps2.sa, const_cast<void*>(a_scales), (uint64_t)m, (uint64_t)k / 16) ||
+            !scale_map(&maps2.sb, const_cast<void*>(b_scales), (uint64_t)n, (uint64_t)k / 16))
             return ABS_ERR_CUDA;
         SplitOperand so[2];
         for (int op = 0; op < 2; ++op) {
@@ -850,24 +852,28 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
         if (blocks > 148 * 8) blocks = 148 * 8;
         if (launch_pdl(if4_split_kernel, dim3((unsigned)blocks), 256, 0, s, so[0], so[1], (int*)ws) != cudaSuccess) return ABS_ERR_CUDA;
     } else {
+        if (!plane_map(&maps1.a[0], const_cast<void*>(a_codes), (uint64_t)m, (uint64_t)k / 2) ||
+            !plane_map(&maps1.b[0], const_cast<void*>(b_codes), (uint64_t)n, (uint64_t)k / 2))
+            return ABS_ERR_CUDA;
         TileOperand to[2];
         for (int op = 0; op < 2; ++op) {
             to[op].scales = (const uint8_t*)(op ? b_scales : a_scales);
             to[op].tiled = ws + (op ? L.off_sfb : L.off_sfa);
             to[op].rows = op ? n : m;
             to[op].items = (to[op].rows + 127) / 128 * (k / kStageK) * 32;
+            to[op].pitch = (uint32_t)(k / 16);
+            to[op].ksteps = (uint32_t)(k / kStageK);
         }
         int64_t blocks = (to[0].items + to[1].items + 255) / 256;
         if (blocks > 148 * 8) blocks = 148 * 8;
-        if (launch_pdl(sf_tile_kernel, dim3((unsigned)blocks), 256, 0, s, to[0], to[1], (uint32_t)(k / kStageK), (int*)ws) != cudaSuccess)
-            return ABS_ERR_CUDA;
+        if (launch_pdl(sf_tile_kernel, dim3((unsigned)blocks), 256, 0, s, to[0], to[1], (int*)ws) != cudaSuccess) return ABS_ERR_CUDA;
     }
     const int32_t tiles_m = (int32_t)((m + kTileM - 1) / kTileM), tiles_n = (int32_t)(n / kTileN);
     const int64_t num_tiles = (int64_t)tiles_m * tiles_n;
     const dim3 pgrid((unsigned)(num_tiles < sm_count[dev] ? num_tiles : sm_count[dev]));
     cudaError_t e;
 #define ABS_LAUNCH_GEMM(P, O, B)                                                                                        \
-    e = launch_pdl(if4_gemm_kernel<P, O, B>, pgrid, kGemmThreads<P>, kGemmSmemBytes<P, B>, s, maps, (const uint8_t*)(ws + L.off_sfa), \
+    e = launch_pdl(if4_gemm_kernel<P, O, B>, pgrid, kGemmThreads<P>, kGemmSmemBytes<P, B>, s, maps##P, (const uint8_t*)(ws + L.off_sfa), \
                    (const uint8_t*)(ws + L.off_sfb), a_alpha, b_alpha, c_f32, tiles_m, tiles_n,                           \
                    (int32_t)(k / (kStageK * B)), (int32_t)m, (int*)ws, stall_step, next_alpha, next_denom)
     const bool long_steps = !has_int && k % (2 * kStageK) == 0;      // NVFP4: K-steps of 512 where K allows
