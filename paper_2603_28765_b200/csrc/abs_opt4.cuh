@@ -10,26 +10,34 @@ namespace absq {
 constexpr float kMagic = 12582912.0f;                 // 1.5 * 2^23: x + kMagic leaves RNE(x) in the low mantissa bits
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
-__device__ __forceinline__ float min3f(float a, float b, float c) {
-    float d;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ float max3f(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ uint32_t sign_of(float y) { return __float_as_uint(y) & 0x80000000u; }
-
 __device__ __forceinline__ uint64_t add2_rp(uint64_t a, uint64_t b) {
     uint64_t d;
     asm("add.rp.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
-__device__ __forceinline__ uint64_t fma2_rp(uint64_t a, uint64_t b, uint64_t c) {
+__device__ __forceinline__ uint64_t add2_rm(uint64_t a, uint64_t b) {
     uint64_t d;
-    asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t mul2_rp(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rp.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// Eight magnitudes 0..7 (nibbles of m), negated in two's complement where bit 3 of the nibble of s is set (s has no other bits):
+// 8 - m borrows from no neighbour, and its bit 3 flipped is 16 - m, or 0 for m = 0.
+__device__ __forceinline__ uint32_t negate_nibbles(uint32_t m, uint32_t s) {
+    const uint32_t neg = m & (s - (s >> 3));                 // the magnitudes to negate
+    return (m ^ neg) | ((s - neg) ^ s);
+}
+
+// c + (-w) * (one 16-bit field of rnd): the field is picked, weighted and subtracted by one instruction.
+template <int W, bool UPPER>
+__device__ __forceinline__ uint32_t minus_field(uint32_t rnd, uint32_t c) {
+    constexpr uint32_t weight = (uint32_t)(256 - W) << (UPPER ? 8 : 0);      // signed byte -W for the wanted field, 0 for the other
+    uint32_t d;
+    asm("dp2a.lo.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(rnd), "r"(weight), "r"(c));
     return d;
 }
 
@@ -37,126 +45,99 @@ __device__ __forceinline__ uint64_t fma2_rp(uint64_t a, uint64_t b, uint64_t c) 
 // rounded stochastically, App. B).  rnd[i] holds the two 16-bit random fields h of elements 2i (low half)
 // and 2i+1; u = (h + 1/2) * 2^-16.
 //
-// The rule "lo if a == lo, else hi iff u < (a - lo) / (hi - lo)" is evaluated as a ceiling.  With phi the
-// grid's fractional-index map (grid point g_i -> i, linear in between), the rounded index is ceil(phi(a) - u):
-// for phi = n + f it is n when u >= f and n + 1 when u < f.  For E2M1 phi(a) = min(2a, a + 2, a/2 + 4); the
-// pieces, the subtraction of u and the final add of 1.5 * 2^23 (which leaves the ceiling in the low mantissa
-// bits) all round toward +infinity, and that changes nothing: u is an odd multiple of 2^-17, every rounding
-// here is to a grid at least as fine as 2^-21, so a sum rounded up crosses neither u nor an integer that the
-// exact sum does not reach.  The value of an index is max(i/2, i - 2, 2i - 8).  The integer candidate is the
-// same ceiling on |z|, z = y * 7/6 rounded to FP32 as in the round-to-nearest path, clamped to 7.
-template <bool HAS_INT>
+// The rule "lo if a == lo, else hi iff u < (a - lo) / (hi - lo)" is a ceiling: with phi the grid's fractional-index
+// map (grid point g_i -> i, linear in between), the rounded index is ceil(phi(a) - u).  Both candidates are formed on
+// magnitudes -- an error and its square do not see a common sign of x, value and code -- and take u off as an integer:
+//   E2M1: phi is linear in the bit pattern of a float with one mantissa bit and the smallest normal exponent at 1, so b =
+//   bits(a * 2^-126) (rounded up; below 1 an FP32 subnormal) is phi(a) * 2^22, and the index is bits 22.. of
+//   b + 2^22 - 33 - 64 h (2^22 u = 64 h + 32).  Those bits alone are the pattern of value * 2^-126.
+//   Integer: the pattern of |z| + 65 - 2^-16 (rounded up; ulp 2^-17), minus 2 h, is that of 64 + k + a fraction, z = y * 7/6
+//   rounded to FP32 as in the round-to-nearest path; an add that rounds down drops the fraction.
+// Rounding up to a grid on which 2^22 u, or 2^17 u, lies crosses neither u nor an integer that the exact value does not reach.
+// What bounds the kernels that call this is the arithmetic pipes, so the count of instructions: 36 -> 25 per pair of elements against three
+// float pieces for phi, a float subtraction of u and signs put back on both values.  IF4, 8192 x 8192, 17/16 option, us before and after:
+// rows with Hadamard 92.3 / 76.0, rows 84.0 / 69.9, columns with Hadamard 104.6 / 86.2; NVFP4 63.5 / 53.4, 53.4 / 47.1, 73.9 / 64.4.
+// CLAMP: |y| may exceed 6 (then |z| 7; fl(6 * fp32(7/6)) is 7, so one clamp serves both).  With the 17/16 option and a
+// scale byte that is neither subnormal nor saturated it stays below 6 (1 + 7 * 2^-24), and neither index passes 7.
+template <bool HAS_INT, bool CLAMP>
 __device__ __forceinline__ void encode_body4_sr(const float (&x)[16], const uint32_t (&rnd)[8], uint32_t sb, float d,
                                                 float r, uint32_t& sbyte, uint32_t& c_lo, uint32_t& c_hi) {
     const uint64_t R2 = pack2(r, r);
-    const uint64_t TWO = pack2(2.0f, 2.0f), HALF = pack2(0.5f, 0.5f), FOUR = pack2(4.0f, 4.0f);
-    const uint64_t MG = pack2(kMagic, kMagic), NMG = pack2(-kMagic, -kMagic);
-    const uint64_t NSC16 = pack2(-1.0f / 65536.0f, -1.0f / 65536.0f);
-    const uint64_t P128MH = pack2(128.0f - 1.0f / 131072.0f, 128.0f - 1.0f / 131072.0f);   // 128 - 2^-17, 24 bits
-
+    constexpr float kTiny = 1.17549435e-38f, kHuge = 8.507059173e37f;          // 2^-126, 2^126
+    const uint64_t TINY = pack2(kTiny, kTiny), HUGE2 = pack2(kHuge, kHuge);
     const float c_pre = __uint_as_float(0x3F955555u);    // fp32(7/6)
     const float c_post = __uint_as_float(0x3F5B6DB7u);   // fp32(6/7)
     const float d_int = __fmul_rn(d, c_post);
     const uint64_t ND2 = pack2(-d, -d), NDI2 = pack2(-d_int, -d_int), CP2 = pack2(c_pre, c_pre);
-    const uint64_t MG8 = pack2(kMagic8, kMagic8);
-    const uint64_t NMGH = pack2(-0.5f * kMagic, -0.5f * kMagic), NMG2 = pack2(-(kMagic + 2.0f), -(kMagic + 2.0f));
-    const uint64_t NMG8 = pack2(-(2.0f * kMagic + 8.0f), -(2.0f * kMagic + 8.0f));
+    constexpr float kBase = 65.0f - 1.0f / 65536.0f;
+    const uint64_t BASE = pack2(kBase, kBase), FLOOR = pack2(kMagic - 64.0f, kMagic - 64.0f), NMG = pack2(-kMagic, -kMagic);
 
     uint64_t accF[2], accI[2];
-    uint32_t fw[2], kb[16], ib[16];
+    uint32_t word[2], sign[2], kb[16];
 #pragma unroll
     for (int hgrp = 0; hgrp < 2; ++hgrp) {
-        float vs[8], ys[8];
+        float vs[8], xs[8];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int e = 8 * hgrp + 2 * i;
-            const uint64_t X = pack2(x[e], x[e + 1]);
-            const uint64_t Y = mul2(X, R2);                                    // E1 (step 3)
-            float y0, y1;
-            unpack2(Y, y0, y1);
-            ys[2 * i] = y0; ys[2 * i + 1] = y1;
-            // -u = -(h + 1/2) * 2^-16 from the 16-bit fields: 2^23 + h as a float, then one multiply-add whose exact
-            // result -(2^23 + h) * 2^-16 + 128 - 2^-17 has 17 significant bits, so nothing is rounded
+            xs[2 * i] = x[e]; xs[2 * i + 1] = x[e + 1];
             const uint32_t rw = rnd[e >> 1];
-            const float m0 = __uint_as_float((rw & 0xFFFFu) | 0x4B000000u);
-            const float m1 = __uint_as_float(__byte_perm(rw, 0x4B00u, 0x5432));
-            const uint64_t NU = fma2(pack2(m0, m1), NSC16, P128MH);
-            // E2 under stochastic rounding: index = ceil(phi(a) - u)
-            const float a0 = fminf(fabsf(y0), 6.0f), a1 = fminf(fabsf(y1), 6.0f);
-            const uint64_t A = pack2(a0, a1);
-            float p00, p01, p10, p11, p20, p21;
-            unpack2(add2(A, A), p00, p01);                                     // exact
-            unpack2(add2_rp(A, TWO), p10, p11);
-            unpack2(fma2_rp(A, HALF, FOUR), p20, p21);
-            const uint64_t PHI = pack2(min3f(p00, p10, p20), min3f(p01, p11, p21));
-            const uint64_t IM = add2_rp(add2_rp(PHI, NU), MG);                 // low mantissa bits = index 0..7
-            float im0, im1;
-            unpack2(IM, im0, im1);
-            ib[e] = __float_as_uint(im0);
-            ib[e + 1] = __float_as_uint(im1);
+            const uint64_t X = pack2(fabsf(x[e]), fabsf(x[e + 1]));
+            uint64_t Y = mul2(X, R2);                                          // E1 (step 3)
+            if constexpr (CLAMP) {
+                float y0, y1;
+                unpack2(Y, y0, y1);
+                Y = pack2(fminf(y0, 6.0f), fminf(y1, 6.0f));
+            }
+            // E2 under stochastic rounding
+            float b0, b1, v0, v1;
+            unpack2(mul2_rp(Y, TINY), b0, b1);
+            constexpr uint32_t kOffset = (1u << 22) - 33u, kIndex = 0xFFC00000u;
+            v0 = __uint_as_float(minus_field<64, false>(rw, __float_as_uint(b0) + kOffset) & kIndex);
+            v1 = __uint_as_float(minus_field<64, true>(rw, __float_as_uint(b1) + kOffset) & kIndex);
+            const uint64_t V = mul2(pack2(v0, v1), HUGE2);                     // value of the index (exact)
+            unpack2(V, vs[2 * i], vs[2 * i + 1]);
             if constexpr (HAS_INT) {
-                // value of the index i = IM - kMagic: max(i/2, i - 2, 2i - 8), each piece formed from IM in one
-                // exact operation (kMagic / 2, kMagic + 2 and 2 * kMagic + 8 are all FP32 numbers)
-                float q00, q01, q10, q11, q20, q21;
-                unpack2(fma2(IM, HALF, NMGH), q00, q01);
-                unpack2(add2(IM, NMG2), q10, q11);
-                unpack2(fma2(IM, TWO, NMG8), q20, q21);
-                const float v0 = max3f(q00, q10, q20), v1 = max3f(q01, q11, q21);          // value of the index
-                const float vs0 = __uint_as_float((__float_as_uint(v0) & 0x7FFFFFFFu) | sign_of(y0));
-                const float vs1 = __uint_as_float((__float_as_uint(v1) & 0x7FFFFFFFu) | sign_of(y1));
-                vs[2 * i] = vs0; vs[2 * i + 1] = vs1;
-                const uint64_t E = fma2(pack2(vs0, vs1), ND2, X);              // E3 (steps 5-6), negated; squared below
+                const uint64_t E = fma2(V, ND2, X);                            // E3 (steps 5-6), negated; squared below
                 accF[hgrp] = (i == 0) ? mul2(E, E) : fma2(E, E, accF[hgrp]);
-                // E4 (step 7) under stochastic rounding: |k| = ceil(min(|z|, 7) - u), sign of z put back
-                float z0, z1;
-                unpack2(mul2(Y, CP2), z0, z1);
-                const uint64_t AZ = pack2(fminf(fabsf(z0), 7.0f), fminf(fabsf(z1), 7.0f));
-                float k0, k1;
-                unpack2(add2(add2_rp(add2_rp(AZ, NU), MG), NMG), k0, k1);
-                const float ks0 = __uint_as_float((__float_as_uint(k0) & 0x7FFFFFFFu) | sign_of(z0));
-                const float ks1 = __uint_as_float((__float_as_uint(k1) & 0x7FFFFFFFu) | sign_of(z1));
-                const uint64_t KS = pack2(ks0, ks1);
-                const uint64_t FI = fma2(KS, NDI2, X);                         // E5 (steps 8-9)
+                // E4 (step 7) under stochastic rounding
+                float z0, z1, k0, k1;
+                unpack2(add2_rp(mul2(Y, CP2), BASE), z0, z1);
+                z0 = __uint_as_float(minus_field<2, false>(rw, __float_as_uint(z0)));
+                z1 = __uint_as_float(minus_field<2, true>(rw, __float_as_uint(z1)));
+                const uint64_t KM = add2_rm(pack2(z0, z1), FLOOR);             // kMagic + k
+                const uint64_t FI = fma2(add2(KM, NMG), NDI2, X);              // E5 (steps 8-9)
                 accI[hgrp] = (i == 0) ? mul2(FI, FI) : fma2(FI, FI, accI[hgrp]);
-                float km0, km1;
-                unpack2(add2(KS, MG8), km0, km1);                              // low nibble = k + 8
-                kb[e] = __float_as_uint(km0);
-                kb[e + 1] = __float_as_uint(km1);
+                unpack2(KM, k0, k1);
+                kb[e] = __float_as_uint(k0);
+                kb[e + 1] = __float_as_uint(k1);
             }
         }
-        if constexpr (HAS_INT) fw[hgrp] = e2m1x8_encode(vs);                   // exact: the values are on the grid
-        else fw[hgrp] = e2m1x8_encode(ys) & 0x88888888u;                       // only the signs of y
+        word[hgrp] = e2m1x8_encode(vs);                                        // exact: the values are on the grid
+        sign[hgrp] = e2m1x8_encode(xs) & 0x88888888u;                          // the sign bits alone
     }
-    if constexpr (!HAS_INT) {
-        // codes = index nibbles by Horner on the raw sums (each holds kMagicBits + index) | sign bits
-        constexpr uint32_t kConstI = kMagicBits * 0x11111111u;
-        uint32_t il = ib[7], ih = ib[15];
-#pragma unroll
-        for (int j = 6; j >= 0; --j) {
-            il = il * 16u + ib[j];
-            ih = ih * 16u + ib[8 + j];
-        }
-        c_lo = (il - kConstI) | fw[0];
-        c_hi = (ih - kConstI) | fw[1];
-        sbyte = sb;
-    } else {
+    c_lo = word[0] | sign[0];
+    c_hi = word[1] | sign[1];
+    sbyte = sb;
+    if constexpr (HAS_INT) {
         float f0, f1, f2, f3, i0, i1, i2, i3;
         unpack2(accF[0], f0, f1); unpack2(accF[1], f2, f3);
         unpack2(accI[0], i0, i1); unpack2(accI[1], i2, i3);
         const float E_fp = __fadd_rn(__fadd_rn(f0, f1), __fadd_rn(f2, f3));     // S1-S2 (step 10)
         const float E_int = __fadd_rn(__fadd_rn(i0, i1), __fadd_rn(i2, i3));
         const bool flag = E_int < E_fp;
-        constexpr uint32_t kConst = kMagic8Bits * 0x11111111u - 0x88888888u;
+        // magnitudes 0..7 by Horner on the raw sums (each holds kMagicBits + k), then two's complement where the sign is set
+        constexpr uint32_t kConst = kMagicBits * 0x11111111u;
         uint32_t il = kb[7], ih = kb[15];
 #pragma unroll
         for (int j = 6; j >= 0; --j) {
             il = il * 16u + kb[j];
             ih = ih * 16u + kb[8 + j];
         }
-        il = (il - kConst) ^ 0x88888888u;
-        ih = (ih - kConst) ^ 0x88888888u;
-        c_lo = flag ? il : fw[0];
-        c_hi = flag ? ih : fw[1];
+        il = negate_nibbles(il - kConst, sign[0]);
+        ih = negate_nibbles(ih - kConst, sign[1]);
+        c_lo = flag ? il : c_lo;
+        c_hi = flag ? ih : c_hi;
         sbyte = sb | (flag ? 0x80u : 0u);
     }
 }
@@ -249,7 +230,10 @@ quantize4_opt_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
         const float d = dr.x, r = dr.y;
         uint32_t sbyte = 0u, c_lo = 0u, c_hi = 0u;
         if constexpr (SR) {
-            if (sb != 0u) encode_body4_sr<HAS_INT>(x, rnd, sb, d, r, sbyte, c_lo, c_hi);      // G4: zero scale -> zeros
+            // without the clamp where it cannot act (IF4 with Hadamard, 8192 x 8192: 77.9 -> 76.0 us; the transposed kernel, which
+            // unrolls four groups, gained nothing from a second copy)
+            if ((sb - 8u) < 118u && scale_mul > 1.0f) encode_body4_sr<HAS_INT, false>(x, rnd, sb, d, r, sbyte, c_lo, c_hi);
+            else if (sb != 0u) encode_body4_sr<HAS_INT, true>(x, rnd, sb, d, r, sbyte, c_lo, c_hi);      // G4: zero scale -> zeros
         } else {
             if ((sb - 8u) >= 118u) {
                 if (sb != 0u) encode_body4<HAS_INT, HAS_INT>(x, sb, d, r, sbyte, c_lo, c_hi);

@@ -182,7 +182,7 @@ __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __rest
                         const uint4 p0 = philox4x32_10((uint32_t)i8, (uint32_t)(i8 >> 32), keys);
                         const uint4 p1 = philox4x32_10((uint32_t)i8 + 1u, (uint32_t)(i8 >> 32), keys);
                         const uint32_t rnd[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-                        encode_body4_sr<HAS_INT>(x, rnd, sb, d, r, sbyte, c_lo, c_hi);
+                        encode_body4_sr<HAS_INT, true>(x, rnd, sb, d, r, sbyte, c_lo, c_hi);
                     }
                 } else if ((sb - 8u) >= 118u) {
                     if (sb != 0u) encode_body4<HAS_INT, HAS_INT>(x, sb, d, r, sbyte, c_lo, c_hi);
