@@ -36,6 +36,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <mutex>
+#include <type_traits>
 
 namespace absq {
 
@@ -598,6 +599,8 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
 
 }  // namespace absq
 
+#include "abs_pair.cuh"
+
 // ----------------------------------------------------------------------------- host side
 
 namespace {
@@ -738,6 +741,19 @@ bool rows_rule(abs_fmt_t fmt, int64_t m, int64_t n, int64_t k, int sm_count) {
         return (m <= 4 && chunks <= 10 && 2 * turns < 3 * warps) || 10 * kRowsChunk * turns * chunks * chunks <= (m <= 4 ? 43 : 30) * warps * k;
     return m <= 4 || k % (2 * kStageK) != 0 || n * chunks <= (int64_t)kTileN * sm_count;
 }
+// NVFP4: which products take their tiles in pairs (abs_pair.cuh) and not one by one.  More than one round of tiles, and what pairs save has to outweigh
+// that the last round is one of pairs or of single tiles: bf16 from one and a quarter rounds on, FP32, whose stores take longer, from three; with
+// K >= 3072 always.  One by one / in pairs, us, bf16 and FP32: 257 x 8192 x 256 (192 tiles) 7.4 / 6.9, 7.9 / 7.4; 1000 x 4096 x 512 (256) 7.8 / 7.6, 8.2 / 8.7;
+// 300 x 14336 x 2048 (336) 14.1 / 13.6, 14.9 / 15.4; 2048 x 4096 x 512 (512) 10.9 / 9.8, 11.9 / 11.6; 600 x 4096 x 1024 (160) 8.6 / 8.5, 9.1 / 9.2;
+// 600 x 4096 x 4096 15.6 / 14.5, 16.0 / 15.2; 1000 x 14336 x 4096 41.9 / 36.3, 54.4 / 44.4; back to back for longer, at the power cap, 8192 x 14336 x 4096
+// 321 / 274, 388 / 326.
+// An odd number of tile columns leaves pairs of one tile; where the rounds then are a sixth longer (FP32: at all), tiles go one by one.
+bool pair_rule(bool out_bf16, int64_t tiles_m, int64_t tiles_n, int64_t k, int sm_count) {
+    const int64_t tiles = tiles_m * tiles_n, pairs = tiles_m * ((tiles_n + 1) / 2), rest = pairs % sm_count;
+    if (tiles <= sm_count || (k < 3072 && (out_bf16 ? 4 * tiles < 5 * (int64_t)sm_count : tiles < 3 * (int64_t)sm_count))) return false;
+    const int64_t one_by_one = (tiles + sm_count - 1) / sm_count, in_pairs = pairs / sm_count * 2 + (rest == 0 ? 0 : 2 * rest <= sm_count ? 1 : 2);
+    return out_bf16 ? 6 * in_pairs <= 7 * one_by_one : in_pairs <= one_by_one;
+}
 typedef void (*RowsKernel)(RowsArgs);
 template <int M> RowsKernel rows_kernel_for(bool has_int, bool out_bf16) {
     return has_int ? (out_bf16 ? rows_kernel<M, true, true> : rows_kernel<M, true, false>)
@@ -847,6 +863,10 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
         ABS_GEMM_ATTR(1, false, 2); ABS_GEMM_ATTR(1, true, 2);
 #undef ABS_GEMM_ATTR
         if (attr_err[dev] == cudaSuccess)
+            attr_err[dev] = cudaFuncSetAttribute(nvfp4_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes);
+        if (attr_err[dev] == cudaSuccess)
+            attr_err[dev] = cudaFuncSetAttribute(nvfp4_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes);
+        if (attr_err[dev] == cudaSuccess)
             attr_err[dev] = cudaFuncSetAttribute(skinny_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkinnySmemBytes);
         if (attr_err[dev] == cudaSuccess)
             attr_err[dev] = cudaFuncSetAttribute(skinny_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkinnySmemBytes);
@@ -912,6 +932,11 @@ static abs_status_t matmul_impl(abs_fmt_t fmt, const void* a_codes, const void* 
 #define ABS_LAUNCH_GEMM(P, O, B)                                                                                        \
     e = launch_pdl(if4_gemm_kernel<P, O, B>, pgrid, kGemmThreads<P>, kGemmSmemBytes<P, B>, s, maps##P, a_alpha, b_alpha, c_f32, tiles_m, tiles_n, \
                    (int32_t)(k / (kStageK * B)), (int32_t)m, (int*)ws, stall_step, next_alpha, next_denom)
+    if (!has_int && pair_rule(out_bf16, tiles_m, tiles_n, k, sm_count[dev])) {
+        e = launch_pdl(out_bf16 ? nvfp4_pair_kernel<true> : nvfp4_pair_kernel<false>, dim3((unsigned)sm_count[dev]), kPairThreads, kPairSmemBytes, s, maps1,
+                       a_alpha, b_alpha, c_f32, tiles_m, tiles_n, (int32_t)(k / kStageK), (int32_t)m, (int*)ws, stall_step, next_alpha, next_denom);
+        return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
+    }
     const bool long_steps = !has_int && k % (2 * kStageK) == 0;      // NVFP4: K-steps of 512 where K allows
     if (has_int && out_bf16) ABS_LAUNCH_GEMM(2, true, 1);
     else if (has_int) ABS_LAUNCH_GEMM(2, false, 1);
