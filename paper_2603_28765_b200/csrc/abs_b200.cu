@@ -795,14 +795,16 @@ static abs_status_t quantize_transposed_impl(abs_fmt_t fmt, const void* in_bf16,
                            ((rblocks + kTransTileRowBlocks - 1) / kTransTileRowBlocks);
     if (ntiles > (int64_t)0x7FFFFFFF) return ABS_ERR_SIZE;      // the kernel indexes tiles with 32 bits
     // 64 KiB of shared memory per block: 3 blocks per SM.  The arithmetic-bound variants (IF4, options) and the
-    // emulation pass run best as several waves with about four tiles per block; plain NVFP4 as one wave of
-    // persistent blocks.
+    // emulation pass run best as several waves with about four tiles per block, and at least two waves as soon as there are more tiles
+    // than resident blocks (1 / 2 waves, us: IF4 Hadamard SR 4096 x 4096, 2.3 tiles per resident block, 25.4 / 22.6, IF4 12.6 / 11.9, IF4 Hadamard
+    // emulation 23.2 / 21.0; between 1.5 and 6 tiles 0.84 to 1.0 times as long, at 8192 x 4096 up to 3 % longer); plain NVFP4 as one
+    // wave of persistent blocks.
     const int64_t resident = (int64_t)st->sm_count * 3;
     const bool heavy = fmt == ABS_FMT_IF4 || (o.flags & (ABS_F_HADAMARD16 | ABS_F_STOCHASTIC)) || out_bf16 != nullptr;
     int64_t tgrid = ntiles < resident ? ntiles : resident;
     if (heavy && ntiles > resident) {
         int64_t waves = (ntiles + 2 * resident) / (4 * resident);
-        if (waves < 1) waves = 1;
+        if (waves < 2) waves = 2;
         tgrid = waves * resident < ntiles ? waves * resident : ntiles;
     }
     cudaLaunchConfig_t cfg = {};

@@ -78,12 +78,6 @@ __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __rest
                                                           bool store_codes) {
     extern __shared__ __align__(16) uint16_t trans_smem[];
     pdl_launch_dependents();
-    pdl_wait();
-    float alpha = 1.0f, inv_a6 = 1.0f;
-    if constexpr (MODE == 0) {
-        alpha = resolve_alpha<FROM_SLOT>(alpha_src);                         // T2
-        inv_a6 = __frcp_rn(__fmul_rn(alpha, 6.0f));                          // T3
-    }
     uint32_t local_max = 0u;
     const int64_t rblocks = rows / 16;
     const int64_t ntx = (cols + kTransTileCols - 1) / kTransTileCols;
@@ -132,7 +126,17 @@ __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __rest
     int64_t t = blockIdx.x;
     const uint32_t ntx32 = (uint32_t)ntx, step_y = gridDim.x / ntx32, step_x = gridDim.x - step_y * ntx32;
     uint32_t ty = blockIdx.x / ntx32, tx = blockIdx.x - ty * ntx32;
-    issue(t, ty, tx, 0);
+    {   // before the wait (see prefetch_l2): the block's first tile, a line of 128 bytes per thread
+        const int64_t r = (int64_t)ty * 16 * kTransTileRowBlocks + (threadIdx.x >> 2), c = (int64_t)tx * kTransTileCols + 64 * (threadIdx.x & 3);
+        if (r < rows && c < cols) prefetch_l2(in + r * cols + c);
+    }
+    pdl_wait();
+    issue(t, ty, tx, 0);                             // its copies are on their way while alpha is read
+    float alpha = 1.0f, inv_a6 = 1.0f;
+    if constexpr (MODE == 0) {
+        alpha = resolve_alpha<FROM_SLOT>(alpha_src);                         // T2
+        inv_a6 = __frcp_rn(__fmul_rn(alpha, 6.0f));                          // T3
+    }
     for (; t < ntiles; t += gridDim.x, s ^= 1) {
         uint32_t ty_next = ty + step_y, tx_next = tx + step_x;
         if (tx_next >= ntx32) { tx_next -= ntx32; ++ty_next; }
