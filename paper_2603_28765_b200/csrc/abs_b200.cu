@@ -26,7 +26,8 @@ constexpr int kMaxDevices = 64;
 
 // Launch with programmatic stream serialization: the kernel may be scheduled while the previous
 // kernel of the stream drains; every kernel here calls pdl_wait() before its first global access.
-// cooperative: the blocks wait for one another (one_pass_alpha), so all of them have to be resident.
+// cooperative: the blocks wait for one another (one_pass_alpha), so all of them have to be resident.  A single block needs no such launch, which costs
+// half a microsecond more on the host (2.45 us instead of 1.93) and lets nothing overlap: such kernels start 4.1 us apart on a stream.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_any(bool cooperative, void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -40,7 +41,7 @@ cudaError_t launch_any(bool cooperative, void (*kernel)(KArgs...), int grid, int
     attr[1].id = cudaLaunchAttributeCooperative;
     attr[1].val.cooperative = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = cooperative ? 2 : 1;
+    cfg.numAttrs = cooperative && grid > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 template <typename... KArgs, typename... Args>

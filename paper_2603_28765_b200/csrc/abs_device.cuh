@@ -411,9 +411,15 @@ __device__ __forceinline__ float one_pass_alpha(const AlphaSrc& a, uint32_t loca
     if (threadIdx.x == 0) {
         uint32_t m = 0u;
         for (int w = 0; w < warps; ++w) m = max(m, warp_max[w]);
-        atomicMax(a.cells + blockIdx.x, ((unsigned long long)a.gen << 32) | m);
+        if (gridDim.x == 1) {            // nothing to exchange (1 x 4096, back to back on a stream: 4.1 -> 2.7 us)
+            alpha_shared = m == 0u ? 1.0f : __fdiv_rn(__uint_as_float(m), a.denom);
+            *a.alpha_out = alpha_shared;
+        } else {
+            atomicMax(a.cells + blockIdx.x, ((unsigned long long)a.gen << 32) | m);
+        }
     }
     __syncthreads();
+    if (gridDim.x == 1) return alpha_shared;
     uint32_t m = 0u;
     bool lost = false;
     for (uint32_t c = threadIdx.x; c < gridDim.x && !lost; c += blockDim.x) {
