@@ -55,7 +55,7 @@ def build_call(force: bool = False) -> str:
     tmp = path + f".tmp{os.getpid()}"
     cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
     cmd += [x for p in inc for x in ("-isystem", p)] + ["-o", tmp, CALL_SOURCES[0], "-L" + os.path.join(root, "lib")]
-    cmd += ["-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10", "-Wl,-rpath," + os.path.join(root, "lib")]
+    cmd += ["-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10", "-Wl,-rpath," + os.path.join(root, "lib")]
     subprocess.run(cmd, check=True)
     os.replace(tmp, path)
     return path
