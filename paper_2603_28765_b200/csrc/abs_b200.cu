@@ -823,18 +823,18 @@ static abs_status_t quantize_transposed_impl(abs_fmt_t fmt, const void* in_bf16,
     uint2* ct = (uint2*)codes_t_u8;
     uint8_t* stp = (uint8_t*)scales_t_e4m3;
     const uint32_t mask = o.had_sign_mask;
-#define ABS_LAUNCH_TE(I, S, R, Q, M, E, SLOT, GEN)                                                                  \
+#define ABS_LAUNCH_TE(I, S, R, Q, E)                                                                                \
     do {                                                                                                            \
-        e = cudaFuncSetAttribute(transposed_kernel<I, S, R, Q, M, E>(), cudaFuncAttributeMaxDynamicSharedMemorySize, \
+        e = cudaFuncSetAttribute(transposed_kernel<I, S, R, Q, E>(), cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                  kTransSmemBytes);                                                                  \
         if (e == cudaSuccess)                                                                                       \
-            e = cudaLaunchKernelEx(&cfg, transposed_kernel<I, S, R, Q, M, E>(), in, ct, stp, src, rows, cols, mask, \
-                                   SLOT, GEN, mul, pk, ctr, (uint16_t*)out_bf16, store_codes);                      \
+            e = cudaLaunchKernelEx(&cfg, transposed_kernel<I, S, R, Q, E>(), in, ct, stp, src, rows, cols, mask, \
+                                   mul, pk, ctr, (uint16_t*)out_bf16, store_codes);                      \
     } while (0)
-#define ABS_LAUNCH_T(I, S, R, Q, M, SLOT, GEN)                                                                      \
+#define ABS_LAUNCH_T(I, S, R, Q)                                                                                    \
     do {                                                                                                            \
-        if (M == 0 && out_bf16) ABS_LAUNCH_TE(I, S, R, Q, 0, true, SLOT, GEN);                                      \
-        else ABS_LAUNCH_TE(I, S, R, Q, M, false, SLOT, GEN);                                                        \
+        if (out_bf16) ABS_LAUNCH_TE(I, S, R, Q, true);                                                              \
+        else ABS_LAUNCH_TE(I, S, R, Q, false);                                                                      \
     } while (0)
 
     const bool sr = o.flags & ABS_F_STOCHASTIC;
@@ -849,9 +849,11 @@ static abs_status_t quantize_transposed_impl(abs_fmt_t fmt, const void* in_bf16,
         if (rs != ABS_OK) return rs;
         const float denom = 6.0f * 448.0f;
         if (rht) {
-            // the maximum is taken over the transformed column groups: same tile walk, MODE 1
-            ABS_LAUNCH_T(false, false, true, false, 1, slot, gen);
-            if (e != cudaSuccess) return ABS_ERR_CUDA;
+            // the maximum is taken over the transformed column groups
+            const int64_t chunks = cols / 4;
+            if (launch_pdl(amax_columns_kernel, grid_for(st->sm_count, rblocks * chunks, kAmaxColumnsBlocks), kThreads, s, (const uint2*)in_bf16, rblocks, chunks,
+                           mask, slot, gen) != cudaSuccess)
+                return ABS_ERR_CUDA;
         } else {
             abs_status_t rc = launch_amax(st->sm_count, in_bf16, ngroups, o, false, slot, gen, tensor_scale_f32, denom, s);
             if (rc != ABS_OK) return rc;
@@ -861,11 +863,10 @@ static abs_status_t quantize_transposed_impl(abs_fmt_t fmt, const void* in_bf16,
         src.denom = denom;
         src.overrun = st->overrun_dev;
     }
-    unsigned long long* no_slot = nullptr;
 #define ABS_LAUNCH_T2(I, R, Q)                                                                                      \
     do {                                                                                                            \
-        if (src.slot) ABS_LAUNCH_T(I, true, R, Q, 0, no_slot, 0u);                                                  \
-        else ABS_LAUNCH_T(I, false, R, Q, 0, no_slot, 0u);                                                          \
+        if (src.slot) ABS_LAUNCH_T(I, true, R, Q);                                                                  \
+        else ABS_LAUNCH_T(I, false, R, Q);                                                                           \
     } while (0)
 #define ABS_LAUNCH_T3(I)                                                                                            \
     do {                                                                                                            \

@@ -60,25 +60,21 @@ __device__ __forceinline__ void hadamard16_pairs(float (&x)[16], uint32_t sign_m
     for (int i = 0; i < 8; ++i) unpack2(mul2(P[i], QUARTER), x[2 * i], x[2 * i + 1]);
 }
 
-// MODE 0: quantize.  MODE 1: only the maximum of the Hadamard-transformed column groups (the amax pass of
-// the transposed path with the Hadamard option; publishes a tagged maximum like amax_kernel).
 // SR: stochastic rounding of both candidates (App. B); element indices, and so the Philox counters, are
 // those of the transposed matrix.  scale_mul is 17/16 with that option and 1 otherwise.
-// EMUL (MODE 0 only): the emulation pass of Sec. 4.1 along the columns.  Every group is decoded from the
+// EMUL: the emulation pass of Sec. 4.1 along the columns.  Every group is decoded from the
 // registers that hold its codes and written back over its own input values in the shared-memory tile; the
 // finished tile then leaves with coalesced 16-byte stores to `out`, a [rows, cols] matrix in the ORIGINAL
 // orientation.  Codes and scales (transposed layout) are stored only when `store_codes` is set.
-template <bool HAS_INT, bool FROM_SLOT, bool RHT, bool SR, int MODE, bool EMUL>
+template <bool HAS_INT, bool FROM_SLOT, bool RHT, bool SR, bool EMUL>
 __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __restrict__ in, uint2* __restrict__ codes_t,
                                                           uint8_t* __restrict__ scales_t, const AlphaSrc alpha_src,
                                                           int64_t rows, int64_t cols, uint32_t sign_mask,
-                                                          unsigned long long* amax_slot, uint32_t amax_gen,
                                                           float scale_mul, const PhiloxKeys& keys,
                                                           uint64_t ctr_base, uint16_t* __restrict__ out,
                                                           bool store_codes) {
     extern __shared__ __align__(16) uint16_t trans_smem[];
     pdl_launch_dependents();
-    uint32_t local_max = 0u;
     const int64_t rblocks = rows / 16;
     const int64_t ntx = (cols + kTransTileCols - 1) / kTransTileCols;
     const int64_t nty = (rblocks + kTransTileRowBlocks - 1) / kTransTileRowBlocks;
@@ -132,11 +128,8 @@ __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __rest
     }
     pdl_wait();
     issue(t, ty, tx, 0);                             // its copies are on their way while alpha is read
-    float alpha = 1.0f, inv_a6 = 1.0f;
-    if constexpr (MODE == 0) {
-        alpha = resolve_alpha<FROM_SLOT>(alpha_src);                         // T2
-        inv_a6 = __frcp_rn(__fmul_rn(alpha, 6.0f));                          // T3
-    }
+    const float alpha = resolve_alpha<FROM_SLOT>(alpha_src);                 // T2
+    const float inv_a6 = __frcp_rn(__fmul_rn(alpha, 6.0f));                  // T3
     for (; t < ntiles; t += gridDim.x, s ^= 1) {
         uint32_t ty_next = ty + step_y, tx_next = tx + step_x;
         if (tx_next >= ntx32) { tx_next -= ntx32; ++ty_next; }
@@ -165,11 +158,6 @@ __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __rest
 #pragma unroll
                 for (int i = 0; i < 16; ++i) x[i] = __uint_as_float((uint32_t)colp[i * kTransTileCols] << 16);
                 if constexpr (RHT) hadamard16_pairs(x, sign_mask);   // along the group, i.e. down the column
-                if constexpr (MODE == 1) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) local_max = max(local_max, __float_as_uint(x[i]) & 0x7FFFFFFFu);
-                    continue;
-                }
                 const float m0 = max3abs(x[0], x[1], x[2]), m1 = max3abs(x[3], x[4], x[5]);
                 const float m2 = max3abs(x[6], x[7], x[8]), m3 = max3abs(x[9], x[10], x[11]);
                 const float m4 = max3abs(x[12], x[13], x[14]);
@@ -223,7 +211,7 @@ __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __rest
                     codes_t[g] = make_uint2(c_lo, c_hi);
                 }
             }
-            if (MODE == 0 && vec && (!EMUL || store_codes)) {
+            if (vec && (!EMUL || store_codes)) {
                 const int64_t g0 = (c0 + c) * rblocks + rb0;
                 store32B<true>(codes_t + g0, reinterpret_cast<const uint32_t(&)[8]>(cw));
                 *reinterpret_cast<uint32_t*>(scales_t + g0) = sbytes;
@@ -245,49 +233,111 @@ __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __rest
         ty = ty_next;
         tx = tx_next;
     }
-    if constexpr (MODE == 1) {
-        __shared__ uint32_t warp_max[8];
-        local_max = __reduce_max_sync(0xFFFFFFFFu, local_max);
-        if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = local_max;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t m = 0u;
-#pragma unroll
-            for (int w = 0; w < 8; ++w) m = max(m, warp_max[w]);
-            atomicMax(amax_slot, ((unsigned long long)amax_gen << 32) | m);
+}
+
+// The amax pass of the transposed path with the Hadamard option: the maximum of the transformed column groups, published like amax_kernel's.  Bound by
+// memory: a thread reads 16 rows of four columns, 8 bytes at a time (256 contiguous bytes per warp and row), the butterflies run on
+// pairs of columns (h = 1, 2, 4, 8, packed add and fused subtract, the arithmetic of hadamard16_pairs), and 1/4 is applied to the maximum alone.
+// us, as the tile walk of the quantize kernel and as this: 8192 x 14336 45.5 / 37.6 (6.25 TB/s), 8192 x 4096 17.6 / 13.5, 4096 x 4096 10.9 / 7.6, 2048 x 4096 7.5 / 4.9.
+// Three blocks per SM and no more of them: four (64 registers) spill, 46.7 us; several waves 38.4 - 39.7.
+constexpr int kAmaxColumnsBlocks = 3;
+__global__ void __launch_bounds__(256, kAmaxColumnsBlocks)
+amax_columns_kernel(const uint2* __restrict__ in, int64_t rblocks, int64_t chunks, uint32_t sign_mask, unsigned long long* __restrict__ slot, uint32_t gen) {
+    pdl_launch_dependents();
+    // item i: row block i / chunks, columns 4 (i % chunks) ..; a thread's items are i, i + stride, ...
+    const int64_t items = rblocks * chunks, stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t step_y = stride / chunks, step_x = stride - step_y * chunks;
+    int64_t y = i / chunks, x = i - y * chunks;
+    {   // before the wait (see prefetch_l2): a line of 128 bytes of one of the 16 rows per thread, two lines per warp and row
+        const int64_t first = i - (threadIdx.x & 31) + 16 * (threadIdx.x & 1);
+        if (first < items) {
+            const int64_t fy = first / chunks;
+            prefetch_l2(in + (fy * 16 + (threadIdx.x >> 1 & 15)) * chunks + (first - fy * chunks));
         }
+    }
+    pdl_wait();
+    const uint64_t NEG1 = pack2(-1.0f, -1.0f);
+    float m0 = 0.0f, m1 = 0.0f;
+    for (; i < items; i += stride) {
+        const uint2* at = in + y * 16 * chunks + x;
+        uint2 w[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) w[r] = __ldg(at + r * chunks);
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            uint64_t P[16];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const uint32_t v = (half ? w[r].y : w[r].x) ^ ((sign_mask >> r & 1u) ? 0x80008000u : 0u);
+                P[r] = pack2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
+            }
+#pragma unroll
+            for (int h = 1; h < 16; h <<= 1) {
+#pragma unroll
+                for (int base = 0; base < 16; base += 2 * h) {
+#pragma unroll
+                    for (int j = base; j < base + h; ++j) {
+                        const uint64_t p = P[j], q = P[j + h];
+                        P[j] = add2(p, q);
+                        P[j + h] = fma2(q, NEG1, p);
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < 16; r += 2) {
+                float a, b, c, d;
+                unpack2(P[r], a, b);
+                unpack2(P[r + 1], c, d);
+                m0 = max3abs(m0, a, b);
+                m1 = max3abs(m1, c, d);
+            }
+        }
+        y += step_y;
+        x += step_x;
+        if (x >= chunks) { x -= chunks; ++y; }
+    }
+    uint32_t local = __float_as_uint(__fmul_rn(fmaxf(m0, m1), 0.25f));
+    __shared__ uint32_t warp_max[8];
+    local = __reduce_max_sync(0xFFFFFFFFu, local);
+    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = local;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t m = 0u;
+#pragma unroll
+        for (int v = 0; v < 8; ++v) m = max(m, warp_max[v]);
+        atomicMax(slot, ((unsigned long long)gen << 32) | m);
     }
 }
 
 #define ABS_TRANS_PARAMS                                                                                              \
     const uint16_t *__restrict__ in, uint2 *__restrict__ codes_t, uint8_t *__restrict__ scales_t,                     \
-        const AlphaSrc alpha_src, int64_t rows, int64_t cols, uint32_t sign_mask, unsigned long long *amax_slot,      \
-        uint32_t amax_gen, float scale_mul, const PhiloxKeys keys, uint64_t ctr_base,                                   \
+        const AlphaSrc alpha_src, int64_t rows, int64_t cols, uint32_t sign_mask, float scale_mul, const PhiloxKeys keys, uint64_t ctr_base,                                   \
         uint16_t *__restrict__ out, bool store_codes
 #define ABS_TRANS_ARGS                                                                                                \
-    in, codes_t, scales_t, alpha_src, rows, cols, sign_mask, amax_slot, amax_gen, scale_mul, keys,                    \
+    in, codes_t, scales_t, alpha_src, rows, cols, sign_mask, scale_mul, keys,                    \
         ctr_base, out, store_codes
 
 // Round-to-nearest and Hadamard instances are held to the registers of three blocks per SM (what the shared
 // memory allows): left alone the compiler takes up to 124 and only two blocks fit.
-template <bool HAS_INT, bool FROM_SLOT, bool RHT, int MODE, bool EMUL>
+template <bool HAS_INT, bool FROM_SLOT, bool RHT, bool EMUL>
 __global__ void __launch_bounds__(256, 3) quantize4_transposed_kernel(ABS_TRANS_PARAMS) {
-    quantize4_transposed_body<HAS_INT, FROM_SLOT, RHT, false, MODE, EMUL>(ABS_TRANS_ARGS);
+    quantize4_transposed_body<HAS_INT, FROM_SLOT, RHT, false, EMUL>(ABS_TRANS_ARGS);
 }
 // The stochastic-rounding instances measured 3-7 % faster with the compiler's own register choice (about 80,
 // no spills) than held to three or to two blocks per SM.
-template <bool HAS_INT, bool FROM_SLOT, bool RHT, int MODE, bool EMUL>
+template <bool HAS_INT, bool FROM_SLOT, bool RHT, bool EMUL>
 __global__ void __launch_bounds__(256) quantize4_transposed_sr_kernel(ABS_TRANS_PARAMS) {
-    quantize4_transposed_body<HAS_INT, FROM_SLOT, RHT, true, MODE, EMUL>(ABS_TRANS_ARGS);
+    quantize4_transposed_body<HAS_INT, FROM_SLOT, RHT, true, EMUL>(ABS_TRANS_ARGS);
 }
 #undef ABS_TRANS_PARAMS
 #undef ABS_TRANS_ARGS
 
 // The kernel instance for a set of options (both wrappers have the same signature).
-template <bool HAS_INT, bool FROM_SLOT, bool RHT, bool SR, int MODE, bool EMUL>
+template <bool HAS_INT, bool FROM_SLOT, bool RHT, bool SR, bool EMUL>
 constexpr auto transposed_kernel() {
-    if constexpr (SR) return &quantize4_transposed_sr_kernel<HAS_INT, FROM_SLOT, RHT, MODE, EMUL>;
-    else return &quantize4_transposed_kernel<HAS_INT, FROM_SLOT, RHT, MODE, EMUL>;
+    if constexpr (SR) return &quantize4_transposed_sr_kernel<HAS_INT, FROM_SLOT, RHT, EMUL>;
+    else return &quantize4_transposed_kernel<HAS_INT, FROM_SLOT, RHT, EMUL>;
 }
 
 }  // namespace absq
