@@ -26,7 +26,7 @@
 // the copy engine brings 110 bytes per cycle and SM, and the tensor core queues two MMAs: what used to take 93 cycles per MMA was the issuing thread,
 // busy for 470 cycles between the MMAs of two steps.  Operands and split included, back to back: IF4 2048 x 4096 x 4096 72.2 -> 64.2
 // us, 1000 x 14336 x 4096 133 -> 122 us, 8192 x 14336 x 4096 845 -> 787 us.  (Nine MMAs per K-block: 1440 us for the largest.)  NVFP4 26.8, 45.6 and
-// 324 us: its issuing thread is as it was (see there).
+// 324 us one tile at a time; such products take their tiles in pairs (abs_pair.cuh).
 #include "../../include/abs_b200.h"
 #include "abs_tc.cuh"
 #include "abs_rows.cuh"
@@ -53,14 +53,14 @@ constexpr int kSfBufs = 3, kScaleBoxBytes = kTileM * (kStageK / 16);
 template <int PLANES> constexpr int kSfRingBytes = PLANES == 2 ? kSfBufs * 2 * kScaleBoxBytes : 0;
 // Epilogue warps: IF4, whose accumulators fill the tensor memory, takes eight, two per quarter of the accumulator lanes,
 // that have everything in registers before they store (the MMAs of the next tile wait only for that); NVFP4 has two sets
-// of accumulators and streams each through four warps.  Staging: a warp turns 16 rows x 128 bytes (IF4) or 32 rows x 128
-// bytes (NVFP4) of output at a time through shared memory, rows 144 bytes apart: 16-byte aligned and free of bank
-// conflicts for 128-bit accesses both ways.
+// of accumulators and streams each through four warps.  A thread stores the columns of its row 32 bytes at a time, whole sectors, straight from its
+// registers (store_columns16).  Turned through shared memory, so that an instruction writes four rows of 128 bytes, the products took longer: IF4 100 x
+// 4096 x 512 8.0 -> 7.3 us, 2048 x 4096 x 4096 57.3 -> 56.0, 4096 x 4096 x 512 24.4 -> 22.3, FP32 27.8 -> 25.0, at the power cap 8192 x 14336 x 4096 791 -> 779;
+// NVFP4 300 x 4096 x 4096 11.4 -> 11.0, 1000 x 4096 x 1024 8.8 -> 8.2, FP32 9.3 -> 8.6.
 template <int PLANES> constexpr int kEpiWarps = PLANES == 2 ? 8 : 4;
 template <int PLANES> constexpr int kGemmThreads = 32 * (2 + kEpiWarps<PLANES> + 4);
-constexpr int kStagePitch = 36, kStagingBytes = 4 * 32 * kStagePitch * 4;
 template <int PLANES, int KBOXES> constexpr int kGemmSmemBytes =
-    kStages<PLANES, KBOXES> * kStageBytes<PLANES, KBOXES> + kSfRingBytes<PLANES> + 1024 /* alignment slack */ + 512 /* barriers */ + kStagingBytes;
+    kStages<PLANES, KBOXES> * kStageBytes<PLANES, KBOXES> + kSfRingBytes<PLANES> + 1024 /* alignment slack */ + 512 /* barriers */;
 
 // ----------------------------------------------------------------------------- operand split
 
@@ -416,7 +416,8 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
         const int quarter = warp & 3;
         const float scale = __fmul_rn(__ldg(alpha_a), __ldg(alpha_b));
         uint32_t j = 0;
-        uint32_t out_max = 0u;                  // bf16 output with next_alpha: largest |C| bit pattern this thread has written
+        uint32_t out_max = 0u;                  // bf16 output with next_alpha: largest |C| bit patterns this thread has written (see store_columns16)
+        const bool out_aligned32 = (reinterpret_cast<uintptr_t>(c_out) & 31u) == 0;
         bool all_tiles = true;
         if constexpr (PLANES == 2) {
             // Two warps per quarter of tensor memory; a warp owns the accumulator lanes (rows of the tile) 32 (w % 4) ..
@@ -424,15 +425,12 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
             // back, and only then stores.
             constexpr int kCols = kTileN / 2;
             const int col0 = ((warp - 2) >> 2) * kCols;
-            uint32_t* staging = reinterpret_cast<uint32_t*>(gemm_smem_raw + (bars - raw) + 512) + (warp - 2) * 16 * kStagePitch;
             const float c1 = __uint_as_float(0x3E124925u), c2 = __uint_as_float(0x3CA72F05u);      // fp32(1/7), fp32(1/49)
             for (int32_t t = blockIdx.x; t < num_tiles && all_tiles; t += gridDim.x) {
                 int32_t tile_m, tile_n;
                 tile_of(t, tiles_m, tiles_n, tile_m, tile_n);
                 const bool own_row_valid = tile_m * kTileM + quarter * 32 + lane < m_rows;   // the row whose values this thread holds
-                // this thread's part of every store: row (lane / 8) of each group of four rows, 16 bytes at byte 16 (lane % 8)
-                const int32_t row0 = tile_m * kTileM + quarter * 32 + (lane >> 3);
-                const size_t first = (size_t)row0 * (size_t)n_cols + (size_t)tile_n * kTileN + col0;
+                const size_t first = (size_t)(tile_m * kTileM + quarter * 32 + lane) * (size_t)n_cols + (size_t)tile_n * kTileN + col0;
                 float v[kCols];
                 for (int32_t k0 = 0; k0 < k_iters; k0 += kChunkSteps, ++j) {
                     const uint32_t buf = j % kAccBufs;
@@ -469,44 +467,13 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
                     if (lane == 0) mbar_arrive(acc_empty0 + 8 * buf);    // the MMAs of the next chunk or tile may start
                 }
                 if (!all_tiles) break;
-                // A thread holds 64 columns of ONE row; stored as they are, every store instruction of the warp would touch
-                // 32 different rows.  Through shared memory each instruction writes four rows of 128 contiguous bytes.
-                constexpr int kPart = OUT_BF16 ? 64 : 32;                 // columns of 128 bytes
+                if (own_row_valid) {
 #pragma unroll
-                for (int part = 0; part < kCols / kPart; ++part) {
-                    uint32_t pk[32];
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        if constexpr (OUT_BF16) {
-                            pk[e] = bf16x2_bits(__fmul_rn(v[2 * e], scale), __fmul_rn(v[2 * e + 1], scale));
-                            if (next_alpha != nullptr && own_row_valid) out_max = max(out_max, max(pk[e] & 0x7FFFu, (pk[e] >> 16) & 0x7FFFu));
-                        } else {
-                            pk[e] = __float_as_uint(__fmul_rn(v[part * kPart + e], scale));
-                        }
-                    }
-#pragma unroll 1
-                    for (int h = 0; h < 2; ++h) {                          // rows 16 h .. 16 h + 15 of the warp's 32
-                        if ((lane >> 4) == h) {
-#pragma unroll
-                            for (int q = 0; q < 8; ++q) *reinterpret_cast<uint4*>(staging + (lane & 15) * kStagePitch + 4 * q) = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-                        }
-                        __syncwarp();
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const uint4 x = *reinterpret_cast<const uint4*>(staging + (4 * i + (lane >> 3)) * kStagePitch + 4 * (lane & 7));
-                            if (row0 + 16 * h + 4 * i < m_rows) {          // the last row block may be partial
-                                const size_t at = first + (size_t)(16 * h + 4 * i) * n_cols + part * kPart;
-                                if constexpr (OUT_BF16) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(c_out) + at + 8 * (lane & 7)) = x;
-                                else *reinterpret_cast<uint4*>(reinterpret_cast<float*>(c_out) + at + 4 * (lane & 7)) = x;
-                            }
-                        }
-                        __syncwarp();
-                    }
+                    for (int q = 0; q < kCols / 16; ++q) store_columns16<OUT_BF16>(c_out, first + 16 * q, v + 16 * q, scale, out_aligned32, next_alpha != nullptr, out_max);
                 }
             }
         } else {
             // A warp owns the accumulator lanes (rows of the tile) 32 (w % 4) .. 32 (w % 4) + 31.
-            float* staging = reinterpret_cast<float*>(gemm_smem_raw + (bars - raw) + 512) + (warp - 2) * 32 * kStagePitch;
             for (int32_t t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
                 int32_t tile_m, tile_n;
                 tile_of(t, tiles_m, tiles_n, tile_m, tile_n);
@@ -517,12 +484,7 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
                 if (!have) { all_tiles = false; break; }
                 tc_fence_after();
                 const bool own_row_valid = tile_m * kTileM + quarter * 32 + lane < m_rows;   // the row whose values this thread holds
-                // this thread's part of every store.  FP32: row (lane / 8) of each group of four rows, 16 bytes at column
-                // 4 (lane % 8); bf16: row (lane / 4) of each group of eight rows, 16 bytes at column 8 (lane % 4)
-                const int32_t row0 = tile_m * kTileM + quarter * 32 + (OUT_BF16 ? (lane >> 2) : (lane >> 3));
-                float* out = reinterpret_cast<float*>(c_out) + (size_t)row0 * (size_t)n_cols + (size_t)tile_n * kTileN + 4 * (lane & 7);
-                __nv_bfloat16* out16 = reinterpret_cast<__nv_bfloat16*>(c_out) + (size_t)row0 * (size_t)n_cols + (size_t)tile_n * kTileN +
-                                       8 * (lane & 3);
+                const size_t first = (size_t)(tile_m * kTileM + quarter * 32 + lane) * (size_t)n_cols + (size_t)tile_n * kTileN;
                 const uint32_t lane_base = tmem + buf * kTileN + ((uint32_t)(quarter * 32) << 16);
                 for (int chunk = 0; chunk < kTileN / 32; ++chunk) {
                     uint32_t r0[32];
@@ -535,51 +497,19 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
                     }
                     float v[32];
 #pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) v[jj] = __fmul_rn(__uint_as_float(r0[jj]), scale);
-                    // A thread holds 32 columns of ONE row; stored as they are, every store instruction of the warp would
-                    // touch 32 different rows.  Through shared memory each instruction writes four rows of 128 contiguous bytes.
-                    if constexpr (!OUT_BF16) {
+                    for (int jj = 0; jj < 32; ++jj) v[jj] = __uint_as_float(r0[jj]);
+                    if (own_row_valid) {
 #pragma unroll
-                        for (int jj = 0; jj < 32; jj += 4)
-                            *reinterpret_cast<float4*>(staging + lane * kStagePitch + jj) = make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
-                        __syncwarp();
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const float4 x = *reinterpret_cast<const float4*>(staging + (4 * i + (lane >> 3)) * kStagePitch + 4 * (lane & 7));
-                            if (row0 + 4 * i < m_rows)                      // the last row block may be partial
-                                *reinterpret_cast<float4*>(out + (size_t)(4 * i) * n_cols + chunk * 32) = x;
-                        }
-                    } else {
-                        // 32 bf16 = 64 bytes per row, rows 20 words apart; a store instruction writes eight rows of 64 bytes
-                        uint32_t* stg = reinterpret_cast<uint32_t*>(staging);
-#pragma unroll
-                        for (int jj = 0; jj < 32; jj += 8) {
-                            uint4 pk;
-                            pk.x = bf16x2_bits(v[jj], v[jj + 1]); pk.y = bf16x2_bits(v[jj + 2], v[jj + 3]);
-                            pk.z = bf16x2_bits(v[jj + 4], v[jj + 5]); pk.w = bf16x2_bits(v[jj + 6], v[jj + 7]);
-                            *reinterpret_cast<uint4*>(stg + lane * 20 + jj / 2) = pk;
-                            if (next_alpha != nullptr && own_row_valid) {
-                                const uint32_t w4[4] = {pk.x, pk.y, pk.z, pk.w};
-#pragma unroll
-                                for (int q = 0; q < 4; ++q) out_max = max(out_max, max(w4[q] & 0x7FFFu, (w4[q] >> 16) & 0x7FFFu));
-                            }
-                        }
-                        __syncwarp();
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const uint4 x = *reinterpret_cast<const uint4*>(stg + (8 * i + (lane >> 2)) * 20 + 4 * (lane & 3));
-                            if (row0 + 8 * i < m_rows)
-                                *reinterpret_cast<uint4*>(out16 + (size_t)(8 * i) * n_cols + chunk * 32) = x;
-                        }
+                        for (int q = 0; q < 2; ++q)
+                            store_columns16<OUT_BF16>(c_out, first + chunk * 32 + 16 * q, v + 16 * q, scale, out_aligned32, next_alpha != nullptr, out_max);
                     }
-                    __syncwarp();
                 }
             }
         }
         // The global maximum of |C| as written (bf16), for the next quantizer's tensor scale (Eq. 1): every epilogue
         // warp publishes its maximum with an atomic and takes a ticket; the last of all warps converts and writes alpha.
         if (OUT_BF16 && next_alpha != nullptr && all_tiles) {
-            const uint32_t wmax = __reduce_max_sync(0xFFFFFFFFu, out_max);
+            const uint32_t wmax = __reduce_max_sync(0xFFFFFFFFu, max(out_max & 0xFFFFu, out_max >> 16));
             if (lane == 0) {
                 atomicMax(reinterpret_cast<unsigned int*>(error) + 1, wmax);
                 __threadfence();
@@ -741,18 +671,17 @@ bool rows_rule(abs_fmt_t fmt, int64_t m, int64_t n, int64_t k, int sm_count) {
         return (m <= 4 && chunks <= 10 && 2 * turns < 3 * warps) || 10 * kRowsChunk * turns * chunks * chunks <= (m <= 4 ? 43 : 30) * warps * k;
     return m <= 4 || k % (2 * kStageK) != 0 || n * chunks <= (int64_t)kTileN * sm_count;
 }
-// NVFP4: which products take their tiles in pairs (abs_pair.cuh) and not one by one.  More than one round of tiles, and what pairs save has to outweigh
-// that the last round is one of pairs or of single tiles: bf16 from one and a quarter rounds on, FP32, whose stores take longer, from three; with
-// K >= 3072 always.  One by one / in pairs, us, bf16 and FP32: 257 x 8192 x 256 (192 tiles) 7.4 / 6.9, 7.9 / 7.4; 1000 x 4096 x 512 (256) 7.8 / 7.6, 8.2 / 8.7;
-// 300 x 14336 x 2048 (336) 14.1 / 13.6, 14.9 / 15.4; 2048 x 4096 x 512 (512) 10.9 / 9.8, 11.9 / 11.6; 600 x 4096 x 1024 (160) 8.6 / 8.5, 9.1 / 9.2;
-// 600 x 4096 x 4096 15.6 / 14.5, 16.0 / 15.2; 1000 x 14336 x 4096 41.9 / 36.3, 54.4 / 44.4; back to back for longer, at the power cap, 8192 x 14336 x 4096
-// 321 / 274, 388 / 326.
-// An odd number of tile columns leaves pairs of one tile; where the rounds then are a sixth longer (FP32: at all), tiles go one by one.
+// NVFP4: which products take their tiles in pairs (abs_pair.cuh) and not one by one: those that need no more rounds so (an odd number of tile columns leaves
+// pairs of one tile, and the last round is one of pairs or of single tiles), with more than one round and a long K, where the feed counts, or with three
+// rounds or more, where the overlap of the ends does too (FP32, whose stores weigh more, from K = 1024 on).  One by one / in pairs, us, bf16 and FP32:
+// 600 x 4096 x 1024 (160 tiles) 8.0 / 8.6, 8.5 / 9.1; 1000 x 4096 x 2048 (256) 10.7 / 10.8, 11.1 / 11.5; 1000 x 4096 x 3072 12.9 / 12.6, 13.9 / 13.4; 300 x 14336 x
+// 1024 (336) 10.0 / 10.1, 10.6 / 11.5; 2048 x 4096 x 512 (512) 9.7 / 9.5, 11.3 / 11.5; 2048 x 4096 x 2048 15.9 / 15.3, 17.9 / 17.3; 1000 x 14336 x 256 (896)
+// 12.5 / 11.4, 15.3 / 15.9; 1000 x 14336 x 1024 16.6 / 15.6, 20.1 / 19.5; 3000 x 4736 x 2048 (888; six rounds or seven) 21.1 / 22.6, 25.0 / 27.7; back to back for
+// longer, at the power cap, 8192 x 14336 x 4096 321 / 274, 388 / 326.
 bool pair_rule(bool out_bf16, int64_t tiles_m, int64_t tiles_n, int64_t k, int sm_count) {
     const int64_t tiles = tiles_m * tiles_n, pairs = tiles_m * ((tiles_n + 1) / 2), rest = pairs % sm_count;
-    if (tiles <= sm_count || (k < 3072 && (out_bf16 ? 4 * tiles < 5 * (int64_t)sm_count : tiles < 3 * (int64_t)sm_count))) return false;
-    const int64_t one_by_one = (tiles + sm_count - 1) / sm_count, in_pairs = pairs / sm_count * 2 + (rest == 0 ? 0 : 2 * rest <= sm_count ? 1 : 2);
-    return out_bf16 ? 6 * in_pairs <= 7 * one_by_one : in_pairs <= one_by_one;
+    if (tiles <= sm_count || (k < 3072 && (tiles < 3 * (int64_t)sm_count || !(out_bf16 || k >= 1024)))) return false;
+    return pairs / sm_count * 2 + (rest == 0 ? 0 : 2 * rest <= sm_count ? 1 : 2) <= (tiles + sm_count - 1) / sm_count;
 }
 typedef void (*RowsKernel)(RowsArgs);
 template <int M> RowsKernel rows_kernel_for(bool has_int, bool out_bf16) {

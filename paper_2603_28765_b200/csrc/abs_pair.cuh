@@ -10,8 +10,7 @@
 // warps, its `empty` barrier frees its shared memory and its slot of scales.  A step, eight MMAs of 64 cycles, takes some 750 cycles (1130 for eight MMAs in
 // if4_gemm_kernel<1>); waiting for the next step's operands before the last MMAs of a step, as the IF4 loop does, made it 10 % slower: with two slots
 // the next step's scales come after the MMAs of the step before.
-// The epilogue stores 32 bytes of its row per thread as they come from tensor memory, whole sectors (turned through shared memory for whole
-// lines the bf16 products took 2 - 18 % longer, most with a short K).
+// The epilogue stores as in if4_gemm_kernel (turned through shared memory for whole lines, bf16 products took 2 - 18 % longer, most with a short K).
 // 1000 x 14336 x 4096, bf16, 41.9 -> 36.3 us, 2048 x 4096 x 4096 27.4 -> 23.5, 4096^3 42.0 -> 36.2; at the power cap 8192 x 14336 x 4096 321 -> 274 (FP32 388 -> 326),
 // 2048 x 8192 x 14336 161 -> 132.  The results are those of if4_gemm_kernel<1>, bit for bit.
 #pragma once
@@ -261,26 +260,13 @@ nvfp4_pair_kernel(const __grid_constant__ GemmMaps<1> maps, const float* __restr
                         __syncwarp();
                         if (lane == 0) mbar_arrive(acc_empty0 + 8 * buf);
                     }
+                    float v[32];
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__fmul_rn(__uint_as_float(r[e]), scale));
-                    constexpr int kPieces = OUT_BF16 ? 2 : 4;              // of 32 bytes
+                    for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
+                    if (own_row_valid) {                                   // the last row block may be partial
 #pragma unroll
-                    for (int q = 0; q < kPieces; ++q) {
-                        uint32_t o[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            if constexpr (OUT_BF16) {
-                                o[e] = bf16x2_bits(__uint_as_float(r[16 * q + 2 * e]), __uint_as_float(r[16 * q + 2 * e + 1]));
-                                if (next_alpha != nullptr && own_row_valid) out_max = __vmaxu2(out_max, o[e] & 0x7FFF7FFFu);
-                            } else {
-                                o[e] = r[8 * q + e];
-                            }
-                        }
-                        if (own_row_valid) {                               // the last row block may be partial
-                            uint8_t* to = reinterpret_cast<uint8_t*>(c_out) + (first + chunk * 32) * (OUT_BF16 ? 2 : 4) + 32 * q;
-                            if (out_aligned32) store32B<true>(to, o);
-                            else store32B<false>(to, o);
-                        }
+                        for (int q = 0; q < 2; ++q)
+                            store_columns16<OUT_BF16>(c_out, first + chunk * 32 + 16 * q, v + 16 * q, scale, out_aligned32, next_alpha != nullptr, out_max);
                     }
                 }
                 buf = buf + 1 == kPairAccBufs ? 0u : buf + 1;

@@ -158,6 +158,27 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
+// Sixteen neighbouring columns of a row of C times `scale`, from column index `at` on: 64 (FP32) or 32 (bf16) contiguous bytes of one thread, in whole sectors where C
+// is 32-byte aligned.  keep_max: the larger of out_max and the bf16 magnitudes written, per half word.
+template <bool OUT_BF16>
+__device__ __forceinline__ void store_columns16(void* c_out, size_t at, const float* v, float scale, bool aligned32, bool keep_max, uint32_t& out_max) {
+#pragma unroll
+    for (int q = 0; q < (OUT_BF16 ? 1 : 2); ++q) {
+        uint32_t o[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            if constexpr (OUT_BF16) {
+                o[e] = bf16x2_bits(__fmul_rn(v[2 * e], scale), __fmul_rn(v[2 * e + 1], scale));
+                if (keep_max) out_max = __vmaxu2(out_max, o[e] & 0x7FFF7FFFu);
+            } else {
+                o[e] = __float_as_uint(__fmul_rn(v[8 * q + e], scale));
+            }
+        }
+        uint8_t* const to = reinterpret_cast<uint8_t*>(c_out) + at * (OUT_BF16 ? 2 : 4) + 32 * q;
+        if (aligned32) store32B<true>(to, o);
+        else store32B<false>(to, o);
+    }
+}
 __device__ __forceinline__ void tmem_load_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // 32 lanes x 16 columns of 32 bits: thread t of the warp writes columns c .. c+15 of lane (warp % 4) * 32 + t.
 __device__ __forceinline__ void tmem_store16(uint32_t addr, const uint4& a, const uint4& b, const uint4& c, const uint4& d) {
