@@ -26,10 +26,12 @@ constexpr int kMaxDevices = 64;
 
 // Launch with programmatic stream serialization: the kernel may be scheduled while the previous
 // kernel of the stream drains; every kernel here calls pdl_wait() before its first global access.
-// cooperative: the blocks wait for one another (one_pass_alpha), so all of them have to be resident.  A single block needs no such launch, which costs
-// half a microsecond more on the host (2.45 us instead of 1.93) and lets nothing overlap: such kernels start 4.1 us apart on a stream.
+// together: the blocks wait for one another, so all of them have to be resident: as a cluster (one_cluster_alpha; the grid is at most kMaxCluster blocks) or by a
+// cooperative launch (one_pass_alpha).  A single block needs neither; the latter costs half a microsecond more on the host (2.45 us instead of
+// 1.93) and lets nothing overlap: such kernels start 4.1 us apart on a stream.
+enum Together { kApart, kCooperative, kCluster };
 template <typename... KArgs, typename... Args>
-cudaError_t launch_any(bool cooperative, void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
+cudaError_t launch_any(Together together, void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
@@ -38,15 +40,21 @@ cudaError_t launch_any(bool cooperative, void (*kernel)(KArgs...), int grid, int
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeCooperative;
-    attr[1].val.cooperative = 1;
+    if (together == kCluster) {
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)grid;
+        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    } else {
+        attr[1].id = cudaLaunchAttributeCooperative;
+        attr[1].val.cooperative = 1;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = cooperative && grid > 1 ? 2 : 1;
+    cfg.numAttrs = together != kApart && grid > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
-    return launch_any(false, kernel, grid, block, s, args...);
+    return launch_any(kApart, kernel, grid, block, s, args...);
 }
 // Internal status: a cooperative grid was refused because its blocks do not all fit what the stream may use (a green context, an
 // MPS share: fewer SMs than the device has).  Nothing was enqueued; the call takes the two kernels.
@@ -223,8 +231,16 @@ bool one_pass(int fmt, const abs_opts_t& o, int sm_count, int64_t ngroups, bool 
     }
     return !(o.flags & ABS_F_INDEX64) && ngroups <= (int64_t)grid_for(sm_count < kMaxCells ? sm_count : kMaxCells, ngroups, 1) * kThreads * per_thread;
 }
+// Whether such a call is one cluster: the round-to-nearest 4-bit kernels with up to three groups per thread of it (two groups of 8 blocks' threads: 3.3 us instead of
+// 4.1 - 4.3; three 3.9 instead of 4.2; with four the single cluster's arithmetic takes longer than the exchange through the L2 that it saves).  Calls of
+// two to four blocks keep the cells: their report of an overrun is exercised with such calls.
+bool one_cluster(int fmt, const abs_opts_t& o, int64_t ngroups) {
+    return (fmt == ABS_FMT_NVFP4 || fmt == ABS_FMT_IF4) && !(o.flags & (ABS_F_HADAMARD16 | ABS_F_STOCHASTIC)) && ngroups > 4 * kThreads &&
+           ngroups <= 3 * kMaxCluster * kThreads;
+}
 // Grid of a quantize kernel: see one_pass and grid_waves.
 int quantize_grid(const AlphaSrc& alpha, int sm_count, int64_t ngroups, int resident_per_sm, int target_iters) {
+    if (alpha.cluster) return kMaxCluster;
     if (alpha.cells) return grid_for(sm_count < kMaxCells ? sm_count : kMaxCells, ngroups, 1);
     return grid_waves(sm_count, ngroups, resident_per_sm, target_iters);
 }
@@ -260,7 +276,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
             // fits the L2 (about 100 MB of the 126 MB stay resident behind a streaming read)
             const bool pf = !alpha.slot || ngroups * 32 > (int64_t)96 << 20;
 #define ABS_LAUNCH_F3(IDX, A32, SRC, MUL)                                                                            \
-    e = launch_any(SRC == kOnePass, swz ? quantize4_fast_kernel<kInt, IDX, A32, SRC, MUL, true>                       \
+    e = launch_any(SRC == kOnePass ? kCooperative : SRC == kOneCluster ? kCluster : kApart, swz ? quantize4_fast_kernel<kInt, IDX, A32, SRC, MUL, true>                       \
                                         : quantize4_fast_kernel<kInt, IDX, A32, SRC, MUL, false>, pgrid, kThreads, s, \
                    (const uint4*)in, (uint2*)codes, (uint8_t*)scales, alpha, (IDX)ngroups, gpr, ktiles, pf)
 #define ABS_LAUNCH_F2(IDX, A32, SRC)                                                                                 \
@@ -270,7 +286,8 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
     } while (0)
 #define ABS_LAUNCH_F(IDX, A32)                                                                                       \
     do {                                                                                                             \
-        if (alpha.cells) ABS_LAUNCH_F2(int32_t, A32, kOnePass);      /* few groups: always 32-bit indices */          \
+        if (alpha.cluster) ABS_LAUNCH_F2(int32_t, A32, kOneCluster); /* few groups: always 32-bit indices */          \
+        else if (alpha.cells) ABS_LAUNCH_F2(int32_t, A32, kOnePass);                                                 \
         else if (alpha.slot) ABS_LAUNCH_F2(IDX, A32, kFromSlot);                                                     \
         else ABS_LAUNCH_F2(IDX, A32, kGiven);                                                                        \
     } while (0)
@@ -281,6 +298,10 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
 #undef ABS_LAUNCH_F
 #undef ABS_LAUNCH_F2
 #undef ABS_LAUNCH_F3
+            if (alpha.cluster && e != cudaSuccess) {         // no room for a cluster: as for a cooperative grid
+                cudaGetLastError();
+                return kNotResident;
+            }
             return quantize_launched(e, s);
         }
     }
@@ -292,7 +313,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             cudaError_t e;
 #define ABS_LAUNCH_O(R, S)                                                                                        \
-    e = launch_any(alpha.cells != nullptr, alpha.cells ? quantize4_opt_kernel<kInt, R, S, kOnePass, false>         \
+    e = launch_any(alpha.cells ? kCooperative : kApart, alpha.cells ? quantize4_opt_kernel<kInt, R, S, kOnePass, false>         \
                                            : alpha.slot ? quantize4_opt_kernel<kInt, R, S, kFromSlot, false>       \
                                                         : quantize4_opt_kernel<kInt, R, S, kGiven, false>,         \
                    ogrid, kThreads, s, (const uint4*)in, (uint2*)codes, (uint8_t*)scales, alpha, (int32_t)ngroups, mul, \
@@ -313,7 +334,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             const auto kernel = emul_out ? (alpha.cells ? quantize4_bs8_kernel<kInt, kOnePass, true> : alpha.slot ? quantize4_bs8_kernel<kInt, kFromSlot, true> : quantize4_bs8_kernel<kInt, kGiven, true>)
                                          : (alpha.cells ? quantize4_bs8_kernel<kInt, kOnePass, false> : alpha.slot ? quantize4_bs8_kernel<kInt, kFromSlot, false> : quantize4_bs8_kernel<kInt, kGiven, false>);
-            const cudaError_t e = launch_any(alpha.cells != nullptr, kernel, bgrid, kThreads, s, (const uint4*)in, (uint2*)codes, (uint16_t*)scales, alpha,
+            const cudaError_t e = launch_any(alpha.cells ? kCooperative : kApart, kernel, bgrid, kThreads, s, (const uint4*)in, (uint2*)codes, (uint16_t*)scales, alpha,
                                              (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
             return quantize_launched(e, s);
         }
@@ -326,7 +347,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             const auto kernel = emul_out ? (alpha.cells ? quantize6_fast_kernel<FMT, kOnePass, true> : alpha.slot ? quantize6_fast_kernel<FMT, kFromSlot, true> : quantize6_fast_kernel<FMT, kGiven, true>)
                                          : (alpha.cells ? quantize6_fast_kernel<FMT, kOnePass, false> : alpha.slot ? quantize6_fast_kernel<FMT, kFromSlot, false> : quantize6_fast_kernel<FMT, kGiven, false>);
-            const cudaError_t e = launch_any(alpha.cells != nullptr, kernel, sgrid, kThreads, s, (const uint4*)in, (uint32_t*)codes, (uint8_t*)scales, alpha,
+            const cudaError_t e = launch_any(alpha.cells ? kCooperative : kApart, kernel, sgrid, kThreads, s, (const uint4*)in, (uint32_t*)codes, (uint8_t*)scales, alpha,
                                              (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
             return quantize_launched(e, s);
         }
@@ -340,7 +361,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             const auto kernel = emul_out ? (alpha.cells ? quantize3_fast_kernel<kG, kOnePass, true> : alpha.slot ? quantize3_fast_kernel<kG, kFromSlot, true> : quantize3_fast_kernel<kG, kGiven, true>)
                                          : (alpha.cells ? quantize3_fast_kernel<kG, kOnePass, false> : alpha.slot ? quantize3_fast_kernel<kG, kFromSlot, false> : quantize3_fast_kernel<kG, kGiven, false>);
-            const cudaError_t e = launch_any(alpha.cells != nullptr, kernel, tgrid, kThreads, s, (const uint4*)in, (uint16_t*)codes, (uint8_t*)scales, alpha,
+            const cudaError_t e = launch_any(alpha.cells ? kCooperative : kApart, kernel, tgrid, kThreads, s, (const uint4*)in, (uint16_t*)codes, (uint8_t*)scales, alpha,
                                              (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
             return quantize_launched(e, s);
         }
@@ -625,7 +646,7 @@ abs_status_t abs_quantize_ex(abs_fmt_t fmt, const void* in_bf16, int64_t rows, i
     if (device_state(&st) != ABS_OK) return ABS_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t ngroups = rows * cols / 16;
-    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr};
+    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr, false};
     // the quantize kernel, with src as it then is
     auto quantize = [&]() {
         switch (fmt) {
@@ -648,8 +669,10 @@ abs_status_t abs_quantize_ex(abs_fmt_t fmt, const void* in_bf16, int64_t rows, i
         src.overrun = st->overrun_dev;
         if (one_pass(fmt, o, st->sm_count, ngroups, false)) {
             src.cells = st->cells + (size_t)(gen % ABS_MAX_INFLIGHT) * kMaxCells;
+            src.cluster = one_cluster(fmt, o, ngroups);
             if ((rc = quantize()) != kNotResident) return rc;
             src.cells = nullptr;
+            src.cluster = false;
         }
         rc = launch_amax(st->sm_count, in_bf16, ngroups, o, false, slot, gen, tensor_scale_f32, src.denom, s);
         if (rc != ABS_OK) return rc;
@@ -692,7 +715,7 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
     const bool rht = o.flags & ABS_F_HADAMARD16, sr = o.flags & ABS_F_STOCHASTIC;
     const int grid = grid_waves(st->sm_count, ngroups, opt_blocks_per_sm(sr, rht), (rht || sr) ? kOptIters : kFastIters);
     if (ngroups >= (int64_t)0x7FFFFFFF - (int64_t)grid * kThreads) return ABS_ERR_SIZE;    // 32-bit group indices only
-    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr};
+    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr, false};
     const bool store = codes_u8 != nullptr;
     const float mul = (o.flags & ABS_F_SR_SCALE_17_16) ? 1.0625f : 1.0f;
     const uint64_t ctr = o.sr_index_offset / 8;
@@ -716,7 +739,7 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
         cudaError_t e = cudaSuccess;
         const int egrid = quantize_grid(src, st->sm_count, ngroups, opt_blocks_per_sm(sr, rht), (rht || sr) ? kOptIters : kFastIters);
 #define ABS_LAUNCH_E2(I, R, S)                                                                                      \
-        e = launch_any(src.cells != nullptr, src.cells ? quantize4_opt_kernel<I, R, S, kOnePass, true>                   \
+        e = launch_any(src.cells ? kCooperative : kApart, src.cells ? quantize4_opt_kernel<I, R, S, kOnePass, true>                   \
                                              : src.slot ? quantize4_opt_kernel<I, R, S, kFromSlot, true>                 \
                                                         : quantize4_opt_kernel<I, R, S, kGiven, true>, egrid, kThreads, s, \
                        (const uint4*)in_bf16, (uint2*)codes_u8, (uint8_t*)scales_e4m3, src, (int32_t)ngroups, mul,        \
@@ -841,7 +864,7 @@ static abs_status_t quantize_transposed_impl(abs_fmt_t fmt, const void* in_bf16,
     const float mul = (o.flags & ABS_F_SR_SCALE_17_16) ? 1.0625f : 1.0f;
     const uint64_t ctr = o.sr_index_offset / 8;
     const PhiloxKeys pk = philox_keys(o.sr_seed);
-    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr};
+    AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr, false};
     if (!(o.flags & ABS_F_ALPHA_GIVEN)) {
         unsigned long long* slot = nullptr;
         uint32_t gen = 0;
@@ -917,7 +940,7 @@ abs_status_t abs_quantize_noalloc(abs_fmt_t fmt, const void* in_bf16, int64_t ro
                                                         fmt_mfp((int)fmt) * 448.0f);
     if (cudaGetLastError() != cudaSuccess) return ABS_ERR_CUDA;
     const abs_opts_t o = {0, 0, 0, 0, 0};
-    const AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr};   // alpha was written by the chunked pass
+    const AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr, false};   // alpha was written by the chunked pass
     switch (fmt) {
         case ABS_FMT_NVFP4: return launch_quantize_fmt<0>(na.sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
         case ABS_FMT_IF4: return launch_quantize_fmt<1>(na.sm_count, in_bf16, ngroups, codes_u8, scales_e4m3, src, o, s, cols);
