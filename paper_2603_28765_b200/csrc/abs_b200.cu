@@ -156,8 +156,8 @@ int grid_for(int sm_count, int64_t work_items, int blocks_per_sm) {
 // amortise the prologue and keep the prefetch running; several waves let blocks that start later overlap
 // their first loads with the arithmetic of the others (measured: about seven items per thread is best for
 // the IF4 kernel, 10 % faster than one wave of long-running blocks).
-int grid_waves(int sm_count, int64_t work_items, int resident_per_sm, int target_iters) {
-    const int64_t want = (work_items + kThreads - 1) / kThreads;
+int grid_waves(int sm_count, int64_t work_items, int resident_per_sm, int target_iters, int threads = kThreads) {
+    const int64_t want = (work_items + threads - 1) / threads;
     const int64_t resident = (int64_t)sm_count * resident_per_sm;
     if (want <= resident) return (int)(want < 1 ? 1 : want);
     int64_t waves = (want + (int64_t)target_iters * resident / 2) / ((int64_t)target_iters * resident);
@@ -225,7 +225,7 @@ bool one_pass(int fmt, const abs_opts_t& o, int sm_count, int64_t ngroups, bool 
     const bool rht = o.flags & ABS_F_HADAMARD16, sr = o.flags & ABS_F_STOCHASTIC;
     int per_thread = 0;
     switch (fmt) {
-        case ABS_FMT_NVFP4: case ABS_FMT_IF4: per_thread = (rht || sr || emulate) ? opt_blocks_per_sm(sr, rht) : kFastMinBlocks; break;
+        case ABS_FMT_NVFP4: case ABS_FMT_IF4: per_thread = (rht || sr || emulate) ? opt_blocks_per_sm(false, sr, rht, kOnePass) : kFastMinBlocks; break;
         case ABS_FMT_NVFP4_BS8: case ABS_FMT_IF4_BS8: per_thread = (rht || sr) ? 0 : 4; break;
         default: per_thread = (rht || sr) ? 0 : 3; break;       // IF3, IF6
     }
@@ -239,10 +239,10 @@ bool one_cluster(int fmt, const abs_opts_t& o, int64_t ngroups) {
            ngroups <= 3 * kMaxCluster * kThreads;
 }
 // Grid of a quantize kernel: see one_pass and grid_waves.
-int quantize_grid(const AlphaSrc& alpha, int sm_count, int64_t ngroups, int resident_per_sm, int target_iters) {
+int quantize_grid(const AlphaSrc& alpha, int sm_count, int64_t ngroups, int resident_per_sm, int target_iters, int threads = kThreads) {
     if (alpha.cluster) return kMaxCluster;
     if (alpha.cells) return grid_for(sm_count < kMaxCells ? sm_count : kMaxCells, ngroups, 1);
-    return grid_waves(sm_count, ngroups, resident_per_sm, target_iters);
+    return grid_waves(sm_count, ngroups, resident_per_sm, target_iters, threads);
 }
 
 template <int FMT>
@@ -307,16 +307,17 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
     }
     if constexpr (FMT == ABS_FMT_NVFP4 || FMT == ABS_FMT_IF4) {
         // Hadamard / stochastic-rounding options of the 4-bit formats: the packed persistent kernel
-        const int ogrid = quantize_grid(alpha, sm_count, ngroups, opt_blocks_per_sm(sr, rht), kOptIters);
-        if (!(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)ogrid * kThreads) {
-            constexpr bool kInt = FMT == ABS_FMT_IF4;
+        constexpr bool kInt = FMT == ABS_FMT_IF4;
+        const int osrc = alpha.cells ? kOnePass : kGiven, othreads = opt_threads(kInt, sr, osrc);
+        const int ogrid = quantize_grid(alpha, sm_count, ngroups, opt_blocks_per_sm(kInt, sr, rht, osrc), kOptIters, othreads);
+        if (!(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)ogrid * othreads) {
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             cudaError_t e;
 #define ABS_LAUNCH_O(R, S)                                                                                        \
     e = launch_any(alpha.cells ? kCooperative : kApart, alpha.cells ? quantize4_opt_kernel<kInt, R, S, kOnePass, false>         \
                                            : alpha.slot ? quantize4_opt_kernel<kInt, R, S, kFromSlot, false>       \
                                                         : quantize4_opt_kernel<kInt, R, S, kGiven, false>,         \
-                   ogrid, kThreads, s, (const uint4*)in, (uint2*)codes, (uint8_t*)scales, alpha, (int32_t)ngroups, mul, \
+                   ogrid, othreads, s, (const uint4*)in, (uint2*)codes, (uint8_t*)scales, alpha, (int32_t)ngroups, mul, \
                    (uint32_t)o.had_sign_mask, pk, ctr, a32, (uint4*)nullptr, false, true)
             if (rht && sr) ABS_LAUNCH_O(true, true);
             else if (rht) ABS_LAUNCH_O(true, false);
@@ -713,7 +714,7 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t ngroups = rows * cols / 16;
     const bool rht = o.flags & ABS_F_HADAMARD16, sr = o.flags & ABS_F_STOCHASTIC;
-    const int grid = grid_waves(st->sm_count, ngroups, opt_blocks_per_sm(sr, rht), (rht || sr) ? kOptIters : kFastIters);
+    const int grid = grid_waves(st->sm_count, ngroups, opt_blocks_per_sm(false, sr, rht, kGiven), (rht || sr) ? kOptIters : kFastIters);
     if (ngroups >= (int64_t)0x7FFFFFFF - (int64_t)grid * kThreads) return ABS_ERR_SIZE;    // 32-bit group indices only
     AlphaSrc src = {tensor_scale_f32, nullptr, 0u, 0.0f, tensor_scale_f32, nullptr, nullptr, false};
     const bool store = codes_u8 != nullptr;
@@ -737,11 +738,14 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
             return (!handled && r == ABS_ERR_FLAGS) ? ABS_ERR_SIZE : r;
         }
         cudaError_t e = cudaSuccess;
-        const int egrid = quantize_grid(src, st->sm_count, ngroups, opt_blocks_per_sm(sr, rht), (rht || sr) ? kOptIters : kFastIters);
+        const bool has_int = fmt == ABS_FMT_IF4;
+        const int esrc = src.cells ? kOnePass : kGiven, ethreads = opt_threads(has_int, sr, esrc);
+        int egrid = quantize_grid(src, st->sm_count, ngroups, opt_blocks_per_sm(has_int, sr, rht, esrc), (rht || sr) ? kOptIters : kFastIters, ethreads);
+        if (ngroups >= (int64_t)0x7FFFFFFF - (int64_t)egrid * ethreads) egrid = (int)((int64_t)grid * kThreads / ethreads);      // the stride that the check above has seen
 #define ABS_LAUNCH_E2(I, R, S)                                                                                      \
         e = launch_any(src.cells ? kCooperative : kApart, src.cells ? quantize4_opt_kernel<I, R, S, kOnePass, true>                   \
                                              : src.slot ? quantize4_opt_kernel<I, R, S, kFromSlot, true>                 \
-                                                        : quantize4_opt_kernel<I, R, S, kGiven, true>, egrid, kThreads, s, \
+                                                        : quantize4_opt_kernel<I, R, S, kGiven, true>, egrid, ethreads, s, \
                        (const uint4*)in_bf16, (uint2*)codes_u8, (uint8_t*)scales_e4m3, src, (int32_t)ngroups, mul,        \
                        (uint32_t)o.had_sign_mask, pk, ctr, a32, (uint4*)out_bf16, o32, store)
 #define ABS_LAUNCH_E(I)                                                                                             \

@@ -142,10 +142,12 @@ __device__ __forceinline__ void encode_body4_sr(const float (&x)[16], const uint
     }
 }
 
-// Resident blocks of 256 threads per SM the kernel is compiled and launched for: the stochastic-rounding
-// instances need about 120 registers, the Hadamard-only ones run best with three blocks, the plain
-// round-to-nearest instance (used by the emulation pass only) with four.
-constexpr int opt_blocks_per_sm(bool sr, bool rht = true) { return sr ? 2 : (rht ? 3 : 4); }
+// Threads of a block, and resident blocks per SM the kernel is compiled and launched for.  IF4 with stochastic rounding takes 93 registers: five blocks
+// of 128 threads (20 warps) instead of two of 256 (8192 x 8192, us: 69.8 -> 66.1, with Hadamard 76.0 -> 73.9, emulation 82.1 -> 78.0; NVFP4 46.8 / 47.2, so it
+// stays); the Hadamard-only kernels run best with three blocks of 256, the plain round-to-nearest one (used by the emulation pass only) with four.  A grid
+// of one block per SM (kOnePass) has blocks of 256.
+constexpr int opt_threads(bool has_int, bool sr, int src) { return has_int && sr && src != kOnePass ? 128 : 256; }
+constexpr int opt_blocks_per_sm(bool has_int, bool sr, bool rht, int src) { return sr ? (opt_threads(has_int, sr, src) == 128 ? 5 : 2) : (rht ? 3 : 4); }
 
 // Persistent grid-stride kernel, one group of 16 per thread and iteration, next group's 32 bytes fetched
 // before the current one is encoded.  scale_mul is 17/16 with that option and 1 otherwise (times 1 is exact).
@@ -154,7 +156,7 @@ constexpr int opt_blocks_per_sm(bool sr, bool rht = true) { return sr ? 2 : (rht
 // the dequantize kernel, and written to `out` as bf16; codes and scale bytes are stored only when
 // `store_codes` is set.
 template <bool HAS_INT, bool RHT, bool SR, int SRC, bool EMUL>
-__global__ void __launch_bounds__(256, opt_blocks_per_sm(SR, RHT))
+__global__ void __launch_bounds__(opt_threads(HAS_INT, SR, SRC), opt_blocks_per_sm(HAS_INT, SR, RHT, SRC))
 quantize4_opt_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, uint8_t* __restrict__ scales,
                      const AlphaSrc alpha_src, int32_t ngroups, float scale_mul, uint32_t sign_mask,
                      const PhiloxKeys keys, uint64_t ctr_base, bool aligned32, uint4* __restrict__ out, bool out_aligned32,
