@@ -342,13 +342,14 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
     }
     if constexpr (FMT == ABS_FMT_IF6_E2M3 || FMT == ABS_FMT_IF6_E3M2) {
         // 6-bit formats, round-to-nearest
-        const int sgrid = quantize_grid(alpha, sm_count, ngroups, 3, kIf6Iters);
-        if (!rht && !sr && !(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)sgrid * kThreads) {
+        const int wsrc = alpha.cells ? kOnePass : kGiven, wthreads = wide_threads(wsrc);
+        const int sgrid = quantize_grid(alpha, sm_count, ngroups, wide_blocks_per_sm(wsrc), kIf6Iters, wthreads);
+        if (!rht && !sr && !(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)sgrid * wthreads) {
             if (handled) *handled = true;
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             const auto kernel = emul_out ? (alpha.cells ? quantize6_fast_kernel<FMT, kOnePass, true> : alpha.slot ? quantize6_fast_kernel<FMT, kFromSlot, true> : quantize6_fast_kernel<FMT, kGiven, true>)
                                          : (alpha.cells ? quantize6_fast_kernel<FMT, kOnePass, false> : alpha.slot ? quantize6_fast_kernel<FMT, kFromSlot, false> : quantize6_fast_kernel<FMT, kGiven, false>);
-            const cudaError_t e = launch_any(alpha.cells ? kCooperative : kApart, kernel, sgrid, kThreads, s, (const uint4*)in, (uint32_t*)codes, (uint8_t*)scales, alpha,
+            const cudaError_t e = launch_any(alpha.cells ? kCooperative : kApart, kernel, sgrid, wthreads, s, (const uint4*)in, (uint32_t*)codes, (uint8_t*)scales, alpha,
                                              (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
             return quantize_launched(e, s);
         }
@@ -356,13 +357,14 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
     if constexpr (FMT == ABS_FMT_IF3 || FMT == ABS_FMT_IF3_BS8) {
         // IF3 and its block-size-8 variant, round-to-nearest
         constexpr int kG = FMT == ABS_FMT_IF3 ? 16 : 8;
-        const int tgrid = quantize_grid(alpha, sm_count, ngroups, kIf3MinBlocks, kIf6Iters);
-        if (!rht && !sr && !(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)tgrid * kThreads) {
+        const int wsrc = alpha.cells ? kOnePass : kGiven, wthreads = wide_threads(wsrc);
+        const int tgrid = quantize_grid(alpha, sm_count, ngroups, wide_blocks_per_sm(wsrc), kIf6Iters, wthreads);
+        if (!rht && !sr && !(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)tgrid * wthreads) {
             if (handled) *handled = true;
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             const auto kernel = emul_out ? (alpha.cells ? quantize3_fast_kernel<kG, kOnePass, true> : alpha.slot ? quantize3_fast_kernel<kG, kFromSlot, true> : quantize3_fast_kernel<kG, kGiven, true>)
                                          : (alpha.cells ? quantize3_fast_kernel<kG, kOnePass, false> : alpha.slot ? quantize3_fast_kernel<kG, kFromSlot, false> : quantize3_fast_kernel<kG, kGiven, false>);
-            const cudaError_t e = launch_any(alpha.cells ? kCooperative : kApart, kernel, tgrid, kThreads, s, (const uint4*)in, (uint16_t*)codes, (uint8_t*)scales, alpha,
+            const cudaError_t e = launch_any(alpha.cells ? kCooperative : kApart, kernel, tgrid, wthreads, s, (const uint4*)in, (uint16_t*)codes, (uint8_t*)scales, alpha,
                                              (int32_t)ngroups, mul, a32, (uint4*)emul_out, o32, emul_store || !emul_out);
             return quantize_launched(e, s);
         }
