@@ -28,9 +28,9 @@
  *     quantizes with alpha = 1, and raises a flag that makes the NEXT such call on the device
  *     return ABS_ERR_SIZE once, so the overrun cannot pass unseen.
  *   - Small tensors (up to 1.2 to 2.4 million elements on 148 SMs, by format and options): abs_quantize* and
- *     abs_quantize_dequantize along the rows are one cooperatively launched kernel whose blocks wait for one another's
- *     maxima.  Where such a grid does not fit (a green context or an MPS share of the device) the call takes the two kernels
- *     of larger tensors.  The wait is bounded (one second; it can run out only if the process is kept off the GPU for that long in
+ *     abs_quantize_dequantize along the rows are one kernel: one block for the smallest, one cluster of blocks or a cooperatively
+ *     launched grid, whose blocks wait for one another's maxima, for the others.  Where cluster or grid does not fit (a green
+ *     context or an MPS share of the device) the call takes the two kernels of larger tensors.  The wait of the grid is bounded (one second; it can run out only if the process is kept off the GPU for that long in
  *     the middle of the kernel); if it runs out, the call counts as overrun: alpha = 1, and the NEXT such call returns
  *     ABS_ERR_SIZE.
  *   - CUDA graphs: the slot and its tag are kernel arguments fixed at enqueue time, so a captured

@@ -225,7 +225,8 @@ quantize4_bs8_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
 // ----------------------------------------------------------------------------- 6-bit formats (IF6)
 
 // Threads of a block and resident blocks per SM of the IF6 and IF3 kernels: seven blocks of 128 threads at 72 registers, 28 warps, instead of three of
-// 256 at 76 - 80, 24 warps (round trip, us: IF3 4096 x 14336 92.2 -> 89.8, IF6 16384 x 8192 194.7 -> 191.9).  A grid of one block per SM (kOnePass) has blocks of 256.
+// 256 at 76 - 80, 24 warps (the kernels at 16384 x 8192, us: IF6 79.9 -> 75.6, IF3 90.2 -> 89.0; round trips of 4096 x 14336 and 16384 x 8192: IF3 90.9 -> 90.4, IF6 199.5
+// -> 196.6).  A grid of one block per SM (kOnePass) has blocks of 256.
 constexpr int wide_threads(int src) { return src == kOnePass ? 256 : 128; }
 constexpr int wide_blocks_per_sm(int src) { return src == kOnePass ? 3 : 7; }
 
