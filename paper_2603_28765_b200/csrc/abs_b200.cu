@@ -824,22 +824,23 @@ static abs_status_t quantize_transposed_impl(abs_fmt_t fmt, const void* in_bf16,
     const int64_t ntiles = ((cols + kTransTileCols - 1) / kTransTileCols) *
                            ((rblocks + kTransTileRowBlocks - 1) / kTransTileRowBlocks);
     if (ntiles > (int64_t)0x7FFFFFFF) return ABS_ERR_SIZE;      // the kernel indexes tiles with 32 bits
-    // 64 KiB of shared memory per block: 3 blocks per SM.  The arithmetic-bound variants (IF4, options) and the
-    // emulation pass run best as several waves with about four tiles per block, and at least two waves as soon as there are more tiles
-    // than resident blocks (1 / 2 waves, us: IF4 Hadamard SR 4096 x 4096, 2.3 tiles per resident block, 25.4 / 22.6, IF4 12.6 / 11.9, IF4 Hadamard
-    // emulation 23.2 / 21.0; between 1.5 and 6 tiles 0.84 to 1.0 times as long, at 8192 x 4096 up to 3 % longer); plain NVFP4 as one
-    // wave of persistent blocks.
-    const int64_t resident = (int64_t)st->sm_count * 3;
-    const bool heavy = fmt == ABS_FMT_IF4 || (o.flags & (ABS_F_HADAMARD16 | ABS_F_STOCHASTIC)) || out_bf16 != nullptr;
-    int64_t tgrid = ntiles < resident ? ntiles : resident;
-    if (heavy && ntiles > resident) {
-        int64_t waves = (ntiles + 2 * resident) / (4 * resident);
+    // The grid: several waves of some five blocks per SM with about four tiles per block, and at least two as soon as there are more tiles
+    // than that, so that blocks that start later overlap their first loads with the arithmetic of the others (1 / 2 / 3 or more waves, us: IF4 4096 x
+    // 4096 13.9 / 11.4 / 11.1, 8192 x 8192 40.7 / 37.9 / 37.4, 8192 x 14336 68.3 / 64.5 / 62.7, as one tile per block 66.6).  Plain NVFP4, which memory bounds, takes one
+    // wave of the six blocks that fit for up to half as many tiles again (2048 x 4096 5.2 / 5.5, 4096 x 4096 8.25 / 8.0, 8192 x 14336 52.6 / 52.6 / 46.8).
+    const int64_t wave = (int64_t)st->sm_count * 5, full = (int64_t)st->sm_count * 6;
+    const bool plain_nvfp4 = fmt != ABS_FMT_IF4 && !(o.flags & (ABS_F_HADAMARD16 | ABS_F_STOCHASTIC)) && !out_bf16;
+    int64_t tgrid;
+    if (plain_nvfp4 && 2 * ntiles < 3 * full) {
+        tgrid = ntiles < full ? ntiles : full;
+    } else {
+        int64_t waves = (ntiles + 2 * wave) / (4 * wave);
         if (waves < 2) waves = 2;
-        tgrid = waves * resident < ntiles ? waves * resident : ntiles;
+        tgrid = waves * wave < ntiles ? waves * wave : ntiles;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)tgrid);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kTransTileCols);
     cfg.dynamicSmemBytes = kTransSmemBytes;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -853,13 +854,7 @@ static abs_status_t quantize_transposed_impl(abs_fmt_t fmt, const void* in_bf16,
     uint8_t* stp = (uint8_t*)scales_t_e4m3;
     const uint32_t mask = o.had_sign_mask;
 #define ABS_LAUNCH_TE(I, S, R, Q, E)                                                                                \
-    do {                                                                                                            \
-        e = cudaFuncSetAttribute(transposed_kernel<I, S, R, Q, E>(), cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                 kTransSmemBytes);                                                                  \
-        if (e == cudaSuccess)                                                                                       \
-            e = cudaLaunchKernelEx(&cfg, transposed_kernel<I, S, R, Q, E>(), in, ct, stp, src, rows, cols, mask, \
-                                   mul, pk, ctr, (uint16_t*)out_bf16, store_codes);                      \
-    } while (0)
+    e = cudaLaunchKernelEx(&cfg, quantize4_transposed_kernel<I, S, R, Q, E>, in, ct, stp, src, rows, cols, mask, mul, pk, ctr, (uint16_t*)out_bf16, store_codes)
 #define ABS_LAUNCH_T(I, S, R, Q)                                                                                    \
     do {                                                                                                            \
         if (out_bf16) ABS_LAUNCH_TE(I, S, R, Q, true);                                                              \

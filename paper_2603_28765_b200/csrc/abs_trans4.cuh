@@ -13,17 +13,27 @@ namespace absq {
 // consecutive ROWS of one column (Sec. 4.1: both operands of the weight-gradient product are quantized
 // along the token dimension).  Output = what the plain kernel would give for the [cols, rows] matrix:
 // codes_t [cols, rows/2 bytes], scales_t [cols, rows/16].
-// Persistent blocks walk over tiles of 64 rows x 256 columns.  A tile is brought into shared memory with
+// Blocks of 128 threads walk over tiles of 64 rows x 128 columns.  A tile is brought into shared memory with
 // 16-byte asynchronous copies (cp.async), double buffered: the copies of the block's next tile are in
 // flight while it encodes the current one.  Thread c reads its column's values down the tile and encodes
 // the four groups of 16 rows; those are neighbours in the transposed output, so their codes leave as one
 // 256-bit store and their scale bytes as one 32-bit store whenever the tile is complete and the output
 // addresses allow it.
 constexpr int kTransUnroll = 4;
-constexpr int kTransTileCols = 256;
+constexpr int kTransTileCols = 128;                                                 // one thread per column
 constexpr int kTransTileRowBlocks = 4;
+constexpr int kTransRowChunks = kTransTileCols / 8, kTransRowLines = kTransTileCols / 64;   // 16-byte chunks, 128-byte lines of a row
 constexpr int kTransStageElems = 16 * kTransTileRowBlocks * kTransTileCols;        // bf16 elements per stage
-constexpr int kTransSmemBytes = 2 * kTransStageElems * 2;                           // two stages
+constexpr int kTransSmemBytes = 2 * kTransStageElems * 2;                           // two stages: 32 KB, which needs no attribute
+static_assert(kTransSmemBytes <= 48 * 1024 - 64, "dynamic shared memory without an attribute");
+
+// Blocks per SM the kernels are compiled for (shared memory would allow six).  What bounds them is the arithmetic pipes, so what helps is that another block
+// runs while one waits at a barrier or for its tile: blocks of 128 threads and columns instead of 256 (three per SM; with stochastic rounding two).
+// us, kernel alone, 256 / 128 columns, 8192 x 14336, 4096 x 4096 and 2048 x 2048: IF4 67.7 / 62.7, 11.9 / 11.4, 5.9 / 5.5; Hadamard 85.5 / 80.5, 14.7 / 13.8,
+// 7.0 / 6.2; Hadamard and SR 142.5 / 140.0, 25.3 / 22.4, 10.6 / 9.4; as the emulation pass 199 / 195, 34.7 / 30.6, 10.2 / 10.2; NVFP4 52.8 / 46.8, 8.2 / 8.0,
+// 4.2 / 4.2.  64 columns: equal or slower.  Six against five blocks: IF4 with Hadamard 1 to 10 % slower (fewer registers), the others up to 4 % faster where tiles abound;
+// SR with five against four: 2 to 5 % faster from 2048 x 4096 up, but the emulation pass of 2048 x 2048 18 % slower.
+constexpr int trans_blocks_per_sm(bool has_int, bool rht, bool sr, bool emul) { return sr ? (emul ? 4 : 5) : has_int && rht ? 5 : 6; }
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
@@ -67,12 +77,10 @@ __device__ __forceinline__ void hadamard16_pairs(float (&x)[16], uint32_t sign_m
 // finished tile then leaves with coalesced 16-byte stores to `out`, a [rows, cols] matrix in the ORIGINAL
 // orientation.  Codes and scales (transposed layout) are stored only when `store_codes` is set.
 template <bool HAS_INT, bool FROM_SLOT, bool RHT, bool SR, bool EMUL>
-__device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __restrict__ in, uint2* __restrict__ codes_t,
-                                                          uint8_t* __restrict__ scales_t, const AlphaSrc alpha_src,
-                                                          int64_t rows, int64_t cols, uint32_t sign_mask,
-                                                          float scale_mul, const PhiloxKeys& keys,
-                                                          uint64_t ctr_base, uint16_t* __restrict__ out,
-                                                          bool store_codes) {
+__global__ void __launch_bounds__(kTransTileCols, trans_blocks_per_sm(HAS_INT, RHT, SR, EMUL))
+quantize4_transposed_kernel(const uint16_t* __restrict__ in, uint2* __restrict__ codes_t, uint8_t* __restrict__ scales_t, const AlphaSrc alpha_src,
+                            int64_t rows, int64_t cols, uint32_t sign_mask, float scale_mul, const PhiloxKeys keys, uint64_t ctr_base,
+                            uint16_t* __restrict__ out, bool store_codes) {
     extern __shared__ __align__(16) uint16_t trans_smem[];
     pdl_launch_dependents();
     const int64_t rblocks = rows / 16;
@@ -92,17 +100,17 @@ __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __rest
             uint16_t* stage = trans_smem + s * kTransStageElems;
             const uint16_t* src = in + rb0 * 16 * cols + c0;
             if (ncols == kTransTileCols && nrb == kTransTileRowBlocks) {
-                // complete tile: 2048 chunks of 16 bytes, chunk ch = thread + 256 j lands at stage + 8 ch and comes
-                // from row (thread / 32) + 8 j, columns 8 (thread % 32) ...
+                // complete tile: chunk ch = thread + threads * j of 16 bytes lands at stage + 8 ch and comes
+                // from row (thread / chunks of a row) + 8 j, columns 8 (thread % chunks of a row) ...
                 uint16_t* dst = stage + 8 * threadIdx.x;
-                const uint16_t* from = src + (int64_t)(threadIdx.x >> 5) * cols + 8 * (threadIdx.x & 31);
+                const uint16_t* from = src + (int64_t)(threadIdx.x / kTransRowChunks) * cols + 8 * (threadIdx.x % kTransRowChunks);
                 const int64_t step = 8 * cols;
 #pragma unroll
-                for (int j = 0; j < 16 * kTransTileRowBlocks * (kTransTileCols / 8) / 256; ++j)
-                    cp_async16(dst + j * 8 * 256, from + j * step);
-            } else if (ncols == kTransTileCols) {        // full-width tile: 32 chunks of 16 bytes per row
-                for (int ch = threadIdx.x; ch < 16 * nrb * (kTransTileCols / 8); ch += blockDim.x) {
-                    const int r = ch >> 5, q = ch & 31;
+                for (int j = 0; j < 2 * kTransTileRowBlocks; ++j)
+                    cp_async16(dst + j * 8 * kTransTileCols, from + j * step);
+            } else if (ncols == kTransTileCols) {        // full-width tile
+                for (int ch = threadIdx.x; ch < 16 * nrb * kTransRowChunks; ch += blockDim.x) {
+                    const int r = ch / kTransRowChunks, q = ch % kTransRowChunks;
                     cp_async16(stage + r * kTransTileCols + q * 8, src + (int64_t)r * cols + q * 8);
                 }
             } else {                                     // ragged last column tile
@@ -117,13 +125,13 @@ __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __rest
     };
 
     int s = 0;
-    // Tile counts fit 32 bits (a tile is 16384 elements).  The block's tiles are t, t + grid, ...: their
+    // Tile counts fit 32 bits (a tile is 8192 elements).  The block's tiles are t, t + grid, ...: their
     // coordinates advance by (grid / ntx, grid % ntx) with one carry, so only the first needs a division.
     int64_t t = blockIdx.x;
     const uint32_t ntx32 = (uint32_t)ntx, step_y = gridDim.x / ntx32, step_x = gridDim.x - step_y * ntx32;
     uint32_t ty = blockIdx.x / ntx32, tx = blockIdx.x - ty * ntx32;
     {   // before the wait (see prefetch_l2): the block's first tile, a line of 128 bytes per thread
-        const int64_t r = (int64_t)ty * 16 * kTransTileRowBlocks + (threadIdx.x >> 2), c = (int64_t)tx * kTransTileCols + 64 * (threadIdx.x & 3);
+        const int64_t r = (int64_t)ty * 16 * kTransTileRowBlocks + threadIdx.x / kTransRowLines, c = (int64_t)tx * kTransTileCols + 64 * (threadIdx.x % kTransRowLines);
         if (r < rows && c < cols) prefetch_l2(in + r * cols + c);
     }
     pdl_wait();
@@ -141,7 +149,7 @@ __device__ __forceinline__ void quantize4_transposed_body(const uint16_t* __rest
         const int ncols = (int)min((int64_t)kTransTileCols, cols - c0);
         uint16_t* stage = trans_smem + s * kTransStageElems;
         const int c = threadIdx.x;
-        // FULL: a complete 64 x 256 tile whose outputs may leave as vector stores (the usual case): no per-group
+        // FULL: a complete tile whose outputs may leave as vector stores (the usual case): no per-group
         // bounds checks.  Otherwise the ragged-tile path with the same arithmetic.
         auto encode_column = [&](auto full_tag) {
             constexpr bool FULL = decltype(full_tag)::value;
@@ -308,36 +316,6 @@ amax_columns_kernel(const uint2* __restrict__ in, int64_t rblocks, int64_t chunk
         for (int v = 0; v < 8; ++v) m = max(m, warp_max[v]);
         atomicMax(slot, ((unsigned long long)gen << 32) | m);
     }
-}
-
-#define ABS_TRANS_PARAMS                                                                                              \
-    const uint16_t *__restrict__ in, uint2 *__restrict__ codes_t, uint8_t *__restrict__ scales_t,                     \
-        const AlphaSrc alpha_src, int64_t rows, int64_t cols, uint32_t sign_mask, float scale_mul, const PhiloxKeys keys, uint64_t ctr_base,                                   \
-        uint16_t *__restrict__ out, bool store_codes
-#define ABS_TRANS_ARGS                                                                                                \
-    in, codes_t, scales_t, alpha_src, rows, cols, sign_mask, scale_mul, keys,                    \
-        ctr_base, out, store_codes
-
-// Round-to-nearest and Hadamard instances are held to the registers of three blocks per SM (what the shared
-// memory allows): left alone the compiler takes up to 124 and only two blocks fit.
-template <bool HAS_INT, bool FROM_SLOT, bool RHT, bool EMUL>
-__global__ void __launch_bounds__(256, 3) quantize4_transposed_kernel(ABS_TRANS_PARAMS) {
-    quantize4_transposed_body<HAS_INT, FROM_SLOT, RHT, false, EMUL>(ABS_TRANS_ARGS);
-}
-// The stochastic-rounding instances measured 3-7 % faster with the compiler's own register choice (about 80,
-// no spills) than held to three or to two blocks per SM.
-template <bool HAS_INT, bool FROM_SLOT, bool RHT, bool EMUL>
-__global__ void __launch_bounds__(256) quantize4_transposed_sr_kernel(ABS_TRANS_PARAMS) {
-    quantize4_transposed_body<HAS_INT, FROM_SLOT, RHT, true, EMUL>(ABS_TRANS_ARGS);
-}
-#undef ABS_TRANS_PARAMS
-#undef ABS_TRANS_ARGS
-
-// The kernel instance for a set of options (both wrappers have the same signature).
-template <bool HAS_INT, bool FROM_SLOT, bool RHT, bool SR, bool EMUL>
-constexpr auto transposed_kernel() {
-    if constexpr (SR) return &quantize4_transposed_sr_kernel<HAS_INT, FROM_SLOT, RHT, EMUL>;
-    else return &quantize4_transposed_kernel<HAS_INT, FROM_SLOT, RHT, EMUL>;
 }
 
 }  // namespace absq
