@@ -309,7 +309,10 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
         // Hadamard / stochastic-rounding options of the 4-bit formats: the packed persistent kernel
         constexpr bool kInt = FMT == ABS_FMT_IF4;
         const int osrc = alpha.cells ? kOnePass : kGiven, othreads = opt_threads(kInt, sr, osrc);
-        const int ogrid = quantize_grid(alpha, sm_count, ngroups, opt_blocks_per_sm(kInt, sr, rht, osrc), kOptIters, othreads);
+        int ogrid = quantize_grid(alpha, sm_count, ngroups, opt_blocks_per_sm(kInt, sr, rht, osrc), kOptIters, othreads);
+        // NVFP4 with stochastic rounding takes 58 registers, so four blocks fit: tensors whose waves of two leave half of that idle get four (backward
+        // pass of a layer of 2048 x 4096 x 4096 119.6 -> 115.1 us); waves of four at 16384 x 8192 take longer, 98.7 -> 105.6 us.
+        if (!kInt && sr && !alpha.cells && ogrid < 4 * sm_count) ogrid = grid_for(sm_count, ngroups, 4);
         if (!(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)ogrid * othreads) {
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             cudaError_t e;
