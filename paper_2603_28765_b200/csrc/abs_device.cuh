@@ -510,12 +510,13 @@ __device__ __forceinline__ float alpha_of(const AlphaSrc& a, const uint32_t (&w)
     else return resolve_alpha_per_thread<SRC == kFromSlot>(a);
 }
 
-// Per-block table of G5 for every scale byte 0x00..0x7E: d = Delta * alpha and its IEEE reciprocal depend only on
-// the byte, so a block computes the 127 pairs once and a group reads its pair with one 8-byte load instead of a
+// Per-block table of G5 for every scale byte: d = Delta * alpha and its IEEE reciprocal depend only on
+// the byte, so a block computes the pairs once and a group reads its pair with one 8-byte load instead of a
 // multiply, a multiply and a reciprocal (same operations, same bits).  Every thread of the block must call this
-// (it ends with a barrier); entry 0 (d = 0) is never read.
+// (it ends with a barrier); blocks have at least 128 threads.  Entry 0x7F is what t is encoded to when it is not a number: a zero
+// group under a tensor scale so small that 1 / (6 alpha) overflows.
 __device__ __forceinline__ void fill_scale_table(float2* table, float alpha) {
-    if (threadIdx.x < 127) {
+    if (threadIdx.x < 128) {
         const float d = __fmul_rn(e4m3_value(threadIdx.x), alpha);
         table[threadIdx.x] = make_float2(d, __frcp_rn(d));
     }
