@@ -240,6 +240,12 @@ __device__ __forceinline__ float max3abs(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(fabsf(a)), "f"(fabsf(b)), "f"(fabsf(c)));
     return d;
 }
+// The same, but NaN if any of them is (max3abs drops a NaN beside a number).
+__device__ __forceinline__ float max3abs_nan(float a, float b, float c) {
+    float d;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(fabsf(a)), "f"(fabsf(b)), "f"(fabsf(c)));
+    return d;
+}
 
 // ----------------------------------------------------------------------------- Hadamard option
 

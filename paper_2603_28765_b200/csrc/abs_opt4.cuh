@@ -57,8 +57,14 @@ __device__ __forceinline__ uint32_t minus_field(uint32_t rnd, uint32_t c) {
 // What bounds the kernels that call this is the arithmetic pipes, so the count of instructions: 36 -> 25 per pair of elements against three
 // float pieces for phi, a float subtraction of u and signs put back on both values.  IF4, 8192 x 8192, 17/16 option, us before and after:
 // rows with Hadamard 92.3 / 76.0, rows 84.0 / 69.9, columns with Hadamard 104.6 / 86.2; NVFP4 63.5 / 53.4, 53.4 / 47.1, 73.9 / 64.4.
-// CLAMP: |y| may exceed 6 (then |z| 7; fl(6 * fp32(7/6)) is 7, so one clamp serves both).  With the 17/16 option and a
-// scale byte that is neither subnormal nor saturated it stays below 6 (1 + 7 * 2^-24), and neither index passes 7.
+// CLAMP: |y| may exceed 6 (then |z| 7; fl(6 * fp32(7/6)) is 7, so one clamp serves both).  It stays below 6 (1 + 7 * 2^-24), and neither index passes 7, with
+// the 17/16 option, a scale byte that is neither subnormal nor saturated, and an alpha between 2^-120 and 2^117, which keeps 6 alpha, d and their
+// reciprocals normal (alphas of supported tensors lie between 2^-112 and 2^117; a given alpha can be anything).  The clamp makes 6 of a y that is not a
+// number, too; without it, such a y leaves its nibble.
+__device__ __forceinline__ bool alpha_keeps_y_below_the_clamp(float alpha) {
+    constexpr uint32_t kLow = (127u - 120u) << 23, kHigh = (127u + 117u) << 23;        // 2^-120, 2^117
+    return __float_as_uint(alpha) - kLow <= kHigh - kLow;
+}
 template <bool HAS_INT, bool CLAMP>
 __device__ __forceinline__ void encode_body4_sr(const float (&x)[16], const uint32_t (&rnd)[8], uint32_t sb, float d,
                                                 float r, uint32_t& sbyte, uint32_t& c_lo, uint32_t& c_hi) {
@@ -193,6 +199,7 @@ quantize4_opt_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
     fill_scale_table(scale_table, alpha);                                    // G5 for every scale byte, once per block
     if (!active) return;
     const float inv_a6 = __frcp_rn(__fmul_rn(alpha, 6.0f));                  // T3
+    const bool bounded = scale_mul > 1.0f && alpha_keeps_y_below_the_clamp(alpha);   // see encode_body4_sr
     while (true) {
         const int32_t gn = g + stride;
         const bool more = gn < ngroups;
@@ -221,21 +228,37 @@ quantize4_opt_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
             rnd[4] = p1.x; rnd[5] = p1.y; rnd[6] = p1.z; rnd[7] = p1.w;
         }
         // G1: group maximum with three-input max.
-        const float m0 = max3abs(x[0], x[1], x[2]), m1 = max3abs(x[3], x[4], x[5]);
-        const float m2 = max3abs(x[6], x[7], x[8]), m3 = max3abs(x[9], x[10], x[11]);
-        const float m4 = max3abs(x[12], x[13], x[14]);
-        const float gmax = fmaxf(max3abs(m0, m1, m2), max3abs(m3, m4, x[15]));
-        // G2-G3 (Eq. 2), with the 17/16 option folded into scale_mul.
-        const float t = __fmul_rn(__fmul_rn(gmax, inv_a6), scale_mul);
-        const uint32_t sb = e4m3_encode(t);
-        const float2 dr = scale_table[sb];                                 // G5: d = Delta * alpha and 1 / d
-        const float d = dr.x, r = dr.y;
+        const auto group_max = [&](auto max3) {
+            const float m0 = max3(x[0], x[1], x[2]), m1 = max3(x[3], x[4], x[5]);
+            const float m2 = max3(x[6], x[7], x[8]), m3 = max3(x[9], x[10], x[11]);
+            const float m4 = max3(x[12], x[13], x[14]);
+            return max3(max3(m0, m1, m2), max3(m3, m4, x[15]), x[15]);
+        };
+        const auto drop_nan = [](float a, float b, float c) { return max3abs(a, b, c); };
+        const auto keep_nan = [](float a, float b, float c) { return max3abs_nan(a, b, c); };
+        // G2-G3 (Eq. 2), with the 17/16 option folded into scale_mul; G5: d = Delta * alpha and 1 / d.
+        uint32_t sb;
+        float d, r;
+        const auto scale_of = [&](float gmax) {
+            sb = e4m3_encode(__fmul_rn(__fmul_rn(gmax, inv_a6), scale_mul));
+            const float2 dr = scale_table[sb];
+            d = dr.x;
+            r = dr.y;
+        };
+        // With a NaN among them t is one and its byte 0x7F, which leads off the path without the clamp: no instruction more on that path (8192 x 8192,
+        // before and after, us, with Hadamard: IF4 73.5 / 73.3, without 17/16 75.0 / 76.2, NVFP4 52.9 / 53.2); a test of its own there cost 2 - 3 %.
+        if constexpr (SR) scale_of(group_max(keep_nan));
+        else scale_of(group_max(drop_nan));
         uint32_t sbyte = 0u, c_lo = 0u, c_hi = 0u;
         if constexpr (SR) {
             // without the clamp where it cannot act (IF4 with Hadamard, 8192 x 8192: 77.9 -> 76.0 us; the transposed kernel, which
             // unrolls four groups, gained nothing from a second copy)
-            if ((sb - 8u) < 118u && scale_mul > 1.0f) encode_body4_sr<HAS_INT, false>(x, rnd, sb, d, r, sbyte, c_lo, c_hi);
-            else if (sb != 0u) encode_body4_sr<HAS_INT, true>(x, rnd, sb, d, r, sbyte, c_lo, c_hi);      // G4: zero scale -> zeros
+            if ((sb - 8u) < 118u && bounded) {
+                encode_body4_sr<HAS_INT, false>(x, rnd, sb, d, r, sbyte, c_lo, c_hi);
+            } else {
+                if (sb == 0x7Fu) scale_of(group_max(drop_nan));            // the scale is that of the numbers of the group
+                if (sb != 0u) encode_body4_sr<HAS_INT, true>(x, rnd, sb, d, r, sbyte, c_lo, c_hi);      // G4: zero scale -> zeros
+            }
         } else {
             if ((sb - 8u) >= 118u) {
                 if (sb != 0u) encode_body4<HAS_INT, HAS_INT>(x, sb, d, r, sbyte, c_lo, c_hi);
