@@ -246,6 +246,7 @@ quantize4_transposed_kernel(const uint16_t* __restrict__ in, uint2* __restrict__
 // The amax pass of the transposed path with the Hadamard option: the maximum of the transformed column groups, published like amax_kernel's.  Bound by
 // memory: a thread reads 16 rows of four columns, 8 bytes at a time (256 contiguous bytes per warp and row), the butterflies run on
 // pairs of columns (h = 1, 2, 4, 8, packed add and fused subtract, the arithmetic of hadamard16_pairs), and 1/4 is applied to the maximum alone.
+// A transformed value that is not a number (a NaN in the input, or sums beyond the largest float) makes a NaN of the tensor scale and does not go unseen.
 // us, as the tile walk of the quantize kernel and as this: 8192 x 14336 45.5 / 37.6 (6.25 TB/s), 8192 x 4096 17.6 / 13.5, 4096 x 4096 10.9 / 7.6, 2048 x 4096 7.5 / 4.9.
 // Three blocks per SM and no more of them: four (64 registers) spill, 46.7 us; several waves 38.4 - 39.7.
 constexpr int kAmaxColumnsBlocks = 3;
@@ -297,15 +298,15 @@ amax_columns_kernel(const uint2* __restrict__ in, int64_t rblocks, int64_t chunk
                 float a, b, c, d;
                 unpack2(P[r], a, b);
                 unpack2(P[r + 1], c, d);
-                m0 = max3abs(m0, a, b);
-                m1 = max3abs(m1, c, d);
+                m0 = max3abs_nan(m0, a, b);
+                m1 = max3abs_nan(m1, c, d);
             }
         }
         y += step_y;
         x += step_x;
         if (x >= chunks) { x -= chunks; ++y; }
     }
-    uint32_t local = __float_as_uint(__fmul_rn(fmaxf(m0, m1), 0.25f));
+    uint32_t local = __float_as_uint(__fmul_rn(max3abs_nan(m0, m1, m1), 0.25f));
     __shared__ uint32_t warp_max[8];
     local = __reduce_max_sync(0xFFFFFFFFu, local);
     if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = local;
