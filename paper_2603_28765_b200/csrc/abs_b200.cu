@@ -14,6 +14,7 @@
 #include "abs_fastx.cuh"
 #include "abs_trans4.cuh"
 #include "abs_generic.cuh"
+#include "abs_launch.h"
 
 #include <atomic>
 #include <mutex>
@@ -23,42 +24,6 @@ using namespace absq;
 namespace {
 
 constexpr int kMaxDevices = 64;
-
-// Launch with programmatic stream serialization: the kernel may be scheduled while the previous
-// kernel of the stream drains; every kernel here calls pdl_wait() before its first global access.
-// together: the blocks wait for one another, so all of them have to be resident: as a cluster (one_cluster_alpha; the grid is at most kMaxCluster blocks) or by a
-// cooperative launch (one_pass_alpha).  A single block needs neither; the latter costs half a microsecond more on the host (2.45 us instead of
-// 1.93) and lets nothing overlap: such kernels start 4.1 us apart on a stream.
-enum Together { kApart, kCooperative, kCluster };
-template <typename... KArgs, typename... Args>
-cudaError_t launch_any(Together together, void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    if (together == kCluster) {
-        attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = (unsigned)grid;
-        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    } else {
-        attr[1].id = cudaLaunchAttributeCooperative;
-        attr[1].val.cooperative = 1;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = together != kApart && grid > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
-    return launch_any(kApart, kernel, grid, block, s, args...);
-}
-// Internal status: a cooperative grid was refused because its blocks do not all fit what the stream may use (a green context, an
-// MPS share: fewer SMs than the device has).  Nothing was enqueued; the call takes the two kernels.
-constexpr abs_status_t kNotResident = (abs_status_t)-1;
 
 // ------------------------------------------------------------------------------------------ host state
 
@@ -81,20 +46,6 @@ struct DeviceState {
     cudaEvent_t d2h_done = nullptr;
 };
 DeviceState g_dev[kMaxDevices];
-
-// Optional CUDA events recorded around the group-quantize kernel (abs_profile_events).
-cudaEvent_t g_ev_quant_begin = nullptr, g_ev_quant_end = nullptr;
-
-// Status of the launch of a quantize kernel on s; also ends the interval of abs_profile_events.
-abs_status_t quantize_launched(cudaError_t e, cudaStream_t s, bool profile = true) {
-    if (e == cudaErrorCooperativeLaunchTooLarge) {
-        cudaGetLastError();                  // the refusal is answered here: it is not left for the caller's own error checks
-        return kNotResident;
-    }
-    if (e != cudaSuccess) return ABS_ERR_CUDA;
-    if (profile && g_ev_quant_end) cudaEventRecord(g_ev_quant_end, s);
-    return cudaGetLastError() == cudaSuccess ? ABS_OK : ABS_ERR_CUDA;
-}
 
 abs_status_t device_state(DeviceState** out) {
     int dev = 0;
@@ -298,10 +249,6 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
 #undef ABS_LAUNCH_F
 #undef ABS_LAUNCH_F2
 #undef ABS_LAUNCH_F3
-            if (alpha.cluster && e != cudaSuccess) {         // no room for a cluster: as for a cooperative grid
-                cudaGetLastError();
-                return kNotResident;
-            }
             return quantize_launched(e, s);
         }
     }
