@@ -1,12 +1,14 @@
 // The calls of binding.py that allocate their outputs and enqueue kernels, without the interpreter in between: argument
-// unpacking, output allocation (at::empty), device guard, current stream, and the call through the C ABI of
+// unpacking, output allocation, device guard, current stream, and the call through the C ABI of
 // include/abs_b200.h, whose addresses binding.py passes in.  A quantize call is two kernels of a few microseconds on small
 // tensors, and marshalling it from Python took 31 us, with a fill kernel for the one float of the tensor scale.
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
+#include <ATen/record_function.h>
 #include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
+#include <c10/core/impl/LocalDispatchKeySet.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -87,11 +89,16 @@ class Work {
         if (!stream && PyErr_Occurred()) throw Raised();
         other = stream != current;
     }
+    // Whether outputs are allocated through the dispatcher, which is a third of the 0.9 us that at::empty takes (a quantize call allocates three tensors): where
+    // somebody listens there (dispatch modes, fake tensors, transforms and tracers put a key of their own into the thread's set; profilers
+    // record the operator), or deterministic algorithms are asked for, with which at::empty fills what it allocates.
+    static bool dispatched() {
+        const c10::DispatchKeySet keys = c10::impl::tls_local_dispatch_key_set().included_;
+        return !(keys - c10::default_included_set).empty() || at::hasCallbacks() || at::globalContext().deterministicAlgorithms();
+    }
     at::Tensor empty(at::IntArrayRef sizes, at::ScalarType type) const {
-        // Past the dispatcher, which is a third of the 0.9 us that at::empty takes (a quantize call allocates three tensors); not where
-        // deterministic algorithms are asked for, with which at::empty fills what it allocates.
-        at::Tensor t = at::globalContext().deterministicAlgorithms() ? at::empty(sizes, at::TensorOptions().dtype(type).device(device))
-                                                                      : at::Tensor(at::detail::empty_cuda(sizes, type, device, std::nullopt));
+        at::Tensor t = dispatched() ? at::empty(sizes, at::TensorOptions().dtype(type).device(device))
+                                    : at::Tensor(at::detail::empty_cuda(sizes, type, device, std::nullopt));
         if (other && t.numel() > 0) c10::cuda::CUDACachingAllocator::recordStream(t.storage().data_ptr(), torch_stream());
         return t;
     }
