@@ -418,6 +418,7 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
         uint32_t j = 0;
         uint32_t out_max = 0u;                  // bf16 output with next_alpha: largest |C| bit patterns this thread has written (see store_columns16)
         const bool out_aligned32 = (reinterpret_cast<uintptr_t>(c_out) & 31u) == 0;
+        uint4 held = make_uint4(0u, 0u, 0u, 0u);   // see store_columns16
         bool all_tiles = true;
         if constexpr (PLANES == 2) {
             // Two warps per quarter of tensor memory; a warp owns the accumulator lanes (rows of the tile) 32 (w % 4) ..
@@ -467,10 +468,7 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
                     if (lane == 0) mbar_arrive(acc_empty0 + 8 * buf);    // the MMAs of the next chunk or tile may start
                 }
                 if (!all_tiles) break;
-                if (own_row_valid) {
-#pragma unroll
-                    for (int q = 0; q < kCols / 16; ++q) store_columns16<OUT_BF16>(c_out, first + 16 * q, v + 16 * q, scale, out_aligned32, next_alpha != nullptr, out_max);
-                }
+                if (own_row_valid) store_columns<OUT_BF16, kCols / 16>(c_out, first, v, scale, out_aligned32, true, true, held, next_alpha != nullptr, out_max);
             }
         } else {
             // A warp owns the accumulator lanes (rows of the tile) 32 (w % 4) .. 32 (w % 4) + 31.
@@ -498,11 +496,8 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
                     float v[32];
 #pragma unroll
                     for (int jj = 0; jj < 32; ++jj) v[jj] = __uint_as_float(r0[jj]);
-                    if (own_row_valid) {
-#pragma unroll
-                        for (int q = 0; q < 2; ++q)
-                            store_columns16<OUT_BF16>(c_out, first + chunk * 32 + 16 * q, v + 16 * q, scale, out_aligned32, next_alpha != nullptr, out_max);
-                    }
+                    if (own_row_valid)
+                        store_columns<OUT_BF16, 2>(c_out, first + chunk * 32, v, scale, out_aligned32, chunk == 0, chunk == kTileN / 32 - 1, held, next_alpha != nullptr, out_max);
                 }
             }
         }

@@ -158,12 +158,18 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-// Sixteen neighbouring columns of a row of C times `scale`, from column index `at` on: 64 (FP32) or 32 (bf16) contiguous bytes of one thread, in whole sectors where C
-// is 32-byte aligned.  keep_max: the larger of out_max and the bf16 magnitudes written, per half word.
-template <bool OUT_BF16>
-__device__ __forceinline__ void store_columns16(void* c_out, size_t at, const float* v, float scale, bool aligned32, bool keep_max, uint32_t& out_max) {
+// Sixteen neighbouring columns of a row of C times `scale`, from column index `at` on: 64 (FP32) or 32 (bf16) contiguous bytes of one thread, which takes a run
+// of such columns in order, first to last.  Whole sectors leave at a time: where C is 32-byte aligned as they are, otherwise (C is 16-byte aligned, rows
+// are whole sectors long) the second half of 32 bytes is held back for the first of the next, and only the ends of the run are half sectors.  (As
+// two 16-byte stores each, whose sectors the next one completes, FP32 products into such a C took up to 1.4 times as long: NVFP4 4096 x 4096 x 512 20.2 us by lines
+// turned through shared memory, 28.5 so, 18.3 held back; 2048 x 4096 x 4096 bf16 27.3, 26.2, 24.0.)
+// keep_max: the larger of out_max and the bf16 magnitudes written, per half word.
+template <bool OUT_BF16, bool ALIGNED32>
+__device__ __forceinline__ void store_columns16(void* c_out, size_t at, const float* v, float scale, bool first, bool last, uint4& held, bool keep_max,
+                                                uint32_t& out_max) {
+    constexpr int kPieces = OUT_BF16 ? 1 : 2;
 #pragma unroll
-    for (int q = 0; q < (OUT_BF16 ? 1 : 2); ++q) {
+    for (int q = 0; q < kPieces; ++q) {
         uint32_t o[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
@@ -175,8 +181,31 @@ __device__ __forceinline__ void store_columns16(void* c_out, size_t at, const fl
             }
         }
         uint8_t* const to = reinterpret_cast<uint8_t*>(c_out) + at * (OUT_BF16 ? 2 : 4) + 32 * q;
-        if (aligned32) store32B<true>(to, o);
-        else store32B<false>(to, o);
+        if constexpr (ALIGNED32) {
+            store32B<true>(to, o);
+        } else {
+            if (first && q == 0) {
+                *reinterpret_cast<uint4*>(to) = make_uint4(o[0], o[1], o[2], o[3]);
+            } else {
+                const uint32_t sector[8] = {held.x, held.y, held.z, held.w, o[0], o[1], o[2], o[3]};
+                store32B<true>(to - 16, sector);
+            }
+            held = make_uint4(o[4], o[5], o[6], o[7]);
+            if (last && q == kPieces - 1) *reinterpret_cast<uint4*>(to + 16) = held;
+        }
+    }
+}
+// N x 16 columns of such a run, the first of them at its start, the last at its end, as told.
+template <bool OUT_BF16, int N>
+__device__ __forceinline__ void store_columns(void* c_out, size_t at, const float* v, float scale, bool aligned32, bool first, bool last, uint4& held,
+                                              bool keep_max, uint32_t& out_max) {
+    if (aligned32) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) store_columns16<OUT_BF16, true>(c_out, at + 16 * q, v + 16 * q, scale, false, false, held, keep_max, out_max);
+    } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q)
+            store_columns16<OUT_BF16, false>(c_out, at + 16 * q, v + 16 * q, scale, first && q == 0, last && q == N - 1, held, keep_max, out_max);
     }
 }
 __device__ __forceinline__ void tmem_load_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
