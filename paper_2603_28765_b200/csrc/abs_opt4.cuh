@@ -199,7 +199,9 @@ quantize4_opt_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
     fill_scale_table(scale_table, alpha);                                    // G5 for every scale byte, once per block
     if (!active) return;
     const float inv_a6 = __frcp_rn(__fmul_rn(alpha, 6.0f));                  // T3
-    const bool bounded = scale_mul > 1.0f && alpha_keeps_y_below_the_clamp(alpha);   // see encode_body4_sr
+    // Scale bytes 8 .. 125 go without the clamp where the rest of encode_body4_sr's conditions hold.  (A number and not a truth value: kept over the loop, that took two
+    // registers more, and the emulation pass of NVFP4 with Hadamard 7.6 us instead of 6.1, back to back at 1000 x 4096.)
+    const uint32_t unclamped = scale_mul > 1.0f && alpha_keeps_y_below_the_clamp(alpha) ? 118u : 0u;
     while (true) {
         const int32_t gn = g + stride;
         const bool more = gn < ngroups;
@@ -246,14 +248,14 @@ quantize4_opt_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
             r = dr.y;
         };
         // With a NaN among them t is one and its byte 0x7F, which leads off the path without the clamp: no instruction more on that path (8192 x 8192,
-        // before and after, us, with Hadamard: IF4 73.5 / 73.3, without 17/16 75.0 / 76.2, NVFP4 52.9 / 53.2); a test of its own there cost 2 - 3 %.
+        // before and after, us, with Hadamard: IF4 73.4 / 73.4, without 17/16 74.9 / 75.8, NVFP4 52.9 / 53.2); a test of its own there cost 2 - 3 %.
         if constexpr (SR) scale_of(group_max(keep_nan));
         else scale_of(group_max(drop_nan));
         uint32_t sbyte = 0u, c_lo = 0u, c_hi = 0u;
         if constexpr (SR) {
             // without the clamp where it cannot act (IF4 with Hadamard, 8192 x 8192: 77.9 -> 76.0 us; the transposed kernel, which
             // unrolls four groups, gained nothing from a second copy)
-            if ((sb - 8u) < 118u && bounded) {
+            if ((sb - 8u) < unclamped) {
                 encode_body4_sr<HAS_INT, false>(x, rnd, sb, d, r, sbyte, c_lo, c_hi);
             } else {
                 if (sb == 0x7Fu) scale_of(group_max(drop_nan));            // the scale is that of the numbers of the group
