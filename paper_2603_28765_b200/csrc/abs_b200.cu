@@ -16,6 +16,7 @@
 #include "abs_generic.cuh"
 #include "abs_launch.h"
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
@@ -196,6 +197,19 @@ int quantize_grid(const AlphaSrc& alpha, int sm_count, int64_t ngroups, int resi
     return grid_waves(sm_count, ngroups, resident_per_sm, target_iters, threads);
 }
 
+// Grid of quantize4_opt_kernel: waves of the blocks it is compiled for.  NVFP4 with stochastic rounding is compiled for two and takes so few registers (60)
+// that four fit: where one wave of two would leave half of that idle, all that fit (kNvSrFit; backward pass of a layer of 2048 x 4096 x 4096 119.6 -> 115.1 us).  Waves
+// of four take longer on large tensors (16384 x 8192 98.7 -> 105.6 us), and so does the kernel when it is compiled for four (8192 x 8192 with
+// Hadamard 53.2 -> 57.6 us), so the launch bound does not say what fits: a test does, against the grid of a call.  The emulation pass, of
+// which three or four fit, keeps one wave of two: with four, 1000 x 4096 takes 5.7 us instead of 6.9, with Hadamard 6.4 instead of 6.1 (4096 x 4096 17.1 -> 16.7).
+constexpr int kNvSrFit = 4;
+int opt_grid(const AlphaSrc& alpha, int sm_count, int64_t ngroups, bool has_int, bool sr, bool rht, bool emulated, int target_iters) {
+    const int src = alpha.cells ? kOnePass : kGiven;
+    const int grid = quantize_grid(alpha, sm_count, ngroups, opt_blocks_per_sm(has_int, sr, rht, src), target_iters, opt_threads(has_int, sr, src));
+    if (has_int || !sr || alpha.cells || emulated) return grid;
+    return std::max(grid, grid_for(sm_count, ngroups, kNvSrFit));
+}
+
 template <int FMT>
 // emul_out != nullptr asks for the emulation pass (abs_quantize_dequantize) of the formats handled by the
 // kernels of abs_fastx.cuh: bf16 output, codes stored only when emul_store.  *handled tells the caller whether
@@ -256,10 +270,7 @@ abs_status_t launch_quantize_fmt(int sm_count, const void* in, int64_t ngroups, 
         // Hadamard / stochastic-rounding options of the 4-bit formats: the packed persistent kernel
         constexpr bool kInt = FMT == ABS_FMT_IF4;
         const int osrc = alpha.cells ? kOnePass : kGiven, othreads = opt_threads(kInt, sr, osrc);
-        int ogrid = quantize_grid(alpha, sm_count, ngroups, opt_blocks_per_sm(kInt, sr, rht, osrc), kOptIters, othreads);
-        // NVFP4 with stochastic rounding takes 58 registers, so four blocks fit: tensors whose waves of two leave half of that idle get four (backward
-        // pass of a layer of 2048 x 4096 x 4096 119.6 -> 115.1 us); waves of four at 16384 x 8192 take longer, 98.7 -> 105.6 us.
-        if (!kInt && sr && !alpha.cells && ogrid < 4 * sm_count) ogrid = grid_for(sm_count, ngroups, 4);
+        const int ogrid = opt_grid(alpha, sm_count, ngroups, kInt, sr, rht, false, kOptIters);
         if (!(o.flags & ABS_F_INDEX64) && ngroups < (int64_t)0x7FFFFFFF - (int64_t)ogrid * othreads) {
             const bool a32 = (reinterpret_cast<uintptr_t>(in) & 31u) == 0;
             cudaError_t e;
@@ -692,7 +703,7 @@ abs_status_t abs_quantize_dequantize(abs_fmt_t fmt, const void* in_bf16, int64_t
         cudaError_t e = cudaSuccess;
         const bool has_int = fmt == ABS_FMT_IF4;
         const int esrc = src.cells ? kOnePass : kGiven, ethreads = opt_threads(has_int, sr, esrc);
-        int egrid = quantize_grid(src, st->sm_count, ngroups, opt_blocks_per_sm(has_int, sr, rht, esrc), (rht || sr) ? kOptIters : kFastIters, ethreads);
+        int egrid = opt_grid(src, st->sm_count, ngroups, has_int, sr, rht, true, (rht || sr) ? kOptIters : kFastIters);
         if (ngroups >= (int64_t)0x7FFFFFFF - (int64_t)egrid * ethreads) egrid = (int)((int64_t)grid * kThreads / ethreads);      // the stride that the check above has seen
 #define ABS_LAUNCH_E2(I, R, S)                                                                                      \
         e = launch_any(src.cells ? kCooperative : kApart, src.cells ? quantize4_opt_kernel<I, R, S, kOnePass, true>                   \
