@@ -468,7 +468,11 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
                     if (lane == 0) mbar_arrive(acc_empty0 + 8 * buf);    // the MMAs of the next chunk or tile may start
                 }
                 if (!all_tiles) break;
-                if (own_row_valid) store_columns<OUT_BF16, kCols / 16>(c_out, first, v, scale, out_aligned32, true, true, held, next_alpha != nullptr, out_max);
+                if (own_row_valid) {
+#pragma unroll
+                    for (int q = 0; q < kCols / 16; ++q)
+                        store_columns16<OUT_BF16, -1>(c_out, first + 16 * q, v + 16 * q, scale, out_aligned32, q == 0, q == kCols / 16 - 1, held, next_alpha != nullptr, out_max);
+                }
             }
         } else {
             // A warp owns the accumulator lanes (rows of the tile) 32 (w % 4) .. 32 (w % 4) + 31.
@@ -496,8 +500,16 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
                     float v[32];
 #pragma unroll
                     for (int jj = 0; jj < 32; ++jj) v[jj] = __uint_as_float(r0[jj]);
-                    if (own_row_valid)
-                        store_columns<OUT_BF16, 2>(c_out, first + chunk * 32, v, scale, out_aligned32, chunk == 0, chunk == kTileN / 32 - 1, held, next_alpha != nullptr, out_max);
+                    const auto store = [&](auto whole) __attribute__((always_inline)) {
+#pragma unroll
+                        for (int q = 0; q < 2; ++q)
+                            store_columns16<OUT_BF16, decltype(whole)::value>(c_out, first + chunk * 32 + 16 * q, v + 16 * q, scale, false, chunk + q == 0,
+                                                                              chunk == kTileN / 32 - 1 && q == 1, held, next_alpha != nullptr, out_max);
+                    };
+                    if (own_row_valid) {
+                        if (out_aligned32) store(std::integral_constant<int, 1>{});
+                        else store(std::integral_constant<int, 0>{});
+                    }
                 }
             }
         }
