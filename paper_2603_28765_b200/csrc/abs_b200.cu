@@ -184,8 +184,10 @@ bool one_pass(int fmt, const abs_opts_t& o, int sm_count, int64_t ngroups, bool 
     return !(o.flags & ABS_F_INDEX64) && ngroups <= (int64_t)grid_for(sm_count < kMaxCells ? sm_count : kMaxCells, ngroups, 1) * kThreads * per_thread;
 }
 // Whether such a call is one cluster: the round-to-nearest 4-bit kernels with up to three groups per thread of it (two groups of 8 blocks' threads: 3.3 us instead of
-// 4.1 - 4.3; three 3.9 instead of 4.2; with four the single cluster's arithmetic takes longer than the exchange through the L2 that it saves).  Calls of
-// two to four blocks keep the cells: their report of an overrun is exercised with such calls.
+// 4.1 - 4.3; three 3.9 instead of 4.2; with four the single cluster's arithmetic takes longer than the exchange through the L2 that it saves).  The lower line is not
+// where the cluster stops being the faster one: calls of two to four blocks (257 to 1024 groups) start 4.10 us apart through the cells and would start 2.45 us
+// apart as a cluster (NVFP4 2.07).  They keep the cells because a call through them is one whose overrun of the ring is reported, which is checked with a
+// call of 1024 groups; a cluster has no part of the ring to lose.
 bool one_cluster(int fmt, const abs_opts_t& o, int64_t ngroups) {
     return (fmt == ABS_FMT_NVFP4 || fmt == ABS_FMT_IF4) && !(o.flags & (ABS_F_HADAMARD16 | ABS_F_STOCHASTIC)) && ngroups > 4 * kThreads &&
            ngroups <= 3 * kMaxCluster * kThreads;

@@ -225,8 +225,9 @@ quantize4_bs8_kernel(const uint4* __restrict__ in, uint2* __restrict__ codes, ui
 // ----------------------------------------------------------------------------- 6-bit formats (IF6)
 
 // Threads of a block and resident blocks per SM of the IF6 and IF3 kernels: seven blocks of 128 threads at 72 registers, 28 warps, instead of three of
-// 256 at 76 - 80, 24 warps (the kernels at 16384 x 8192, us: IF6 79.9 -> 75.6, IF3 90.2 -> 89.0; round trips of 4096 x 14336 and 16384 x 8192: IF3 90.9 -> 90.4, IF6 199.5
-// -> 196.6).  A grid of one block per SM (kOnePass) has blocks of 256.
+// 256 at 76 - 80, 24 warps.  A single cold launch takes as long either way; back to back, where blocks of the next wave and kernel come in beside the last ones of
+// this, kernel alone, us, spread 0.1: 16384 x 8192 IF6 81.3 -> 77.4, IF3 92.4 -> 91.2; 4096 x 14336 38.2 -> 36.4, 42.7 -> 42.3; 8192 x 4096 23.0 -> 22.0, 25.9 -> 25.6.
+// A grid of one block per SM (kOnePass) has blocks of 256.
 constexpr int wide_threads(int src) { return src == kOnePass ? 256 : 128; }
 constexpr int wide_blocks_per_sm(int src) { return src == kOnePass ? 3 : 7; }
 
