@@ -71,8 +71,16 @@ struct Opts {
 // released when the call returns, or an output that is dropped, must not be handed out again while the kernels are pending), and
 // fills run there too, before the kernels.
 class Work {
+    // Whether the call's outputs are allocated through the dispatcher, which is a third of the 0.9 us that at::empty takes (a quantize call allocates three tensors): where
+    // somebody listens there (dispatch modes, fake tensors, transforms and tracers put a key of their own into the thread's set; profilers
+    // record the operator), or deterministic algorithms are asked for, with which at::empty fills what it allocates.
+    static bool dispatched() {
+        const c10::DispatchKeySet keys = c10::impl::tls_local_dispatch_key_set().included_;
+        return !(keys - c10::default_included_set).empty() || at::hasCallbacks() || at::globalContext().deterministicAlgorithms();
+    }
     c10::Device device;
     bool other = false;                  // not the current stream
+    const bool dispatch = dispatched();
 
     c10::cuda::CUDAStream torch_stream() const { return c10::cuda::getStreamFromExternal((cudaStream_t)stream, device.index()); }
 
@@ -89,16 +97,9 @@ class Work {
         if (!stream && PyErr_Occurred()) throw Raised();
         other = stream != current;
     }
-    // Whether outputs are allocated through the dispatcher, which is a third of the 0.9 us that at::empty takes (a quantize call allocates three tensors): where
-    // somebody listens there (dispatch modes, fake tensors, transforms and tracers put a key of their own into the thread's set; profilers
-    // record the operator), or deterministic algorithms are asked for, with which at::empty fills what it allocates.
-    static bool dispatched() {
-        const c10::DispatchKeySet keys = c10::impl::tls_local_dispatch_key_set().included_;
-        return !(keys - c10::default_included_set).empty() || at::hasCallbacks() || at::globalContext().deterministicAlgorithms();
-    }
     at::Tensor empty(at::IntArrayRef sizes, at::ScalarType type) const {
-        at::Tensor t = dispatched() ? at::empty(sizes, at::TensorOptions().dtype(type).device(device))
-                                    : at::Tensor(at::detail::empty_cuda(sizes, type, device, std::nullopt));
+        at::Tensor t = dispatch ? at::empty(sizes, at::TensorOptions().dtype(type).device(device))
+                                : at::Tensor(at::detail::empty_cuda(sizes, type, device, std::nullopt));
         if (other && t.numel() > 0) c10::cuda::CUDACachingAllocator::recordStream(t.storage().data_ptr(), torch_stream());
         return t;
     }
