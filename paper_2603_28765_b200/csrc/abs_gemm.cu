@@ -470,8 +470,10 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
                 if (!all_tiles) break;
                 if (own_row_valid) {
 #pragma unroll
-                    for (int q = 0; q < kCols / 16; ++q)
-                        store_columns16<OUT_BF16, -1>(c_out, first + 16 * q, v + 16 * q, scale, out_aligned32, q == 0, q == kCols / 16 - 1, held, next_alpha != nullptr, out_max);
+                    for (int q = 0; q < kCols / 16; ++q) {
+                        if (out_aligned32) store_columns16<OUT_BF16, true>(c_out, first + 16 * q, v + 16 * q, scale, false, false, held, next_alpha != nullptr, out_max);
+                        else store_columns16<OUT_BF16, false>(c_out, first + 16 * q, v + 16 * q, scale, q == 0, q == kCols / 16 - 1, held, next_alpha != nullptr, out_max);
+                    }
                 }
             }
         } else {
@@ -503,12 +505,12 @@ if4_gemm_kernel(const __grid_constant__ GemmMaps<PLANES> maps, const float* __re
                     const auto store = [&](auto whole) __attribute__((always_inline)) {
 #pragma unroll
                         for (int q = 0; q < 2; ++q)
-                            store_columns16<OUT_BF16, decltype(whole)::value>(c_out, first + chunk * 32 + 16 * q, v + 16 * q, scale, false, chunk + q == 0,
+                            store_columns16<OUT_BF16, decltype(whole)::value>(c_out, first + chunk * 32 + 16 * q, v + 16 * q, scale, chunk + q == 0,
                                                                               chunk == kTileN / 32 - 1 && q == 1, held, next_alpha != nullptr, out_max);
                     };
                     if (own_row_valid) {
-                        if (out_aligned32) store(std::integral_constant<int, 1>{});
-                        else store(std::integral_constant<int, 0>{});
+                        if (out_aligned32) store(std::true_type{});
+                        else store(std::false_type{});
                     }
                 }
             }

@@ -269,13 +269,13 @@ nvfp4_pair_kernel(const __grid_constant__ GemmMaps<1> maps, const float* __restr
                         if (own_row_valid) {                               // the last row block may be partial
 #pragma unroll
                             for (int q = 0; q < 2; ++q)
-                                store_columns16<OUT_BF16, decltype(whole)::value>(c_out, first + chunk * 32 + 16 * q, v + 16 * q, scale, false, chunk + q == 0,
+                                store_columns16<OUT_BF16, decltype(whole)::value>(c_out, first + chunk * 32 + 16 * q, v + 16 * q, scale, chunk + q == 0,
                                                                                   chunk == kTileN / 32 - 1 && q == 1, held, next_alpha != nullptr, out_max);
                         }
                     }
                 };
-                if (out_aligned32) columns(std::integral_constant<int, 1>{});
-                else columns(std::integral_constant<int, 0>{});
+                if (out_aligned32) columns(std::true_type{});
+                else columns(std::false_type{});
                 buf = buf + 1 == kPairAccBufs ? 0u : buf + 1;
             }
         }

@@ -163,15 +163,14 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
 // are whole sectors long) the second half of 32 bytes is held back for the first of the next, and only the ends of the run are half sectors.  (As
 // two 16-byte stores each, whose sectors the next one completes, FP32 products into such a C took up to 1.4 times as long: NVFP4 4096 x 4096 x 512 20.2 us by lines
 // turned through shared memory, 28.5 so, 18.3 held back; 2048 x 4096 x 4096 bf16 27.3, 26.2, 24.0.)
-// WHOLE: 1 where C is known to be 32-byte aligned, 0 where it is known not to be, -1 where `whole` says, without a branch.  Which form costs aligned outputs nothing
-// differs: IF4 with -1 (a branch around its 64 columns 0.7 % more in FP32 at 4096^3, one per 32 bytes 2.5 % at 4096 x 4096 x 512), NVFP4 with a copy
-// for either (-1: 2 % more in bf16 at 1000 x 4096 x 1024).
+// WHOLE: whether C is 32-byte aligned.  How far the choice lies from the stores is a matter of what it costs aligned outputs: IF4 makes it per 16 columns (around all 64 of
+// a thread FP32 products take 0.5 - 1 % longer, by selects 0.5 - 0.8 %, per 32 bytes 2.5 % at 4096 x 4096 x 512; so, 0.8 % there and nothing elsewhere), NVFP4 per
+// 32 columns, its pairs of tiles per tile (by selects 2 % more in bf16 at 1000 x 4096 x 1024).
 // keep_max: the larger of out_max and the bf16 magnitudes written, per half word.
-template <bool OUT_BF16, int WHOLE>
-__device__ __forceinline__ void store_columns16(void* c_out, size_t at, const float* v, float scale, bool whole, bool first, bool last, uint4& held,
-                                                bool keep_max, uint32_t& out_max) {
+template <bool OUT_BF16, bool WHOLE>
+__device__ __forceinline__ void store_columns16(void* c_out, size_t at, const float* v, float scale, bool first, bool last, uint4& held, bool keep_max,
+                                                uint32_t& out_max) {
     constexpr int kPieces = OUT_BF16 ? 1 : 2;
-    if constexpr (WHOLE >= 0) whole = WHOLE;
 #pragma unroll
     for (int q = 0; q < kPieces; ++q) {
         uint32_t o[8];
@@ -185,12 +184,18 @@ __device__ __forceinline__ void store_columns16(void* c_out, size_t at, const fl
             }
         }
         uint8_t* const to = reinterpret_cast<uint8_t*>(c_out) + at * (OUT_BF16 ? 2 : 4) + 32 * q;
-        const uint32_t sector[8] = {whole ? o[0] : held.x, whole ? o[1] : held.y, whole ? o[2] : held.z, whole ? o[3] : held.w,
-                                    whole ? o[4] : o[0],   whole ? o[5] : o[1],   whole ? o[6] : o[2],   whole ? o[7] : o[3]};
-        if (first && q == 0 && !whole) *reinterpret_cast<uint4*>(to) = make_uint4(o[0], o[1], o[2], o[3]);
-        else store32B<true>(whole ? to : to - 16, sector);
-        held = make_uint4(o[4], o[5], o[6], o[7]);
-        if (last && q == kPieces - 1 && !whole) *reinterpret_cast<uint4*>(to + 16) = held;
+        if constexpr (WHOLE) {
+            store32B<true>(to, o);
+        } else {
+            if (first && q == 0) {
+                *reinterpret_cast<uint4*>(to) = make_uint4(o[0], o[1], o[2], o[3]);
+            } else {
+                const uint32_t sector[8] = {held.x, held.y, held.z, held.w, o[0], o[1], o[2], o[3]};
+                store32B<true>(to - 16, sector);
+            }
+            held = make_uint4(o[4], o[5], o[6], o[7]);
+            if (last && q == kPieces - 1) *reinterpret_cast<uint4*>(to + 16) = held;
+        }
     }
 }
 __device__ __forceinline__ void tmem_load_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
