@@ -148,7 +148,7 @@ __device__ __forceinline__ void encode_body4_sr(const float (&x)[16], const uint
     }
 }
 
-// Threads of a block, and resident blocks per SM the kernel is compiled and launched for.  IF4 with stochastic rounding takes 93 registers: five blocks
+// Threads of a block, and resident blocks per SM the kernel is compiled for (opt_grid says what it is launched for).  IF4 with stochastic rounding takes 91 to 94 registers: five blocks
 // of 128 threads (20 warps) instead of two of 256 (8192 x 8192, us: 69.8 -> 66.1, with Hadamard 76.0 -> 73.9, emulation 82.1 -> 78.0; NVFP4 46.8 / 47.2, so it
 // stays); the Hadamard-only kernels run best with three blocks of 256, the plain round-to-nearest one (used by the emulation pass only) with four.  A grid
 // of one block per SM (kOnePass) has blocks of 256.

@@ -163,9 +163,9 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
 // are whole sectors long) the second half of 32 bytes is held back for the first of the next, and only the ends of the run are half sectors.  (As
 // two 16-byte stores each, whose sectors the next one completes, FP32 products into such a C took up to 1.4 times as long: NVFP4 4096 x 4096 x 512 20.2 us by lines
 // turned through shared memory, 28.5 so, 18.3 held back; 2048 x 4096 x 4096 bf16 27.3, 26.2, 24.0.)
-// WHOLE: whether C is 32-byte aligned.  How far the choice lies from the stores is a matter of what it costs aligned outputs: IF4 makes it per 16 columns (around all 64 of
-// a thread FP32 products take 0.5 - 1 % longer, by selects 0.5 - 0.8 %, per 32 bytes 2.5 % at 4096 x 4096 x 512; so, 0.8 % there and nothing elsewhere), NVFP4 per
-// 32 columns, its pairs of tiles per tile (by selects 2 % more in bf16 at 1000 x 4096 x 1024).
+// WHOLE: whether C is 32-byte aligned.  Where the choice lies follows from what it costs aligned outputs.  IF4, FP32: per 16 columns nothing (0.8 % at
+// 4096 x 4096 x 512), around all 64 of a thread 0.5 - 1 %, by selects instead of a branch 0.1 - 0.8 %, per 32 bytes 2.5 % at 4096 x 4096 x 512.  NVFP4: per 32 columns, and in the
+// pairs of tiles per tile, nothing; by selects 2 % in bf16 at 1000 x 4096 x 1024.
 // keep_max: the larger of out_max and the bf16 magnitudes written, per half word.
 template <bool OUT_BF16, bool WHOLE>
 __device__ __forceinline__ void store_columns16(void* c_out, size_t at, const float* v, float scale, bool first, bool last, uint4& held, bool keep_max,
